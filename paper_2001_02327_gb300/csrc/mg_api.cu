@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <map>
 #include <new>
 #include <string>
 #include <vector>
@@ -49,6 +50,8 @@ struct LevelData {
     int Lc[2] = {-1, -1};          // first level handled by the cluster kernel (-1: none)
     int Llim[2] = {0, 0};          // the level-size limit that chose it
     MgBottom bt[2];
+    int Lslab[2] = {-1, -1};       // first level handled by the slab kernel (-1: none)
+    MgSlabPlan slab;               // its plan, for the precision of the V-cycles
     // device image of the one-block kernel's plan for the precision the
     // V-cycles run in, sized for the largest bottom the level admits
     void *bplan = nullptr;
@@ -140,6 +143,7 @@ void plan_tiles(LevelData &ld, int dim, int nu_pre, int nu_post)
 // times the choices; the batched kernels (MG_BATCHED=1) run plain levels
 // only.  Changing the layout clears the level's FP32 arrays (their ghost
 // layer must read zero in either layout).
+int first_fused(const LevelData &ld, bool fp32);
 constexpr int kTileSplit = 1 << 16;   // mg_tuning / tuning-cache code of a split level
 constexpr int kSplitMinN = 192;
 
@@ -147,7 +151,7 @@ int split_default(const LevelData &ld)
 {
     if (ld.Lc[1] >= 0 || ld.frozen)   // the cluster kernel runs plain levels
         return 0;
-    const int Ls = ld.Ls[1];
+    const int Ls = first_fused(ld, true);
     if (const char *v = std::getenv("MG_SPLIT"))
         if (*v)
             return std::max(0, std::min(std::atoi(v), Ls));
@@ -163,7 +167,7 @@ int split_default(const LevelData &ld)
 
 cudaError_t plan_split(LevelData &ld, int dim, int S, cudaStream_t s)
 {
-    S = std::max(0, std::min(S, ld.Ls[1]));
+    S = std::max(0, std::min(S, first_fused(ld, true)));
     if (ld.Lc[1] >= 0)
         S = 0;
     const bool changed = S != ld.nsplit;
@@ -308,6 +312,31 @@ void plan_cluster(LevelData &ld, int dim, int csize, const mg_options &o, int li
     }
 }
 
+// The slab kernel (mg_slab.cu) takes the multigrid levels from the first of at
+// most slab_limit cells per edge down, unless the environment asks for one of
+// the other plans of those levels; of them, those of more than slab_cut cells
+// per edge are split over its CTAs.  The limits are the largest levels whose
+// V-cycle is shorter there than as launches of the whole GPU (3D 34^3: 31 us
+// FP32 and 48 us FP64 against 52 and 70 us) and that fit its shared memory.
+int slab_limit(int dim, bool) { return dim == 3 ? 34 : 160; }
+int slab_cut(int dim) { return dim == 3 ? 9 : 24; }
+
+bool slab_wanted(bool fp32)
+{
+    for (const char *name : {fp32 ? "MG_BOTTOM_N32" : "MG_BOTTOM_N64", fp32 ? "MG_CLUSTER_N32" : "MG_CLUSTER_N64",
+                             "MG_WAVE", "MG_WAVE_PLAN", "MG_TB_TILE"})
+        if (const char *v = std::getenv(name))
+            if (*v)
+                return false;
+    return true;
+}
+
+// first level that the per-level launches leave to the slab or one-block kernel
+int first_fused(const LevelData &ld, bool fp32)
+{
+    return ld.Lslab[fp32 ? 1 : 0] >= 0 ? ld.Lslab[fp32 ? 1 : 0] : ld.Ls[fp32 ? 1 : 0];
+}
+
 // Sec. 2.2: N^L = round(M / 2^L), halves rounded up, until N^L = 1.
 int level_sizes(int M, int *N, int cap)
 {
@@ -403,6 +432,8 @@ struct mg_hierarchy {
     // solve graph
     bool use_graph = true;          // MG_SOLVE_GRAPH=0: host-driven loop (for kernel profilers)
     int csize = 0;                  // CTAs per cluster of the cluster kernel (0: unavailable)
+    int ssize = 0;                  // the same of the slab kernel
+    std::map<std::pair<int, int>, int *> slab_img;   // its plan images by (M, first level)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     std::vector<char> graph_sig;
@@ -682,6 +713,61 @@ cudaError_t refresh_bottom_plan(mg_hierarchy *h, LevelData &ld)
     return e;
 }
 
+// The slab kernel's plan of a level, for the precision of the V-cycles; its
+// image is shared by all levels of the handle with the same sizes and built
+// at creation or tuning (synchronous).
+cudaError_t plan_slab(mg_hierarchy *h, LevelData &ld, bool on)
+{
+    const bool fp32 = h->opt.precision == MG_MIXED;
+    const int w = fp32 ? 1 : 0, lim = slab_limit(h->dim, fp32);
+    ld.Lslab[w] = -1;
+    // mixed batches: graph branches of several hierarchies share the SMs, which
+    // small launches of all of them fill better than clusters of 16 (batch of 32
+    // uneven hierarchies: 40 ms against 47 ms)
+    if (!on || h->ssize <= 0 || !slab_wanted(fp32) || (fp32 && h->batch > 1))
+        return cudaSuccess;
+    for (int L = 0; L + 1 < ld.nmg; L++) {
+        if (ld.g[L].N > lim)
+            continue;
+        MgSlabPlan &p = ld.slab;
+        if (!mg_slab_layout(h->dim, fp32, h->ssize, &ld.g[L], ld.nmg - L, slab_cut(h->dim), h->opt.nu_pre,
+                            h->opt.nu_post, p))
+            continue;
+        int *&img = h->slab_img[{ld.M, L}];
+        const size_t ib = align256(mg_slab_image_bytes(p)), nd = (size_t)p.dn * p.dn;
+        if (!img) {
+            // the dense matrix behind the plan words
+            const int Ld = L + p.nlev - 1;
+            std::vector<double> mat(nd);
+            mg_slab_dense(h->dim, &ld.g[Ld], ld.nmg - Ld, h->opt.nu_pre, h->opt.nu_post, mat.data());
+            std::vector<float> m32(nd);
+            std::vector<long long> m64(nd);
+            for (size_t i = 0; i < nd; i++) {
+                m32[i] = (float)mat[i];
+                m64[i] = std::llrint(std::ldexp(mat[i], 60));
+            }
+            cudaError_t e = cudaMalloc((void **)&img, ib + nd * (fp32 ? 4 : 8));
+            if (e == cudaSuccess)
+                e = mg_launch_slab_plan(h->dim, p, img, h->stream);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync((char *)img + ib, fp32 ? (const void *)m32.data() : (const void *)m64.data(),
+                                    nd * (fp32 ? 4 : 8), cudaMemcpyHostToDevice, h->stream);
+            if (e == cudaSuccess)
+                e = cudaStreamSynchronize(h->stream);
+            if (e)
+                return e;
+        }
+        p.dense = (const char *)img + ib;
+        p.img = img;
+        p.zero_start = L > 0;
+        p.phi = fp32 ? (void *)ld.phi32[L] : (void *)ld.phi[L];
+        p.f = fp32 ? (const void *)ld.f32[L] : (const void *)ld.f[L];
+        ld.Lslab[w] = L;
+        break;
+    }
+    return cudaSuccess;
+}
+
 // the V-cycle of Sec. 2.3 (steps 2-13) on the arrays of one refinement level,
 // `ncyc` times; the levels from Lc down run in the cluster kernel (when
 // Lc < Ls), those from Ls down in the one-block kernel
@@ -700,7 +786,8 @@ cudaError_t vcycle(mg_hierarchy *h, const LevelData &ld, bool fp32, cudaStream_t
     const MgBottom &bt = ld.bt[fp32 ? 1 : 0];
     const int Lc = ld.Lc[fp32 ? 1 : 0];
     const bool clu = Lc >= 0 && h->csize > 0;
-    const int Lstop = clu ? Lc : Ls;
+    const int Lslab = ld.Lslab[fp32 ? 1 : 0];
+    const int Lstop = Lslab >= 0 ? Lslab : clu ? Lc : Ls;
     auto bottom = [&]() {
         return timed(h, KK_BOTTOM, 3.0 * w * cells_d(ld.g[Ls].E, dim),
                      [&] { return mg_launch_bottom(dim, fp32, P(Ls), F(Ls), bt, o.nu_pre, o.nu_post, s); });
@@ -720,8 +807,33 @@ cudaError_t vcycle(mg_hierarchy *h, const LevelData &ld, bool fp32, cudaStream_t
             by += w * cells_d(ld.g[Lc + q].N, dim) * (4.0 * (o.nu_pre + o.nu_post) + 5.0);
         return timed(h, KK_CLUSTER, by * cycles, [&] { return mg_launch_cluster(fp32, p, h->csize, smem, s); });
     };
+    auto slab = [&](int cycles, bool count) {
+        MgSlabPlan p = ld.slab;
+        p.cycles = cycles;
+        if (count) {
+            p.ctl = ctl;
+            p.hi = hi;
+        }
+        // one launch that runs every kind of phase: it counts under each, its
+        // time and bytes under the bottom's
+        if (h->prof.on)
+            for (int kind : {KK_SMOOTH, KK_RESTRICT, KK_PROLONG})
+                h->prof.launches[kind]++;
+        return timed(h, KK_BOTTOM, 3.0 * w * cells_d(ld.g[Lslab].E, dim) * cycles,
+                     [&] { return mg_launch_slab(dim, fp32, p, s); });
+    };
     cudaError_t e;
     if (Lstop == 0) {                                                                     // whole cycle
+        if (Lslab >= 0) {
+            if (ctl && counted)
+                *counted = true;
+            if (!h->prof.on)
+                return slab(ncyc, ctl && counted);
+            for (int c = 0; c < ncyc; c++)   // per-kernel timing: one launch per V-cycle
+                if ((e = slab(1, false)))
+                    return e;
+            return cudaSuccess;
+        }
         if (clu)
             return cluster(ncyc);
         for (int c = 0; c < ncyc; c++)
@@ -779,7 +891,7 @@ cudaError_t vcycle(mg_hierarchy *h, const LevelData &ld, bool fp32, cudaStream_t
             return e;
         red_done = fuse;
     }
-    if ((e = clu ? cluster(1) : bottom()))                                                // steps 6-11, L >= Lstop
+    if ((e = Lslab >= 0 ? slab(1, false) : clu ? cluster(1) : bottom()))                  // steps 6-11, L >= Lstop
         return e;
     // ascent: prolongation + correction, then nu_post sweeps (steps 10-11)
     for (int L = Lstop; L > 0; L--) {
@@ -1745,6 +1857,7 @@ mg_status solve_graph(mg_hierarchy *h, mg_level_stats *stats)
 // correction arrays (scratch: rewritten by the next defect), so tuning does
 // not disturb a solve.
 // --------------------------------------------------------------------------
+constexpr int kBottomSlab = 1 << 16;   // TuneEntry::bottom_n: the slab kernel instead of the one-block kernel
 struct TuneEntry {
     int dim, n, nu_pre, nu_post, bottom_n;
     int tile[MG_MAX_MG];
@@ -1833,11 +1946,15 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
     te.nu_pre = o.nu_pre;
     te.nu_post = o.nu_post;
     // 1. the bottom limit, with the default tiles
-    const int nbs[3] = {4, 8, 17};
+    const int nbs[4] = {4, 8, 17, kBottomSlab};
     float best = 1e30f;
     int bestnb = 8;
     for (int nb : nbs) {
-        plan_bottom(ld, dim, nb);
+        if ((err = plan_slab(h, ld, nb == kBottomSlab)))
+            return false;
+        if (nb == kBottomSlab && ld.Lslab[1] < 0)
+            continue;
+        plan_bottom(ld, dim, nb == kBottomSlab ? 8 : nb);
         if ((err = refresh_bottom_plan(h, ld)))
             return false;
         plan_tiles(ld, dim, o.nu_pre, o.nu_post);
@@ -1852,7 +1969,9 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
             bestnb = nb;
         }
     }
-    plan_bottom(ld, dim, bestnb);
+    if ((err = plan_slab(h, ld, bestnb == kBottomSlab)))
+        return false;
+    plan_bottom(ld, dim, bestnb == kBottomSlab ? 8 : bestnb);
     if ((err = refresh_bottom_plan(h, ld)))
         return false;
     plan_cluster(ld, h->dim, h->csize, h->opt);
@@ -1860,7 +1979,7 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
         return false;
     te.bottom_n = bestnb;
     // 2. per level above the bottom: the tile of its pre/post pair
-    const int Ls = ld.Ls[1];
+    const int Ls = first_fused(ld, true);
     for (int L = 0; L < MG_MAX_MG; L++)
         te.tile[L] = 0;
     for (int L = 0; L < Ls; L++) {
@@ -1960,13 +2079,16 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
 
 cudaError_t apply_entry(mg_hierarchy *h, LevelData &ld, const TuneEntry &te)
 {
-    plan_bottom(ld, h->dim, te.bottom_n);
-    cudaError_t e = refresh_bottom_plan(h, ld);
+    cudaError_t e = plan_slab(h, ld, te.bottom_n == kBottomSlab);
+    plan_bottom(ld, h->dim, te.bottom_n == kBottomSlab ? 8 : te.bottom_n);
+    if (!e)
+        e = refresh_bottom_plan(h, ld);
+    const int Ls = first_fused(ld, true);
     int S = 0;
-    while (S < ld.Ls[1] && te.tile[S] == kTileSplit)
+    while (S < Ls && te.tile[S] == kTileSplit)
         S++;
     for (int L = 0; L < ld.nmg; L++)
-        ld.tile[L] = L < ld.Ls[1] && te.tile[L] != kTileSplit ? te.tile[L] : 0;
+        ld.tile[L] = L < Ls && te.tile[L] != kTileSplit ? te.tile[L] : 0;
     plan_cluster(ld, h->dim, h->csize, h->opt);
     if (!e)
         e = plan_split(ld, h->dim, S, h->stream);
@@ -2198,6 +2320,8 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
     if (e == cudaSuccess)
         h->csize = mg_cluster_prepare();
     if (e == cudaSuccess)
+        h->ssize = mg_slab_prepare();
+    if (e == cudaSuccess)
         e = mg_launch_zero(h->arena, bytes, h->stream);
     if (e == cudaSuccess)   // the table copies below do not run on the caller's stream
         e = cudaStreamSynchronize(h->stream);
@@ -2223,6 +2347,8 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
                 e = refresh_bottom_plan(h, ld);
             plan_tiles(ld, dim, o.nu_pre, o.nu_post);
             plan_cluster(ld, h->dim, h->csize, h->opt);
+            if (e == cudaSuccess)
+                e = plan_slab(h, ld, true);
             if (e == cudaSuccess && o.precision == MG_MIXED)
                 e = plan_split(ld, dim, split_default(ld), h->stream);
         }
@@ -2239,6 +2365,8 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
         e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        for (auto &im : h->slab_img)
+            cudaFree(im.second);
         cudaFreeHost(h->hscal);
         cudaFreeHost(h->hctl);
         cudaFree(h->arena);
@@ -2621,7 +2749,7 @@ int mg_tuning(const mg_hierarchy *h, int b, int level, int *tiles, int cap)
     const LevelData &ld = h->lev[b][level];
     for (int L = 0; L < cap && L < ld.nmg; L++)
         tiles[L] = L < ld.nsplit ? kTileSplit : ld.tile[L];
-    return ld.g[ld.Ls[1]].N;
+    return ld.g[first_fused(ld, true)].N;
 }
 
 mg_status mg_destroy(mg_hierarchy *h)
@@ -2635,6 +2763,8 @@ mg_status mg_destroy(mg_hierarchy *h)
     for (cudaEvent_t e : h->prof.pool)
         cudaEventDestroy(e);
     destroy_graph(h);
+    for (auto &im : h->slab_img)
+        cudaFree(im.second);
     if (h->persist_mem)
         cudaFree(h->persist_mem);
     if (h->cap_p)

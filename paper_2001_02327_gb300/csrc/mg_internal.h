@@ -129,6 +129,51 @@ struct MgClusterPlan {
     MgBottom bt;
 };
 
+// The levels of a V-cycle from a size limit down in one thread-block cluster
+// (mg_slab.cu): levels 0..nlev-1 of the plan, the first nclu of them split by
+// planes of the outermost axis over the cluster's CTAs, the others in CTA 0.
+// FP32, or FP64 arrays computed in 64-bit fixed point.
+#define MG_SLAB_THREADS 512
+#define MG_SLAB_MAXLEV 12
+#define MG_SLAB_MAXK 6                 // pairs of cells per thread and level
+#define MG_SLAB_CTRL (72 * MG_SLAB_MAXLEV)   // control words in shared memory
+#define MG_SLAB_SMEM_MAX (226 * 1024)
+struct MgSolveCtl;
+struct MgSlabPlan {
+    int nlev, nclu, csize, lgc;    // lgc: log2 of csize
+    int nu_pre, nu_post, cycles;
+    int zero_start;                // the first level's potential is zero: not read
+    MgGeom g[MG_SLAB_MAXLEV];
+    int po[MG_SLAB_MAXLEV];        // planes per CTA (without its copies of the neighbours' planes)
+    int off[MG_SLAB_MAXLEV];       // words: the level's potential (two colours)
+    int K[MG_SLAB_MAXLEV];         // pairs of cells per thread
+    int slot[MG_SLAB_MAXLEV];      // first slot of the level's pairs
+    int tb[MG_SLAB_MAXLEV];        // fixed point: bits of the largest right-hand side a level starts from
+    int top[MG_SLAB_MAXLEV];       // ... and of the largest correction added to it
+    int KG[MG_SLAB_MAXLEV];        // ghost cells of the staged planes per thread
+    int bcd[MG_SLAB_MAXLEV], ghost[MG_SLAB_MAXLEV];   // their words in the plan image
+    int cri[MG_SLAB_MAXLEV];       // fixed point: right-ghost factor, floor and fraction * 2^62
+    long long crf[MG_SLAB_MAXLEV];
+    int nslot, nimg, words;        // slots; words per thread in shared memory, in the image
+    int dn, dmat, dvec, dpos;      // cells of the last level; its matrix and vectors (words), cell positions (plan word)
+    int scratch, fs, tabs, ctrl, zero16;   // words; 16-byte units zeroed at the start
+    size_t smem;                   // dynamic shared memory per CTA
+    const int *img;                // plan image (mg_launch_slab_plan)
+    const void *dense;             // matrix of the last level and those below, column by column, for h^2 f: FP32 or
+                                   // fixed point * 2^60
+    void *phi;                     // the first level's global arrays
+    const void *f;
+    MgSolveCtl *ctl;               // not NULL: the launch also counts one V-cycle of a nested loop (condition hi)
+    cudaGraphConditionalHandle hi;
+};
+int mg_slab_prepare();             // CTAs per cluster (0: unavailable); once per device before the first launch
+bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, int cut, int nu_pre, int nu_post,
+                    MgSlabPlan &p);
+size_t mg_slab_image_bytes(const MgSlabPlan &p);
+void mg_slab_dense(int dim, const MgGeom *g, int nlev, int nu_pre, int nu_post, double *mat);
+cudaError_t mg_launch_slab_plan(int dim, const MgSlabPlan &p, int *img, cudaStream_t s);
+cudaError_t mg_launch_slab(int dim, bool fp32, const MgSlabPlan &p, cudaStream_t s);
+
 size_t mg_bottom_smem(int dim, bool fp32, const MgBottom &bt);
 size_t mg_bottom_plan_bytes(int dim, bool fp32, const MgBottom &bt);
 // writes the per-cell plan of bt's levels to `img` (mg_bottom_plan_bytes)

@@ -1,0 +1,1507 @@
+// mg_slab.cu -- the coarse part of the V-cycle (Sec. 2.3 steps 2-13 on the
+// multigrid levels from a size limit down) in one launch of one thread-block
+// cluster.  Every array of those levels lives on chip: the potentials in the
+// shared memory of the cluster's CTAs (the larger levels as slabs of planes
+// along the outermost axis, z in 3D and y in 2D, the smaller ones whole in CTA
+// 0), the right-hand sides and coefficients with the threads that use them.
+//
+// What bounds these levels is latency, not arithmetic or bandwidth: a level of
+// 33^3 cells has 18k updates per colour, less than a microsecond of work for
+// the whole GPU, but one launch per phase costs about 2.2 us (a graph node with
+// programmatic dependent launch about 0.9 us, the loads' round trip to L2 the
+// rest).  So everything here removes steps from the dependent chain of a phase:
+//   - a thread owns fixed pairs of neighbouring cells (2x+1, 2x+2) of a row on
+//     every level; where they are, which boundary class they have and where
+//     their children and parents are comes packed from a plan image in global
+//     memory, written once per level configuration and copied to shared memory
+//     before the kernel waits for its predecessor, so no phase divides;
+//   - each CTA keeps copies of its neighbours' boundary planes, and the owner
+//     pushes every new value into the copies by distributed shared memory
+//     stores, which the phase's barrier completes: sweeps load locally only;
+//   - the first red half-sweep on a level (whose correction starts from zero)
+//     is done with the restriction into it, the potential that a finer level
+//     interpolates is copied to where it reads it right after the level's last
+//     sweep, and the pair sums of the restriction come from the residual pass;
+//   - from the first level of at most 64 cells down, one V-cycle from a zero
+//     correction is a fixed linear map of that level's right-hand side: its
+//     matrix is built once (in FP64) and applied as a matrix-vector product,
+//     one phase in place of the 25 or so of those levels.
+//
+// FP64 V-cycles run in 64-bit fixed point.  The part issues one FP64
+// instruction per sub-partition every 64 cycles but a 64-bit integer addition
+// every 2.3 (measured), so an update of the 7-point stencil (five additions,
+// one FMA, one product) takes 450 cycles a warp in FP64 and about 45 as
+// integers: the neighbour sum and the right-hand side are exact, the product
+// by the reciprocal diagonal is a 64 x 64 bit high product.  Every level has a
+// power-of-two scale of its own, taken from the largest right-hand side (and
+// potential) it starts from; a coarse correction too large for the finer
+// level's scale lowers that scale first (prolong_from), so nothing overflows
+// and a right-hand side keeps 53 bits or more below its largest value.
+#include <algorithm>
+#include <cmath>
+#include <cstdlib>
+#include <vector>
+
+#include "mg_internal.h"
+
+namespace {
+
+constexpr int kT = MG_SLAB_THREADS;
+
+typedef long long fix;   // fixed-point value: real * 2^scale
+
+__device__ __forceinline__ unsigned cluster_rank_()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// every thread of every CTA of the cluster, from converged code
+__device__ __forceinline__ void cluster_sync_()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Shared memory by 32-bit address: the same location in CTA `rank` of the
+// cluster, and loads and stores there
+__device__ __forceinline__ unsigned cluster_addr(unsigned a, int rank)
+{
+    unsigned out;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(a), "r"(rank));
+    return out;
+}
+__device__ __forceinline__ void st_cluster(unsigned a, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(unsigned a, long long v)
+{
+    asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(unsigned a, unsigned v)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void ld_cluster(float &v, unsigned a)
+{
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ld_cluster(long long &v, unsigned a)
+{
+    asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+}
+template <typename T>
+__device__ __forceinline__ unsigned shared_addr(const T *p)
+{
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+
+// (v * K) >> (32 + S) for |v|, |K| < 2^62, K = kh 2^32 + kl with kl signed; the
+// product of the low words (below one unit) is dropped.
+template <int S>
+__device__ __forceinline__ fix qmul(fix v, fix K)
+{
+    const int kl = (int)K, kh = (int)((K - kl) >> 32);
+    const int vh = (int)(v >> 32);
+    const unsigned vl = (unsigned)v;
+    const fix mid = (fix)vh * kl + (fix)vl * kh;
+    return (((fix)vh * kh) << (32 - S)) + (mid >> S);
+}
+
+__device__ __forceinline__ fix shift_by(fix v, int s)   // v * 2^s, floor
+{
+    return s >= 0 ? v << min(s, 63) : v >> min(-s, 63);
+}
+
+// x * 2^scale, truncated (|result| < 2^62 by the choice of the scale; x finite)
+__device__ __forceinline__ fix to_fix(double x, int scale)
+{
+    const int hi = __double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const int e = (hi >> 20) & 0x7ff;
+    if (e == 0)
+        return 0;   // zero or denormal
+    const fix m = (fix)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | lo);
+    const fix a = shift_by(m, e - 1075 + scale);
+    return hi < 0 ? -a : a;
+}
+
+// v * 2^-scale rounded to nearest (ties away from zero)
+__device__ __forceinline__ double from_fix(fix v, int scale)
+{
+    if (v == 0)
+        return 0.0;
+    const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
+    const int lz = __clzll((fix)a);
+    const unsigned long long n = a << lz;
+    const unsigned long long q = (n >> 11) + ((n >> 10) & 1);   // 2^52 .. 2^53
+    const int e = 63 - lz - scale + 1023;
+    unsigned long long bits;
+    if (e <= 0)
+        bits = 0;
+    else if (e >= 2047)
+        bits = 0x7ffull << 52;
+    else
+        bits = ((unsigned long long)(e - 1) << 52) + q;         // the carry of q = 2^53 reaches the exponent
+    if (v < 0)
+        bits |= 1ull << 63;
+    return __longlong_as_double((long long)bits);
+}
+
+// Working precision: storage type T of the shared-memory arrays and G of the
+// global ones; words per boundary class of the coefficient tables.
+struct PrecF32 {
+    typedef float T;
+    typedef float G;
+    static constexpr bool kFix = false;
+    static constexpr int kTab = 2;   // negated reciprocal diagonal, diagonal
+};
+struct PrecFix {
+    typedef fix T;
+    typedef double G;
+    static constexpr bool kFix = true;
+    static constexpr int kTab = 3;   // reciprocal of -diagonal * 2^63, floor(-diagonal), its fraction * 2^62
+};
+
+// The plan image: per item (a pair of cells of a thread) four words.
+//   A  bits 0-13 b, the index of the odd cell 2x+1 within its colour (the even
+//      cell is at b + 1 of the other colour); 14 colour of the odd cell; 15, 16
+//      odd, even cell exists; 17-18, 19-20 boundary class along the second and
+//      third axis (bit 0 first, bit 1 last cell); 21-22 the odd cell's along x;
+//      23 even cell last along x; 24, 25 the plane before, after is another CTA's
+//   B  bits 0-13 index of (near plane, near row, column x) among the staged
+//      coarse planes; 14, 15 the far row, plane is the next one (else previous)
+//   C  bits 0-13 index of the first child pair in the finer level's pair sums;
+//      14-17 CTA of the first child plane, 18-21 of the second; 22 the second
+//      plane, 23 the second row exists; 24 the second plane is the first of its CTA
+//   D  level 0: x (bits 0-9), row (10-19), plane (20-29); other levels: bits
+//      0-12 index of the odd cell within a staged plane, 13-16 the first CTA
+//      that interpolates from this plane, 17-20 how many do, 21-30 the plane
+// In the image (and in shared memory) the A words of all slots come first,
+// then B, C, D of the slots of the levels with one pair per thread; those of
+// the other levels follow and stay in global memory (read once per V-cycle).
+// Then, per level of the plan but the last, the ghost cells of the staged
+// planes: bits 0-12 the cell, 13-25 the cell it comes from, and two bits per
+// axis (x lowest) for the factor: 0 one, 1 minus one, 2 cR.
+constexpr int kA = 0, kB = 1, kC = 2, kD = 3;
+
+// One level as one CTA sees it.  Colour c of plane k, row j, storage half
+// index m at ph[c cs + ((k - k0 + 1) R + j) H + m].
+struct Shape {
+    int N, H, R, cs, rows, ha, k0, k1, total;
+};
+
+// planes 1..N of a distributed level over the C CTAs: CTA r owns [plane_first(r), plane_first(r + 1)),
+// and plane k belongs to CTA plane_owner(k); the other levels are CTA 0's
+__host__ __device__ __forceinline__ bool slab_dist(const MgSlabPlan &p, int q) { return q < p.nclu; }
+__host__ __device__ __forceinline__ int plane_first(const MgSlabPlan &p, int q, int r)
+{
+    return slab_dist(p, q) ? 1 + ((r * p.g[q].N) >> p.lgc) : (r == 0 ? 1 : p.g[q].N + 1);
+}
+__host__ __device__ __forceinline__ int plane_owner(const MgSlabPlan &p, int q, int k)
+{
+    return slab_dist(p, q) ? ((k << p.lgc) - 1) / p.g[q].N : 0;
+}
+// first and last staged plane of level q + 1 in CTA r: those around its planes
+// of level q (and the source of the right ghost plane where x_N = 1)
+__host__ __device__ __forceinline__ int staged_first(const MgSlabPlan &p, int q, int r)
+{
+    const int K = plane_first(p, q, r) >> 1;
+    const MgGeom &c = p.g[q + 1];
+    return c.tie && plane_first(p, q, r + 1) > p.g[q].N && K > c.N - 1 ? c.N - 1 : K;
+}
+__host__ __device__ __forceinline__ int staged_last(const MgSlabPlan &p, int q, int r)
+{
+    return ((plane_first(p, q, r + 1) - 1) >> 1) + 1;
+}
+
+template <int DIM>
+__host__ __device__ __forceinline__ Shape shape_of(const MgSlabPlan &p, int q, int rank)
+{
+    Shape s;
+    s.N = p.g[q].N;
+    s.H = (s.N + 3) >> 1;
+    s.R = DIM == 3 ? s.N + 2 : 1;
+    s.cs = (p.po[q] + 2) * s.R * s.H;
+    s.rows = DIM == 3 ? s.N : 1;
+    s.ha = (s.N + 1) >> 1;
+    s.k0 = plane_first(p, q, rank);
+    s.k1 = plane_first(p, q, rank + 1);
+    s.total = s.ha * s.rows * (s.k1 - s.k0);
+    return s;
+}
+
+// Item t of level q in CTA `rank` (t = thread + 512 slot; the pair sums of the
+// residual pass are stored at t)
+template <int DIM>
+__host__ __device__ void plan_item(const MgSlabPlan &p, int q, int rank, int t, int (&w)[4])
+{
+    const Shape s = shape_of<DIM>(p, q, rank);
+    w[0] = w[1] = w[2] = w[3] = 0;
+    if (t >= s.total)
+        return;
+    const int x = t % s.ha, r = t / s.ha;
+    const int j = DIM == 3 ? r % s.rows + 1 : 0, kk = r / s.rows, k = s.k0 + kk;
+    const int b = ((kk + 1) * s.R + j) * s.H + x;
+    const bool even = 2 * x + 2 <= s.N;
+    auto cls = [&](int v) { return (v == 1 ? 1 : 0) | (v == s.N ? 2 : 0); };
+    const bool ring = p.g[q].L == 0;
+    const int c2 = ring ? 0 : DIM == 3 ? cls(j) : cls(k), c3 = ring || DIM == 2 ? 0 : cls(k);
+    w[kA] = b | (((1 + j + k) & 1) << 14) | (1 << 15) | ((even ? 1 : 0) << 16) | (c2 << 17) | (c3 << 19) |
+            ((ring ? 0 : cls(2 * x + 1)) << 21) | ((!ring && 2 * x + 2 == s.N ? 1 : 0) << 23) |
+            ((slab_dist(p, q) && kk == 0 && k > 1 ? 1 : 0) << 24) |
+            ((slab_dist(p, q) && k == s.k1 - 1 && k < s.N ? 1 : 0) << 25);
+    w[kD] = x | (j << 10) | (k << 20);
+    if (q > 0) {
+        // the CTAs with planes 2 k - 2 .. 2 k + 1 of the finer level (and its last plane, whose
+        // right ghost comes from cell N - 1 where x_N = 1)
+        const int Nf = p.g[q - 1].N, ka = max(2 * k - 2, 1);
+        const int kb = p.g[q].tie && k == s.N - 1 ? Nf : min(2 * k + 1, Nf);
+        const int oa = plane_owner(p, q - 1, ka), ob = plane_owner(p, q - 1, kb);
+        w[kD] = (j * (s.N + 2) + 2 * x + 1) | (oa << 13) | ((ob - oa + 1) << 17) | (k << 21);
+    }
+    if (q + 1 < p.nlev) {
+        const int Ec = p.g[q + 1].N + 2, Ra = DIM == 3 ? Ec : 1;
+        const int zn = (k + 1) >> 1, yn = DIM == 3 ? (j + 1) >> 1 : 0;
+        w[kB] = (((zn - staged_first(p, q, rank)) * Ra + yn) * Ec + x) | ((DIM == 3 && !(j & 1) ? 1 : 0) << 14) |
+                ((!(k & 1) ? 1 : 0) << 15);
+    }
+    if (q > 0) {
+        const int Nf = p.g[q - 1].N, haf = (Nf + 1) >> 1, rowsf = DIM == 3 ? Nf : 1;
+        const int k1 = 2 * k - 1, o1 = plane_owner(p, q - 1, k1);
+        const int row = DIM == 3 ? 2 * j - 2 : 0;
+        const bool pl2 = k1 + 1 <= Nf, row2 = DIM == 3 && 2 * j <= Nf;
+        const int o2 = pl2 ? plane_owner(p, q - 1, k1 + 1) : o1;
+        w[kC] = (((k1 - plane_first(p, q - 1, o1)) * rowsf + row) * haf + 2 * x) | (o1 << 14) | (o2 << 18) |
+                ((pl2 ? 1 : 0) << 22) | ((row2 ? 1 : 0) << 23) | ((o2 != o1 ? 1 : 0) << 24);
+    }
+}
+
+// Ghost cell t of the staged planes of level q + 1 in CTA `rank` (-1: none)
+template <int DIM>
+__host__ __device__ int plan_ghost(const MgSlabPlan &p, int q, int rank, int t)
+{
+    const MgGeom &g = p.g[q + 1];
+    const int N = g.N, Ec = N + 2, Ra = DIM == 3 ? Ec : 1;
+    const int Ka = staged_first(p, q, rank), Kb = staged_last(p, q, rank);
+    if (plane_first(p, q, rank) >= plane_first(p, q, rank + 1))
+        return -1;
+    // the active index a ghost index comes from (itself where active), and the factor's kind
+    auto from = [&](int v, int &kind) {
+        kind = 0;
+        if (v >= 1 && v <= N)
+            return v;
+        if (v == 0) {
+            kind = 1;
+            return 1;
+        }
+        if (g.tie) {
+            kind = N >= 2 ? 1 : 0;
+            return N >= 2 ? N - 1 : 1;
+        }
+        kind = 2;
+        return N;
+    };
+    int n = 0;
+    for (int K = Ka; K <= Kb; K++) {
+        const bool kg = K < 1 || K > N;
+        const int in_plane = kg ? Ra * Ec : DIM == 3 ? Ec * Ec - N * N : 2;
+        if (t >= n + in_plane) {
+            n += in_plane;
+            continue;
+        }
+        int r = t - n, I, J = 0;
+        if (kg) {
+            J = r / Ec;
+            I = r - J * Ec;
+        } else if (DIM == 2) {
+            I = r ? N + 1 : 0;
+        } else if (r < 2 * Ec) {       // first and last row
+            J = r < Ec ? 0 : N + 1;
+            I = r < Ec ? r : r - Ec;
+        } else {                       // two columns of the other rows
+            r -= 2 * Ec;
+            J = 1 + (r >> 1);
+            I = r & 1 ? N + 1 : 0;
+        }
+        int kx, ky = 0, kz;
+        const int i = from(I, kx), j = DIM == 3 ? from(J, ky) : 0, k = from(K, kz);
+        const int dst = ((K - Ka) * Ra + J) * Ec + I, src = ((k - Ka) * Ra + j) * Ec + i;
+        return dst | (src << 13) | ((kx | (ky << 2) | (kz << 4)) << 26);
+    }
+    return -1;
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kT) k_slab_plan(const __grid_constant__ MgSlabPlan p, int *img)
+{
+    const int rank = blockIdx.x;
+    int *o = img + (size_t)rank * p.words * kT + threadIdx.x;
+    for (int q = 0; q < p.nlev; q++) {
+        for (int u = 0; u < p.K[q]; u++) {
+            int w[4];
+            plan_item<DIM>(p, q, rank, (int)threadIdx.x + u * kT, w);
+            o[(p.slot[q] + u) * kT] = w[kA];
+            for (int a = kB; a <= kD; a++)
+                o[(p.bcd[q] + 3 * u + a - 1) * kT] = w[a];
+        }
+        for (int u = 0; u < p.KG[q]; u++)
+            o[(p.ghost[q] + u) * kT] = plan_ghost<DIM>(p, q, rank, (int)threadIdx.x + u * kT);
+    }
+    const int t = threadIdx.x;
+    o[p.dpos * kT] = 0;
+    if (t < p.dn) {
+        const Shape s = shape_of<DIM>(p, p.nlev - 1, 0);
+        const int i = t % s.N + 1, r = t / s.N, j = DIM == 3 ? r % s.N + 1 : 0, k = DIM == 3 ? r / s.N + 1 : r + 1;
+        o[p.dpos * kT] = ((i + j + k) & 1) * s.cs + (k * s.R + j) * s.H + (i >> 1);
+    }
+}
+
+template <class P, int DIM>
+struct Engine {
+    typedef typename P::T T;
+    static constexpr bool kFix = P::kFix;
+    static constexpr int kW = sizeof(T);
+    const MgSlabPlan &pl;
+    int rank, tid;
+
+    __device__ explicit Engine(const MgSlabPlan &p) : pl(p), rank((int)cluster_rank_()), tid((int)threadIdx.x) {}
+
+    // ---- shared memory: word arrays (potentials, scratch = pair sums or
+    // staged coarse planes, right-hand sides, dense matrix, tables), then the
+    // control words, then the plan words
+    __device__ __forceinline__ static T *W()
+    {
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        return reinterpret_cast<T *>(smem_raw);
+    }
+    __device__ __forceinline__ T *scratch() const { return W() + pl.scratch; }
+    __device__ __forceinline__ T *fs() const { return W() + pl.fs; }
+    __device__ __forceinline__ T *tab(int q) const { return W() + pl.tabs + P::kTab * 64 * q; }
+    __device__ __forceinline__ int *ctrl() const { return reinterpret_cast<int *>(W() + pl.ctrl); }
+    __device__ __forceinline__ int *sc() const { return ctrl(); }                       // fixed point: scale of every level
+    __device__ __forceinline__ int *psc() const { return ctrl() + MG_SLAB_MAXLEV; }     // ... of its published potential
+    // OR of magnitudes, [2 MAXLEV] pairs: residuals of level q at q, published
+    // potentials at MAXLEV + q; orw: over this CTA, slots: of every CTA
+    __device__ __forceinline__ unsigned *orw() const { return reinterpret_cast<unsigned *>(ctrl() + 2 * MG_SLAB_MAXLEV); }
+    __device__ __forceinline__ unsigned *slots() const { return orw() + 4 * MG_SLAB_MAXLEV; }
+    __device__ __forceinline__ int *img() const { return ctrl() + MG_SLAB_CTRL; }
+    __device__ __forceinline__ const int *gimg() const { return pl.img + (size_t)rank * pl.words * kT; }
+
+    __device__ __forceinline__ bool dist(int q) const { return q < pl.nclu; }
+    __device__ __forceinline__ int word_a(int slot) const { return img()[slot * kT + tid]; }
+    // word B, C or D of pair u of level q
+    __device__ __forceinline__ int word(int q, int u, int a) const
+    {
+        const int i = (pl.bcd[q] + 3 * u + a - 1) * kT + tid;
+        return pl.K[q] == 1 ? img()[i] : gimg()[i];
+    }
+    // barrier between two phases: the cluster's, or this block's when the level lives in CTA 0
+    __device__ __forceinline__ void sync(bool cluster) const
+    {
+        if (cluster)
+            cluster_sync_();
+        else
+            __syncthreads();
+    }
+
+    // where this CTA keeps level q (word offset) and its neighbours keep the
+    // copies of its first and last plane (byte address of the same word)
+    struct Lev {
+        int ph, cs, H, RH;
+        unsigned prev, next;
+        bool tie;
+    };
+    __device__ __forceinline__ Lev level(int q) const
+    {
+        const Shape s = shape_of<DIM>(pl, q, rank);
+        Lev L;
+        L.ph = pl.off[q];
+        L.cs = s.cs;
+        L.H = s.H;
+        L.RH = s.R * s.H;
+        L.tie = pl.g[q].L > 0 && pl.g[q].tie && s.N >= 2;
+        L.prev = L.next = 0u;
+        if (dist(q) && s.total > 0) {
+            const unsigned w0 = shared_addr(W());
+            if (s.k0 > 1) {
+                const int o = plane_owner(pl, q, s.k0 - 1);
+                L.prev = cluster_addr(w0, o) + (s.k0 - plane_first(pl, q, o)) * L.RH * kW;
+            }
+            if (s.k1 <= s.N)
+                L.next = cluster_addr(w0, plane_owner(pl, q, s.k1)) - (s.k1 - s.k0) * L.RH * kW;
+        }
+        return L;
+    }
+
+    __device__ __forceinline__ static int cls_odd(int A) { return ((A >> 21) & 3) | ((A >> 15) & 0x3c); }
+    __device__ __forceinline__ static int cls_even(int A) { return ((A >> 22) & 2) | ((A >> 15) & 0x3c); }
+    // the pair's cell of colour c: 0 the odd one, 1 the even one; whether it exists
+    __device__ __forceinline__ static int s_of(int A, int c) { return ((A >> 14) & 1) ^ c; }
+    __device__ __forceinline__ static bool has(int A, int c) { return (A >> (15 + s_of(A, c))) & 1; }
+
+    __device__ __forceinline__ void put(const Lev &L, int A, int i, T v) const
+    {
+        W()[i] = v;
+        if ((A >> 24) & 3) {
+            if ((A >> 24) & 1)
+                st_cluster(L.prev + i * kW, v);
+            if ((A >> 25) & 1)
+                st_cluster(L.next + i * kW, v);
+        }
+    }
+
+    // neighbour sum of a pair's cell of colour c (s = 0: the odd, 1: the even
+    // cell).  Ghost layers read zero on coarse levels; where x_N = 1 the ghost
+    // cancels the left neighbour of the last cell (Sec. 2.4).
+    __device__ __forceinline__ T nsum(const Lev &L, int A, int c, int s) const
+    {
+        const T *o = W() + L.ph + (1 - c) * L.cs + (A & 0x3fff);
+        T sx = o[0] + o[1];
+        o += s;
+        T sy = T(0), sz;
+        if (DIM == 3) {
+            sy = o[-L.H] + o[L.H];
+            sz = o[-L.RH] + o[L.RH];
+        } else {
+            sz = o[-L.H] + o[L.H];
+        }
+        if (L.tie) {
+            if (s ? (A >> 23) & 1 : (A >> 22) & 1)
+                sx = T(0);
+            if (DIM == 3) {
+                if ((A >> 18) & 1)
+                    sy = T(0);
+                if ((A >> 20) & 1)
+                    sz = T(0);
+            } else if ((A >> 18) & 1) {
+                sz = T(0);
+            }
+        }
+        return DIM == 3 ? (sx + sy) + sz : sx + sz;
+    }
+
+    // What a thread needs of K of its pairs to sweep: per pair the plan word,
+    // and per colour the right-hand side and the reciprocal diagonal.  A level
+    // of one pair per thread keeps them in registers from sweep to sweep; the
+    // others read two pairs at a time from shared memory in every sweep, which
+    // keeps the code small enough for the instruction cache.
+    template <int K>
+    struct Items {
+        int A[K];
+        T f[2][K], n[2][K];
+    };
+
+    // pairs u0 .. u0 + K - 1 of level q, colours c0 .. c1
+    template <int K>
+    __device__ __forceinline__ void load_items(int q, int u0, Items<K> &it, bool with_f, int c0 = 0, int c1 = 1) const
+    {
+        const int slot = pl.slot[q] + u0;
+        const T *tb = tab(q);
+#pragma unroll
+        for (int u = 0; u < K; u++) {
+            const int A = word_a(slot + u);
+            it.A[u] = A;
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                it.n[c][u] = it.f[c][u] = T(0);
+                if (c < c0 || c > c1)
+                    continue;
+                it.n[c][u] = tb[s_of(A, c) ? cls_even(A) : cls_odd(A)];
+                if (with_f)
+                    it.f[c][u] = fs()[(2 * (slot + u) + c) * kT + tid];
+            }
+        }
+    }
+
+    // fn(items, u0) over all pairs of level q: in registers already (one pair), or two at a time
+    template <bool ONE, class It, class Fn>
+    __device__ __forceinline__ void pairs(int q, It &it, int c0, int c1, Fn &&fn) const
+    {
+        if constexpr (ONE) {
+            if (__any_sync(0xffffffffu, (it.A[0] >> 15) & 1))   // a warp without pairs skips the phase
+                fn(it, 0);
+        } else {
+            const int K = pl.K[q];
+#pragma unroll 1
+            for (int u0 = 0; u0 < K; u0 += 2) {
+                load_items<2>(q, u0, it, true, c0, c1);
+                fn(it, u0);
+            }
+        }
+    }
+
+    __device__ __forceinline__ T update(int q, T s, T f, T n) const
+    {
+        if constexpr (kFix)
+            return qmul<31>(s - f, n);
+        else
+            return (s - pl.g[q].h2f * f) * n;
+    }
+
+    // colour c of a red-black sweep
+    template <int c, int K>
+    __device__ __forceinline__ void pass(int q, const Lev &L, const Items<K> &it) const
+    {
+        T v[K];
+#pragma unroll
+        for (int u = 0; u < K; u++)
+            if (has(it.A[u], c))
+                v[u] = update(q, nsum(L, it.A[u], c, s_of(it.A[u], c)), it.f[c][u], it.n[c][u]);
+#pragma unroll
+        for (int u = 0; u < K; u++)
+            if (has(it.A[u], c))
+                put(L, it.A[u], L.ph + c * L.cs + (it.A[u] & 0x3fff) + s_of(it.A[u], c), v[u]);
+    }
+
+    // OR of the magnitudes m over this CTA into word pair w of orw
+    __device__ __forceinline__ void block_or(fix m, int w) const
+    {
+        const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)((unsigned long long)m >> 32));
+        const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
+        if ((tid & 31) == 0) {
+            if (hi)
+                atomicOr(orw() + 2 * w, hi);
+            else if (lo)
+                atomicOr(orw() + 2 * w + 1, lo);
+        }
+    }
+    // ... and to every CTA of the cluster
+    __device__ __forceinline__ void share_or(int w) const
+    {
+        __syncthreads();
+        if (tid < pl.csize) {
+            const unsigned dst = cluster_addr(shared_addr(slots() + (w * 16 + rank) * 2), tid);
+            st_cluster(dst, orw()[2 * w]);
+            st_cluster(dst + 4, orw()[2 * w + 1]);
+            if (w >= MG_SLAB_MAXLEV && rank == 0)
+                st_cluster(cluster_addr(shared_addr(psc() + (w - MG_SLAB_MAXLEV)), tid),
+                           (unsigned)sc()[w - MG_SLAB_MAXLEV]);
+        }
+    }
+    __device__ __forceinline__ void clear_or(int w) const
+    {
+        if (tid == 0)
+            orw()[2 * w] = orw()[2 * w + 1] = 0u;
+    }
+    // bits of the largest magnitude, after the barrier that follows block_or (and share_or)
+    __device__ __forceinline__ int or_bits(int w, bool cluster) const
+    {
+        unsigned hi = 0, lo = 0;
+        if (cluster) {
+            for (int t = 0; t < pl.csize; t++) {
+                hi |= slots()[(w * 16 + t) * 2];
+                lo |= slots()[(w * 16 + t) * 2 + 1];
+            }
+        } else {
+            hi = orw()[2 * w];
+            lo = orw()[2 * w + 1];
+        }
+        return hi ? 64 - __clz(hi) : 32 - __clz(lo);
+    }
+    __device__ __forceinline__ static fix mag(fix v) { return v < 0 ? ~v : v; }
+
+    // Residual (step 4) of both cells of every pair, summed over the pair.
+    template <int K>
+    __device__ __forceinline__ fix residual(int q, const Lev &L, const Items<K> &it, int u0) const
+    {
+        const T *tb = tab(q);
+        const float ih2 = pl.g[q].inv_h2f;
+        fix big = 0;
+#pragma unroll
+        for (int u = 0; u < K; u++) {
+            const int A = it.A[u];
+            T sum = T(0);
+#pragma unroll
+            for (int c = 0; c < 2; c++)
+                if (has(A, c)) {
+                    const int s = s_of(A, c), cls = s ? cls_even(A) : cls_odd(A);
+                    const T ns = nsum(L, A, c, s);
+                    const T v = W()[L.ph + c * L.cs + (A & 0x3fff) + s];
+                    if constexpr (kFix) {
+                        T d = (2 * DIM) * v;
+                        if (cls)
+                            d = tb[64 + cls] * v + qmul<30>(v, tb[128 + cls]);
+                        sum += it.f[c][u] - ns + d;
+                    } else {
+                        sum += it.f[c][u] - (ns + tb[64 + cls] * v) * ih2;
+                    }
+                }
+            if ((A >> 15) & 1)
+                scratch()[tid + (u0 + u) * kT] = sum;
+            if constexpr (kFix)
+                big |= mag(sum);
+        }
+        return big;
+    }
+
+    // The scale of level q from the largest residual of level q - 1; the shift
+    // of its pair sums into it (h_c^2 = 4 h_f^2, 2^-d average).
+    __device__ __forceinline__ int restrict_scale(int q) const
+    {
+        const int bits = or_bits(q - 1, dist(q - 1)), s0 = sc()[q - 1];
+        const int s1 = bits ? s0 + pl.tb[q] - (bits + 1) : s0;
+        if (tid == 0)
+            sc()[q] = s1;
+        return s1 - s0 - (DIM == 3 ? 1 : 0);
+    }
+
+    // The right-hand sides of K pairs of level q: the 2^d-child average (step
+    // 5) of level q - 1's residual.
+    template <int K>
+    __device__ __forceinline__ void restrict_into(int q, int u0, Items<K> &it, int sh, bool keep) const
+    {
+        const bool dup = dist(q - 1);
+        const int slot = pl.slot[q] + u0;
+        const int Nf = pl.g[q - 1].N, haf = (Nf + 1) >> 1, planef = haf * (DIM == 3 ? Nf : 1);
+        const unsigned r0 = shared_addr(scratch());
+#pragma unroll
+        for (int u = 0; u < K; u++) {
+            const int A = it.A[u];
+            T o = T(0), e = T(0);
+            if ((A >> 15) & 1) {
+                const int w = word(q, u0 + u, kC);
+                const bool even = (A >> 16) & 1, row2 = DIM == 3 && ((w >> 23) & 1), pl2 = (w >> 22) & 1;
+                const int i1 = w & 0x3fff, i2 = (w >> 24) & 1 ? i1 % planef : i1 + planef;
+                T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0), c0 = T(0), c1 = T(0), d0 = T(0), d1 = T(0);
+                auto quad = [&](auto &&ld) {
+                    ld(a0, 0, i1);
+                    if (even)
+                        ld(a1, 0, i1 + 1);
+                    if (row2) {
+                        ld(b0, 0, i1 + haf);
+                        if (even)
+                            ld(b1, 0, i1 + haf + 1);
+                    }
+                    if (pl2) {
+                        ld(c0, 1, i2);
+                        if (even)
+                            ld(c1, 1, i2 + 1);
+                        if (row2) {
+                            ld(d0, 1, i2 + haf);
+                            if (even)
+                                ld(d1, 1, i2 + haf + 1);
+                        }
+                    }
+                };
+                if (dup) {
+                    const unsigned r1 = cluster_addr(r0, (w >> 14) & 15), r2 = cluster_addr(r0, (w >> 18) & 15);
+                    quad([&](T &v, int p, int i) { ld_cluster(v, (p ? r2 : r1) + i * kW); });
+                } else {
+                    quad([&](T &v, int, int i) { v = scratch()[i]; });
+                }
+                o = (a0 + b0) + (c0 + d0);
+                e = (a1 + b1) + (c1 + d1);
+            }
+            if constexpr (kFix) {
+                o = shift_by(o, sh);
+                e = shift_by(e, sh);
+            } else {
+                o *= DIM == 3 ? 0.125f : 0.25f;
+                e *= DIM == 3 ? 0.125f : 0.25f;
+            }
+            const bool odd0 = s_of(A, 0) == 0;   // the odd cell is red
+            it.f[0][u] = odd0 ? o : e;
+            it.f[1][u] = odd0 ? e : o;
+            if (keep) {
+                fs()[(2 * (slot + u)) * kT + tid] = it.f[0][u];
+                fs()[(2 * (slot + u) + 1) * kT + tid] = it.f[1][u];
+            }
+        }
+    }
+
+    // The potential of a level that starts from zero after its first red
+    // half-sweep, which sees zero neighbours
+    template <int K>
+    __device__ __forceinline__ void first_red(int q, const Lev &L, const Items<K> &it) const
+    {
+        const bool on = pl.nu_pre > 0;
+#pragma unroll
+        for (int u = 0; u < K; u++) {
+            const int A = it.A[u], i = L.ph + (A & 0x3fff);
+            if (has(A, 0))
+                put(L, A, i + s_of(A, 0), on ? update(q, T(0), it.f[0][u], it.n[0][u]) : T(0));
+            if (has(A, 1))
+                put(L, A, i + L.cs + s_of(A, 1), T(0));
+        }
+    }
+
+    // The last level of the plan and everything below it: the matrix of one
+    // V-cycle times the right-hand side.  CTA 0; pl.dn cells, cell t at word
+    // dpos[t] of the level; eight partial sums per cell.
+    __device__ __forceinline__ void dense_solve(int q, const Lev &L, const Items<1> &it) const
+    {
+        const int n = pl.dn;
+        T *vec = W() + pl.dvec, *part = vec + 64;
+        const T *mat = W() + pl.dmat;
+        const int *pos = img() + pl.dpos * kT;
+        // right-hand sides by cell number (x fastest)
+        const int A = it.A[0];
+        if ((A >> 15) & 1) {
+            const int w = 2 * tid - (pl.g[q].N & 1) * (tid / ((pl.g[q].N + 1) >> 1));
+            const bool odd0 = s_of(A, 0) == 0;
+            T o = odd0 ? it.f[0][0] : it.f[1][0], e = odd0 ? it.f[1][0] : it.f[0][0];
+            if constexpr (!kFix) {
+                o *= pl.g[q].h2f;
+                e *= pl.g[q].h2f;
+            }
+            vec[w] = o;
+            if ((A >> 16) & 1)
+                vec[w + 1] = e;
+        }
+        __syncthreads();
+        const int i = tid & 63, p = tid >> 6;
+        T s = T(0);
+        if (i < n)
+            for (int j = p; j < n; j += 8) {
+                if constexpr (kFix)
+                    s += qmul<28>(vec[j], mat[j * n + i]);
+                else
+                    s += mat[j * n + i] * vec[j];
+            }
+        part[tid] = s;
+        __syncthreads();
+        if (tid < n) {
+            T v = T(0);
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                v += part[tid + 64 * k];
+            W()[L.ph + pos[tid]] = v;
+        }
+        __syncthreads();
+    }
+
+    // The potential of level q into the staged planes of the CTAs that
+    // interpolate from it.
+    __device__ __forceinline__ void publish(int q, const Lev &L) const
+    {
+        const int Ec = pl.g[q].N + 2, ps = (DIM == 3 ? Ec : 1) * Ec;
+        const bool dup = dist(q - 1);
+        const unsigned s0 = shared_addr(scratch());
+        fix big = 0;
+        const int K = pl.K[q];
+#pragma unroll 1
+        for (int u = 0; u < K; u++) {
+            const int A = word_a(pl.slot[q] + u), d = word(q, u, kD);
+            if (!((A >> 15) & 1))
+                continue;
+            const int c1 = (A >> 14) & 1, b = L.ph + (A & 0x3fff), k = d >> 21;
+            const bool even = (A >> 16) & 1;
+            const T vo = W()[b + c1 * L.cs], ve = even ? W()[b + (1 - c1) * L.cs + 1] : T(0);
+            if constexpr (kFix)
+                big |= mag(vo) | mag(ve);
+            if (!dup) {
+                T *dst = scratch() + k * ps + (d & 0x1fff);
+                dst[0] = vo;
+                if (even)
+                    dst[1] = ve;
+                continue;
+            }
+            const int o1 = (d >> 13) & 15, n = (d >> 17) & 15;
+            for (int o = o1; o < o1 + n; o++) {
+                if (plane_first(pl, q - 1, o) == plane_first(pl, q - 1, o + 1))
+                    continue;
+                const unsigned dst = cluster_addr(s0, o) + ((k - staged_first(pl, q - 1, o)) * ps + (d & 0x1fff)) * kW;
+                st_cluster(dst, vo);
+                if (even)
+                    st_cluster(dst + kW, ve);
+            }
+        }
+        if constexpr (kFix) {
+            block_or(big, MG_SLAB_MAXLEV + q);
+            if (dup)
+                share_or(MG_SLAB_MAXLEV + q);
+        }
+    }
+
+    // The ghost cells of the staged planes of level q + 1 by the rule of Sec.
+    // 2.4: left ghost -Phi_1, right ghost cR Phi_N, or -Phi_{N-1} where x_N = 1.
+    __device__ __forceinline__ void fill_ghosts(int q) const
+    {
+        const int K = pl.KG[q];
+#pragma unroll 1
+        for (int u = 0; u < K; u++) {
+            const int w = img()[(pl.ghost[q] + u) * kT + tid];
+            if (w == -1)
+                continue;
+            T v = scratch()[(w >> 13) & 0x1fff];
+#pragma unroll
+            for (int a = 0; a < DIM; a++) {
+                const int kind = (w >> (26 + 2 * (DIM == 2 && a ? 2 : a))) & 3;
+                if (kind == 1)
+                    v = -v;
+                if (kind == 2) {
+                    if constexpr (kFix)
+                        v = pl.cri[q + 1] * v + qmul<30>(v, pl.crf[q + 1]);
+                    else
+                        v = pl.g[q + 1].cRf * v;
+                }
+            }
+            scratch()[w & 0x1fff] = v;
+        }
+    }
+
+    // The shift of level q + 1's potential to level q's scale, which is lowered
+    // first if the correction is beyond its range.
+    __device__ __forceinline__ int prolong_scale(int q, const Lev &L) const
+    {
+        const bool cl = dist(q);
+        const int bits = or_bits(MG_SLAB_MAXLEV + q + 1, cl), s1 = cl ? psc()[q + 1] : sc()[q + 1], s0 = sc()[q];
+        const int low = bits ? max(0, bits + s0 - s1 - pl.top[q]) : 0;
+        if (low) {
+            __syncthreads();   // every thread has read the scale
+            if (tid == 0)
+                sc()[q] = s0 - low;
+            for (int t = tid; t < 2 * L.cs; t += kT)
+                W()[L.ph + t] = shift_by(W()[L.ph + t], -low);
+            T *f = fs() + 2 * pl.slot[q] * kT + tid;
+            for (int u = 0; u < 2 * pl.K[q]; u++)
+                f[u * kT] = shift_by(f[u * kT], -low);
+            sync(cl);
+        }
+        return s0 - low - s1;
+    }
+
+    // Prolongation and correction (step 10) of K pairs of level q from the
+    // staged planes of level q + 1.
+    template <int K>
+    __device__ __forceinline__ void prolong_from(int q, int u0, const Lev &L, const Items<K> &it, int sh) const
+    {
+        const int Ec = pl.g[q + 1].N + 2, ps = (DIM == 3 ? Ec : 1) * Ec;
+        // 3/4 - 1/4 interpolation along one axis
+        auto mix = [](T near, T far) -> T {
+            if constexpr (kFix)
+                return (3 * near + far) >> 2;
+            else
+                return 0.75f * near + 0.25f * far;
+        };
+#pragma unroll
+        for (int u = 0; u < K; u++) {
+            const int A = it.A[u];
+            if (!((A >> 15) & 1))
+                continue;
+            const int bw = word(q, u0 + u, kB);
+            const T *b = scratch() + (bw & 0x3fff);
+            const int dy = (bw >> 14) & 1 ? Ec : -Ec, dz = (bw >> 15) & 1 ? ps : -ps;
+            auto plane = [&](const T *z, T &o, T &e) {
+                o = mix(z[1], z[0]);
+                e = mix(z[1], z[2]);
+                if (DIM == 3) {
+                    const T *y = z + dy;
+                    o = mix(o, mix(y[1], y[0]));
+                    e = mix(e, mix(y[1], y[2]));
+                }
+            };
+            T o0, e0, o1, e1;
+            plane(b, o0, e0);
+            plane(b + dz, o1, e1);
+            T po = mix(o0, o1), pe = mix(e0, e1);
+            if constexpr (kFix) {
+                po = shift_by(po, sh);
+                pe = shift_by(pe, sh);
+            }
+            const int c1 = (A >> 14) & 1, i = L.ph + (A & 0x3fff), io = i + c1 * L.cs, ie = i + (1 - c1) * L.cs + 1;
+            put(L, A, io, W()[io] + po);
+            if ((A >> 16) & 1)
+                put(L, A, ie, W()[ie] + pe);
+        }
+    }
+
+    // descent on level q: its right-hand side from the finer level (q > 0),
+    // pre-smoothing, residual; the last level is solved
+    template <bool ONE>
+    __device__ __forceinline__ void descend(int q, bool fresh) const
+    {
+        const Lev L = level(q);
+        const bool cl = dist(q);
+        Items<ONE ? 1 : 2> it;
+        if constexpr (kFix)
+            clear_or(MG_SLAB_MAXLEV + q);
+        const bool red = q > 0 || fresh, last = q + 1 == pl.nlev;
+        if (q > 0) {
+            int sh = 0;
+            if constexpr (kFix)
+                sh = restrict_scale(q);
+            const int K = pl.K[q];
+#pragma unroll 1
+            for (int u0 = 0; u0 < K; u0 += ONE ? 1 : 2) {
+                load_items(q, u0, it, false);
+                restrict_into(q, u0, it, sh, !last);
+                if (!last)
+                    first_red(q, L, it);
+            }
+            if constexpr (ONE)
+                if (last) {
+                    dense_solve(q, L, it);
+                    return;
+                }
+        } else {
+            if constexpr (ONE)
+                load_items(0, 0, it, true);
+            if (fresh)
+                pairs<ONE>(q, it, 0, 1, [&](auto &t, int) { first_red(q, L, t); });
+        }
+        if (red)
+            sync(cl);
+#pragma unroll 1
+        for (int s = 0; s < pl.nu_pre; s++) {
+            if (s > 0 || !red) {
+                pairs<ONE>(q, it, 0, 0, [&](auto &t, int) { this->template pass<0>(q, L, t); });
+                sync(cl);
+            }
+            pairs<ONE>(q, it, 1, 1, [&](auto &t, int) { this->template pass<1>(q, L, t); });
+            sync(cl);
+        }
+        fix big = 0;
+        pairs<ONE>(q, it, 0, 1, [&](auto &t, int u0) { big |= residual(q, L, t, u0); });
+        if constexpr (kFix) {
+            block_or(big, q);
+            if (cl)
+                share_or(q);
+        }
+        sync(cl);
+    }
+
+    // ascent on level q: correction from level q + 1, post-smoothing (after
+    // the last sweep the own cells alone are read: no barrier)
+    template <bool ONE>
+    __device__ __forceinline__ void ascend(int q, bool last) const
+    {
+        const Lev L = level(q);
+        const bool cl = dist(q);
+        Items<ONE ? 1 : 2> it;
+        int sh = 0;
+        if constexpr (kFix) {
+            clear_or(q);
+            sh = prolong_scale(q, L);
+        }
+        fill_ghosts(q);
+        if constexpr (ONE)
+            load_items(q, 0, it, true);
+        __syncthreads();
+        pairs<ONE>(q, it, 0, 1, [&](auto &t, int u0) { prolong_from(q, u0, L, t, sh); });
+        const bool fin = q > 0 || last;
+        sync(cl);   // also: no CTA may publish into staged planes that another still reads
+#pragma unroll 1
+        for (int s = 0; s < pl.nu_post; s++) {
+            pairs<ONE>(q, it, 0, 0, [&](auto &t, int) { this->template pass<0>(q, L, t); });
+            sync(cl);
+            pairs<ONE>(q, it, 1, 1, [&](auto &t, int) { this->template pass<1>(q, L, t); });
+            if (!fin || s + 1 < pl.nu_post)
+                sync(cl);
+        }
+    }
+
+    // coefficient tables of every level, the dense matrix
+    __device__ __forceinline__ void fill_tables() const
+    {
+        for (int t = tid; t < 64 * pl.nlev; t += kT) {
+            const int q = t >> 6, c = t & 63;
+            const MgGeom &g = pl.g[q];
+            T *tb = tab(q);
+            double d = -2.0 * DIM, nid = 1.0 / (2 * DIM);
+            if (c && g.tab64) {
+                d = g.tab64[c];
+                nid = g.tab64[64 + c];
+            }
+            if constexpr (kFix) {
+                tb[c] = (fix)(nid * 9223372036854775808.0);
+                const double fl = floor(-d);
+                tb[64 + c] = (fix)fl;
+                tb[128 + c] = (fix)((-d - fl) * 4611686018427387904.0);
+            } else {
+                tb[c] = (float)nid;
+                tb[64 + c] = (float)d;
+            }
+        }
+        if (rank == 0) {
+            const T *src = static_cast<const T *>(pl.dense);
+            T *dst = W() + pl.dmat;
+            const int n = pl.dn * pl.dn;
+#pragma unroll 4
+            for (int t = tid; t < n; t += kT)
+                dst[t] = src[t];
+        }
+    }
+};
+
+// exponent bound: |x| < 2^result for the largest magnitude with this high word
+__device__ __forceinline__ int exp_bound(unsigned hi) { return hi ? (int)(hi >> 20) - 1022 : -4000; }
+
+template <class P, int DIM>
+__global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPlan pl)
+{
+    typedef typename P::T T;
+    typedef typename P::G G;
+    __shared__ unsigned s_max[2], s_all[2][16];
+    const Engine<P, DIM> en(pl);
+    const int tid = threadIdx.x, rank = en.rank, C = pl.csize;
+    const int wid = tid >> 5, lane = tid & 31, nw = kT / 32;
+    // before the predecessor has finished: the plan image, the tables, the
+    // potentials to zero (their ghost layers stay zero)
+    {
+        const int nw16 = pl.nimg * (kT / 4);
+        const uint4 *src = reinterpret_cast<const uint4 *>(en.gimg());
+        uint4 *dst = reinterpret_cast<uint4 *>(en.img());
+#pragma unroll 4
+        for (int t = tid; t < nw16; t += kT)
+            dst[t] = src[t];
+    }
+    for (int t = tid; t < pl.zero16; t += kT)
+        reinterpret_cast<uint4 *>(en.W())[t] = make_uint4(0, 0, 0, 0);
+    en.fill_tables();
+    for (int t = tid; t < MG_SLAB_CTRL; t += kT)
+        en.ctrl()[t] = 0;
+    if (tid < 2)
+        s_max[tid] = 0u;
+    __syncthreads();
+    pdl_begin();
+    const Shape S = shape_of<DIM>(pl, 0, rank);
+    const MgGeom &g0 = pl.g[0];
+    const int N = g0.N, E = N + 2;
+    T *ph0 = en.W() + pl.off[0];
+    const G *gphi = static_cast<const G *>(pl.phi), *gf = static_cast<const G *>(pl.f);
+    auto gidx = [&](int i, int j, int k) { return (size_t)(DIM == 3 ? k * E + j : k) * E + i; };
+    // level 0 of the plan from global memory: the right-hand side to its
+    // threads, the potential (with its ring) to the slab, a warp per row
+    unsigned mphi = 0, mf = 0;
+    for (int u = 0; u < pl.K[0]; u++) {
+        const int A = en.word_a(u), d = en.word(0, u, kD);
+        const int x = d & 0x3ff, j = (d >> 10) & 0x3ff, k = d >> 20;
+        G o = G(0), e = G(0);
+        if ((A >> 15) & 1)
+            o = gf[gidx(2 * x + 1, j, k)];
+        if ((A >> 16) & 1)
+            e = gf[gidx(2 * x + 2, j, k)];
+        const bool odd0 = ((A >> 14) & 1) == 0;
+        const G r = odd0 ? o : e, b = odd0 ? e : o;
+        if constexpr (P::kFix) {
+            en.fs()[(2 * u) * kT + tid] = __double_as_longlong(r);
+            en.fs()[(2 * u + 1) * kT + tid] = __double_as_longlong(b);
+            mf = max(mf, max((unsigned)__double2hiint(r) & 0x7fffffffu, (unsigned)__double2hiint(b) & 0x7fffffffu));
+        } else {
+            en.fs()[(2 * u) * kT + tid] = r;
+            en.fs()[(2 * u + 1) * kT + tid] = b;
+        }
+    }
+    if (!pl.zero_start && S.total > 0) {
+        const int rows = DIM == 3 ? E : 1, ka = S.k0 - 1, nr = rows * (S.k1 - S.k0 + 2);
+        constexpr int U = 4;
+        for (int i0 = 0; i0 < E; i0 += 32)
+            for (int r0 = wid; r0 < nr; r0 += nw * U) {
+                const int i = i0 + lane;
+                G v[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int r = r0 + u * nw, kz = r / rows;
+                    v[u] = G(0);
+                    if (r < nr && i < E)
+                        v[u] = gphi[gidx(i, r - kz * rows, ka + kz)];
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int r = r0 + u * nw, kz = r / rows, j = r - kz * rows;
+                    if (r < nr && i < E) {
+                        T &d = ph0[((i + j + ka + kz) & 1) * S.cs + (kz * S.R + j) * S.H + (i >> 1)];
+                        if constexpr (P::kFix) {
+                            d = __double_as_longlong(v[u]);
+                            mphi = max(mphi, (unsigned)__double2hiint(v[u]) & 0x7fffffffu);
+                        } else {
+                            d = v[u];
+                        }
+                    }
+                }
+            }
+    }
+    bool bad = false;
+    if constexpr (P::kFix) {
+        // the scale of the plan's first level from the largest magnitudes over
+        // the cluster; infinities and NaN make every result NaN
+        mphi = __reduce_max_sync(0xffffffffu, mphi);
+        mf = __reduce_max_sync(0xffffffffu, mf);
+        if (lane == 0) {
+            atomicMax(&s_max[0], mphi);
+            atomicMax(&s_max[1], mf);
+        }
+        cluster_sync_();   // every CTA has started: its shared memory may be written
+        if (tid < C) {
+            st_cluster(cluster_addr(shared_addr(&s_all[0][rank]), tid), s_max[0]);
+            st_cluster(cluster_addr(shared_addr(&s_all[1][rank]), tid), s_max[1]);
+        }
+        cluster_sync_();
+        mphi = mf = 0;
+        for (int t = 0; t < C; t++) {
+            mphi = max(mphi, s_all[0][t]);
+            mf = max(mf, s_all[1][t]);
+        }
+        bad = mphi >= 0x7ff00000u || mf >= 0x7ff00000u;
+        const int gb = mf ? exp_bound(mf) + exp_bound((unsigned)__double2hiint(g0.h2)) : -4000;
+        const int s0 = mf || mphi ? pl.tb[0] - max(gb, exp_bound(mphi)) : 0;
+        if (tid == 0)
+            en.sc()[0] = s0;
+        if (!pl.zero_start)
+            for (int t = tid; t < 2 * S.cs; t += kT)
+                ph0[t] = to_fix(__longlong_as_double(ph0[t]), s0);
+        for (int u = 0; u < 2 * pl.K[0]; u++) {
+            T &f = en.fs()[u * kT + tid];
+            f = to_fix(__longlong_as_double(f) * g0.h2, s0);
+        }
+        __syncthreads();
+    } else {
+        cluster_sync_();
+    }
+    if (!bad) {
+        for (int cyc = 0; cyc < pl.cycles; cyc++) {
+            int q = 0;
+            for (;; q++) {
+                // a level in CTA 0 alone: the other CTAs wait for its staged planes
+                if (en.dist(q) || rank == 0) {
+                    const bool fresh = pl.zero_start && cyc == 0;
+                    if (pl.K[q] == 1)
+                        en.template descend<true>(q, fresh);
+                    else
+                        en.template descend<false>(q, fresh);
+                }
+                if (q + 1 == pl.nlev)
+                    break;
+            }
+            for (; q > 0; q--) {
+                if (en.dist(q) || rank == 0)
+                    en.publish(q, en.level(q));
+                if (en.dist(q - 1))
+                    cluster_sync_();
+                else if (rank == 0)
+                    __syncthreads();
+                if (en.dist(q - 1) || rank == 0) {
+                    const bool last = cyc + 1 == pl.cycles;
+                    if (pl.K[q - 1] == 1)
+                        en.template ascend<true>(q - 1, last);
+                    else
+                        en.template ascend<false>(q - 1, last);
+                }
+            }
+        }
+    }
+    // the potential of the plan's first level back to global memory
+    {
+        G *out = static_cast<G *>(pl.phi);
+        int s0 = 0;
+        if constexpr (P::kFix)
+            s0 = en.sc()[0];
+        for (int u = 0; u < pl.K[0]; u++) {
+            const int A = en.word_a(u), d = en.word(0, u, kD);
+            const int x = d & 0x3ff, j = (d >> 10) & 0x3ff, k = d >> 20, c1 = (A >> 14) & 1, b = A & 0x3fff;
+            for (int s = 0; s < 2; s++)
+                if ((A >> (15 + s)) & 1) {
+                    const T v = ph0[(s ? 1 - c1 : c1) * S.cs + b + s];
+                    G o;
+                    if constexpr (P::kFix)
+                        o = bad ? __longlong_as_double(0x7ff8000000000000ll) : from_fix(v, s0);
+                    else
+                        o = v;
+                    out[gidx(2 * x + 1 + s, j, k)] = o;
+                }
+        }
+    }
+    if (pl.ctl && rank == 0 && tid == 0)
+        inner_step_count(pl.ctl, pl.hi);
+    cluster_sync_();   // no CTA leaves while another may still write to its shared memory
+}
+
+template <class P, int DIM>
+cudaError_t slab_prepare()
+{
+    cudaError_t e = cudaFuncSetAttribute(k_slab<P, DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, MG_SLAB_SMEM_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_slab<P, DIM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
+void slab_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, int csize, size_t smem, cudaStream_t s)
+{
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(csize);
+    cfg.blockDim = dim3(kT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = csize;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = mg_pdl_enabled() ? 2 : 1;
+}
+
+}  // namespace
+
+// The largest cluster (16 CTAs, else 8) that the device can hold at the
+// largest shared-memory size, 0 if none.
+int mg_slab_prepare()
+{
+    if (slab_prepare<PrecF32, 2>() || slab_prepare<PrecF32, 3>() || slab_prepare<PrecFix, 2>() ||
+        slab_prepare<PrecFix, 3>()) {
+        cudaGetLastError();
+        return 0;
+    }
+    for (int cs : {16, 8}) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at[2];
+        slab_config(cfg, at, cs, MG_SLAB_SMEM_MAX, nullptr);
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_slab<PrecFix, 3>, &cfg) == cudaSuccess && n > 0)
+            return cs;
+        cudaGetLastError();
+    }
+    return 0;
+}
+
+// Shared-memory layout of levels g[0..nlev-1]; the levels of more than `cut`
+// cells per edge are distributed.  False when it does not fit.
+bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, int cut, int nu_pre, int nu_post,
+                    MgSlabPlan &p)
+{
+    // the plan ends with the first level of at most 64 cells
+    int last = 1;
+    while (last < nlev && std::pow((double)g[last].N, dim) > 64.5)
+        last++;
+    if ((csize != 8 && csize != 16) || last >= nlev || last >= MG_SLAB_MAXLEV)
+        return false;
+    nlev = last + 1;
+    p = MgSlabPlan{};
+    p.nlev = nlev;
+    p.csize = csize;
+    p.lgc = csize == 16 ? 4 : 3;
+    p.nu_pre = nu_pre;
+    p.nu_post = nu_post;
+    const size_t w = fp32 ? 4 : 8;
+    size_t off = 0, scratch = 0;
+    const int lognu = (int)std::ceil(std::log2(1.0 + nu_pre + nu_post));
+    auto align = [](size_t v) { return (v + 3) & ~(size_t)3; };
+    for (int q = 0; q < nlev; q++) {
+        p.g[q] = g[q];
+        if (g[q].N > cut && q == p.nclu && q + 1 < nlev)
+            p.nclu = q + 1;
+    }
+    for (int q = 0; q < nlev; q++) {
+        const int N = g[q].N, H = (N + 3) >> 1, R = dim == 3 ? N + 2 : 1, ha = (N + 1) >> 1, rows = dim == 3 ? N : 1;
+        p.po[q] = q < p.nclu ? (N + csize - 1) / csize : N;
+        const size_t cs = (size_t)(p.po[q] + 2) * R * H, items = (size_t)p.po[q] * rows * ha;
+        if (cs > 0x3fff || items > 0x3fff || N > 1020)   // fields of the plan words
+            return false;
+        p.off[q] = (int)off;
+        off = align(off + 2 * cs);
+        const int k = (int)((items + kT - 1) / kT);
+        if (k > MG_SLAB_MAXK)
+            return false;
+        p.K[q] = k == 1 ? 1 : (k + 1) & ~1;
+        p.slot[q] = p.nslot;
+        p.nslot += p.K[q];
+        scratch = std::max(scratch, items);
+        if (q + 1 < nlev) {
+            const size_t Ec = g[q + 1].N + 2, planes = q < p.nclu ? (size_t)p.po[q] / 2 + 5 : Ec + 1;
+            const size_t staged = planes * Ec * (dim == 3 ? Ec : 1);
+            if (staged > 0x1fff)
+                return false;
+            scratch = std::max(scratch, staged);
+            for (int r = 0; r < csize; r++) {
+                if (plane_first(p, q, r) >= plane_first(p, q, r + 1))
+                    continue;
+                size_t cells = 0;   // ghost cells of this CTA's staged planes
+                for (int K = staged_first(p, q, r); K <= staged_last(p, q, r); K++) {
+                    const bool whole = K < 1 || K > g[q + 1].N;
+                    const size_t Nc = Ec - 2;
+                    cells += dim == 3 ? Ec * Ec - (whole ? 0 : Nc * Nc) : whole ? Ec : 2;
+                }
+                p.KG[q] = std::max(p.KG[q], (int)((cells + kT - 1) / kT));
+            }
+        }
+        const double fl = std::floor(g[q].cR);
+        p.cri[q] = (int)fl;
+        p.crf[q] = (long long)((g[q].cR - fl) * 4611686018427387904.0);
+        // fixed point: the boundary cells' diagonals can be larger than 2 d
+        double dmax = 2.0 * dim;
+        for (int c = 0; c < 64; c++) {
+            double d = mg_axis_diag(c & 3, g[q]) + mg_axis_diag((c >> 2) & 3, g[q]);
+            if (dim == 3)
+                d += mg_axis_diag((c >> 4) & 3, g[q]);
+            if (g[q].L > 0)
+                dmax = std::max(dmax, -d);
+        }
+        const int db = (int)std::ceil(std::log2(dmax / 6.0 > 1.0 ? dmax / 6.0 : 1.0));
+        p.tb[q] = std::min(57 - db - lognu, q + 1 == nlev ? 54 : 57);
+        p.top[q] = 57 - db;
+    }
+    // plan words: A of every slot, B C D of the levels with one pair per thread, ghosts (copied to
+    // shared memory), then B C D of the other levels
+    p.words = p.nslot;
+    for (int q = 0; q < nlev; q++)
+        if (p.K[q] == 1) {
+            p.bcd[q] = p.words;
+            p.words += 3;
+        }
+    for (int q = 0; q < nlev; q++) {
+        p.ghost[q] = p.words;
+        p.words += p.KG[q];
+    }
+    p.dpos = p.words++;          // word offset of every cell of the last level
+    p.nimg = p.words;
+    for (int q = 0; q < nlev; q++)
+        if (p.K[q] > 1) {
+            p.bcd[q] = p.words;
+            p.words += 3 * p.K[q];
+        }
+    p.zero16 = (int)(off * w / 16);
+    p.scratch = (int)off;
+    off = align(off + scratch);
+    p.fs = (int)off;
+    off += (size_t)2 * (p.nslot - 1) * kT;   // the last level's right-hand side is used at once
+    p.dn = 1;
+    for (int a = 0; a < dim; a++)
+        p.dn *= g[nlev - 1].N;
+    p.dmat = (int)off;
+    off = align(off + (size_t)p.dn * p.dn);
+    p.dvec = (int)off;
+    off += 64 + kT;
+    p.tabs = (int)off;
+    off = align(off + (size_t)(fp32 ? 2 : 3) * 64 * nlev);
+    p.ctrl = (int)off;
+    p.smem = off * w + (size_t)MG_SLAB_CTRL * 4 + (size_t)p.nimg * kT * 4;
+    return p.K[nlev - 1] == 1 && p.smem <= MG_SLAB_SMEM_MAX;
+}
+
+// Matrix of one V-cycle from a zero potential on levels g[0..nlev-1] (all of
+// them, down to one cell): column j holds the potential of level 0 for the
+// right-hand side h^2 f = unit vector j, cells x fastest.  FP64 on the host,
+// at most 64 cells.
+void mg_slab_dense(int dim, const MgGeom *g, int nlev, int nu_pre, int nu_post, double *mat)
+{
+    struct L {
+        int N, E, n;
+        std::vector<double> phi, f;   // (N + 2)^d, ghosts zero; f as h^2 f
+    };
+    std::vector<L> v(nlev);
+    for (int q = 0; q < nlev; q++) {
+        v[q].N = g[q].N;
+        v[q].E = g[q].N + 2;
+        v[q].n = dim == 3 ? v[q].E * v[q].E * v[q].E : v[q].E * v[q].E;
+        v[q].phi.assign(v[q].n, 0.0);
+        v[q].f.assign(v[q].n, 0.0);
+    }
+    auto id = [&](const L &l, int i, int j, int k) { return (k * l.E + j) * l.E + i; };
+    auto cells = [&](const L &l, auto &&fn) {
+        for (int k = dim == 3 ? 1 : 0; k <= (dim == 3 ? l.N : 0); k++)
+            for (int j = 1; j <= l.N; j++)
+                for (int i = 1; i <= l.N; i++)
+                    fn(i, j, k);
+    };
+    // neighbour sum and diagonal with the ghost rule folded in
+    auto stencil = [&](int q, int i, int j, int k, double &s, double &d) {
+        const L &l = v[q];
+        const MgGeom &G = g[q];
+        const int st[3] = {1, l.E, l.E * l.E}, a[3] = {i, j, k}, p = id(l, i, j, k);
+        s = d = 0.0;
+        for (int x = 0; x < dim; x++) {
+            const bool lo = a[x] == 1, hi = a[x] == l.N;
+            d += mg_axis_diag((lo ? 1 : 0) | (hi ? 2 : 0), G);
+            if (!lo && !(hi && G.tie && l.N >= 2))
+                s += l.phi[p - st[x]];
+            if (!hi)
+                s += l.phi[p + st[x]];
+        }
+    };
+    auto smooth = [&](int q, int sweeps) {
+        for (int sw = 0; sw < (v[q].N == 1 && sweeps > 0 ? 1 : sweeps); sw++)
+            for (int c = 0; c < 2; c++)
+                cells(v[q], [&](int i, int j, int k) {
+                    if (((i + j + k) & 1) != c)
+                        return;
+                    double s, d;
+                    stencil(q, i, j, k, s, d);
+                    const int p = id(v[q], i, j, k);
+                    v[q].phi[p] = (s - v[q].f[p]) / -d;
+                });
+    };
+    auto ghost = [&](int q, int I, double &c) {   // coarse index with ghosts -> active index, factor
+        const int N = v[q].N;
+        c = 1.0;
+        if (I >= 1 && I <= N)
+            return I;
+        if (I == 0) {
+            c = -1.0;
+            return 1;
+        }
+        if (g[q].tie) {
+            c = N >= 2 ? -1.0 : 1.0;
+            return N >= 2 ? N - 1 : 1;
+        }
+        c = g[q].cR;
+        return N;
+    };
+    const int N0 = v[0].N, n0 = dim == 3 ? N0 * N0 * N0 : N0 * N0;
+    for (int col = 0; col < n0; col++) {
+        std::fill(v[0].phi.begin(), v[0].phi.end(), 0.0);
+        std::fill(v[0].f.begin(), v[0].f.end(), 0.0);
+        v[0].f[id(v[0], 1 + col % N0, 1 + (col / N0) % N0, dim == 3 ? 1 + col / (N0 * N0) : 0)] = 1.0;
+        smooth(0, nu_pre);
+        for (int q = 0; q + 1 < nlev; q++) {
+            L &c = v[q + 1];
+            std::fill(c.phi.begin(), c.phi.end(), 0.0);
+            std::fill(c.f.begin(), c.f.end(), 0.0);
+            cells(v[q], [&](int i, int j, int k) {   // h_c^2 = 4 h_f^2, 2^-d average
+                const int I = (i + 1) / 2, J = (j + 1) / 2, K = (k + 1) / 2;
+                if (I > c.N || J > c.N || K > c.N)
+                    return;
+                double s, d;
+                stencil(q, i, j, k, s, d);
+                const int p = id(v[q], i, j, k);
+                c.f[id(c, I, J, K)] += (dim == 3 ? 0.5 : 1.0) * (v[q].f[p] - s - d * v[q].phi[p]);
+            });
+            smooth(q + 1, nu_pre);
+        }
+        for (int q = nlev - 2; q >= 0; q--) {
+            cells(v[q], [&](int i, int j, int k) {
+                double e = 0.0;
+                for (int m = 0; m < (1 << dim); m++) {
+                    double w = 1.0;
+                    int at[3] = {0, 0, 0};
+                    const int a[3] = {i, j, k};
+                    for (int x = 0; x < dim; x++) {
+                        const int near = (a[x] + 1) / 2, far = near + (a[x] & 1 ? -1 : 1);
+                        double c;
+                        at[x] = ghost(q + 1, (m >> x) & 1 ? far : near, c);
+                        w *= c * ((m >> x) & 1 ? 0.25 : 0.75);
+                    }
+                    e += w * v[q + 1].phi[id(v[q + 1], at[0], at[1], at[2])];
+                }
+                v[q].phi[id(v[q], i, j, k)] += e;
+            });
+            smooth(q, nu_post);
+        }
+        int row = 0;
+        cells(v[0], [&](int i, int j, int k) { mat[(size_t)col * n0 + row++] = v[0].phi[id(v[0], i, j, k)]; });
+    }
+}
+
+size_t mg_slab_image_bytes(const MgSlabPlan &p) { return (size_t)p.csize * p.words * kT * sizeof(int); }
+
+cudaError_t mg_launch_slab_plan(int dim, const MgSlabPlan &p, int *img, cudaStream_t s)
+{
+    if (dim == 3)
+        k_slab_plan<3><<<p.csize, kT, 0, s>>>(p, img);
+    else
+        k_slab_plan<2><<<p.csize, kT, 0, s>>>(p, img);
+    return cudaGetLastError();
+}
+
+cudaError_t mg_launch_slab(int dim, bool fp32, const MgSlabPlan &p, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[2];
+    slab_config(cfg, at, p.csize, p.smem, s);
+    if (fp32)
+        return dim == 3 ? cudaLaunchKernelEx(&cfg, k_slab<PrecF32, 3>, p) : cudaLaunchKernelEx(&cfg, k_slab<PrecF32, 2>, p);
+    return dim == 3 ? cudaLaunchKernelEx(&cfg, k_slab<PrecFix, 3>, p) : cudaLaunchKernelEx(&cfg, k_slab<PrecFix, 2>, p);
+}

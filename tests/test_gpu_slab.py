@@ -1,0 +1,69 @@
+"""GPU parity of the slab kernel (csrc/mg_slab.cu: the coarse part of the
+V-cycle in one thread-block cluster) with the oracle and with the one-block
+and per-phase launches, at sizes where its plan changes: one to three planes
+per CTA, empty CTAs, tie (x_N = 1) and odd levels, the smallest level."""
+import numpy as np
+import pytest
+
+from paper_2001_02327_gb300 import inputs as I
+from tests.test_gpu_parity import gpu_solve, mg, omega, random_single_level, relmax  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dim,n", [(3, 4), (3, 7), (3, 8), (3, 9), (3, 16), (3, 17), (3, 31), (3, 32), (3, 33),
+                                   (2, 6), (2, 22), (2, 23), (2, 64), (2, 127), (2, 158), (2, 159)])
+@pytest.mark.parametrize("nu", [(1, 1), (3, 0), (0, 2)])
+def test_fp64_slab_matches_oracle(mg, oracle, dim, n, nu):  # noqa: F811
+    """Fixed-point V-cycles against the FP64 oracle after three cycles on
+    random data (the parity bar of the FP64 path)."""
+    H, inp = random_single_level(dim, n, 1000 * dim + n)
+    _, g = gpu_solve(mg, H, inp, nu_pre=nu[0], nu_post=nu[1], max_cycles=3, rel_tol=0.0)
+    ref = oracle.solve_hierarchy(H, inp, nu[0], nu[1], 3, 0.0)
+    assert relmax(g[0]["phi"], omega(ref[0]["phi"], n, dim)) < 1e-12
+
+
+@pytest.mark.parametrize("dim,n", [(3, 30), (2, 126), (2, 158)])
+def test_fp64_slab_smooth_source_far_above_its_right_hand_side(mg, oracle, dim, n):  # noqa: F811
+    """A constant density with a zero boundary: the potential is thousands of
+    times the right-hand side h^2 f that fixes the first scale, so the scale
+    has to give way during the ascent."""
+    H = I.Hierarchy(dim, [n], [tuple([0.0] * dim)], 1.0 / n, 1.0, [], "const")
+    inp = [{"rho": np.ones((n,) * dim), "bc_rho": np.ones((n + 2,) * dim), "bc_phi": np.zeros((n + 4,) * dim)}]
+    _, g = gpu_solve(mg, H, inp, max_cycles=3, rel_tol=0.0)
+    ref = oracle.solve_hierarchy(H, inp, 2, 1, 3, 0.0)
+    assert relmax(g[0]["phi"], omega(ref[0]["phi"], n, dim)) < 1e-12
+
+
+@pytest.mark.parametrize("scale", [1e-130, 1e-30, 1e130])
+def test_fp64_slab_extreme_magnitudes(mg, scale):  # noqa: F811
+    """The potential scales with the data over the whole range of exponents."""
+    H, inp = random_single_level(3, 16, 5)
+    big = [{k: v * scale for k, v in inp[0].items()}]
+    _, a = gpu_solve(mg, H, inp, max_cycles=3, rel_tol=0.0)
+    _, b = gpu_solve(mg, H, big, max_cycles=3, rel_tol=0.0)
+    assert relmax(b[0]["phi"] / scale, a[0]["phi"]) < 1e-12
+
+
+@pytest.mark.parametrize("dim,n", [(3, 16), (3, 33), (3, 47), (2, 64), (2, 127)])
+@pytest.mark.parametrize("nu", [(2, 2), (1, 0), (0, 1)])
+def test_fp32_slab_matches_phase_launches(mg, monkeypatch, dim, n, nu):  # noqa: F811
+    """One FP32 correction step of two V-cycles in the slab kernel and as
+    launches per phase differ by FP32 rounding only: some 50 dependent
+    operations of 2^-24 each per cycle on a correction of the potential's own
+    size, below 1e-5 of its largest value."""
+    H, inp = random_single_level(dim, n, 77 + n)
+    kw = dict(nu_pre=nu[0], nu_post=nu[1], max_cycles=2, rel_tol=0.0, precision=mg.MG_MIXED, inner_cycles=2)
+    _, a = gpu_solve(mg, H, inp, **kw)
+    monkeypatch.setenv("MG_BOTTOM_N32", "8")
+    _, b = gpu_solve(mg, H, inp, **kw)
+    assert relmax(a[0]["phi"], b[0]["phi"]) < 1e-5
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_fp64_slab_non_finite_density_reports_ediverged(mg, bad):  # noqa: F811
+    H, inp = random_single_level(3, 16, 6)
+    inp[0]["rho"][3, 4, 5] = bad
+    with pytest.raises(mg.MGError) as ei:
+        gpu_solve(mg, H, inp, max_cycles=5, rel_tol=1e-10)
+    assert ei.value.status == mg.MG_EDIVERGED
