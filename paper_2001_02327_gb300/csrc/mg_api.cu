@@ -415,7 +415,7 @@ struct mg_hierarchy {
     size_t arena_bytes = 0;
     double *stage = nullptr;        // device staging for host-pointer I/O
     size_t stage_elems = 0;
-    double *partials = nullptr;     // MG_BRANCHES * 2 * MG_NORM_BLOCKS_MAX reduction scratch
+    double *partials = nullptr;     // MG_BRANCHES * 2 * MG_MARCH_BLOCKS reduction scratch
     unsigned *counters = nullptr;   // MG_BRANCHES block counters of the norm kernel
     unsigned long long *fmax = nullptr; // MG_BRANCHES maxima of the force-change test
     double *scal = nullptr;         // device scalars: [b][l][2] = ||b||^2, ||r||^2
@@ -953,7 +953,7 @@ cudaError_t norms(mg_hierarchy *h, const LevelData &ld, int which, double *scal,
     const bool fd = (which & 2) && fused_defect(h);
     return timed(h, KK_NORM, (fd ? 24.0 : 16.0) * cells_d(ld.g[0].N, h->dim), [&] {
         return mg_launch_norms2(h->dim, ld.phi[0], ld.f[0], ld.g[0], which,
-                                h->partials + (size_t)branch * 2 * MG_NORM_BLOCKS_MAX, h->counters + branch, scal, s,
+                                h->partials + (size_t)branch * 2 * MG_MARCH_BLOCKS, h->counters + branch, scal, s,
                                 fd ? ld.f32[0] : nullptr, fd ? ld.phi32[0] : nullptr);
     });
 }
@@ -2265,7 +2265,7 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
     }
     h->stage_elems = stage;
     slots.push_back({(void **)&h->stage, align256(stage * sizeof(double))});
-    slots.push_back({(void **)&h->partials, align256((size_t)MG_BRANCHES * 2 * MG_NORM_BLOCKS_MAX * sizeof(double))});
+    slots.push_back({(void **)&h->partials, align256((size_t)MG_BRANCHES * 2 * MG_MARCH_BLOCKS * sizeof(double))});
     slots.push_back({(void **)&h->counters, align256((size_t)MG_BRANCHES * sizeof(unsigned))});
     slots.push_back({(void **)&h->fmax, align256((size_t)MG_BRANCHES * sizeof(unsigned long long))});
     slots.push_back({(void **)&h->ctl, align256((size_t)batch * MG_MAX_LEVELS * sizeof(MgSolveCtl))});

@@ -26,7 +26,9 @@
 #include <vector>
 
 #include "../../include/mg_box.h"
+#include "mg_fix.cuh"
 #include "mg_internal.h"
+#include "mg_march.cuh"
 
 namespace {
 
@@ -39,6 +41,7 @@ struct BoxGeom {
     double cR[3];     // right ghost = cR Phi_N when !tie (Sec. 2.4)
     double ih2[3];    // 1 / h_a^2, h_a this axis's cell size on this level
     double d0, inv0;  // diagonal of a cell with no ghost folded in (-2 sum ih2) and its reciprocal
+    int iso;          // every axis has the same cell size
     int H;            // FP32 colour-split storage: cells of one colour per row, (E_x + 1) / 2
     long long half;   //   and per colour array, H E_y E_z
     float cRf[3], ih2f[3], d0f, inv0f;
@@ -101,6 +104,28 @@ __device__ __forceinline__ int gx() { return blockIdx.x * blockDim.x + threadIdx
 __device__ __forceinline__ int gy() { return blockIdx.y * blockDim.y + threadIdx.y; }
 __device__ __forceinline__ int gz() { return blockIdx.z; }
 
+// no ghost neighbour on a coarse level
+template <int DIM>
+__device__ __forceinline__ bool box_inner(const BoxGeom &g, int i, int j, int k)
+{
+    return g.L == 0 || (i > 1 && i < g.N[0] && j > 1 && j < g.N[1] && (DIM == 2 || (k > 1 && k < g.N[2])));
+}
+template <int DIM>
+__device__ __forceinline__ void box_neighbours(const double *__restrict__ phi, const BoxGeom &g, int i, int j, int k,
+                                               double (&v)[2 * DIM])
+{
+    const double *c = phi + box_index(g, i, j, k);
+    v[0] = c[-1];
+    v[1] = c[1];
+    v[2] = c[-g.E[0]];
+    v[3] = c[g.E[0]];
+    if (DIM == 3) {
+        const long long sz = (long long)g.E[0] * g.E[1];
+        v[2 * DIM - 2] = c[-sz];
+        v[2 * DIM - 1] = c[sz];
+    }
+}
+
 // The off-diagonal sum of cell (i, j, k)'s equation and what ghosts add to
 // its diagonal (Sec. 2.3 stencil, per-axis cell sizes): per axis the two
 // neighbours, except on coarse levels where a neighbour in the ghost layer is
@@ -116,6 +141,15 @@ __device__ __forceinline__ bool box_terms(const T *__restrict__ phi, const BoxGe
     const int id[3] = {i, j, k};
     other = T(0);
     fold = T(0);
+    if constexpr (sizeof(T) == sizeof(double) && !S) {
+        // equal cell sizes, no ghost: the sum on the integer pipe (mg_fix.cuh)
+        if (g.iso && box_inner<DIM>(g, i, j, k)) {
+            double v[2 * DIM];
+            box_neighbours<DIM>(phi, g, i, j, k, v);
+            other = fx_nsum<DIM>(v) * g.ih2[0];
+            return false;
+        }
+    }
     bool folded = false;
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
@@ -261,6 +295,14 @@ template <typename T, int DIM, bool S>
 __device__ __forceinline__ T box_resid(const T *__restrict__ phi, const T *__restrict__ f, const BoxGeom &g, int i,
                                        int j, int k)
 {
+    if constexpr (sizeof(T) == sizeof(double) && !S) {
+        if (g.iso && box_inner<DIM>(g, i, j, k)) {
+            double v[2 * DIM];
+            box_neighbours<DIM>(phi, g, i, j, k, v);
+            const long long p = box_index(g, i, j, k);
+            return fma(-fx_lap<DIM>(v, phi[p]), g.ih2[0], f[p]);
+        }
+    }
     T other, fold;
     box_terms<T, DIM, S>(phi, g, i, j, k, other, fold);
     const long long p = lidx<S>(g, i, j, k);
@@ -640,6 +682,34 @@ __device__ __forceinline__ double block_sum(double v)
     return s;
 }
 
+// a cell next to the ring: what its ghost neighbours take from the right-hand side (kept out of line, mg_fix.cuh)
+__device__ __noinline__ double ring_term(double res, double left, double right, double ih2)
+{
+    return res - (left + right) * ih2;
+}
+
+// The residual norm of a large 3D level 0 (mg_march.cuh), per block
+struct BoxIndex {
+    long long half;
+    int E1, H;
+    __device__ __forceinline__ long long operator()(int i, int j, int k) const
+    {
+        return ((i + j + k) & 1) * half + ((long long)k * E1 + j) * H + (i >> 1);
+    }
+};
+__global__ void __launch_bounds__(256, 5) kx_norm_march(const double *__restrict__ phi, const double *__restrict__ f,
+                                                        BoxGeom g, MarchGrid m, double *__restrict__ part,
+                                                        float *__restrict__ f32, float *__restrict__ e32)
+{
+    pdl_begin();
+    MarchResidual<BoxIndex> fn{phi, f, m.sy, m.sz, g.N[0], g.N[1], g.N[2], g.ih2[0], false, f32, e32,
+                               {g.half, g.E[1], g.H}, 0.0, 0.0, 0.0};
+    march<1, 6>(phi, m, fn);
+    const double s = block_sum(fn.r2);
+    if (threadIdx.x == 0)
+        part[blockIdx.x] = s;
+}
+
 // ||f - A Phi||^2 over the active cells of multigrid level 0 in FP64 (Sec.
 // 2.3 step 14), per block into part[blockIdx.x]; block b takes rows b,
 // b + gridDim.x, ...  zero_inside: the potential taken as zero on the active
@@ -665,19 +735,17 @@ __global__ void __launch_bounds__(kNormThreads) kx_resid_norm(const double *__re
                 // only the ghost-layer neighbours (level 0: boundary data) remain
                 const long long st[3] = {1, g.E[0], (long long)g.E[0] * g.E[1]};
                 const int id[3] = {i, j, k};
-                double other = 0.0;
-                for (int a = 0; a < DIM; a++) {
-                    const double left = id[a] == 1 ? phi[p - st[a]] : 0.0;
-                    const double right = id[a] == g.N[a] ? phi[p + st[a]] : 0.0;
-                    other = other + (left + right) * g.ih2[a];
-                }
-                res = f[p] - other;
+                res = f[p];
+                for (int a = 0; a < DIM; a++)
+                    if (id[a] == 1 || id[a] == g.N[a])
+                        res = ring_term(res, id[a] == 1 ? phi[p - st[a]] : 0.0, id[a] == g.N[a] ? phi[p + st[a]] : 0.0,
+                                        g.ih2[a]);
             } else {
                 res = box_resid<double, DIM, false>(phi, f, g, i, j, k);
             }
             if (f32) {
                 const long long q = lidx<true>(g, i, j, k);
-                f32[q] = (float)res;
+                f32[q] = fx_to_float(res);
                 e32[q] = 0.0f;
             }
             acc += res * res;
@@ -792,34 +860,19 @@ __global__ void __launch_bounds__(256) kx_interface(PatchDims dc, PatchDims dp, 
     const int ring = block_ring(dc, dim, s);
     if (mode == 1 && ring == 0)
         return;
-    const int off[3] = {o0, o1, o2};
-    int p0[3];
-    double tw[3];
-    for (int a = 0; a < 3; a++) {
-        if (a < dim) {
-            const double q = off[a] + 1.5 + (s[a] - 1.5) * 0.5;
-            p0[a] = (int)floor(q);
-            tw[a] = q - p0[a];
-        } else {
-            p0[a] = 0;
-            tw[a] = 0.0;
-        }
-    }
+    // parent coordinate off + 3/4 + s/2: the second cell weighs 3/4 where s is even
+    const int p0[3] = {o0 + ((s[0] + 1) >> 1), o1 + ((s[1] + 1) >> 1), dim == 3 ? o2 + ((s[2] + 1) >> 1) : 0};
+    const bool far[3] = {!(s[0] & 1), !(s[1] & 1), !(s[2] & 1)};
     auto interp = [&](const double *src) {
-        double v = 0.0;
-        const int nz = dim == 3 ? 2 : 1;
-        for (int cx = 0; cx < 2; cx++)
-            for (int cy = 0; cy < 2; cy++)
-                for (int cz = 0; cz < nz; cz++) {
-                    double w = 1.0;
-                    w = w * (cx ? tw[0] : 1.0 - tw[0]);
-                    w = w * (cy ? tw[1] : 1.0 - tw[1]);
-                    if (dim == 3)
-                        w = w * (cz ? tw[2] : 1.0 - tw[2]);
-                    const long long q = ((long long)(p0[2] + cz) * dp.B[1] + (p0[1] + cy)) * dp.B[0] + (p0[0] + cx);
-                    v += w * src[q];
-                }
-        return v;
+        const double *r = src + ((long long)p0[2] * dp.B[1] + p0[1]) * dp.B[0] + p0[0];
+        const long long sy = dp.B[0], sz = (long long)dp.B[0] * dp.B[1];
+        if (dim == 3) {
+            const double v[8] = {r[0],  r[1],      r[sy],      r[sy + 1],
+                                 r[sz], r[sz + 1], r[sz + sy], r[sz + sy + 1]};
+            return fx_interp<3>(v, far);
+        }
+        const double v[4] = {r[0], r[1], r[sy], r[sy + 1]};
+        return fx_interp<2>(v, far);
     };
     if (mode == 1) {
         phi_c[t] = interp(phi_p);
@@ -861,6 +914,14 @@ __global__ void __launch_bounds__(256) kx_zero_gamma(PatchDims d, int dim, doubl
 // 1/3 of the one over 4h, i2h = 1/(2h), i4h = 1/(4h); stencil 1: the
 // two-point centred difference), and the potential on Omega.  Component a at
 // F[a * cells + cell].
+__global__ void __launch_bounds__(256, 4) kx_forces_march(PatchDims d, double c, const double *__restrict__ phi, MarchGrid m,
+                                                          double *__restrict__ F, double *__restrict__ phi_out,
+                                                          int stencil)
+{
+    pdl_begin();
+    MarchForces fn{phi, m.sy, m.sz, (long long)d.n[0] * d.n[1] * d.n[2], d.n[0], d.n[1], stencil, c, F, phi_out, 0.0};
+    march<2, 5>(phi, m, fn);
+}
 __global__ void __launch_bounds__(256) kx_forces(PatchDims d, int dim, double i2h, double i4h,
                                                  const double *__restrict__ phi, double *__restrict__ F,
                                                  double *__restrict__ phi_out, int stencil)
@@ -964,6 +1025,7 @@ BoxGeom level_geom(const int n[3], int dim, double h, int L)
     g.inv0f = (float)g.inv0;
     g.H = mg_split_H(g.E[0]);   // a multiple of 4: rows start 16-byte aligned
     g.half = (long long)g.H * g.E[1] * g.E[2];
+    g.iso = g.ih2[0] == g.ih2[1] && (dim == 2 || g.ih2[0] == g.ih2[2]);
     return g;
 }
 
@@ -1201,14 +1263,25 @@ cudaError_t vcycle(const mg_box *b, const BoxPatch &P, cudaStream_t s)
     return e;
 }
 
+// Levels for the marching kernels: tiles of 32 cells along x, enough planes and cells to fill the SMs
+bool march_fits(const int *N) { return N[0] >= 64 && N[2] >= 32 && (double)N[0] * N[1] * N[2] >= 9e5; }
+
 // ||f - A Phi||^2 of level 0 into *out (zero_inside: Phi zero on Gamma);
 // mixed precision with write32: the residual also becomes the FP32 defect
 cudaError_t resid_norm(const mg_box *b, const BoxPatch &P, int zero_inside, bool write32, double *out, cudaStream_t s)
 {
     const BoxLevel &l = P.lv[0];
     float *f32 = write32 ? l.f32 : nullptr, *e32 = write32 ? l.phi32 : nullptr;
-    const int blocks = std::min(kNormBlocks, l.g.N[1] * l.g.N[2]);
-    if (b->dim == 3)
+    int blocks = std::min(kNormBlocks, l.g.N[1] * l.g.N[2]);
+    int mblocks = 0;
+    MarchGrid m{};
+    if (b->dim == 3 && !zero_inside && march_fits(l.g.N))
+        m = march_grid(l.g.N[0], l.g.N[1], l.g.N[2], l.g.E[0], (long long)l.g.E[0] * l.g.E[1], 1, &mblocks);
+    if (mblocks > 0 && mblocks <= MG_MARCH_BLOCKS) {
+        blocks = mblocks;
+        mg_launch_kernel(kx_norm_march, dim3(blocks), dim3(256), 0, s, (const double *)l.phi64, (const double *)l.f64,
+                         l.g, m, b->part, f32, e32);
+    } else if (b->dim == 3)
         mg_launch_kernel(kx_resid_norm<3>, dim3(blocks), dim3(kNormThreads), 0, s, (const double *)l.phi64,
                          (const double *)l.f64, l.g, zero_inside, b->part, f32, e32);
     else
@@ -1411,6 +1484,7 @@ BoxGeom box_from_mg(const MgGeom &g, int dim)
         b.cRf[a] = g.cRf;
         b.ih2f[a] = g.inv_h2f;
     }
+    b.iso = 1;
     b.d0 = -2.0 * dim * g.inv_h2;
     b.inv0 = 1.0 / b.d0;
     b.d0f = (float)b.d0;
@@ -1506,7 +1580,7 @@ mg_status mg_box_create(const mg_box_desc *desc, const mg_options *opt, mg_box *
     const int dim = b->dim;
     b->p.resize(desc->num_patches);
     // layout of the arena
-    size_t bytes = up256(kNormBlocks * sizeof(double));
+    size_t bytes = up256(MG_MARCH_BLOCKS * sizeof(double));
     size_t stage = 0;
     std::vector<std::vector<size_t>> offs(desc->num_patches);
     for (int l = 0; l < desc->num_patches; l++) {
@@ -1758,6 +1832,15 @@ mg_status mg_box_forces(mg_box *b, int patch, double *phi_out, double *F_out)
     const bool F_dev = F_out && device_ptr(F_out), P_dev = phi_out && device_ptr(phi_out);
     double *dF = F_out ? (F_dev ? F_out : b->stage) : nullptr;
     double *dP = phi_out ? (P_dev ? phi_out : b->stage + (size_t)dim * nr) : nullptr;
+    if (dim == 3 && march_fits(P.n)) {
+        int blocks = 0;
+        const MarchGrid m =
+            march_grid(P.n[0], P.n[1], P.n[2], P.d.B[0], (long long)P.d.B[0] * P.d.B[1], 2, &blocks);
+        mg_launch_kernel(kx_forces_march, dim3(blocks), dim3(256), 0, b->stream, P.d,
+                         -1.0 / ((b->opt.force_stencil == 0 ? 12.0 : 2.0) * P.h), (const double *)P.phi, m, dF, dP,
+                         b->opt.force_stencil);
+        BCK(b, cudaGetLastError());
+    } else
     BCK(b, launch3(kx_forces, P.n[0], P.n[1], P.n[2], b->stream, P.d, dim, 1.0 / (2.0 * P.h), 1.0 / (4.0 * P.h),
                    (const double *)P.phi, dF, dP, b->opt.force_stencil));
     bool sync = false;

@@ -240,9 +240,10 @@ cudaError_t mg_launch_prolong(int dim, bool fp32, const void *phi_c, const MgGeo
 #define MG_NORM_BLOCKS 304
 // Single-launch form: out2[0] = ||b||^2 if (which & 1), out2[1] = ||r||^2 if
 // (which & 2); the last block to finish reduces the per-block partials
-// (MG_NORM_BLOCKS_MAX doubles) in a fixed order; counter (one unsigned, zero
+// (2 MG_MARCH_BLOCKS doubles) in a fixed order; counter (one unsigned, zero
 // between launches) tracks finished blocks.
 #define MG_NORM_BLOCKS_MAX 1216
+#define MG_MARCH_BLOCKS 2280   // of the marching kernels (mg_march.cuh): three waves of 152 x 5
 // ||b||^2 / ||r||^2 of a finest level; with r32 set, also the FP32 right-hand
 // side r32 = f - A Phi and a zero correction e32 of the next defect-correction
 // step (what mg_launch_defect writes), from the same residual values.

@@ -5,21 +5,25 @@
 // the force stencil.  Arrays are C order, x fastest.
 //
 // The part runs FP64 at two FMA per clock per SM, so the FP64 kernels are
-// written to minimise double-precision operations per cell: no device
-// divisions (host tables of the boundary diagonals), neighbour folding by
-// selects rather than multiplies, separable interpolation.  Index arithmetic
-// is 32-bit.
+// written to minimise double-precision operations per cell: sums on the
+// integer pipe (mg_fix.cuh), no device divisions (host tables of the boundary
+// diagonals), neighbour folding by selects rather than multiplies, separable
+// interpolation.  Index arithmetic is 32-bit.
 #include <algorithm>
 #include <cstdlib>
 
 #include <math_constants.h>
 
+#include "mg_fix.cuh"
 #include "mg_internal.h"
+#include "mg_march.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
 constexpr int kBottomThreads = 512;
+// cells per edge from which the marching kernels (mg_march.cuh) take a 3D level
+constexpr int kMarchMinN = 96;
 
 inline int grid_for(long work, int cap = 152 * 16)
 {
@@ -115,6 +119,22 @@ __device__ __forceinline__ const double *tab_of<double>(const MgGeom &g) { retur
 template <>
 __device__ __forceinline__ const float *tab_of<float>(const MgGeom &g) { return g.tab32; }
 
+// The sum of a cell's 2 DIM neighbours: FP32 pairwise, FP64 on the integer
+// pipe, rounded once
+template <int DIM>
+__device__ __forceinline__ float pair_sum(const float (&v)[2 * DIM])
+{
+    float s = (v[0] + v[1]) + (v[2] + v[3]);
+    if (DIM == 3)
+        s += v[2 * DIM - 2] + v[2 * DIM - 1];
+    return s;
+}
+template <int DIM>
+__device__ __forceinline__ double pair_sum(const double (&v)[2 * DIM])
+{
+    return fx_nsum<DIM>(v);
+}
+
 // Ghost-folded neighbour sum of the 5/7-point Laplacian (Sec. 2.3 item 1) at
 // active cell (i,j,k) of index p, and the cell's boundary class (0 if it
 // touches no multigrid boundary, always 0 on the finest level where the outer
@@ -127,29 +147,35 @@ __device__ __forceinline__ T neighbour_sum_ptr(const T *c, const T *d, const T *
     const int N = g.N;
     const bool coarse = g.L > 0;
     const bool inner = !coarse || (i > 1 && i < N && j > 1 && j < N && (DIM == 2 || (k > 1 && k < N)));
+    T v[2 * DIM];
     if (inner) {
         cls = 0;
-        T s = (c[-1] + c[1]) + (c[-sy] + c[sy]);
-        if (DIM == 3)
-            s += d[0] + u[0];
-        return s;
+        v[0] = c[-1];
+        v[1] = c[1];
+        v[2] = c[-sy];
+        v[3] = c[sy];
+        if (DIM == 3) {
+            v[2 * DIM - 2] = d[0];
+            v[2 * DIM - 1] = u[0];
+        }
+        return pair_sum<DIM>(v);
     }
     // left neighbour dropped at index 1 (ghost = -self: goes to the diagonal)
     // and at index N when x_N = 1 (ghost = -Phi_{N-1} cancels it); right
     // neighbour dropped at index N (ghost cR Phi_N: diagonal)
     const bool tieN = g.tie && N >= 2;
     cls = 0;
-    auto axis = [&](int a, const T *lp, const T *rp, int shift) -> T {
+    auto axis = [&](int a, const T *lp, const T *rp, int x) {
         const bool lo = a == 1, hi = a == N;
-        cls |= ((lo ? 1 : 0) | (hi ? 2 : 0)) << shift;
-        const T l = (!lo && !(hi && tieN)) ? *lp : T(0);
-        const T r = !hi ? *rp : T(0);
-        return l + r;
+        cls |= ((lo ? 1 : 0) | (hi ? 2 : 0)) << (2 * x);
+        v[2 * x] = (!lo && !(hi && tieN)) ? *lp : T(0);
+        v[2 * x + 1] = !hi ? *rp : T(0);
     };
-    T s = axis(i, c - 1, c + 1, 0) + axis(j, c - sy, c + sy, 2);
+    axis(i, c - 1, c + 1, 0);
+    axis(j, c - sy, c + sy, 1);
     if (DIM == 3)
-        s += axis(k, d, u, 4);
-    return s;
+        axis(k, d, u, DIM - 1);
+    return pair_sum<DIM>(v);
 }
 
 // Ghost-folded neighbour sum at index p of an array with strides (1, sy, sz)
@@ -224,6 +250,18 @@ template <typename T, int DIM>
 __device__ __forceinline__ T residual_ptr(const T *c, const T *d, const T *u, T fv, const MgGeom &g, int i, int j,
                                           int k)
 {
+    if constexpr (sizeof(T) == sizeof(double)) {
+        // a cell without a folded ghost: the centre joins the integer sum
+        const int N = g.N;
+        if (g.L == 0 || (i > 1 && i < N && j > 1 && j < N && (DIM == 2 || (k > 1 && k < N)))) {
+            T v[2 * DIM] = {c[-1], c[1], c[-g.E], c[g.E]};
+            if (DIM == 3) {
+                v[2 * DIM - 2] = d[0];
+                v[2 * DIM - 1] = u[0];
+            }
+            return fma(-fx_lap<DIM>(v, c[0]), g.inv_h2, fv);
+        }
+    }
     int cls;
     const T other = neighbour_sum_ptr<T, DIM>(c, d, u, g, i, j, k, g.E, cls);
     return fv - (other + diag_of<T, DIM>(g, cls) * c[0]) * geo_inv_h2<T>(g);
@@ -309,6 +347,45 @@ __device__ __forceinline__ void ghost_map(int q, const MgGeom &gc, int &idx, T &
 template <typename T, int DIM, typename Planes>
 __device__ __forceinline__ T prolong_combine(const Planes &plane, int Ec, const int (&idx)[3][2], const T (&w)[3][2])
 {
+    if constexpr (sizeof(T) == sizeof(double)) {
+        // without a ghost among the coarse cells the weights are 3/4 and 1/4
+        // on every axis: 27, 9, 3, 1 of the 2^d values on the integer pipe
+        bool plain = true;
+        for (int a = 0; a < DIM; a++)
+            plain = plain && __double_as_longlong(w[a][0]) == 0x3fe8000000000000ll &&
+                    __double_as_longlong(w[a][1]) == 0x3fd0000000000000ll;
+        if (plain) {
+            T v[1 << DIM];
+            int e = 0;
+#pragma unroll
+            for (int m = 0; m < (1 << DIM); m++) {
+                v[m] = plane(DIM == 3 ? idx[2][m >> 2] : 0)[idx[1][(m >> 1) & 1] * Ec + idx[0][m & 1]];
+                e = max(e, fx_exp(v[m]));
+            }
+            if (fx_ok(e)) {
+                long long s[1 << DIM];
+#pragma unroll
+                for (int m = 0; m < (1 << DIM); m++)
+                    s[m] = fx_align<4>(v[m], e);   // weights of 64 in all: 2^6 2^57
+#pragma unroll
+                for (int n = (1 << DIM) / 2; n >= 1; n /= 2)
+#pragma unroll
+                    for (int m = 0; m < n; m++)
+                        s[m] = 3 * s[2 * m] + s[2 * m + 1];
+                return fx_round<4 + 2 * DIM>(s[0], e);
+            }
+        }
+    }
+    if constexpr (sizeof(T) == sizeof(double)) {
+        T z[2] = {};
+        for (int c = 0; c < (DIM == 3 ? 2 : 1); c++) {
+            const T *pl = plane(DIM == 3 ? idx[2][c] : 0);
+            const T *r0 = pl + idx[1][0] * Ec, *r1 = pl + idx[1][1] * Ec;
+            z[c] = fx_rare_mix2(r0[idx[0][0]], r0[idx[0][1]], r1[idx[0][0]], r1[idx[0][1]], w[0][0], w[0][1], w[1][0],
+                                w[1][1]);
+        }
+        return DIM == 3 ? fx_rare_add(fx_rare_mul(w[2][0], z[0]), fx_rare_mul(w[2][1], z[1])) : z[0];
+    }
     if (DIM == 3) {
         T zsum = T(0);
         for (int c = 0; c < 2; c++) {
@@ -342,8 +419,17 @@ __device__ __forceinline__ void prolong_axis(int v, const MgGeom &gc, int &i0, i
     T c0, c1;
     ghost_map<T>(near, gc, i0, c0);
     ghost_map<T>(far, gc, i1, c1);
-    w0 = T(0.75) * c0;
-    w1 = T(0.25) * c1;
+    if constexpr (sizeof(T) == sizeof(double)) {   // FP64 products for ghosts only
+        w0 = T(0.75);
+        w1 = T(0.25);
+        if (near < 1 || near > gc.N)
+            w0 = fx_rare_mul(0.75, c0);
+        if (far < 1 || far > gc.N)
+            w1 = fx_rare_mul(0.25, c1);
+    } else {
+        w0 = T(0.75) * c0;
+        w1 = T(0.25) * c1;
+    }
 }
 
 // P(Phi_c) at fine active cell f
@@ -617,13 +703,14 @@ __device__ __forceinline__ T bottom_plan_nsum(const T *c, int e, int sy, int sz,
     const T *a1 = (e >> (B + 1)) & 1 ? zero : c + 1;
     const T *a2 = (e >> (B + 2)) & 1 ? zero : c - sy;
     const T *a3 = (e >> (B + 3)) & 1 ? zero : c + sy;
-    T s = (*a0 + *a1) + (*a2 + *a3);
+    T v[2 * DIM] = {*a0, *a1, *a2, *a3};
     if (DIM == 3) {
         const T *a4 = (e >> (B + 4)) & 1 ? zero : c - sz;
         const T *a5 = (e >> (B + 5)) & 1 ? zero : c + sz;
-        s += *a4 + *a5;
+        v[2 * DIM - 2] = *a4;
+        v[2 * DIM - 1] = *a5;
     }
-    return s;
+    return pair_sum<DIM>(v);
 }
 
 // one colour of a red-black sweep (the arithmetic of op_smooth_colour)
@@ -678,6 +765,17 @@ __device__ __forceinline__ void bottom_plan_restrict(const T *__restrict__ phi_f
             continue;
         const int p = e & M;
         const T *c = phi_f + p;
+        if constexpr (sizeof(T) == sizeof(double)) {
+            if (!(e >> kPlanCellBits)) {   // no folded ghost: the sum of residual_ptr
+                T v[2 * DIM] = {c[-1], c[1], c[-Ef], c[Ef]};
+                if (DIM == 3) {
+                    v[2 * DIM - 2] = c[-sz];
+                    v[2 * DIM - 1] = c[sz];
+                }
+                r[p] = fma(-fx_lap<DIM>(v, c[0]), ih2, f_f[p]);
+                continue;
+            }
+        }
         const T other = bottom_plan_nsum<T, DIM>(c, e, Ef, sz, zero);
         r[p] = f_f[p] - (other + Pf.dg[t] * c[0]) * ih2;
     }
@@ -1453,14 +1551,16 @@ __device__ __forceinline__ void norm_terms(const double *__restrict__ phi, const
     }
     const int p = lin<DIM>(i, j, k, E);
     if (which & 1) {
-        double o = 0.0;
-        if (i == 1) o += phi[p - 1];
-        if (i == N) o += phi[p + 1];
-        if (j == 1) o += phi[p - E];
-        if (j == N) o += phi[p + E];
-        if (DIM == 3) {
-            if (k == 1) o += phi[p - E * E];
-            if (k == N) o += phi[p + E * E];
+        double o = 0.0;   // the ring's part: cells next to it only
+        if (i == 1 || i == N || j == 1 || j == N || (DIM == 3 && (k == 1 || k == N))) {
+            if (i == 1) o = fx_rare_add(o, phi[p - 1]);
+            if (i == N) o = fx_rare_add(o, phi[p + 1]);
+            if (j == 1) o = fx_rare_add(o, phi[p - E]);
+            if (j == N) o = fx_rare_add(o, phi[p + E]);
+            if (DIM == 3) {
+                if (k == 1) o = fx_rare_add(o, phi[p - E * E]);
+                if (k == N) o = fx_rare_add(o, phi[p + E * E]);
+            }
         }
         const double v = f[p] - o * g.inv_h2;
         b2 += v * v;
@@ -1470,26 +1570,19 @@ __device__ __forceinline__ void norm_terms(const double *__restrict__ phi, const
         r2 += v * v;
         if (r32) {   // the next defect-correction step's right-hand side (k_defect's values)
             const long long q = mg_idx32(g, DIM, i, j, k);
-            r32[q] = (float)v;
+            r32[q] = fx_to_float(v);
             e32[q] = 0.0f;
         }
     }
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(kThreads) k_norms2(const double *__restrict__ phi, const double *__restrict__ f,
-                                                     MgGeom g, int which, double *__restrict__ partials,
-                                                     unsigned *__restrict__ counter, double *__restrict__ out2,
-                                                     float *__restrict__ r32, float *__restrict__ e32)
+// Block sums of b2 and r2 (which bits 0, 1) into out2, the blocks' parts added in
+// a fixed order by the last block to finish.
+__device__ __forceinline__ void norms_reduce(double b2, double r2, int which, double *__restrict__ partials,
+                                             unsigned *__restrict__ counter, double *__restrict__ out2)
 {
-    pdl_begin();
     __shared__ double sm[kThreads / 32];
     __shared__ bool last;
-    const int N = g.N;
-    const int total = N * N * (DIM == 3 ? N : 1);
-    double b2 = 0.0, r2 = 0.0;
-    for (int t = gtid(); t < total; t += gstride())
-        norm_terms<DIM>(phi, f, g, t, which, b2, r2, r32, e32);
     // FP64 reductions cost FP64-pipe time: reduce only what was asked for
     if (which & 1)
         b2 = block_sum(b2, sm);
@@ -1521,6 +1614,41 @@ __global__ void __launch_bounds__(kThreads) k_norms2(const double *__restrict__ 
             out2[1] = sr;
         *counter = 0u;
     }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kThreads) k_norms2(const double *__restrict__ phi, const double *__restrict__ f,
+                                                     MgGeom g, int which, double *__restrict__ partials,
+                                                     unsigned *__restrict__ counter, double *__restrict__ out2,
+                                                     float *__restrict__ r32, float *__restrict__ e32)
+{
+    pdl_begin();
+    const int N = g.N;
+    const int total = N * N * (DIM == 3 ? N : 1);
+    double b2 = 0.0, r2 = 0.0;
+    for (int t = gtid(); t < total; t += gstride())
+        norm_terms<DIM>(phi, f, g, t, which, b2, r2, r32, e32);
+    norms_reduce(b2, r2, which, partials, counter, out2);
+}
+
+// The same for the large 3D levels (mg_march.cuh), bound by the instruction
+// count.  At 258^3 with the fused defect: 379 us with FP64 instructions, 220 us
+// with integer sums per cell, 193 us here; the bytes take 60 us.  Below 96 cells
+// per edge there are too few columns and the per-cell kernel is the faster.
+struct SplitIndex {
+    MgGeom g;
+    __device__ __forceinline__ long long operator()(int i, int j, int k) const { return mg_idx32(g, 3, i, j, k); }
+};
+__global__ void __launch_bounds__(256, 5) k_norms_march(const double *__restrict__ phi, const double *__restrict__ f,
+                                                        MgGeom g, MarchGrid m, int which,
+                                                        double *__restrict__ partials, unsigned *__restrict__ counter,
+                                                        double *__restrict__ out2, float *__restrict__ r32,
+                                                        float *__restrict__ e32)
+{
+    pdl_begin();
+    MarchResidual<SplitIndex> fn{phi, f, m.sy, m.sz, g.N, g.N, g.N, g.inv_h2, (which & 1) != 0, r32, e32, {g}, 0.0, 0.0, 0.0};
+    march<1, 6>(phi, m, fn);
+    norms_reduce(fn.b2, fn.r2, which, partials, counter, out2);
 }
 
 // Two-launch form kept for the allocation-free entry point.
@@ -1575,7 +1703,7 @@ __global__ void __launch_bounds__(kThreads) k_defect(const double *__restrict__ 
             k = 0;
         }
         const long long q = mg_idx32(g, DIM, i, j, k);
-        r32[q] = (float)residual_at<double, DIM>(phi, f, g, i, j, k);
+        r32[q] = fx_to_float(residual_at<double, DIM>(phi, f, g, i, j, k));
         e32[q] = 0.0f;
     }
 }
@@ -1659,17 +1787,16 @@ __device__ __forceinline__ void iface_axis(int s, int off, int &p0, double &t)
 template <int DIM>
 __device__ __forceinline__ double interp(const double *__restrict__ src, int Ep, const int *p0, const double *t)
 {
-    double zs = 0.0;
-    for (int dk = 0; dk < (DIM == 3 ? 2 : 1); dk++) {
-        double ys = 0.0;
-        for (int dj = 0; dj < 2; dj++) {
-            const int row = DIM == 3 ? ((p0[2] + dk) * Ep + p0[1] + dj) * Ep : (p0[1] + dj) * Ep;
-            const double xv = (1.0 - t[0]) * src[row + p0[0]] + t[0] * src[row + p0[0] + 1];
-            ys += (dj ? t[1] : 1.0 - t[1]) * xv;
-        }
-        zs += DIM == 3 ? (dk ? t[2] : 1.0 - t[2]) * ys : ys;
+    double v[1 << DIM];
+#pragma unroll
+    for (int m = 0; m < (1 << DIM); m++) {
+        const int row = DIM == 3 ? ((p0[2] + (m >> 2)) * Ep + p0[1] + ((m >> 1) & 1)) * Ep : (p0[1] + (m >> 1)) * Ep;
+        v[m] = src[row + p0[0] + (m & 1)];
     }
-    return zs;
+    // t is 3/4 or 1/4: compared by its bits, not on the FP64 pipe
+    const bool far[3] = {__double2hiint(t[0]) == 0x3fe80000, __double2hiint(t[1]) == 0x3fe80000,
+                         DIM == 3 && __double2hiint(t[2]) == 0x3fe80000};
+    return fx_interp<DIM>(v, far);
 }
 
 // Storage index of the r-th cell of the two outer rings of a block of edge E
@@ -1780,11 +1907,13 @@ __global__ void __launch_bounds__(kThreads) k_interface(int np, const double *__
 // The interpolated initial guess (Sec. 2.4; Appendix A) on Omega of a child
 // level: per work item the 2^d children s = 2 sigma, 2 sigma + 1 along each
 // axis, which share 3^d parent centres (off + sigma .. off + sigma + 2).  The
-// x interpolation of each parent row serves both children planes, the y
-// combination both child z planes -- about half of interp's FP64 operations
-// per cell, with interp's arithmetic per cell (x, then y, then z).
+// centres are aligned to one exponent and combined as integers (weights 3 and 1
+// per axis), the x interpolation of each parent row serving both children
+// planes, the y combination both child z planes, and each child rounded once:
+// bound by the integer pipe (about 110 instructions a child).  Unusual
+// exponents (mg_fix.cuh) take interp per child.
 template <int DIM>
-__global__ void __launch_bounds__(kThreads) k_iface_guess(int np, const double *__restrict__ phi_p, int nc, int ox,
+__global__ void __launch_bounds__(kThreads, 3) k_iface_guess(int np, const double *__restrict__ phi_p, int nc, int ox,
                                                           int oy, int oz, double *__restrict__ phi_c)
 {
     pdl_begin();
@@ -1798,42 +1927,51 @@ __global__ void __launch_bounds__(kThreads) k_iface_guess(int np, const double *
         const int sy = DIM == 3 ? r - rq * hc : r, sz = DIM == 3 ? rq : 0;
         // parent cells off + sigma .. off + sigma + 2, sigma = s + 1
         const int bx = ox + sx + 1, by = oy + sy + 1, bz = DIM == 3 ? oz + sz + 1 : 0;
-        double xv[NZ][3][2];   // [parent z row][parent y row][child x: even, odd]
+        auto row = [&](int pz, int py) {
+            return phi_p + (DIM == 3 ? ((bz + pz) * Ep + by + py) * Ep : (by + py) * Ep) + bx;
+        };
+        // the largest exponent from the high words (the rows are read again
+        // below: 27 doubles held would leave one block per SM)
+        int e = 0;
+#pragma unroll
+        for (int pz = 0; pz < NZ; pz++)
+#pragma unroll
+            for (int py = 0; py < 3; py++)
+#pragma unroll
+                for (int px = 0; px < 3; px++)
+                    e = max(e, reinterpret_cast<const int *>(row(pz, py) + px)[1] & 0x7ff00000);
+        e >>= 20;
+        const bool ok = fx_ok(e);
+        // the second parent weighs 3/4 for the even child, 1/4 for the odd one
+        long long xv[NZ][3][2];   // [parent z row][parent y row][child x: even, odd]
 #pragma unroll
         for (int pz = 0; pz < NZ; pz++)
 #pragma unroll
             for (int py = 0; py < 3; py++) {
-                const int row = DIM == 3 ? ((bz + pz) * Ep + by + py) * Ep : (by + py) * Ep;
-                const double a = phi_p[row + bx], b = phi_p[row + bx + 1], c = phi_p[row + bx + 2];
-                const double te = 0.75, to = 0.25;   // weight of the second parent: even child, odd child
-                xv[pz][py][0] = (1.0 - te) * a + te * b;
-                xv[pz][py][1] = (1.0 - to) * b + to * c;
+                const double *v = row(pz, py);
+                const long long a = fx_align<4>(v[0], e), b = fx_align<4>(v[1], e), c = fx_align<4>(v[2], e);
+                xv[pz][py][0] = a + 3 * b;
+                xv[pz][py][1] = 3 * b + c;
             }
 #pragma unroll
         for (int cx = 0; cx < 2; cx++)
 #pragma unroll
             for (int cy = 0; cy < 2; cy++) {
-                const double t1 = cy ? 0.25 : 0.75;
-                double ys[NZ];
+                long long ys[NZ];
 #pragma unroll
-                for (int pz = 0; pz < NZ; pz++) {
-                    double v = 0.0;
-                    v += (1.0 - t1) * xv[pz][cy][cx];
-                    v += t1 * xv[pz][cy + 1][cx];
-                    ys[pz] = v;
-                }
+                for (int pz = 0; pz < NZ; pz++)
+                    ys[pz] = 3 * xv[pz][1][cx] + xv[pz][2 * cy][cx];
 #pragma unroll
                 for (int cz = 0; cz < (DIM == 3 ? 2 : 1); cz++) {
-                    double zs = 0.0;
-                    if (DIM == 3) {
-                        const double t2 = cz ? 0.25 : 0.75;
-                        zs += (1.0 - t2) * ys[cz];
-                        zs += t2 * ys[cz + 1];
-                    } else {
-                        zs += ys[0];
-                    }
                     const int i = 2 * (sx + 1) + cx, j = 2 * (sy + 1) + cy, k = DIM == 3 ? 2 * (sz + 1) + cz : 0;
-                    phi_c[lin<DIM>(i, j, k, E)] = zs;
+                    const long long zs = DIM == 3 ? 3 * ys[NZ / 2] + ys[cz ? NZ - 1 : 0] : ys[0];
+                    double out = fx_round<4 + 2 * DIM>(zs, e);
+                    if (!ok) {
+                        const int p0[3] = {bx + cx, by + cy, bz + cz};
+                        const double w[3] = {cx ? 0.25 : 0.75, cy ? 0.25 : 0.75, cz ? 0.25 : 0.75};
+                        out = interp<DIM>(phi_p, Ep, p0, w);
+                    }
+                    phi_c[lin<DIM>(i, j, k, E)] = out;
                 }
             }
     }
@@ -1873,7 +2011,17 @@ __global__ void __launch_bounds__(kThreads) k_copy_guess(int n, const double *__
     }
 }
 
-// F = -grad(Phi) on Omega: Eq. 2 (stencil 0) or the two-point difference.
+// One component of -grad(Phi) at p along the axis of stride st: Eq. 2 (stencil
+// 0) or the two-point difference; c = -1 / (12 h) or -1 / (2 h).
+__device__ __forceinline__ double force_at(const double *__restrict__ phi, int p, int st, double c, int stencil)
+{
+    const double a = phi[p + st], b = phi[p - st];
+    if (stencil != 0)
+        return c * (a - b);
+    return c * fx_diff4(a, b, phi[p + 2 * st], phi[p - 2 * st]);
+}
+
+// F = -grad(Phi) on Omega
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_forces(int n, double h, const double *__restrict__ phi,
                                                      double *__restrict__ F, double *__restrict__ phi_out, int stencil)
@@ -1881,8 +2029,7 @@ __global__ void __launch_bounds__(kThreads) k_forces(int n, double h, const doub
     pdl_begin();
     const int E = n + 4;
     const int total = n * n * (DIM == 3 ? n : 1);
-    const double c1 = stencil == 0 ? (4.0 / 3.0) / (2.0 * h) : 1.0 / (2.0 * h);
-    const double c2 = stencil == 0 ? (1.0 / 3.0) / (4.0 * h) : 0.0;
+    const double c = -1.0 / ((stencil == 0 ? 12.0 : 2.0) * h);
     for (int t = gtid(); t < total; t += gstride()) {
         const int r = div_small(t, n);
         const int i = t - r * n + 2;
@@ -1891,14 +2038,24 @@ __global__ void __launch_bounds__(kThreads) k_forces(int n, double h, const doub
         const int k = DIM == 3 ? rq + 2 : 0;
         const int p = lin<DIM>(i, j, k, E);
         const int st[3] = {1, E, E * E};
-        for (int a = 0; a < DIM; a++) {
-            const double d1 = phi[p + st[a]] - phi[p - st[a]];
-            const double d2 = phi[p + 2 * st[a]] - phi[p - 2 * st[a]];
-            F[(long)a * total + t] = -(c1 * d1 - c2 * d2);
-        }
+#pragma unroll
+        for (int a = 0; a < DIM; a++)
+            F[(long)a * total + t] = force_at(phi, p, st[a], c, stencil);
         if (phi_out)
             phi_out[t] = phi[p];
     }
+}
+
+// The same for large 3D levels (mg_march.cuh): 500 us at 256^3 with FP64
+// instructions, 275 us with integer sums per cell, 190 us here; the bytes take
+// 100 us.
+__global__ void __launch_bounds__(256, 4) k_forces_march(int n, double c, const double *__restrict__ phi, MarchGrid m,
+                                                         double *__restrict__ F, double *__restrict__ phi_out,
+                                                         int stencil)
+{
+    pdl_begin();
+    MarchForces fn{phi, m.sy, m.sz, (long long)n * n * n, n, n, stencil, c, F, phi_out, 0.0};
+    march<2, 5>(phi, m, fn);
 }
 
 // Stopping test of Sec. 3: max over Omega of |F(phi) - F(prev)|^2 into *cmax
@@ -2187,7 +2344,7 @@ __global__ void __launch_bounds__(kThreads) kb_defect(const MgBPart *__restrict_
         int i, j, k;
         active_cell<DIM>(g, t, i, j, k);
         const long long q = mg_idx32(g, DIM, i, j, k);
-        P.f32[0][q] = (float)residual_at<double, DIM>(P.phi, P.f, g, i, j, k);
+        P.f32[0][q] = fx_to_float(residual_at<double, DIM>(P.phi, P.f, g, i, j, k));
         P.phi32[0][q] = 0.0f;
     }
 }
@@ -2496,8 +2653,7 @@ __device__ void persist_level(const MgBPart &P, int nu_pre, int nu_post, double 
     if (P.out_F) {   // registered outputs: potential and forces of Eq. 2 (or the two-point difference)
         const int n = P.n;
         const int total = n * n * (DIM == 3 ? n : 1);
-        const double c1 = stencil == 0 ? (4.0 / 3.0) / (2.0 * P.h) : 1.0 / (2.0 * P.h);
-        const double c2 = stencil == 0 ? (1.0 / 3.0) / (4.0 * P.h) : 0.0;
+        const double c = -1.0 / ((stencil == 0 ? 12.0 : 2.0) * P.h);
         for (int t = tid; t < total; t += nth) {
             const int r = div_small(t, n);
             const int i = t - r * n + 2;
@@ -2506,11 +2662,8 @@ __device__ void persist_level(const MgBPart &P, int nu_pre, int nu_post, double 
             const int k = DIM == 3 ? rq + 2 : 0;
             const int p = lin<DIM>(i, j, k, E);
             const int st[3] = {1, E, E * E};
-            for (int a = 0; a < DIM; a++) {
-                const double d1 = P.phi[p + st[a]] - P.phi[p - st[a]];
-                const double d2 = P.phi[p + 2 * st[a]] - P.phi[p - 2 * st[a]];
-                P.out_F[(long)a * total + t] = -(c1 * d1 - c2 * d2);
-            }
+            for (int a = 0; a < DIM; a++)
+                P.out_F[(long)a * total + t] = force_at(P.phi, p, st[a], c, stencil);
             if (P.out_phi)
                 P.out_phi[t] = P.phi[p];
         }
@@ -2821,6 +2974,14 @@ cudaError_t mg_launch_prolong(int dim, bool fp32, const void *phi_c, const MgGeo
 cudaError_t mg_launch_norms2(int dim, const double *phi, const double *f, const MgGeom &g, int which,
                              double *partials, unsigned *counter, double *out2, cudaStream_t s, float *r32, float *e32)
 {
+    if (dim == 3 && g.N >= kMarchMinN && (which & 2)) {
+        int blocks = 0;
+        const MarchGrid m = march_grid(g.N, g.N, g.N, g.E, (long long)g.E * g.E, 1, &blocks);
+        if (blocks <= MG_MARCH_BLOCKS) {
+            mg_launch_kernel(k_norms_march, blocks, 256, 0, s, phi, f, g, m, which, partials, counter, out2, r32, e32);
+            return cudaGetLastError();
+        }
+    }
     // about four cells per thread: fewer block reductions on the FP64 pipe
     const int grid = std::max(1, std::min<int>((int)((cube(g.N, dim) + 4 * kThreads - 1) / (4 * kThreads)), MG_NORM_BLOCKS_MAX));
     if (dim == 3)
@@ -2910,6 +3071,14 @@ cudaError_t mg_launch_copy_guess(int dim, int n, const double *guess_src, double
 cudaError_t mg_launch_forces(int dim, int n, double h, const double *phi_blk, double *F, double *phi_out, int stencil,
                              cudaStream_t s)
 {
+    if (dim == 3 && n >= kMarchMinN) {
+        int blocks = 0;
+        const int E = n + 4;
+        const MarchGrid m = march_grid(n, n, n, E, (long long)E * E, 2, &blocks);
+        mg_launch_kernel(k_forces_march, blocks, 256, 0, s, n, -1.0 / ((stencil == 0 ? 12.0 : 2.0) * h), phi_blk, m, F,
+                         phi_out, stencil);
+        return cudaGetLastError();
+    }
     const int grid = grid_for(cube(n, dim));
     if (dim == 3)
         mg_launch_kernel(k_forces<3>, grid, kThreads, 0, s, n, h, phi_blk, F, phi_out, stencil);
