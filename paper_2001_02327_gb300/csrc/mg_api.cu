@@ -655,7 +655,7 @@ mg_status wave_status(mg_hierarchy *h)
         return fail_cuda(h, e, "reading the device error word");
     if (w) {
         h->poisoned = true;
-        return fail(h, MG_ETIMEOUT, "a plane-marching sweep's load wait ran out of its clock budget");
+        return fail(h, MG_ETIMEOUT, "a device-side wait ran out of its clock budget");
     }
     return MG_OK;
 }
@@ -768,6 +768,17 @@ cudaError_t plan_slab(mg_hierarchy *h, LevelData &ld, bool on)
     return cudaSuccess;
 }
 
+// A launch of the slab kernel runs every kind of phase: it counts under each,
+// its time and bytes under the bottom's.
+template <class Fn>
+cudaError_t timed_slab(mg_hierarchy *h, double bytes, Fn &&fn)
+{
+    if (h->prof.on)
+        for (int kind : {KK_SMOOTH, KK_RESTRICT, KK_PROLONG})
+            h->prof.launches[kind]++;
+    return timed(h, KK_BOTTOM, bytes, fn);
+}
+
 // the V-cycle of Sec. 2.3 (steps 2-13) on the arrays of one refinement level,
 // `ncyc` times; the levels from Lc down run in the cluster kernel (when
 // Lc < Ls), those from Ls down in the one-block kernel
@@ -814,13 +825,9 @@ cudaError_t vcycle(mg_hierarchy *h, const LevelData &ld, bool fp32, cudaStream_t
             p.ctl = ctl;
             p.hi = hi;
         }
-        // one launch that runs every kind of phase: it counts under each, its
-        // time and bytes under the bottom's
-        if (h->prof.on)
-            for (int kind : {KK_SMOOTH, KK_RESTRICT, KK_PROLONG})
-                h->prof.launches[kind]++;
-        return timed(h, KK_BOTTOM, 3.0 * w * cells_d(ld.g[Lslab].E, dim) * cycles,
-                     [&] { return mg_launch_slab(dim, fp32, p, s); });
+        p.err = h->werr;
+        return timed_slab(h, 3.0 * w * cells_d(ld.g[Lslab].E, dim) * cycles,
+                          [&] { return mg_launch_slab(dim, fp32, p, s); });
     };
     cudaError_t e;
     if (Lstop == 0) {                                                                     // whole cycle
@@ -1107,6 +1114,29 @@ cudaError_t level_iteration(mg_hierarchy *h, int b, int l, cudaStream_t s, int b
     return norms(h, ld, 2, level_scal(h, b, l), s, branch);
 }
 
+// True when one launch of the slab kernel runs all V-cycles of a level and
+// decides after each whether to go on: FP64 levels that it holds whole, under
+// the residual stopping rule.
+bool slab_solves(const mg_hierarchy *h, const LevelData &ld)
+{
+    return h->opt.precision != MG_MIXED && h->opt.stop == MG_STOP_RESIDUAL && ld.Lslab[0] == 0;
+}
+
+// That launch, after level_prelude; level_ctl gets the result.
+cudaError_t slab_solve(mg_hierarchy *h, int b, int l, cudaStream_t s)
+{
+    const LevelData &ld = h->lev[b][l];
+    MgSlabPlan p = ld.slab;
+    p.cycles = h->opt.max_cycles;
+    p.solve = 1;
+    p.tol = h->opt.rel_tol;
+    p.scal = level_scal(h, b, l);
+    p.ctl = level_ctl(h, b, l);
+    p.err = h->werr;
+    return timed_slab(h, 3.0 * 8.0 * cells_d(ld.g[0].E, h->dim),
+                      [&] { return mg_launch_slab(h->dim, false, p, s); });
+}
+
 int cycles_per_iteration(const mg_hierarchy *h) { return h->opt.precision == MG_MIXED ? h->opt.inner_cycles : 1; }
 
 void fill_stats(const mg_hierarchy *h, const MgSolveCtl &c, mg_level_stats *st)
@@ -1150,9 +1180,16 @@ mg_status solve_level_host(mg_hierarchy *h, int b, int l, mg_level_stats *st)
     c.rel = c.bnorm > 0.0 ? std::sqrt(hs[1]) / c.bnorm : 0.0;
     if (!std::isfinite(c.bnorm))
         c.status = 1;
+    if (slab_solves(h, h->lev[b][l])) {
+        CK(h, slab_solve(h, b, l, s));
+        CK(h, cudaMemcpyAsync(h->hctl, level_ctl(h, b, l), sizeof(MgSolveCtl), cudaMemcpyDeviceToHost, s));
+        CK(h, cudaStreamSynchronize(s));
+        c = h->hctl[0];
+    }
     const bool adapt = adaptive_inner(h);
     int inner = o.inner_cycles;   // adaptive: FP32 V-cycles of the next step, as the graph's ctl kernels choose
-    while (c.bnorm > 0.0 && c.status == 0 && c.cycles < o.max_cycles && !(c.rel < o.rel_tol)) {
+    while (!slab_solves(h, h->lev[b][l]) && c.bnorm > 0.0 && c.status == 0 && c.cycles < o.max_cycles &&
+           !(c.rel < o.rel_tol)) {
         const int ncyc = adapt ? std::min(inner, o.max_cycles - c.cycles) : cycles_per_iteration(h);
         CK(h, level_iteration(h, b, l, s, 0, ncyc));
         CK(h, cudaMemcpyAsync(hs, ds, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1212,6 +1249,11 @@ cudaError_t capture_level(mg_hierarchy *h, int b, int l, cudaStream_t s, int bra
     cudaError_t e = cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, nullptr, nullptr, nullptr);
     if (e)
         return e;
+    if (slab_solves(h, h->lev[b][l])) {
+        if ((e = level_prelude(h, b, l, s, branch)) || (e = slab_solve(h, b, l, s)))
+            return e;
+        return level_epilogue(h, b, l, s);
+    }
     cudaGraphConditionalHandle hc;
     if ((e = cudaGraphConditionalHandleCreate(&hc, g, 0, cudaGraphCondAssignDefault)))
         return e;

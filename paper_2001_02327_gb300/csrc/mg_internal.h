@@ -135,8 +135,8 @@ struct MgClusterPlan {
 // FP32, or FP64 arrays computed in 64-bit fixed point.
 #define MG_SLAB_THREADS 512
 #define MG_SLAB_MAXLEV 12
-#define MG_SLAB_MAXK 6                 // pairs of cells per thread and level
-#define MG_SLAB_CTRL (72 * MG_SLAB_MAXLEV)   // control words in shared memory
+#define MG_SLAB_MAXK 4                 // pairs of cells per thread and level
+#define MG_SLAB_CTRL (81 * MG_SLAB_MAXLEV)       // control words in shared memory (a multiple of 4)
 #define MG_SLAB_SMEM_MAX (226 * 1024)
 struct MgSolveCtl;
 struct MgSlabPlan {
@@ -163,8 +163,16 @@ struct MgSlabPlan {
                                    // fixed point * 2^60
     void *phi;                     // the first level's global arrays
     const void *f;
+    long long h2k;                 // fixed point: h^2 of the first level = h2k 2^(h2e - 62)
+    int h2e;
     MgSolveCtl *ctl;               // not NULL: the launch also counts one V-cycle of a nested loop (condition hi)
     cudaGraphConditionalHandle hi;
+    // solve (FP64, the plan's first level the finest): V-cycles until ||r|| <
+    // tol ||b|| or `cycles` of them, from scal = {||b||^2, ||r||^2}; *ctl gets the result
+    int solve;
+    double tol;
+    const double *scal;
+    int *err;                      // MG_ETIMEOUT once a wait for a neighbour's values ran out
 };
 int mg_slab_prepare();             // CTAs per cluster (0: unavailable); once per device before the first launch
 bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, int cut, int nu_pre, int nu_post,

@@ -16,8 +16,12 @@
 //     memory, written once per level configuration and copied to shared memory
 //     before the kernel waits for its predecessor, so no phase divides;
 //   - each CTA keeps copies of its neighbours' boundary planes, and the owner
-//     pushes every new value into the copies by distributed shared memory
-//     stores, which the phase's barrier completes: sweeps load locally only;
+//     pushes every new value into the copies, so that sweeps load locally only;
+//     a colour pass waits for its two neighbours' values alone (asynchronous
+//     stores that count their bytes on an mbarrier, about 300 cycles) and not at
+//     a barrier of the whole cluster (about 600 with its stores);
+//   - a thread holds its cells' right-hand sides and coefficients in registers
+//     from sweep to sweep;
 //   - the first red half-sweep on a level (whose correction starts from zero)
 //     is done with the restriction into it, the potential that a finer level
 //     interpolates is copied to where it reads it right after the level's last
@@ -25,7 +29,16 @@
 //   - from the first level of at most 64 cells down, one V-cycle from a zero
 //     correction is a fixed linear map of that level's right-hand side: its
 //     matrix is built once (in FP64) and applied as a matrix-vector product,
-//     one phase in place of the 25 or so of those levels.
+//     one phase in place of the 25 or so of those levels;
+//   - an FP64 level that fits whole is solved by one launch: the V-cycles of its
+//     loop, the residual norm and the decision after each.  Loading the level
+//     (4 us), its norm kernel, the control kernel and the turn of the graph's
+//     loop then happen once per solve and not once per cycle: a hierarchy of
+//     three 16^3 levels 2.05 -> 1.28 ms, of three 64^2 levels 1.35 -> 0.90 ms
+//     (one launch per phase: 2.73 and 2.34 ms).
+//
+// One V-cycle, launch to launch: 33^3 31 us in FP32 and 47 us in FP64, 17^3 15
+// us (FP32), 18^3 30 us and 66^2 28 us (FP64).
 //
 // FP64 V-cycles run in 64-bit fixed point.  The part issues one FP64
 // instruction per sub-partition every 64 cycles but a 64-bit integer addition
@@ -40,13 +53,17 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <type_traits>
 #include <vector>
+
+#include <math_constants.h>
 
 #include "mg_internal.h"
 
 namespace {
 
 constexpr int kT = MG_SLAB_THREADS;
+constexpr long long kWaitCycles = 2000000000ll;   // bound of one wait, about 1 s
 
 typedef long long fix;   // fixed-point value: real * 2^scale
 
@@ -90,6 +107,37 @@ __device__ __forceinline__ void ld_cluster(float &v, unsigned a)
 __device__ __forceinline__ void ld_cluster(long long &v, unsigned a)
 {
     asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+}
+// a store that counts its bytes on the mbarrier `mb` of the same CTA
+__device__ __forceinline__ void st_async(unsigned a, float v, unsigned mb)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a),
+                 "r"(__float_as_uint(v)), "r"(mb)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async(unsigned a, long long v, unsigned mb)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a), "l"(v), "r"(mb)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_init(unsigned mb)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned mb, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(unsigned mb, unsigned parity)
+{
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok)
+                 : "r"(mb), "r"(parity)
+                 : "memory");
+    return ok != 0;
 }
 template <typename T>
 __device__ __forceinline__ unsigned shared_addr(const T *p)
@@ -174,7 +222,8 @@ struct PrecFix {
 //      coarse planes; 14, 15 the far row, plane is the next one (else previous)
 //   C  bits 0-13 index of the first child pair in the finer level's pair sums;
 //      14-17 CTA of the first child plane, 18-21 of the second; 22 the second
-//      plane, 23 the second row exists; 24 the second plane is the first of its CTA
+//      plane, 23 the second row exists; 24 the second plane is the first of its
+//      CTA; 25-28 the first plane's index within its CTA
 //   D  level 0: x (bits 0-9), row (10-19), plane (20-29); other levels: bits
 //      0-12 index of the odd cell within a staged plane, 13-16 the first CTA
 //      that interpolates from this plane, 17-20 how many do, 21-30 the plane
@@ -239,8 +288,10 @@ __host__ __device__ void plan_item(const MgSlabPlan &p, int q, int rank, int t, 
 {
     const Shape s = shape_of<DIM>(p, q, rank);
     w[0] = w[1] = w[2] = w[3] = 0;
-    if (t >= s.total)
+    if (t >= s.total) {
+        w[kA] = s.R * s.H + (DIM == 3 ? s.H : 0);   // inside the slab
         return;
+    }
     const int x = t % s.ha, r = t / s.ha;
     const int j = DIM == 3 ? r % s.rows + 1 : 0, kk = r / s.rows, k = s.k0 + kk;
     const int b = ((kk + 1) * s.R + j) * s.H + x;
@@ -274,7 +325,8 @@ __host__ __device__ void plan_item(const MgSlabPlan &p, int q, int rank, int t, 
         const bool pl2 = k1 + 1 <= Nf, row2 = DIM == 3 && 2 * j <= Nf;
         const int o2 = pl2 ? plane_owner(p, q - 1, k1 + 1) : o1;
         w[kC] = (((k1 - plane_first(p, q - 1, o1)) * rowsf + row) * haf + 2 * x) | (o1 << 14) | (o2 << 18) |
-                ((pl2 ? 1 : 0) << 22) | ((row2 ? 1 : 0) << 23) | ((o2 != o1 ? 1 : 0) << 24);
+                ((pl2 ? 1 : 0) << 22) | ((row2 ? 1 : 0) << 23) | ((o2 != o1 ? 1 : 0) << 24) |
+                (((k1 - plane_first(p, q - 1, o1)) & 15) << 25);
     }
 }
 
@@ -365,6 +417,8 @@ struct Engine {
     static constexpr int kW = sizeof(T);
     const MgSlabPlan &pl;
     int rank, tid;
+    unsigned npass = 0;     // colour passes on distributed levels so far (the same in every CTA)
+    unsigned phase = 0;     // phase bits of the four mbarriers: [from the previous, next CTA][even, odd pass]
 
     __device__ explicit Engine(const MgSlabPlan &p) : pl(p), rank((int)cluster_rank_()), tid((int)threadIdx.x) {}
 
@@ -386,6 +440,18 @@ struct Engine {
     // potentials at MAXLEV + q; orw: over this CTA, slots: of every CTA
     __device__ __forceinline__ unsigned *orw() const { return reinterpret_cast<unsigned *>(ctrl() + 2 * MG_SLAB_MAXLEV); }
     __device__ __forceinline__ unsigned *slots() const { return orw() + 4 * MG_SLAB_MAXLEV; }
+    // per level, of the CTAs with the planes before and after its own: byte
+    // address of their copies of its first and last plane, and of their
+    // mbarriers for this CTA's values (0: none)
+    __device__ __forceinline__ unsigned *nbr() const { return slots() + 64 * MG_SLAB_MAXLEV; }
+    // this CTA's mbarriers: values from the previous (dir 0) and the next CTA, even and odd passes
+    __device__ __forceinline__ unsigned mbar(int dir, int par) const
+    {
+        return shared_addr(nbr() + 4 * MG_SLAB_MAXLEV) + 8 * (2 * dir + par);
+    }
+    __device__ __forceinline__ int *failed() const { return reinterpret_cast<int *>(nbr() + 4 * MG_SLAB_MAXLEV + 8); }
+    // norm of the residual: 16 warps' and 16 CTAs' sums, the total
+    __device__ __forceinline__ double *sums() const { return reinterpret_cast<double *>(nbr() + 4 * MG_SLAB_MAXLEV + 10); }
     __device__ __forceinline__ int *img() const { return ctrl() + MG_SLAB_CTRL; }
     __device__ __forceinline__ const int *gimg() const { return pl.img + (size_t)rank * pl.words * kT; }
 
@@ -410,29 +476,84 @@ struct Engine {
     // copies of its first and last plane (byte address of the same word)
     struct Lev {
         int ph, cs, H, RH;
-        unsigned prev, next;
+        unsigned prev, next, mprev, mnext;
         bool tie;
     };
     __device__ __forceinline__ Lev level(int q) const
     {
-        const Shape s = shape_of<DIM>(pl, q, rank);
         Lev L;
         L.ph = pl.off[q];
-        L.cs = s.cs;
-        L.H = s.H;
-        L.RH = s.R * s.H;
-        L.tie = pl.g[q].L > 0 && pl.g[q].tie && s.N >= 2;
-        L.prev = L.next = 0u;
-        if (dist(q) && s.total > 0) {
-            const unsigned w0 = shared_addr(W());
-            if (s.k0 > 1) {
-                const int o = plane_owner(pl, q, s.k0 - 1);
-                L.prev = cluster_addr(w0, o) + (s.k0 - plane_first(pl, q, o)) * L.RH * kW;
-            }
-            if (s.k1 <= s.N)
-                L.next = cluster_addr(w0, plane_owner(pl, q, s.k1)) - (s.k1 - s.k0) * L.RH * kW;
-        }
+        L.H = (pl.g[q].N + 3) >> 1;
+        L.RH = (DIM == 3 ? pl.g[q].N + 2 : 1) * L.H;
+        L.cs = (pl.po[q] + 2) * L.RH;
+        L.tie = pl.g[q].L > 0 && pl.g[q].tie && pl.g[q].N >= 2;
+        L.prev = nbr()[4 * q];
+        L.next = nbr()[4 * q + 1];
+        L.mprev = nbr()[4 * q + 2];
+        L.mnext = nbr()[4 * q + 3];
         return L;
+    }
+    // the addresses level() reads, and the neighbours' mbarriers beside them (one thread per level)
+    __device__ __forceinline__ void find_neighbours(int q) const
+    {
+        const Shape s = shape_of<DIM>(pl, q, rank);
+        unsigned *n = nbr() + 4 * q;
+        n[0] = n[1] = n[2] = n[3] = 0u;
+        if (!dist(q) || s.total == 0)
+            return;
+        const unsigned w0 = shared_addr(W());
+        const int RH = s.R * s.H;
+        if (s.k0 > 1) {
+            const int o = plane_owner(pl, q, s.k0 - 1);
+            n[0] = cluster_addr(w0, o) + (s.k0 - plane_first(pl, q, o)) * RH * kW;
+            n[2] = cluster_addr(mbar(1, 0), o);
+        }
+        if (s.k1 <= s.N) {
+            const int o = plane_owner(pl, q, s.k1);
+            n[1] = cluster_addr(w0, o) - (s.k1 - s.k0) * RH * kW;
+            n[3] = cluster_addr(mbar(0, 0), o);
+        }
+    }
+    // bytes of colour c of plane k that a neighbour sends
+    __device__ __forceinline__ unsigned plane_bytes(int q, int c, int k) const
+    {
+        const int N = pl.g[q].N, cells = DIM == 3 ? N * N : N;
+        // 3D: i + j even for half of the cells and the odd one; 2D: i odd
+        const bool more = DIM == 3 ? ((c + k) & 1) == 0 : ((c + k) & 1) == 1;
+        return (unsigned)(kW * ((cells + (more ? 1 : 0)) >> 1));
+    }
+    // After a colour pass on level q: the neighbours' new values have arrived
+    // (bounded: a wait that runs out marks the launch failed, after which no
+    // further wait waits) and every thread of this CTA has written its own.
+    __device__ __forceinline__ void pass_sync(int q, const Lev &L, int c)
+    {
+        if (!dist(q)) {
+            __syncthreads();
+            return;
+        }
+        const int par = npass & 1;
+        npass++;
+        if (tid == 0) {
+            if (L.mprev)
+                mbar_expect(mbar(0, par), plane_bytes(q, c, plane_first(pl, q, rank) - 1));
+            if (L.mnext)
+                mbar_expect(mbar(1, par), plane_bytes(q, c, plane_first(pl, q, rank + 1)));
+        }
+#pragma unroll
+        for (int dir = 0; dir < 2; dir++)
+            if (dir ? L.mnext : L.mprev) {
+                const unsigned bit = 1u << (2 * dir + par);
+                if (!mbar_try(mbar(dir, par), phase & bit ? 1u : 0u) && !*failed()) {
+                    const long long t0 = clock64();
+                    while (!mbar_try(mbar(dir, par), phase & bit ? 1u : 0u))
+                        if (clock64() - t0 > kWaitCycles) {
+                            *failed() = 1;
+                            break;
+                        }
+                }
+                phase ^= bit;
+            }
+        __syncthreads();
     }
 
     __device__ __forceinline__ static int cls_odd(int A) { return ((A >> 21) & 3) | ((A >> 15) & 0x3c); }
@@ -441,6 +562,8 @@ struct Engine {
     __device__ __forceinline__ static int s_of(int A, int c) { return ((A >> 14) & 1) ^ c; }
     __device__ __forceinline__ static bool has(int A, int c) { return (A >> (15 + s_of(A, c))) & 1; }
 
+    // a new value into this CTA's slab and (plain stores, completed by a
+    // cluster barrier) the neighbours' copies
     __device__ __forceinline__ void put(const Lev &L, int A, int i, T v) const
     {
         W()[i] = v;
@@ -449,6 +572,17 @@ struct Engine {
                 st_cluster(L.prev + i * kW, v);
             if ((A >> 25) & 1)
                 st_cluster(L.next + i * kW, v);
+        }
+    }
+    // the same in a colour pass, the copies by stores that pass_sync waits for
+    __device__ __forceinline__ void put_async(const Lev &L, int A, int i, T v, unsigned mb) const
+    {
+        W()[i] = v;
+        if ((A >> 24) & 3) {
+            if ((A >> 24) & 1)
+                st_async(L.prev + i * kW, v, L.mprev + mb);
+            if ((A >> 25) & 1)
+                st_async(L.next + i * kW, v, L.mnext + mb);
         }
     }
 
@@ -482,20 +616,18 @@ struct Engine {
         return DIM == 3 ? (sx + sy) + sz : sx + sz;
     }
 
-    // What a thread needs of K of its pairs to sweep: per pair the plan word,
-    // and per colour the right-hand side and the reciprocal diagonal.  A level
-    // of one pair per thread keeps them in registers from sweep to sweep; the
-    // others read two pairs at a time from shared memory in every sweep, which
-    // keeps the code small enough for the instruction cache.
+    // What a thread keeps of K of its pairs of a level while it sweeps: per
+    // pair the plan word, and per colour the right-hand side and the reciprocal
+    // diagonal.  Pairs that do not exist point at a cell inside the slab, so
+    // everything but the stores is done for all of them without a branch, and
+    // the loads of several pairs are in flight together.
     template <int K>
     struct Items {
         int A[K];
         T f[2][K], n[2][K];
     };
-
-    // pairs u0 .. u0 + K - 1 of level q, colours c0 .. c1
     template <int K>
-    __device__ __forceinline__ void load_items(int q, int u0, Items<K> &it, bool with_f, int c0 = 0, int c1 = 1) const
+    __device__ __forceinline__ void load_items(int q, int u0, Items<K> &it, bool with_f) const
     {
         const int slot = pl.slot[q] + u0;
         const T *tb = tab(q);
@@ -505,30 +637,41 @@ struct Engine {
             it.A[u] = A;
 #pragma unroll
             for (int c = 0; c < 2; c++) {
-                it.n[c][u] = it.f[c][u] = T(0);
-                if (c < c0 || c > c1)
-                    continue;
                 it.n[c][u] = tb[s_of(A, c) ? cls_even(A) : cls_odd(A)];
-                if (with_f)
-                    it.f[c][u] = fs()[(2 * (slot + u) + c) * kT + tid];
+                it.f[c][u] = with_f ? fs()[(2 * (slot + u) + c) * kT + tid] : T(0);
             }
         }
     }
-
-    // fn(items, u0) over all pairs of level q: in registers already (one pair), or two at a time
-    template <bool ONE, class It, class Fn>
-    __device__ __forceinline__ void pairs(int q, It &it, int c0, int c1, Fn &&fn) const
+    // All K pairs of a thread on a level: held in registers from phase to
+    // phase, or (more than two in 64 bits) read two at a time in each phase:
+    // the kernel's shared memory leaves the L1 cache no room for spills.  A warp
+    // without pairs skips the phases.
+    template <int K>
+    struct Held {
+        static constexpr bool kStream = kFix && K > 2;
+        Items<kStream ? 1 : K> it;
+        bool on;
+    };
+    template <int K>
+    __device__ __forceinline__ void hold(int q, Held<K> &h, bool with_f) const
     {
-        if constexpr (ONE) {
-            if (__any_sync(0xffffffffu, (it.A[0] >> 15) & 1))   // a warp without pairs skips the phase
-                fn(it, 0);
-        } else {
-            const int K = pl.K[q];
+        if constexpr (!Held<K>::kStream)
+            load_items(q, 0, h.it, with_f);
+        h.on = K > 1 || __any_sync(0xffffffffu, (h.it.A[0] >> 15) & 1);
+    }
+    template <int K, typename Fn>
+    __device__ __forceinline__ void each(int q, Held<K> &h, Fn &&fn) const
+    {
+        if constexpr (Held<K>::kStream) {
 #pragma unroll 1
-            for (int u0 = 0; u0 < K; u0 += 2) {
-                load_items<2>(q, u0, it, true, c0, c1);
-                fn(it, u0);
+            for (int u = 0; u < K; u += 2) {
+                Items<2> it;
+                load_items(q, u, it, true);
+                if (__any_sync(0xffffffffu, (it.A[0] >> 15) & 1))
+                    fn(it, u);
             }
+        } else if (h.on) {
+            fn(h.it, 0);
         }
     }
 
@@ -540,19 +683,24 @@ struct Engine {
             return (s - pl.g[q].h2f * f) * n;
     }
 
-    // colour c of a red-black sweep
+    // colour c of a red-black sweep; send: the neighbours need the new values
     template <int c, int K>
-    __device__ __forceinline__ void pass(int q, const Lev &L, const Items<K> &it) const
+    __device__ __forceinline__ void pass(int q, const Lev &L, const Items<K> &it, bool send) const
     {
+        const unsigned mb = 8 * (npass & 1);
         T v[K];
 #pragma unroll
         for (int u = 0; u < K; u++)
-            if (has(it.A[u], c))
-                v[u] = update(q, nsum(L, it.A[u], c, s_of(it.A[u], c)), it.f[c][u], it.n[c][u]);
+            v[u] = update(q, nsum(L, it.A[u], c, s_of(it.A[u], c)), it.f[c][u], it.n[c][u]);
 #pragma unroll
         for (int u = 0; u < K; u++)
-            if (has(it.A[u], c))
-                put(L, it.A[u], L.ph + c * L.cs + (it.A[u] & 0x3fff) + s_of(it.A[u], c), v[u]);
+            if (has(it.A[u], c)) {
+                const int i = L.ph + c * L.cs + (it.A[u] & 0x3fff) + s_of(it.A[u], c);
+                if (send)
+                    put_async(L, it.A[u], i, v[u], mb);
+                else
+                    W()[i] = v[u];
+            }
     }
 
     // OR of the magnitudes m over this CTA into word pair w of orw
@@ -614,20 +762,21 @@ struct Engine {
             const int A = it.A[u];
             T sum = T(0);
 #pragma unroll
-            for (int c = 0; c < 2; c++)
-                if (has(A, c)) {
-                    const int s = s_of(A, c), cls = s ? cls_even(A) : cls_odd(A);
-                    const T ns = nsum(L, A, c, s);
-                    const T v = W()[L.ph + c * L.cs + (A & 0x3fff) + s];
-                    if constexpr (kFix) {
-                        T d = (2 * DIM) * v;
-                        if (cls)
-                            d = tb[64 + cls] * v + qmul<30>(v, tb[128 + cls]);
-                        sum += it.f[c][u] - ns + d;
-                    } else {
-                        sum += it.f[c][u] - (ns + tb[64 + cls] * v) * ih2;
-                    }
+            for (int c = 0; c < 2; c++) {
+                const int s = s_of(A, c), cls = s ? cls_even(A) : cls_odd(A);
+                const T ns = nsum(L, A, c, s);
+                const T v = W()[L.ph + c * L.cs + (A & 0x3fff) + s];
+                T d;
+                if constexpr (kFix) {
+                    d = (2 * DIM) * v;
+                    if (cls)
+                        d = tb[64 + cls] * v + qmul<30>(v, tb[128 + cls]);
+                    d = it.f[c][u] - ns + d;
+                } else {
+                    d = it.f[c][u] - (ns + tb[64 + cls] * v) * ih2;
                 }
+                sum += has(A, c) ? d : T(0);
+            }
             if ((A >> 15) & 1)
                 scratch()[tid + (u0 + u) * kT] = sum;
             if constexpr (kFix)
@@ -650,7 +799,7 @@ struct Engine {
     // The right-hand sides of K pairs of level q: the 2^d-child average (step
     // 5) of level q - 1's residual.
     template <int K>
-    __device__ __forceinline__ void restrict_into(int q, int u0, Items<K> &it, int sh, bool keep) const
+    __device__ __forceinline__ void restrict_into(int q, Items<K> &it, int u0, int sh, bool keep) const
     {
         const bool dup = dist(q - 1);
         const int slot = pl.slot[q] + u0;
@@ -663,7 +812,7 @@ struct Engine {
             if ((A >> 15) & 1) {
                 const int w = word(q, u0 + u, kC);
                 const bool even = (A >> 16) & 1, row2 = DIM == 3 && ((w >> 23) & 1), pl2 = (w >> 22) & 1;
-                const int i1 = w & 0x3fff, i2 = (w >> 24) & 1 ? i1 % planef : i1 + planef;
+                const int i1 = w & 0x3fff, i2 = (w >> 24) & 1 ? i1 - ((w >> 25) & 15) * planef : i1 + planef;
                 T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0), c0 = T(0), c1 = T(0), d0 = T(0), d1 = T(0);
                 auto quad = [&](auto &&ld) {
                     ld(a0, 0, i1);
@@ -866,7 +1015,7 @@ struct Engine {
     // Prolongation and correction (step 10) of K pairs of level q from the
     // staged planes of level q + 1.
     template <int K>
-    __device__ __forceinline__ void prolong_from(int q, int u0, const Lev &L, const Items<K> &it, int sh) const
+    __device__ __forceinline__ void prolong_from(int q, const Lev &L, const Items<K> &it, int u0, int sh) const
     {
         const int Ec = pl.g[q + 1].N + 2, ps = (DIM == 3 ? Ec : 1) * Ec;
         // 3/4 - 1/4 interpolation along one axis
@@ -910,51 +1059,47 @@ struct Engine {
 
     // descent on level q: its right-hand side from the finer level (q > 0),
     // pre-smoothing, residual; the last level is solved
-    template <bool ONE>
-    __device__ __forceinline__ void descend(int q, bool fresh) const
+    template <int K>
+    __device__ __forceinline__ void descend(int q, bool fresh)
     {
         const Lev L = level(q);
         const bool cl = dist(q);
-        Items<ONE ? 1 : 2> it;
+        Held<K> h;
         if constexpr (kFix)
             clear_or(MG_SLAB_MAXLEV + q);
         const bool red = q > 0 || fresh, last = q + 1 == pl.nlev;
-        if (q > 0) {
-            int sh = 0;
-            if constexpr (kFix)
+        hold(q, h, q == 0);
+        int sh = 0;
+        if constexpr (kFix)
+            if (q > 0)
                 sh = restrict_scale(q);
-            const int K = pl.K[q];
-#pragma unroll 1
-            for (int u0 = 0; u0 < K; u0 += ONE ? 1 : 2) {
-                load_items(q, u0, it, false);
-                restrict_into(q, u0, it, sh, !last);
-                if (!last)
-                    first_red(q, L, it);
+        if constexpr (K == 1)
+            if (last) {
+                if (h.on)
+                    restrict_into(q, h.it, 0, sh, false);
+                dense_solve(q, L, h.it);
+                return;
             }
-            if constexpr (ONE)
-                if (last) {
-                    dense_solve(q, L, it);
-                    return;
-                }
-        } else {
-            if constexpr (ONE)
-                load_items(0, 0, it, true);
-            if (fresh)
-                pairs<ONE>(q, it, 0, 1, [&](auto &t, int) { first_red(q, L, t); });
-        }
-        if (red)
+        if (red) {
+            each(q, h, [&](auto &it, int u0) {
+                if (q > 0)
+                    restrict_into(q, it, u0, sh, true);
+                first_red(q, L, it);
+            });
             sync(cl);
+        }
+        auto colour = [&](auto c) {
+            each(q, h, [&](auto &it, int) { this->template pass<decltype(c)::value>(q, L, it, true); });
+            pass_sync(q, L, decltype(c)::value);
+        };
 #pragma unroll 1
         for (int s = 0; s < pl.nu_pre; s++) {
-            if (s > 0 || !red) {
-                pairs<ONE>(q, it, 0, 0, [&](auto &t, int) { this->template pass<0>(q, L, t); });
-                sync(cl);
-            }
-            pairs<ONE>(q, it, 1, 1, [&](auto &t, int) { this->template pass<1>(q, L, t); });
-            sync(cl);
+            if (s > 0 || !red)
+                colour(std::integral_constant<int, 0>());
+            colour(std::integral_constant<int, 1>());
         }
         fix big = 0;
-        pairs<ONE>(q, it, 0, 1, [&](auto &t, int u0) { big |= residual(q, L, t, u0); });
+        each(q, h, [&](auto &it, int u0) { big |= residual(q, L, it, u0); });
         if constexpr (kFix) {
             block_or(big, q);
             if (cl)
@@ -963,34 +1108,128 @@ struct Engine {
         sync(cl);
     }
 
-    // ascent on level q: correction from level q + 1, post-smoothing (after
-    // the last sweep the own cells alone are read: no barrier)
-    template <bool ONE>
-    __device__ __forceinline__ void ascend(int q, bool last) const
+    // ascent on level q: correction from level q + 1, post-smoothing (the
+    // last sweep of a level that publishes is read by its own thread alone: no
+    // barrier, nothing sent)
+    template <int K>
+    __device__ __forceinline__ void ascend(int q, bool last)
     {
         const Lev L = level(q);
         const bool cl = dist(q);
-        Items<ONE ? 1 : 2> it;
+        Held<K> h;
         int sh = 0;
         if constexpr (kFix) {
             clear_or(q);
             sh = prolong_scale(q, L);
         }
         fill_ghosts(q);
-        if constexpr (ONE)
-            load_items(q, 0, it, true);
+        hold(q, h, true);
         __syncthreads();
-        pairs<ONE>(q, it, 0, 1, [&](auto &t, int u0) { prolong_from(q, u0, L, t, sh); });
+        each(q, h, [&](auto &it, int u0) { prolong_from(q, L, it, u0, sh); });
         const bool fin = q > 0 || last;
         sync(cl);   // also: no CTA may publish into staged planes that another still reads
 #pragma unroll 1
         for (int s = 0; s < pl.nu_post; s++) {
-            pairs<ONE>(q, it, 0, 0, [&](auto &t, int) { this->template pass<0>(q, L, t); });
-            sync(cl);
-            pairs<ONE>(q, it, 1, 1, [&](auto &t, int) { this->template pass<1>(q, L, t); });
-            if (!fin || s + 1 < pl.nu_post)
-                sync(cl);
+            const bool end = fin && s + 1 == pl.nu_post;
+            each(q, h, [&](auto &it, int) { this->template pass<0>(q, L, it, true); });
+            pass_sync(q, L, 0);
+            each(q, h, [&](auto &it, int) { this->template pass<1>(q, L, it, !end); });
+            if (!end)
+                pass_sync(q, L, 1);
         }
+    }
+
+    __device__ __forceinline__ void descend_any(int q, bool fresh)
+    {
+        if (pl.K[q] == 1)
+            descend<1>(q, fresh);
+        else if (pl.K[q] == 2)
+            descend<2>(q, fresh);
+        else
+            descend<4>(q, fresh);
+    }
+    __device__ __forceinline__ void ascend_any(int q, bool last)
+    {
+        if (pl.K[q] == 1)
+            ascend<1>(q, last);
+        else if (pl.K[q] == 2)
+            ascend<2>(q, last);
+        else
+            ascend<4>(q, last);
+    }
+
+    // One V-cycle on the levels of the plan
+    __device__ __forceinline__ void cycle(bool fresh, bool last)
+    {
+        // a level in CTA 0 alone: the other CTAs wait for its staged planes
+        int q = 0;
+        for (;; q++) {
+            if (dist(q) || rank == 0)
+                descend_any(q, fresh);
+            if (q + 1 == pl.nlev)
+                break;
+        }
+        for (; q > 0; q--) {
+            if (dist(q) || rank == 0)
+                publish(q, level(q));
+            if (dist(q - 1))
+                cluster_sync_();
+            else if (rank == 0)
+                __syncthreads();
+            if (dist(q - 1) || rank == 0)
+                ascend_any(q - 1, last);
+        }
+    }
+
+    // x 2^e (e any)
+    __device__ __forceinline__ static double scaled(double x, int e) { return scalbn(scalbn(x, e / 2), e - e / 2); }
+    // |h^2 r|^2 over level 0 in units of 2^(-2 scale): every CTA gets the sum,
+    // added in a fixed order
+    __device__ __forceinline__ double square_sum(int K) const
+    {
+        const Lev L = level(0);
+        double acc = 0.0;
+#pragma unroll 1
+        for (int u = 0; u < K; u++) {
+            Items<1> it;
+            load_items(0, u, it, true);
+            const int A = it.A[0];
+#pragma unroll
+            for (int c = 0; c < 2; c++)
+                if (has(A, c)) {
+                    const int s = s_of(A, c);
+                    const fix v = W()[L.ph + c * L.cs + (A & 0x3fff) + s];
+                    const double r = from_fix(it.f[c][0] - nsum(L, A, c, s) + (2 * DIM) * v, 0);
+                    acc = fma(r, r, acc);
+                }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            acc += __shfl_down_sync(0xffffffffu, acc, o);
+        double *sm = sums();
+        if ((tid & 31) == 0)
+            sm[tid >> 5] = acc;
+        __syncthreads();
+        if (tid < 32) {
+            acc = tid < kT / 32 ? sm[tid] : 0.0;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+                acc += __shfl_down_sync(0xffffffffu, acc, o);
+            acc = __shfl_sync(0xffffffffu, acc, 0);
+            if (tid < pl.csize)
+                st_cluster(cluster_addr(shared_addr(sm + 16 + rank), tid), __double_as_longlong(acc));
+        }
+        cluster_sync_();
+        if (tid < 32) {
+            acc = tid < pl.csize ? sm[16 + tid] : 0.0;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+                acc += __shfl_down_sync(0xffffffffu, acc, o);
+            if (tid == 0)
+                sm[32] = acc;
+        }
+        __syncthreads();
+        return sm[32];
     }
 
     // coefficient tables of every level, the dense matrix
@@ -1035,7 +1274,7 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
     typedef typename P::T T;
     typedef typename P::G G;
     __shared__ unsigned s_max[2], s_all[2][16];
-    const Engine<P, DIM> en(pl);
+    Engine<P, DIM> en(pl);
     const int tid = threadIdx.x, rank = en.rank, C = pl.csize;
     const int wid = tid >> 5, lane = tid & 31, nw = kT / 32;
     // before the predecessor has finished: the plan image, the tables, the
@@ -1056,6 +1295,13 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
     if (tid < 2)
         s_max[tid] = 0u;
     __syncthreads();
+    if (tid < 4) {
+        mbar_init(en.mbar(tid >> 1, tid & 1));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (tid < pl.nlev)
+        en.find_neighbours(tid);
+    cluster_sync_();   // every CTA has started: its shared memory may be written
     pdl_begin();
     const Shape S = shape_of<DIM>(pl, 0, rank);
     const MgGeom &g0 = pl.g[0];
@@ -1066,23 +1312,16 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
     // level 0 of the plan from global memory: the right-hand side to its
     // threads, the potential (with its ring) to the slab, a warp per row
     unsigned mphi = 0, mf = 0;
-    for (int u = 0; u < pl.K[0]; u++) {
-        const int A = en.word_a(u), d = en.word(0, u, kD);
-        const int x = d & 0x3ff, j = (d >> 10) & 0x3ff, k = d >> 20;
-        G o = G(0), e = G(0);
-        if ((A >> 15) & 1)
-            o = gf[gidx(2 * x + 1, j, k)];
-        if ((A >> 16) & 1)
-            e = gf[gidx(2 * x + 2, j, k)];
-        const bool odd0 = ((A >> 14) & 1) == 0;
-        const G r = odd0 ? o : e, b = odd0 ? e : o;
-        if constexpr (P::kFix) {
-            en.fs()[(2 * u) * kT + tid] = __double_as_longlong(r);
-            en.fs()[(2 * u + 1) * kT + tid] = __double_as_longlong(b);
-            mf = max(mf, max((unsigned)__double2hiint(r) & 0x7fffffffu, (unsigned)__double2hiint(b) & 0x7fffffffu));
-        } else {
-            en.fs()[(2 * u) * kT + tid] = r;
-            en.fs()[(2 * u + 1) * kT + tid] = b;
+    G fo[MG_SLAB_MAXK], fe[MG_SLAB_MAXK];
+#pragma unroll
+    for (int u = 0; u < MG_SLAB_MAXK; u++) {
+        fo[u] = fe[u] = G(0);
+        if (u < pl.K[0] && ((en.word_a(u) >> 15) & 1)) {
+            const int d = en.word(0, u, kD);
+            const G *src = gf + gidx(2 * (d & 0x3ff) + 1, (d >> 10) & 0x3ff, d >> 20);
+            fo[u] = src[0];
+            if ((en.word_a(u) >> 16) & 1)
+                fe[u] = src[1];
         }
     }
     if (!pl.zero_start && S.total > 0) {
@@ -1114,17 +1353,30 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
                 }
             }
     }
+    // right-hand sides by colour to their threads' words
+    auto keep = [&](auto &&conv) {
+#pragma unroll
+        for (int u = 0; u < MG_SLAB_MAXK; u++)
+            if (u < pl.K[0]) {
+                const bool odd0 = ((en.word_a(u) >> 14) & 1) == 0;
+                en.fs()[(2 * u) * kT + tid] = conv(odd0 ? fo[u] : fe[u]);
+                en.fs()[(2 * u + 1) * kT + tid] = conv(odd0 ? fe[u] : fo[u]);
+            }
+    };
     bool bad = false;
     if constexpr (P::kFix) {
         // the scale of the plan's first level from the largest magnitudes over
         // the cluster; infinities and NaN make every result NaN
+#pragma unroll
+        for (int u = 0; u < MG_SLAB_MAXK; u++)
+            mf = max(mf, max((unsigned)__double2hiint(fo[u]) & 0x7fffffffu, (unsigned)__double2hiint(fe[u]) & 0x7fffffffu));
         mphi = __reduce_max_sync(0xffffffffu, mphi);
         mf = __reduce_max_sync(0xffffffffu, mf);
         if (lane == 0) {
             atomicMax(&s_max[0], mphi);
             atomicMax(&s_max[1], mf);
         }
-        cluster_sync_();   // every CTA has started: its shared memory may be written
+        __syncthreads();
         if (tid < C) {
             st_cluster(cluster_addr(shared_addr(&s_all[0][rank]), tid), s_max[0]);
             st_cluster(cluster_addr(shared_addr(&s_all[1][rank]), tid), s_max[1]);
@@ -1136,75 +1388,87 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
             mf = max(mf, s_all[1][t]);
         }
         bad = mphi >= 0x7ff00000u || mf >= 0x7ff00000u;
-        const int gb = mf ? exp_bound(mf) + exp_bound((unsigned)__double2hiint(g0.h2)) : -4000;
+        const int gb = mf ? exp_bound(mf) + pl.h2e : -4000;   // h^2 = h2k 2^(h2e - 62)
         const int s0 = mf || mphi ? pl.tb[0] - max(gb, exp_bound(mphi)) : 0;
         if (tid == 0)
             en.sc()[0] = s0;
         if (!pl.zero_start)
             for (int t = tid; t < 2 * S.cs; t += kT)
                 ph0[t] = to_fix(__longlong_as_double(ph0[t]), s0);
-        for (int u = 0; u < 2 * pl.K[0]; u++) {
-            T &f = en.fs()[u * kT + tid];
-            f = to_fix(__longlong_as_double(f) * g0.h2, s0);
-        }
-        __syncthreads();
+        keep([&](double f) { return qmul<30>(to_fix(f, s0 + pl.h2e), pl.h2k); });
     } else {
-        cluster_sync_();
+        keep([](float f) { return f; });
     }
-    if (!bad) {
-        for (int cyc = 0; cyc < pl.cycles; cyc++) {
-            int q = 0;
-            for (;; q++) {
-                // a level in CTA 0 alone: the other CTAs wait for its staged planes
-                if (en.dist(q) || rank == 0) {
-                    const bool fresh = pl.zero_start && cyc == 0;
-                    if (pl.K[q] == 1)
-                        en.template descend<true>(q, fresh);
-                    else
-                        en.template descend<false>(q, fresh);
-                }
-                if (q + 1 == pl.nlev)
-                    break;
-            }
-            for (; q > 0; q--) {
-                if (en.dist(q) || rank == 0)
-                    en.publish(q, en.level(q));
-                if (en.dist(q - 1))
-                    cluster_sync_();
-                else if (rank == 0)
-                    __syncthreads();
-                if (en.dist(q - 1) || rank == 0) {
-                    const bool last = cyc + 1 == pl.cycles;
-                    if (pl.K[q - 1] == 1)
-                        en.template ascend<true>(q - 1, last);
-                    else
-                        en.template ascend<false>(q - 1, last);
+    cluster_sync_();
+    // V-cycles: `cycles` of them, or (solve; the loop of Sec. 2.3 step 14)
+    // until |r| < tol |b|, both in FP64, |b| and the first |r| from the norm
+    // kernel before this launch.  Compared as squares; r = 0 meets any tol > 0.
+    const bool solve = P::kFix && pl.solve;
+    double bb = 0.0, r2 = 0.0, goal = 0.0;
+    int n = 0;
+    auto more = [&]() { return n < pl.cycles && (!solve || (isfinite(r2) && !(r2 < goal) && !(r2 == 0.0 && goal >= 0.0 && pl.tol > 0.0))); };
+    bool go = pl.cycles > 0;
+    if (solve) {
+        bb = pl.scal[0];
+        r2 = pl.scal[1];
+        goal = pl.tol * pl.tol * bb;
+        // (a first |r| that is not finite: one step finds that out, as in the loop of launches)
+        go = isfinite(bb) && bb > 0.0 && (more() || (!isfinite(r2) && go));
+    }
+    while (go) {
+        if (!bad)
+            en.cycle(pl.zero_start && n == 0, !solve && n + 1 == pl.cycles);
+        n++;
+        if constexpr (P::kFix)
+            if (solve) {
+                r2 = CUDART_NAN;
+                if (!bad) {
+                    const double q = en.square_sum(pl.K[0]);
+                    r2 = en.scaled(q, -2 * en.sc()[0]) * g0.inv_h2 * g0.inv_h2;
                 }
             }
-        }
+        go = more();
+    }
+    if (solve && rank == 0 && tid == 0) {
+        MgSolveCtl c{};
+        c.cycles = c.outer = n;
+        c.bnorm = sqrt(bb);
+        c.rel = c.bnorm > 0.0 ? sqrt(r2) / c.bnorm : 0.0;
+        c.status = isfinite(c.bnorm) && (n == 0 || isfinite(c.rel)) ? 0 : 6;
+        *pl.ctl = c;
+    }
+    if (*en.failed()) {   // (a wait for a neighbour ran out)
+        bad = true;
+        if (pl.err && tid == 0)
+            *pl.err = 7;   // MG_ETIMEOUT
     }
     // the potential of the plan's first level back to global memory
-    {
+    if (n > 0) {
         G *out = static_cast<G *>(pl.phi);
         int s0 = 0;
         if constexpr (P::kFix)
             s0 = en.sc()[0];
-        for (int u = 0; u < pl.K[0]; u++) {
-            const int A = en.word_a(u), d = en.word(0, u, kD);
-            const int x = d & 0x3ff, j = (d >> 10) & 0x3ff, k = d >> 20, c1 = (A >> 14) & 1, b = A & 0x3fff;
-            for (int s = 0; s < 2; s++)
-                if ((A >> (15 + s)) & 1) {
-                    const T v = ph0[(s ? 1 - c1 : c1) * S.cs + b + s];
-                    G o;
-                    if constexpr (P::kFix)
-                        o = bad ? __longlong_as_double(0x7ff8000000000000ll) : from_fix(v, s0);
-                    else
-                        o = v;
-                    out[gidx(2 * x + 1 + s, j, k)] = o;
-                }
+#pragma unroll
+        for (int u = 0; u < MG_SLAB_MAXK; u++) {
+            if (u >= pl.K[0])
+                break;
+            const int A = en.word_a(u);
+            if (!((A >> 15) & 1))
+                continue;
+            const int d = en.word(0, u, kD), c1 = (A >> 14) & 1, b = A & 0x3fff;
+            G *dst = out + gidx(2 * (d & 0x3ff) + 1, (d >> 10) & 0x3ff, d >> 20);
+            auto value = [&](T v) -> G {
+                if constexpr (P::kFix)
+                    return bad ? __longlong_as_double(0x7ff8000000000000ll) : from_fix(v, s0);
+                else
+                    return v;
+            };
+            dst[0] = value(ph0[c1 * S.cs + b]);
+            if ((A >> 16) & 1)
+                dst[1] = value(ph0[(1 - c1) * S.cs + b + 1]);
         }
     }
-    if (pl.ctl && rank == 0 && tid == 0)
+    if (pl.ctl && !solve && rank == 0 && tid == 0)
         inner_step_count(pl.ctl, pl.hi);
     cluster_sync_();   // no CTA leaves while another may still write to its shared memory
 }
@@ -1276,6 +1540,9 @@ bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, in
     p.lgc = csize == 16 ? 4 : 3;
     p.nu_pre = nu_pre;
     p.nu_post = nu_post;
+    int e2 = 0;
+    p.h2k = std::llrint(std::ldexp(std::frexp(g[0].h2, &e2), 62));
+    p.h2e = e2;
     const size_t w = fp32 ? 4 : 8;
     size_t off = 0, scratch = 0;
     const int lognu = (int)std::ceil(std::log2(1.0 + nu_pre + nu_post));
@@ -1289,14 +1556,14 @@ bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, in
         const int N = g[q].N, H = (N + 3) >> 1, R = dim == 3 ? N + 2 : 1, ha = (N + 1) >> 1, rows = dim == 3 ? N : 1;
         p.po[q] = q < p.nclu ? (N + csize - 1) / csize : N;
         const size_t cs = (size_t)(p.po[q] + 2) * R * H, items = (size_t)p.po[q] * rows * ha;
-        if (cs > 0x3fff || items > 0x3fff || N > 1020)   // fields of the plan words
+        if (cs > 0x3fff || items > 0x3fff || N > 1020 || (q < p.nclu && p.po[q] > 16))   // fields of the plan words
             return false;
         p.off[q] = (int)off;
         off = align(off + 2 * cs);
         const int k = (int)((items + kT - 1) / kT);
         if (k > MG_SLAB_MAXK)
             return false;
-        p.K[q] = k == 1 ? 1 : (k + 1) & ~1;
+        p.K[q] = k <= 2 ? k : 4;
         p.slot[q] = p.nslot;
         p.nslot += p.K[q];
         scratch = std::max(scratch, items);

@@ -67,3 +67,28 @@ def test_fp64_slab_non_finite_density_reports_ediverged(mg, bad):  # noqa: F811
     with pytest.raises(mg.MGError) as ei:
         gpu_solve(mg, H, inp, max_cycles=5, rel_tol=1e-10)
     assert ei.value.status == mg.MG_EDIVERGED
+
+
+@pytest.mark.parametrize("dim,n", [(3, 4), (3, 16), (3, 31), (3, 32), (2, 22), (2, 64), (2, 158)])
+@pytest.mark.parametrize("max_cycles", [1, 30])
+def test_fp64_slab_solve_stops_where_the_loop_of_launches_stops(mg, monkeypatch, dim, n, max_cycles):  # noqa: F811
+    """A level solved by one launch takes the cycles that the loop of launches
+    takes.  Residuals of potentials of order one round at 8 n^2 2^-53 of the
+    right-hand side (12), below 2e-12 of it here."""
+    H, inp = random_single_level(dim, n, 31 * n + dim)
+    kw = dict(max_cycles=max_cycles, rel_tol=1e-8)
+    _, a = gpu_solve(mg, H, inp, **kw)
+    monkeypatch.setenv("MG_BOTTOM_N64", "8")
+    _, b = gpu_solve(mg, H, inp, **kw)
+    assert a[0]["cycles"] == b[0]["cycles"] and a[0]["status"] == b[0]["status"]
+    assert abs(a[0]["rel_res"] - b[0]["rel_res"]) < 1e-11 * max(1.0, b[0]["rel_res"])
+    assert relmax(a[0]["phi"], b[0]["phi"]) < 1e-12
+
+
+def test_fp64_slab_solve_of_nothing(mg):  # noqa: F811
+    """A zero right-hand side: no cycle, the zero potential."""
+    n = 16
+    H = I.Hierarchy(3, [n], [(0.0, 0.0, 0.0)], 1.0 / n, 1.0, [], "zero")
+    inp = [{"rho": np.zeros((n,) * 3), "bc_rho": np.zeros((n + 2,) * 3), "bc_phi": np.zeros((n + 4,) * 3)}]
+    _, g = gpu_solve(mg, H, inp, max_cycles=5, rel_tol=1e-10)
+    assert g[0]["cycles"] == 0 and np.all(g[0]["phi"] == 0.0)
