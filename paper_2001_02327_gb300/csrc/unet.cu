@@ -562,24 +562,248 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16 *__restrict__ in, i
         atomicExch(err, 1);
 }
 
-// db[co] += sum_v d[v][co]: a block of 256 threads takes a run of voxels,
-// thread t the channel t % N of voxels v0 + t / N, v0 + t / N + 256 / N, ...
-// (coalesced rows), then sums per channel in shared memory and adds once
-__global__ void __launch_bounds__(256) k_bias_grad(const float *__restrict__ d, int N, int V, int vchunk,
-                                                   float *__restrict__ db)
+// The same gradients on grids of at least 8^3 voxels, without a transposition:
+// with the voxels as K, both operands lie in memory with M and N fastest, so
+// they go to shared memory as they are (16-byte rows of 8 channels) and the
+// MMAs read them M- and N-major.  A stage holds 8 grid rows (y0 .. y0 + 7 of
+// one plane z, all x) of the output gradient and the rows y0 - 1 .. of plane
+// z + dz of the input, per row one line of voxels per 8 channels.  A start
+// address 16 bytes on is a shift by one voxel (dx), and the lines of
+// consecutive rows are evenly spaced, so one MMA takes 128 / CK input rows
+// (M = row, channel) and TB gradient rows (N = row, channel) over 16 voxels of
+// x (two groups of 8 rows on the 8^3 grid): its D holds every dy = input row -
+// gradient row of them, and the rest of D (other row pairs, rows past the
+// tile) is ignored.  A block keeps the three dx (and the MA row groups that
+// TB + 2 input rows need) of one dz in TMEM over all its stages, two in
+// flight, and adds its sums into dW with 16-byte reductions.
+// The gather by tap (k_wgrad_tc) spent its time in the transposing stores,
+// eight-way bank conflicts among them, once per tap: 4 x 64^3 voxels, 32 -> 16
+// channels 1022 -> 123 us and 16 -> 16 608 -> 56 us, 4 x 8^3, 64 -> 64 111 ->
+// 13 us.  What bounds it now is the MMAs' reading of A (4 KB of shared memory,
+// 32 cycles each, for 16 voxels of TB rows) beside the copies of a stage (59
+// KB for 512 voxels, from L2).  Error of the sums against FP64, relative in the
+// 2-norm: 3e-6 -> 2e-6 at 64^3, 1e-6 -> 1e-7 at 8^3 (shorter accumulator
+// chains, see kChain).  Grids of less than 8^3 voxels and layers whose stages
+// do not fit stay with k_wgrad_tc.
+template <int CK, int N>
+struct WgradTile {
+    static constexpr int kRA = 128 / CK;                              // input rows of one MMA
+    static constexpr int kTB = CK == 16 ? 4 : CK == 32 ? 2 : N == 16 ? 2 : 1;   // gradient rows of one MMA
+    static constexpr int kMA = (kTB + 2 + kRA - 1) / kRA;
+    static constexpr int kTY = 8;
+    static constexpr int kRows = kTY - kTB + kRA * kMA;               // input rows an MMA may read
+    // The tensor core adds to its FP32 accumulators with more error than a
+    // rounded addition, so no accumulator takes more than kChain MMAs: stages
+    // take kSets sets of accumulators in turn, and a block at most
+    // kChain kSets / (MMAs of one accumulator per stage) stages.
+    static constexpr int kChain = 256;
+    static constexpr int kSetCols = 3 * kMA * kTB * N;
+    static constexpr int kSets = kSetCols <= 128 ? 4 : 1;
+    static constexpr int kCols = kSets * kSetCols;
+    static constexpr int kAlloc = kCols <= 256 ? 256 : 512;
+    static int items_max(int n) { return kChain * kSets / (kTY / kTB * std::max(n, 16) / 16 / (n == 8 ? 2 : 1)); }
+    // voxels per line: x = -1 .. n and one more (odd: lines of different channels in different banks)
+    __host__ __device__ static int pa(int n) { return n + 3; }
+    __host__ __device__ static int pb(int n) { return n + 1; }
+    __host__ __device__ static int a_bytes(int n) { return kRows * (CK / 8) * pa(n) * 16; }
+    __host__ __device__ static int stage(int n) { return a_bytes(n) + kTY * (N / 8) * pb(n) * 16; }
+    static constexpr int kSmemMax = 226 * 1024;
+    static bool applies(int lg) { return lg >= 3 && 2 * stage(1 << lg) <= kSmemMax; }
+};
+
+__device__ __forceinline__ void red_add4(float *p, const float *v)
 {
-    __shared__ float part[256];
-    const int v0 = blockIdx.x * vchunk, v1 = min(v0 + vchunk, V);
-    const int c = threadIdx.x % N, step = 256 / N;
-    float s = 0.f;
-    for (int v = v0 + threadIdx.x / N; v < v1; v += step)
-        s += d[(size_t)v * N + c];
-    part[threadIdx.x] = s;
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+}
+
+template <int CK, int N>
+__global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in, int Cin, const bf16 *__restrict__ d,
+                                                    float *__restrict__ dW, int lg, int B, int *__restrict__ err)
+{
+    typedef WgradTile<CK, N> W;
+    constexpr int CG = CK / 8, NG = N / 8, TY = W::kTY;
+    // BF16 operands, both M- / N-major
+    constexpr uint32_t IDESC = tc_idesc_bf16(128, W::kTB * N) | (1u << 15) | (1u << 16);
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t mbar[2];
+    __shared__ uint32_t tslot;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const uint32_t sm0 = smem_u32(smem), mb0 = smem_u32(&mbar[0]);
+    if (warp == 0) {
+        tc_alloc(smem_u32(&tslot), W::kAlloc);
+        tc_relinquish();
+    }
+    if (tid == 0) {
+        mbar_init1(mb0);
+        mbar_init1(mb0 + 8);
+        fence_mbar_init();
+    }
+    const int n = 1 << lg, PA = W::pa(n), PB = W::pb(n), sbytes = W::stage(n), abytes = W::a_bytes(n);
+    // the padding voxels x = -1 and x = n of every line stay zero
+    for (int e = tid; e < 2 * W::kRows * CG * 2; e += 256) {
+        const int line = (e >> 1) % (W::kRows * CG), st = (e >> 1) / (W::kRows * CG);
+        *reinterpret_cast<uint4 *>(smem + st * sbytes + (line * PA + (e & 1 ? n + 1 : 0)) * 16) = make_uint4(0, 0, 0, 0);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tslot;
+    const int dz = (int)blockIdx.y - 1;
+    const int lgt = lg - 3, nitem = B << (lg + lgt);   // items: (sample, z, group of 8 rows)
+    auto next_item = [&](int it) {
+        for (; it < nitem; it += gridDim.x) {
+            const int z = ((it >> lgt) & (n - 1)) + dz;
+            if ((unsigned)z < (unsigned)n)
+                break;
+        }
+        return it;
+    };
+    auto fill = [&](int it, int st) {
+        const int y0 = (it & ((1 << lgt) - 1)) * TY, z = (it >> lgt) & (n - 1), b = it >> (lgt + lg);
+        const uint32_t As = sm0 + st * sbytes, Bs = As + abytes;
+        const bf16 *pa = in + ((size_t)(((b << lg) + z + dz) << lg) << lg) * CK;
+        for (int e = tid; e < (TY + 2) * n * CG; e += 256) {
+            const int cg = e & (CG - 1), x = (e / CG) & (n - 1), row = (e / CG) >> lg, y = y0 - 1 + row;
+            const bool ok = (unsigned)y < (unsigned)n;
+            cp16(As + ((row * CG + cg) * PA + x + 1) * 16, ok ? pa + ((size_t)(y << lg) + x) * CK + 8 * cg : pa, ok);
+        }
+        const bf16 *pd = d + ((size_t)((((b << lg) + z) << lg) + y0) << lg) * N;
+        for (int e = tid; e < TY * n * NG; e += 256) {
+            const int ng = e & (NG - 1), x = (e / NG) & (n - 1), row = (e / NG) >> lg;
+            cp16(Bs + ((row * NG + ng) * PB + x) * 16, pd + ((size_t)(row << lg) + x) * N + 8 * ng, true);
+        }
+    };
+    const uint32_t lboA = n == 8 ? W::kTB * CG * PA * 16 : 128, lboB = n == 8 ? W::kTB * NG * PB * 16 : 128;
+    const int ystep = n == 8 ? 2 * W::kTB : W::kTB;
+    int it = next_item(blockIdx.x), issued = 0;
+    uint32_t phases = 0u;
+    bool bad = false;
+    if (it < nitem)
+        fill(it, 0);
+    cp_commit();
+    while (it < nitem) {
+        const int nx = next_item(it + gridDim.x), s = issued & 1;
+        if (nx < nitem) {
+            if (issued > 0) {   // the other stage's MMAs have finished reading it
+                const bool done = mbar_wait_for(mb0 + 8 * (s ^ 1), (phases >> (s ^ 1)) & 1u, kTcBudget);
+                if (__syncthreads_or(!done)) {
+                    bad = true;
+                    break;
+                }
+                phases ^= 1u << (s ^ 1);
+            }
+            fill(nx, s ^ 1);
+        }
+        cp_commit();
+        cp_wait<1>();
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (tid == 0) {
+            const uint32_t a0 = sm0 + s * sbytes, b0 = a0 + abytes;
+            bool first = issued < W::kSets;
+            const uint32_t acc = tmem + (issued & (W::kSets - 1)) * W::kSetCols;
+            for (int yb = 0; yb < TY; yb += ystep)
+                for (int x0 = 0; x0 < n; x0 += 16) {
+                    const uint64_t db = tc_sdesc(b0 + (yb * NG * PB + x0) * 16, lboB, PB * 16);
+                    for (int dx = 0; dx < 3; dx++)
+                        for (int ma = 0; ma < W::kMA; ma++)
+                            tc_mma(acc + (dx * W::kMA + ma) * W::kTB * N,
+                                   tc_sdesc(a0 + ((yb + ma * W::kRA) * CG * PA + x0 + dx) * 16, lboA, PA * 16), db,
+                                   IDESC, first ? 0u : 1u);
+                    first = false;
+                }
+            tc_commit(mb0 + 8 * s);
+        }
+        issued++;
+        it = nx;
+    }
+    cp_wait<0>();
+    bool done = true;
+    if (issued > 0) {
+        const int s = (issued - 1) & 1;   // the last commit covers every MMA issued before it
+        done = mbar_wait_for(mb0 + 8 * s, (phases >> s) & 1u, kTcBudget);
+    }
+    done = !__syncthreads_or(!done);
+    tc_fence_after();
+    if (done && !bad && issued > 0) {
+        const int m = (warp & 3) * 32 + (tid & 31), ci = m & (CK - 1);
+        const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        for (int q = warp >> 2; q < 3 * W::kMA * W::kTB; q += 2) {   // column blocks (dx, row group, gradient row)
+            const int b = q % W::kTB, ma = (q / W::kTB) % W::kMA, dx = q / (W::kTB * W::kMA);
+            const int dy = ma * W::kRA + m / CK - b;
+            float *o = dW + ((size_t)((blockIdx.y * 3 + dy) * 3 + dx) * Cin + ci) * N;
+            for (int c0 = 0; c0 < N; c0 += 16) {
+                float v[16];
+                tc_ld16(lane_base + q * N + c0, v);
+                for (int set = 1; set < min(W::kSets, issued); set++) {
+                    float w[16];
+                    tc_ld16(lane_base + set * W::kSetCols + q * N + c0, w);
+#pragma unroll
+                    for (int i = 0; i < 16; i++)
+                        v[i] += w[i];
+                }
+                if (dy >= 0 && dy < 3 && ci < Cin)
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4)
+                        red_add4(o + c0 + i, v + i);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0)
+        tc_dealloc(tmem, W::kAlloc);
+    if ((bad || !done) && tid == 0)
+        atomicExch(err, 1);
+}
+
+// What the weight and data gradients of a convolution read, in one pass over
+// its output gradient d (N channels, V voxels): d where the activation is
+// positive, else 0, as BF16 (out) and, for grids of less than 8^3 voxels, in
+// FP32 in place; db[c] += its sums.  A thread keeps one group of 8 channels.
+// Bound by memory; as three kernels (mask, sums, rounding) the gradient of 4 x
+// 64^3 x 16 took 77 us, here 22 us.
+__global__ void __launch_bounds__(256) k_grad_prep(float *__restrict__ d, const bf16 *__restrict__ act, int N, long n8,
+                                                   bf16 *__restrict__ out, float *__restrict__ db, int keep)
+{
+    __shared__ float part[256][9];
+    const int ng = N >> 3;
+    float s[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        s[i] = 0.f;
+    // the number of threads is a multiple of the channel groups
+    for (long e = blockIdx.x * 256l + threadIdx.x; e < n8; e += gridDim.x * 256l) {
+        float4 *p = reinterpret_cast<float4 *>(d) + 2 * e;
+        const float4 a = p[0], c = p[1];
+        const uint4 w = reinterpret_cast<const uint4 *>(act)[e];
+        float v[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+        const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const float x = __uint_as_float(i & 1 ? q[i >> 1] & 0xFFFF0000u : q[i >> 1] << 16);
+            if (!(x > 0.f))
+                v[i] = 0.f;
+            s[i] += v[i];
+        }
+        reinterpret_cast<uint4 *>(out)[e] =
+            make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+        if (keep) {
+            p[0] = make_float4(v[0], v[1], v[2], v[3]);
+            p[1] = make_float4(v[4], v[5], v[6], v[7]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        part[threadIdx.x][i] = s[i];
     __syncthreads();
     if (threadIdx.x < N) {
         float t = 0.f;
-        for (int q = threadIdx.x; q < 256; q += N)
-            t += part[q];
+        for (int k = threadIdx.x >> 3; k < 256; k += ng)
+            t += part[k][threadIdx.x & 7];
         atomicAdd(&db[threadIdx.x], t);
     }
 }
@@ -921,16 +1145,6 @@ __global__ void __launch_bounds__(128) k_conv3_halo_p(const __grid_constant__ CU
         tc_dealloc(tmem, 2 * NCOL);
     if (!ok && tid == 0)
         atomicExch(err, 1);
-}
-
-// FP32 -> BF16 (round to nearest even), 8 values per thread
-__global__ void k_to_bf16(const float *__restrict__ src, bf16 *__restrict__ dst, long n8)
-{
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < n8; e += (long)gridDim.x * blockDim.x) {
-        const float4 a = reinterpret_cast<const float4 *>(src)[2 * e], c = reinterpret_cast<const float4 *>(src)[2 * e + 1];
-        reinterpret_cast<uint4 *>(dst)[e] =
-            make_uint4(pack2(a.x, a.y), pack2(a.z, a.w), pack2(c.x, c.y), pack2(c.z, c.w));
-    }
 }
 
 // Weight and bias gradients of a 3x3x3 convolution (FP32 on the CUDA cores):
@@ -1476,24 +1690,19 @@ bool use_halo()
     return on;
 }
 
-// tcgen05 path: FP32 input (the data-gradient pass) is rounded to BF16 first
-// (into scratch), as the mma.sync kernel rounds it when it loads it
+// tcgen05 path: BF16 input; the mma.sync kernel also takes FP32 (the
+// data-gradient pass) and rounds it when it loads it
 template <int NT, bool FLIP, typename TIn>
 cudaError_t conv_launch(const TIn *in, int CK, const bf16 *W, const float *bias, void *out, int out_bf16, int relu,
-                        int lg, int V, int *err, bf16 *scratch, cudaStream_t s)
+                        int lg, int V, int *err, cudaStream_t s)
 {
     if (!use_mma_sync()) {
-        const bf16 *src;
-        if constexpr (sizeof(TIn) == 4) {
-            const long n8 = (long)V * CK / 8;
-            k_to_bf16<<<blocks_for(n8), kT, 0, s>>>(in, scratch, n8);
-            src = scratch;
-        } else {
-            src = in;
+        if constexpr (sizeof(TIn) == 2) {
+            if (use_halo() && halo_applies(CK, NT * 8, lg))
+                return conv_launch_halo<NT * 8, FLIP>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
+            return conv_launch_tc<NT * 8, FLIP>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
         }
-        if (use_halo() && halo_applies(CK, NT * 8, lg))
-            return conv_launch_halo<NT * 8, FLIP>(src, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
-        return conv_launch_tc<NT * 8, FLIP>(src, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
+        return cudaErrorInvalidValue;
     }
     k_conv3<NT, FLIP, TIn><<<(V + 63) / 64, 128, 0, s>>>(in, CK, W, bias, out, out_bf16, relu, lg, V);
     return cudaGetLastError();
@@ -1501,13 +1710,13 @@ cudaError_t conv_launch(const TIn *in, int CK, const bf16 *W, const float *bias,
 
 template <bool FLIP, typename TIn>
 cudaError_t conv_any(const TIn *in, int CK, const bf16 *W, const float *bias, int N, void *out, int out_bf16, int relu,
-                     int lg, int V, int *err, bf16 *scratch, cudaStream_t s)
+                     int lg, int V, int *err, cudaStream_t s)
 {
     switch (N) {
-    case 16: return conv_launch<2, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, scratch, s);
-    case 32: return conv_launch<4, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, scratch, s);
-    case 64: return conv_launch<8, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, scratch, s);
-    case 128: return conv_launch<16, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, scratch, s);
+    case 16: return conv_launch<2, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
+    case 32: return conv_launch<4, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
+    case 64: return conv_launch<8, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
+    case 128: return conv_launch<16, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -1541,7 +1750,7 @@ cudaError_t forward(mg_unet *u, int B, int lg)
     float *P = u->p;
 #define FWD(i, in, out, lgv, V)                                                                                   \
     if ((e = conv_any<false, bf16>(in, C(i).ckin, u->wf[i], P + C(i).boff, C(i).cout, out, 1, 1, lgv, V, u->tcerr, \
-                                   nullptr, s)))                                                                \
+                                   s)))                                                                \
         return e;
     FWD(0, u->x0, u->a0, lg, V0);
     FWD(1, u->a0, u->s0, lg, V0);
@@ -1564,8 +1773,23 @@ cudaError_t forward(mg_unet *u, int B, int lg)
 }
 
 template <int CK, int N>
-cudaError_t wgrad_tc(const bf16 *in, int Cin, const float *g, float *dW, int lg, int V, int *err, cudaStream_t s)
+cudaError_t wgrad_tc(const bf16 *in, int Cin, const float *g, const bf16 *gbf, float *dW, int lg, int V, int *err,
+                     cudaStream_t s)
 {
+    typedef WgradTile<CK, N> W;
+    if (W::applies(lg)) {
+        static cudaError_t attr = cudaFuncSetAttribute(k_wgrad_rows<CK, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       W::kSmemMax);
+        if (attr)
+            return attr;
+        // no more blocks per SM than tensor memory has room for: a block never waits for its columns
+        const int most = 512 / W::kAlloc, smem = std::max(2 * W::stage(1 << lg), W::kSmemMax / (most + 1) + 1024);
+        const int B = V >> (3 * lg), items = B << (2 * lg - 3), per_sm = std::max(1, W::kSmemMax / smem);
+        const int most_items = W::items_max(1 << lg);
+        const dim3 grid(std::max(std::min(items, 152 * per_sm / 3), (items + most_items - 1) / most_items), 3);
+        k_wgrad_rows<CK, N><<<grid, 256, smem, s>>>(in, Cin, gbf, dW, lg, B, err);
+        return cudaGetLastError();
+    }
     constexpr size_t smem = 2 * ((size_t)128 * 64 * 2 + (size_t)N * 64 * 2);
     static cudaError_t attr = cudaFuncSetAttribute(k_wgrad_tc<CK, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)smem);
@@ -1577,47 +1801,54 @@ cudaError_t wgrad_tc(const bf16 *in, int Cin, const float *g, float *dW, int lg,
     return cudaGetLastError();
 }
 
-cudaError_t wgrad_tc_any(int CK, int N, const bf16 *in, int Cin, const float *g, float *dW, int lg, int V, int *err,
-                         cudaStream_t s)
+// whether k_wgrad_rows takes the layer (else k_wgrad_tc, which reads the masked FP32 gradient)
+bool wgrad_by_rows(int CK, int N, int lg)
 {
 #define WG(ck, nn)                   \
     if (CK == ck && N == nn)         \
-        return wgrad_tc<ck, nn>(in, Cin, g, dW, lg, V, err, s);
+        return WgradTile<ck, nn>::applies(lg);
+    WG(16, 16) WG(16, 32) WG(32, 32) WG(32, 64) WG(64, 64) WG(128, 32) WG(64, 16) WG(32, 16)
+#undef WG
+    return false;
+}
+
+cudaError_t wgrad_tc_any(int CK, int N, const bf16 *in, int Cin, const float *g, const bf16 *gbf, float *dW, int lg,
+                         int V, int *err, cudaStream_t s)
+{
+#define WG(ck, nn)                   \
+    if (CK == ck && N == nn)         \
+        return wgrad_tc<ck, nn>(in, Cin, g, gbf, dW, lg, V, err, s);
     WG(16, 16) WG(16, 32) WG(32, 32) WG(32, 64) WG(64, 64) WG(128, 32) WG(64, 16) WG(32, 16)
 #undef WG
     return cudaErrorInvalidValue;
 }
 
-// weight gradients of conv i from its input activation and output gradient g (FP32, N channels)
-cudaError_t wgrad(mg_unet *u, int i, const bf16 *in, const float *g, int lg, int V)
+// weight and bias gradients of conv i from its input activation `in`, its
+// output activation `act` and output gradient g (FP32, N channels); leaves what
+// dgrad reads: the masked g, in BF16 in gbf on the tensor-core path
+cudaError_t wgrad(mg_unet *u, int i, const bf16 *in, const bf16 *act, float *g, int lg, int V)
 {
     const Conv &c = u->conv[i];
+    const long n8 = (long)V * c.cout / 8;
     if (use_mma_sync()) {
+        k_relu_mask<<<blocks_for(8 * n8), kT, 0, u->stream>>>(g, act, 8 * n8);
         const int vpb = 4096;
         dim3 grid((V + vpb - 1) / vpb, 27);
         k_wgrad<<<grid, kT, 0, u->stream>>>(in, c.ckin, c.cin, g, c.cout, u->grad + c.woff, u->grad + c.boff, lg, V,
                                             vpb);
         return cudaGetLastError();
     }
-    cudaError_t e = wgrad_tc_any(c.ckin, c.cout, in, c.cin, g, u->grad + c.woff, lg, V, u->tcerr, u->stream);
-    if (e)
-        return e;
-    const int vchunk = 4096;
-    k_bias_grad<<<(V + vchunk - 1) / vchunk, 256, 0, u->stream>>>(g, c.cout, V, vchunk, u->grad + c.boff);
-    return cudaGetLastError();
+    k_grad_prep<<<blocks_for(n8, 152 * 8), 256, 0, u->stream>>>(g, act, c.cout, n8, u->gbf, u->grad + c.boff,
+                                                                wgrad_by_rows(c.ckin, c.cout, lg) ? 0 : 1);
+    return wgrad_tc_any(c.ckin, c.cout, in, c.cin, g, u->gbf, u->grad + c.woff, lg, V, u->tcerr, u->stream);
 }
 
 cudaError_t dgrad(mg_unet *u, int i, const float *g, float *out, int lg, int V)
 {
     const Conv &c = u->conv[i];
-    return conv_any<true, float>(g, c.cout, u->wd[i], nullptr, c.ckin, out, 0, 0, lg, V, u->tcerr, u->gbf,
-                                 u->stream);
-}
-
-cudaError_t mask(mg_unet *u, float *g, const bf16 *act, long n)
-{
-    k_relu_mask<<<blocks_for(n), kT, 0, u->stream>>>(g, act, n);
-    return cudaGetLastError();
+    if (use_mma_sync())
+        return conv_any<true, float>(g, c.cout, u->wd[i], nullptr, c.ckin, out, 0, 0, lg, V, u->tcerr, u->stream);
+    return conv_any<true, bf16>(u->gbf, c.cout, u->wd[i], nullptr, c.ckin, out, 0, 0, lg, V, u->tcerr, u->stream);
 }
 
 // backward pass (loss gradient from y vs tgt), accumulating into u->grad
@@ -1630,42 +1861,42 @@ cudaError_t backward(mg_unet *u, int B, int lg)
     k_out1_bwd<<<blocks_for(V0, 152 * 4), kT, 0, s>>>(u->y, u->tgt, u->d0, u->p + u->nparam - 17, gA,
                                                      u->grad + u->nparam - 17, u->grad + u->nparam - 1, u->loss, V0);
     // D0 (u0 -> d0), gA = dd0 [V0][16]
-    if ((e = mask(u, gA, u->d0, (long)V0 * 16)) || (e = wgrad(u, 8, u->u0, gA, lg, V0)) ||
+    if ((e = wgrad(u, 8, u->u0, u->d0, gA, lg, V0)) ||
         (e = dgrad(u, 8, gA, gB, lg, V0)))
         return e;                                                        // gB = du0 [V0][32]
     // split du0 -> dd1 (coarse) and ds0 (gC)
     k_upcat_bwd<<<blocks_for((long)V0 * 16), kT, 0, s>>>(gB, 16, 16, gA, gC, lg - 1, V1);   // gA = dd1 [V1][16], gC = ds0 [V0][16]
-    if ((e = mask(u, gA, u->d1, (long)V1 * 16)) || (e = wgrad(u, 7, u->u1, gA, lg - 1, V1)) ||
+    if ((e = wgrad(u, 7, u->u1, u->d1, gA, lg - 1, V1)) ||
         (e = dgrad(u, 7, gA, gB, lg - 1, V1)))
         return e;                                                        // gB = du1 [V1][64]
     // ds1 lives behind ds0 in gC
     float *ds1 = gC + (size_t)V0 * 16;
     k_upcat_bwd<<<blocks_for((long)V1 * 32), kT, 0, s>>>(gB, 32, 32, gA, ds1, lg - 2, V2);  // gA = dd2 [V2][32]
-    if ((e = mask(u, gA, u->d2, (long)V2 * 32)) || (e = wgrad(u, 6, u->u2, gA, lg - 2, V2)) ||
+    if ((e = wgrad(u, 6, u->u2, u->d2, gA, lg - 2, V2)) ||
         (e = dgrad(u, 6, gA, gB, lg - 2, V2)))
         return e;                                                        // gB = du2 [V2][128]
     float *ds2 = ds1 + (size_t)V1 * 32;
     k_upcat_bwd<<<blocks_for((long)V2 * 64), kT, 0, s>>>(gB, 64, 64, gA, ds2, lg - 3, V3);  // gA = da3 [V3][64]
-    if ((e = mask(u, gA, u->a3, (long)V3 * 64)) || (e = wgrad(u, 5, u->p2, gA, lg - 3, V3)) ||
+    if ((e = wgrad(u, 5, u->p2, u->a3, gA, lg - 3, V3)) ||
         (e = dgrad(u, 5, gA, gB, lg - 3, V3)))
         return e;                                                        // gB = dp2 [V3][64]
     k_pool_bwd_add<<<blocks_for((long)V2 * 64), kT, 0, s>>>(gB, ds2, 64, lg - 2, V2);
-    if ((e = mask(u, ds2, u->s2, (long)V2 * 64)) || (e = wgrad(u, 4, u->p1, ds2, lg - 2, V2)) ||
+    if ((e = wgrad(u, 4, u->p1, u->s2, ds2, lg - 2, V2)) ||
         (e = dgrad(u, 4, ds2, gB, lg - 2, V2)))
         return e;                                                        // gB = dp1 [V2][32]
     k_pool_bwd_add<<<blocks_for((long)V1 * 32), kT, 0, s>>>(gB, ds1, 32, lg - 1, V1);
-    if ((e = mask(u, ds1, u->s1, (long)V1 * 32)) || (e = wgrad(u, 3, u->a1, ds1, lg - 1, V1)) ||
+    if ((e = wgrad(u, 3, u->a1, u->s1, ds1, lg - 1, V1)) ||
         (e = dgrad(u, 3, ds1, gB, lg - 1, V1)))
         return e;                                                        // gB = da1 [V1][32]
-    if ((e = mask(u, gB, u->a1, (long)V1 * 32)) || (e = wgrad(u, 2, u->p0, gB, lg - 1, V1)) ||
+    if ((e = wgrad(u, 2, u->p0, u->a1, gB, lg - 1, V1)) ||
         (e = dgrad(u, 2, gB, gA, lg - 1, V1)))
         return e;                                                        // gA = dp0 [V1][16]
     float *ds0 = gC;
     k_pool_bwd_add<<<blocks_for((long)V0 * 16), kT, 0, s>>>(gA, ds0, 16, lg, V0);
-    if ((e = mask(u, ds0, u->s0, (long)V0 * 16)) || (e = wgrad(u, 1, u->a0, ds0, lg, V0)) ||
+    if ((e = wgrad(u, 1, u->a0, u->s0, ds0, lg, V0)) ||
         (e = dgrad(u, 1, ds0, gB, lg, V0)))
         return e;                                                        // gB = da0 [V0][16]
-    if ((e = mask(u, gB, u->a0, (long)V0 * 16)) || (e = wgrad(u, 0, u->x0, gB, lg, V0)))
+    if ((e = wgrad(u, 0, u->x0, u->a0, gB, lg, V0)))
         return e;
     return cudaGetLastError();
 }

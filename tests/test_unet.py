@@ -435,3 +435,29 @@ def test_persistent_halo_kernel_equals_per_tile_kernel(tmp_path):
     g0, g1 = out["0"]["g"].astype(np.float64), out["1"]["g"].astype(np.float64)
     assert _rel(g1, g0) < 1e-5, _rel(g1, g0)
     assert np.isfinite(out["1"]["y"]).all() and np.abs(g1).max() > 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,B", [(8, 3), (16, 2), (32, 1), (64, 1)])
+def test_weight_gradients_by_rows_elementwise_dyadic(un, n, B):
+    """Every weight and bias gradient on the dyadic case (each of its forward
+    sums exact) within the FP32 summation bound V 2^-24 sum |terms| of its
+    terms, at grids of 8^3 (two rows per MMA) to 64^3, with levels below 8^3
+    beside them, so that a wrong row, shift, channel or padding voxel shows."""
+    import torch
+    from oracle import unet_ref as R
+    rho, phi, res, tru, frho, p = _dyadic_case(1, n, B)
+    u = un.mg_unet_create(n, B, seed=0)
+    try:
+        un.mg_unet_set_params(u, p)
+        dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        un.mg_unet_train_step(u, B, n, dev(rho), dev(phi), dev(res), dev(tru), frho, update=False)
+        g = un.mg_unet_get_grad(u).astype(np.float64)
+        T = torch.from_numpy
+        p64 = p.astype(np.float64)
+        _, gr = R.loss_and_grad(p64, T(rho), T(phi), T(res), T(tru), frho, emulate=True)
+        mag = R.weight_grad_magnitude(p64, T(rho), T(phi), T(res), T(tru), frho)
+        assert not (np.abs(g - gr) > B * n ** 3 * 2.0 ** -24 * mag).any()
+        assert (gr != 0).mean() > 0.01
+    finally:
+        un.mg_unet_destroy(u)
