@@ -49,6 +49,16 @@ __device__ __forceinline__ uint32_t pack2(float a, float b)
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t *>(&v);
 }
+// the 8 BF16 values of a 16-byte word
+__device__ __forceinline__ void unpack8(uint4 q, float *f)
+{
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        f[2 * i] = __uint_as_float(w[i] << 16);
+        f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+    }
+}
 
 __device__ __forceinline__ uint32_t ld2(const bf16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
 __device__ __forceinline__ uint32_t ld2(const float *p)
@@ -702,19 +712,22 @@ __global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in,
         __syncthreads();
         tc_fence_after();
         if (tid == 0) {
-            const uint32_t a0 = sm0 + s * sbytes, b0 = a0 + abytes;
+            const uint64_t da0 = tc_sdesc(sm0 + s * sbytes, lboA, PA * 16);
+            const uint64_t db0 = tc_sdesc(sm0 + s * sbytes + abytes, lboB, PB * 16);
             bool first = issued < W::kSets;
-            const uint32_t acc = tmem + (issued & (W::kSets - 1)) * W::kSetCols;
-            for (int yb = 0; yb < TY; yb += ystep)
-                for (int x0 = 0; x0 < n; x0 += 16) {
-                    const uint64_t db = tc_sdesc(b0 + (yb * NG * PB + x0) * 16, lboB, PB * 16);
+            const uint32_t acc = tmem + (issued & (W::kSets - 1)) * W::kSetCols, step = W::kRA * CG * PA;
+            for (int yb = 0; yb < TY; yb += ystep) {
+                uint64_t da = da0 + yb * CG * PA, db = db0 + yb * NG * PB;
+                for (int x0 = 0; x0 < n; x0 += 16, da += 16, db += 16) {
+#pragma unroll
                     for (int dx = 0; dx < 3; dx++)
+#pragma unroll
                         for (int ma = 0; ma < W::kMA; ma++)
-                            tc_mma(acc + (dx * W::kMA + ma) * W::kTB * N,
-                                   tc_sdesc(a0 + ((yb + ma * W::kRA) * CG * PA + x0 + dx) * 16, lboA, PA * 16), db,
-                                   IDESC, first ? 0u : 1u);
+                            tc_mma(acc + (dx * W::kMA + ma) * W::kTB * N, da + dx + ma * step, db, IDESC,
+                                   first ? 0u : 1u);
                     first = false;
                 }
+            }
             tc_commit(mb0 + 8 * s);
         }
         issued++;
@@ -781,11 +794,11 @@ __global__ void __launch_bounds__(256) k_grad_prep(float *__restrict__ d, const 
         const float4 a = p[0], c = p[1];
         const uint4 w = reinterpret_cast<const uint4 *>(act)[e];
         float v[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
-        const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+        float x[8];
+        unpack8(w, x);
 #pragma unroll
         for (int i = 0; i < 8; i++) {
-            const float x = __uint_as_float(i & 1 ? q[i >> 1] & 0xFFFF0000u : q[i >> 1] << 16);
-            if (!(x > 0.f))
+            if (!(x[i] > 0.f))
                 v[i] = 0.f;
             s[i] += v[i];
         }
@@ -815,7 +828,7 @@ __global__ void __launch_bounds__(256) k_grad_prep(float *__restrict__ d, const 
 // 16-byte rows, x fastest.  Tap (dz, dy, dx) is then the 128 x CK operand
 // whose row (x, y) is halo row ((dz+1) 18 + y + dy + 1) 10 + x + dx + 1: a
 // descriptor at that start with 8-row groups one halo row (160 B) apart
-// (SBO) and the channel chunks kHaloChunk apart (LBO) -- no copy per tap.
+// (SBO) and the channel chunks one chunk apart (LBO) -- no copy per tap.
 // All 27 taps' weights (N x CK each) come in by cp.async from every thread,
 // N rows of 16 B per chunk.  One thread issues the TMA and every MMA; the
 // block waits once for the accumulator.
@@ -835,23 +848,39 @@ __device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap *map, 
                  "l"((unsigned long long)map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(mbar)
                  : "memory");
 }
-template <int N, bool FLIP>
-__global__ void __launch_bounds__(128) k_conv3_halo(const __grid_constant__ CUtensorMap tm_in,
-                                                    const bf16 *__restrict__ in, int halo_by_tma,
-                                                    const bf16 *__restrict__ W, int CK,
+// This kernel: tz planes per block (tz accumulators), the halo by cp.async.  A
+// warp copies a line of 10 voxels, 16 bytes per lane, channels fastest, so the
+// reads are whole sectors; the channel chunks in shared memory start in
+// different banks (halo_chunk, and N + 1 rows per weight chunk).  What bounded
+// the one-plane form with one TMA box per chunk was the thread that issues the
+// MMAs, which built two descriptors from run-time sizes for each (100 cycles an
+// MMA; with constant steps 55 to 65, near the 32 its 4 KB of A take), then
+// loading three planes and all weights for one.  4 x 64^3, 16 -> 16 channels 63
+// -> 43 us, 32 -> 16 145 -> 98 us, data gradient 32 <- 16 122 -> 74 us.
+// Layers whose weights do not fit beside the halo stream them, three taps a
+// stage; per tap, the gather of k_conv3_tc took an L1 line per lane: 4 x 16^3,
+// 128 -> 32 channels 54 -> 19 us, 4 x 8^3, 64 -> 64 36 -> 16 us.
+// Every accumulator takes its products in the same order in all these forms.
+__host__ __device__ constexpr int halo_chunk(int tz) { return (180 * (tz + 2) + 1) * 16; }
+// all 27 taps' weights stay beside the halo, else they stream through it three taps at a time
+__host__ __device__ constexpr bool halo_resident(int CK, int N) { return 27 * N * CK * 2 <= 64 * 1024 && CK <= 64; }
+
+template <int N, bool FLIP, int CK>
+__global__ void __launch_bounds__(256) k_conv3_halo(const bf16 *__restrict__ in, const bf16 *__restrict__ W,
                                                     const float *__restrict__ bias, void *__restrict__ out,
-                                                    int out_bf16, int relu, int lg, int B, int fault,
+                                                    int out_bf16, int relu, int lg, int tz, int ncol, int fault,
                                                     int *__restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t mbar[2];   // 0: halo and weights arrived; 1: accumulator complete
+    __shared__ __align__(8) uint64_t mbar[4];   // accumulator of a plane complete; streamed weights: a stage read
     __shared__ uint32_t tslot;
-    constexpr int NCOL = N < 32 ? 32 : N;
     constexpr uint32_t IDESC = tc_idesc_bf16(128, N);
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int nk8 = CK >> 3;
-    const uint32_t halo = smem_u32(smem), wts = halo + nk8 * kHaloChunk;
-    const uint32_t mb_in = smem_u32(&mbar[0]), mb_acc = smem_u32(&mbar[1]);
+    constexpr bool kStream = !halo_resident(CK, N);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int nk8 = CK / 8;
+    const int chunk = halo_chunk(tz);
+    const uint32_t halo = smem_u32(smem), wts = halo + nk8 * chunk;
+    const uint32_t mb0 = smem_u32(&mbar[0]);
     const int n = 1 << lg;
     const int tx = n >> 3, ty = (n + 15) >> 4;          // tiles per row and per column of a plane
     int t = blockIdx.x;
@@ -859,83 +888,115 @@ __global__ void __launch_bounds__(128) k_conv3_halo(const __grid_constant__ CUte
     t /= tx;
     const int y0 = (t % ty) * 16;
     t /= ty;
-    const int z0 = t % n, b = t / n;
+    const int z0 = (t % (n / tz)) * tz, b = t / (n / tz);
     if (warp == 0) {
-        tc_alloc(smem_u32(&tslot), NCOL);
+        tc_alloc(smem_u32(&tslot), ncol);
         tc_relinquish();
     }
     if (tid == 0) {
-        mbar_init1(mb_in);
-        mbar_init1(mb_acc);
+        for (int q = 0; q < 4; q++)
+            mbar_init1(mb0 + 8 * q);
         fence_mbar_init();
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tslot;
-    bool ok = true;
-    if (halo_by_tma) {
-        if (tid == 0) {
-            mbar_expect_tx(mb_in, (uint32_t)(nk8 * kHaloRows * 16));
-            for (int k8 = 0; k8 < nk8; k8++)
-                tma_load5(halo + k8 * kHaloChunk, &tm_in, 8 * k8, x0 - 1, y0 - 1, z0 - 1, b, mb_in);
-        }
-    } else {
-        // the halo rows by every thread, zero outside the grid
-        for (int e = tid; e < nk8 * kHaloRows; e += 128) {
-            const int k8 = e / kHaloRows, row = e - k8 * kHaloRows;
-            const int hx = row % 10, hy = (row / 10) % 18, hz = row / 180;
-            const int gx = x0 - 1 + hx, gy = y0 - 1 + hy, gz = z0 - 1 + hz;
-            const bool inside = (unsigned)gx < (unsigned)n && (unsigned)gy < (unsigned)n && (unsigned)gz < (unsigned)n;
-            const bf16 *src = inside ? in + ((((size_t)b * n + gz) * n + gy) * n + gx) * CK + 8 * k8 : in;
-            cp16(halo + k8 * kHaloChunk + row * 16, src, inside);
+    // the halo, zero outside the grid
+    for (int line = warp; line < 18 * (tz + 2); line += 8) {
+        const int hz = line / 18, hy = line - hz * 18, gz = z0 - 1 + hz, gy = y0 - 1 + hy;
+        const bool inside = (unsigned)gy < (unsigned)n && (unsigned)gz < (unsigned)n;
+        const bf16 *src = in + (((((size_t)b << lg) + gz) << lg) + gy << lg) * CK;
+        for (int c = lane; c < 10 * nk8; c += 32) {
+            const int hx = c / nk8, k8 = c % nk8, gx = x0 - 1 + hx;
+            const bool ok = inside && (unsigned)gx < (unsigned)n;
+            cp16(halo + k8 * chunk + (line * 10 + hx) * 16, ok ? src + (size_t)gx * CK + 8 * k8 : in, ok);
         }
     }
-    // the weights by every thread (16-byte copies), N rows of 16 B per (tap, chunk)
-    for (int e = tid; e < 27 * N * nk8; e += 128) {
-        const int k8 = e % nk8, row = e / nk8;   // row = tap * N + output channel
-        const int tap = row / N, nn = row - tap * N;
-        cp16(wts + ((tap * nk8 + k8) * N + nn) * 16, W + (size_t)row * CK + 8 * k8, true);
-    }
-    cp_commit();
-    cp_wait<0>();
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (tid == 0) {
-        if (halo_by_tma) {
-            ok = mbar_wait_for(mb_in, 0, kTcBudget);
-            if (!ok)
-                mbar_wait_for(mb_in, 0, kTcBudget);   // the copies still in flight land before the block leaves
+    // the weights of taps t0 .. t0 + nt - 1, N rows of 16 B per (tap, chunk)
+    auto weights = [&](int t0, int nt, uint32_t dst) {
+        for (int e = tid; e < nt * N * nk8; e += 256) {
+            const int k8 = e % nk8, row = e / nk8;   // row = tap * N + output channel
+            const int tap = row / N, nn = row - tap * N;
+            cp16(dst + ((tap * nk8 + k8) * (N + 1) + nn) * 16, W + ((size_t)t0 * N + row) * CK + 8 * k8, true);
         }
-        if (ok && !fault) {   // fault (test of the timeout path): nothing is issued, the accumulator wait runs out
+    };
+    // the MMAs of a tap: one thread issues them; with the descriptors' steps as
+    // constants an MMA costs it few instructions
+    auto tap_mmas = [&](int tap, uint32_t d, uint64_t da, uint64_t db) {
+        const int p = FLIP ? 26 - tap : tap;   // position of the tap in the 3 x 3 x 3 box
+        const int off = ((p / 9) * 18 + (p / 3) % 3) * 10 + p % 3;
+#pragma unroll
+        for (int k = 0; k < CK / 16; k++)
+            tc_mma(d, da + off + k * (2 * chunk / 16), db + 2 * k * (N + 1), IDESC, (tap > 0 || k > 0) ? 1u : 0u);
+    };
+    // fault (test of the timeout path): no MMA is issued, the waits for them run out
+    const long long budget = fault ? (1ll << 21) : kTcBudget;
+    bool bad = false;
+    if constexpr (kStream) {
+        // three taps a stage, three stages in a ring; one plane
+        constexpr int SB = 3 * nk8 * (N + 1) * 16;
+        weights(0, 3, wts);
+        cp_commit();
+        weights(3, 3, wts + SB);
+        cp_commit();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        const uint32_t tmem = tslot;
+        for (int st = 0; st < 9; st++) {
+            cp_wait<1>();
+            fence_async_smem();
+            tc_fence_before();
+            __syncthreads();
             tc_fence_after();
-            for (int tap = 0; tap < 27; tap++) {
-                int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-                if (FLIP) {
-                    dz = -dz;
-                    dy = -dy;
-                    dx = -dx;
-                }
-                const uint32_t a0 = halo + (uint32_t)((((dz + 1) * 18 + dy + 1) * 10 + dx + 1) * 16);
-                for (int k = 0; k < CK / 16; k++)
-                    tc_mma(tmem, tc_sdesc(a0 + 2 * k * kHaloChunk, kHaloChunk, 160),
-                           tc_sdesc(wts + (tap * nk8 + 2 * k) * N * 16, N * 16, 128), IDESC,
-                           (tap > 0 || k > 0) ? 1u : 0u);
+            if (tid == 0 && !fault) {
+                const uint64_t da = tc_sdesc(halo, chunk, 160), db = tc_sdesc(wts + (st % 3) * SB, (N + 1) * 16, 128);
+                for (int q = 0; q < 3; q++)
+                    tap_mmas(3 * st + q, tmem, da, db + q * nk8 * (N + 1));
+                tc_commit(mb0 + 8 * (st % 3));
+                if (st == 8)
+                    tc_commit(mb0 + 24);
             }
-            tc_commit(mb_acc);
+            if (st + 2 < 9) {
+                if (st > 0) {   // the MMAs of stage st - 1 have read the ring's third stage
+                    const bool done = mbar_wait_for(mb0 + 8 * ((st - 1) % 3), ((st - 1) / 3) & 1, budget);
+                    if (__syncthreads_or(!done)) {
+                        bad = true;
+                        break;
+                    }
+                }
+                weights(3 * (st + 2), 3, wts + ((st + 2) % 3) * SB);
+            }
+            cp_commit();
         }
+        cp_wait<0>();
+    } else {
+        weights(0, 27, wts);
+        cp_commit();
+        cp_wait<0>();
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (tid == 0 && !fault)
+            for (int zi = 0; zi < tz; zi++) {
+                const uint64_t da = tc_sdesc(halo + zi * 180 * 16, chunk, 160), db = tc_sdesc(wts, (N + 1) * 16, 128);
+#pragma unroll
+                for (int tap = 0; tap < 27; tap++)
+                    tap_mmas(tap, tslot + zi * N, da, db + tap * nk8 * (N + 1));
+                tc_commit(mb0 + 8 * zi);
+            }
     }
-    ok = !__syncthreads_or(!ok);
-    bool done = ok && mbar_wait_for(mb_acc, 0, fault ? (1ll << 21) : kTcBudget);
-    done = !__syncthreads_or(!done);
-    tc_fence_after();
-    if (done) {
-        const int x = x0 + (tid & 7), y = y0 + (tid >> 3);
+    const uint32_t tmem = tslot;
+    const auto acc_bar = [&](int zi) { return mb0 + 8 * (kStream ? 3 : zi); };
+    // four warps cover an accumulator's 128 rows: planes alternate between the two halves of the block
+    for (int zi = warp >> 2; zi < tz && !bad; zi += 2) {
+        bad = !mbar_wait_for(acc_bar(zi), 0, budget);
+        bad = __any_sync(0xffffffffu, bad);
+        if (bad)
+            break;
+        tc_fence_after();
+        const int row = (warp & 3) * 32 + lane, x = x0 + (row & 7), y = y0 + (row >> 3);
         const bool mine = y < n;
-        const size_t r = ((((size_t)b * n + z0) * n + y) * n + x);
-        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+        const size_t r = ((((size_t)b * n + z0 + zi) * n + y) * n + x);
+        const uint32_t lane_base = tmem + zi * N + ((uint32_t)((warp & 3) * 32) << 16);
         for (int c0 = 0; c0 < N; c0 += 16) {
             float v[16];
             tc_ld16(lane_base + c0, v);
@@ -961,11 +1022,14 @@ __global__ void __launch_bounds__(128) k_conv3_halo(const __grid_constant__ CUte
             }
         }
     }
+    // every MMA has completed (or the wait for one ran out) before the block leaves
+    if (!bad)
+        bad = !mbar_wait_for(acc_bar(tz - 1), 0, budget);
     tc_fence_before();
-    __syncthreads();
+    bad = __syncthreads_or(bad);
     if (warp == 0)
-        tc_dealloc(tmem, NCOL);
-    if (!done && tid == 0)
+        tc_dealloc(tmem, ncol);
+    if (bad && tid == 0)
         atomicExch(err, 1);
 }
 
@@ -1245,27 +1309,49 @@ __global__ void k_pack_weights(const float *__restrict__ w, int Cin, int CKin, i
 // 2x2x2 mean pool (BF16, C channels): fine n = 2^lg -> coarse
 __global__ void k_pool(const bf16 *__restrict__ in, bf16 *__restrict__ out, int C, int lgc, int Vc)
 {
-    const int nc = 1 << lgc, m = nc - 1, lgf = lgc + 1;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vc * C; e += gridDim.x * blockDim.x) {
-        const int c = e % C, v = e / C;
+    const int nc = 1 << lgc, m = nc - 1, lgf = lgc + 1, C8 = C >> 3;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vc * C8; e += gridDim.x * blockDim.x) {
+        const int c = 8 * (e % C8), v = e / C8;
         const int x = v & m, y = (v >> lgc) & m, z = (v >> (2 * lgc)) & m, b = v >> (3 * lgc);
-        float s = 0.f;
+        uint4 q[8];
+#pragma unroll
         for (int k = 0; k < 8; k++) {
             const int fz = 2 * z + (k >> 2), fy = 2 * y + ((k >> 1) & 1), fx = 2 * x + (k & 1);
-            s += __bfloat162float(in[(size_t)((((b << lgf | fz) << lgf | fy) << lgf) | fx) * C + c]);
+            q[k] = *reinterpret_cast<const uint4 *>(
+                in + (size_t)((((b << lgf | fz) << lgf | fy) << lgf) | fx) * C + c);
         }
-        out[e] = __float2bfloat16_rn(0.125f * s);
+        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            float f[8];
+            unpack8(q[k], f);
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                s[i] += f[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+            s[i] *= 0.125f;
+        reinterpret_cast<uint4 *>(out)[e] =
+            make_uint4(pack2(s[0], s[1]), pack2(s[2], s[3]), pack2(s[4], s[5]), pack2(s[6], s[7]));
     }
 }
 
 // pool backward, added: dIn[fine] += dOut[coarse] / 8
 __global__ void k_pool_bwd_add(const float *__restrict__ dout, float *__restrict__ din, int C, int lgf, int Vf)
 {
-    const int nf = 1 << lgf, m = nf - 1, lgc = lgf - 1;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vf * C; e += gridDim.x * blockDim.x) {
-        const int c = e % C, v = e / C;
+    const int nf = 1 << lgf, m = nf - 1, lgc = lgf - 1, C4 = C >> 2;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vf * C4; e += gridDim.x * blockDim.x) {
+        const int c = 4 * (e % C4), v = e / C4;
         const int x = v & m, y = (v >> lgf) & m, z = (v >> (2 * lgf)) & m, b = v >> (3 * lgf);
-        din[e] += 0.125f * dout[(size_t)((((b << lgc | (z >> 1)) << lgc | (y >> 1)) << lgc) | (x >> 1)) * C + c];
+        const float4 d = *reinterpret_cast<const float4 *>(
+            dout + (size_t)((((b << lgc | (z >> 1)) << lgc | (y >> 1)) << lgc) | (x >> 1)) * C + c);
+        float4 o = reinterpret_cast<float4 *>(din)[e];
+        o.x += 0.125f * d.x;
+        o.y += 0.125f * d.y;
+        o.z += 0.125f * d.z;
+        o.w += 0.125f * d.w;
+        reinterpret_cast<float4 *>(din)[e] = o;
     }
 }
 
@@ -1273,15 +1359,17 @@ __global__ void k_pool_bwd_add(const float *__restrict__ dout, float *__restrict
 __global__ void k_upcat(const bf16 *__restrict__ low, int Cu, const bf16 *__restrict__ skip, int Cs,
                         bf16 *__restrict__ out, int lgf, int Vf)
 {
-    const int nf = 1 << lgf, m = nf - 1, lgc = lgf - 1, C = Cu + Cs;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vf * C; e += gridDim.x * blockDim.x) {
-        const int c = e % C, v = e / C;
+    const int nf = 1 << lgf, m = nf - 1, lgc = lgf - 1, C8 = (Cu + Cs) >> 3;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vf * C8; e += gridDim.x * blockDim.x) {
+        const int c = 8 * (e % C8), v = e / C8;
+        const bf16 *src;
         if (c < Cu) {
             const int x = v & m, y = (v >> lgf) & m, z = (v >> (2 * lgf)) & m, b = v >> (3 * lgf);
-            out[e] = low[(size_t)((((b << lgc | (z >> 1)) << lgc | (y >> 1)) << lgc) | (x >> 1)) * Cu + c];
+            src = low + (size_t)((((b << lgc | (z >> 1)) << lgc | (y >> 1)) << lgc) | (x >> 1)) * Cu + c;
         } else {
-            out[e] = skip[(size_t)v * Cs + c - Cu];
+            src = skip + (size_t)v * Cs + c - Cu;
         }
+        reinterpret_cast<uint4 *>(out)[e] = *reinterpret_cast<const uint4 *>(src);
     }
 }
 
@@ -1289,21 +1377,31 @@ __global__ void k_upcat(const bf16 *__restrict__ low, int Cu, const bf16 *__rest
 __global__ void k_upcat_bwd(const float *__restrict__ dout, int Cu, int Cs, float *__restrict__ dlow,
                             float *__restrict__ dskip, int lgc, int Vc)
 {
-    const int nc = 1 << lgc, m = nc - 1, lgf = lgc + 1, C = Cu + Cs;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vc * Cu; e += gridDim.x * blockDim.x) {
-        const int c = e % Cu, v = e / Cu;
+    const int nc = 1 << lgc, m = nc - 1, lgf = lgc + 1, C = Cu + Cs, U4 = Cu >> 2, S4 = Cs >> 2;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vc * U4; e += gridDim.x * blockDim.x) {
+        const int c = 4 * (e % U4), v = e / U4;
         const int x = v & m, y = (v >> lgc) & m, z = (v >> (2 * lgc)) & m, b = v >> (3 * lgc);
-        float s = 0.f;
+        float4 d[8];
+#pragma unroll
         for (int k = 0; k < 8; k++) {
             const int fz = 2 * z + (k >> 2), fy = 2 * y + ((k >> 1) & 1), fx = 2 * x + (k & 1);
-            s += dout[(size_t)((((b << lgf | fz) << lgf | fy) << lgf) | fx) * C + c];
+            d[k] = *reinterpret_cast<const float4 *>(
+                dout + (size_t)((((b << lgf | fz) << lgf | fy) << lgf) | fx) * C + c);
         }
-        dlow[e] = s;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            s.x += d[k].x;
+            s.y += d[k].y;
+            s.z += d[k].z;
+            s.w += d[k].w;
+        }
+        reinterpret_cast<float4 *>(dlow)[e] = s;
     }
     const int Vf = Vc * 8;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vf * Cs; e += gridDim.x * blockDim.x) {
-        const int c = e % Cs, v = e / Cs;
-        dskip[e] = dout[(size_t)v * C + Cu + c];
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Vf * S4; e += gridDim.x * blockDim.x) {
+        const int c = 4 * (e % S4), v = e / S4;
+        reinterpret_cast<float4 *>(dskip)[e] = *reinterpret_cast<const float4 *>(dout + (size_t)v * C + Cu + c);
     }
 }
 
@@ -1320,9 +1418,14 @@ __global__ void k_out1(const bf16 *__restrict__ d0, const float *__restrict__ w,
                        float *__restrict__ y, int V)
 {
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
+        const uint4 *q = reinterpret_cast<const uint4 *>(d0) + 2 * (size_t)v;
+        float f[16];
+        unpack8(q[0], f);
+        unpack8(q[1], f + 8);
         float s = b[0];
+#pragma unroll
         for (int c = 0; c < 16; c++)
-            s += __bfloat162float(d0[(size_t)v * 16 + c]) * w[c];
+            s += f[c] * w[c];
         y[v] = s;
     }
 }
@@ -1341,10 +1444,17 @@ __global__ void k_out1_bwd(const float *__restrict__ y, const float *__restrict_
         const float dy = 2.f * r * inv;
         accl += r * r * inv;
         accb += dy;
-        for (int c = 0; c < 16; c++) {
-            accw[c] += dy * __bfloat162float(d0[(size_t)v * 16 + c]);
-            dd0[(size_t)v * 16 + c] = dy * w[c];
-        }
+        const uint4 *q = reinterpret_cast<const uint4 *>(d0) + 2 * (size_t)v;
+        float f[16];
+        unpack8(q[0], f);
+        unpack8(q[1], f + 8);
+#pragma unroll
+        for (int c = 0; c < 16; c++)
+            accw[c] += dy * f[c];
+#pragma unroll
+        for (int c = 0; c < 16; c += 4)
+            *reinterpret_cast<float4 *>(dd0 + (size_t)v * 16 + c) =
+                make_float4(dy * w[c], dy * w[c + 1], dy * w[c + 2], dy * w[c + 3]);
     }
     // block reductions of the 16 weight gradients, the bias gradient and the loss
     float vals[18];
@@ -1467,12 +1577,9 @@ __global__ void k_make_input(const double *__restrict__ rho, const double *__res
         const int x = v & m, y = (v >> lg) & m, z = v >> (2 * lg);
         const size_t q = blk ? (size_t)b * E * E * E + ((size_t)(z + 2) * E + y + 2) * E + x + 2 : (size_t)e;
         const float s = scale[2 * b], sr = scale[2 * b + 1];
-        bf16 *o = x0 + (size_t)e * 16;
-        o[0] = __float2bfloat16_rn((float)(frho[b] * rho[q]) / s);
-        o[1] = __float2bfloat16_rn((float)phi[q] / s);
-        o[2] = __float2bfloat16_rn((float)rh2[e] / sr);
-        for (int c = 3; c < 16; c++)
-            o[c] = __float2bfloat16_rn(0.f);
+        uint4 *o = reinterpret_cast<uint4 *>(x0) + 2 * (size_t)e;
+        o[0] = make_uint4(pack2((float)(frho[b] * rho[q]) / s, (float)phi[q] / s), pack2((float)rh2[e] / sr, 0.f), 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -1558,6 +1665,14 @@ bool use_mma_sync()
     return on;
 }
 
+int ilog2(int n)
+{
+    int l = 0;
+    while ((1 << l) < n)
+        l++;
+    return l;
+}
+
 constexpr int kTcSmemMax = 200 * 1024;  // kTcStages stages of 128 x CK and N x CK BF16 tiles
 
 template <int N, bool FLIP>
@@ -1591,8 +1706,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-// the persistent halo kernel with UNET_HALO_P=1 (measured as fast as the
-// one-tile-per-block kernel at 4 x 64^3: 0.996 vs 0.989 ms a forward pass)
+// the persistent halo kernel with UNET_HALO_P=1 (as fast as the form of
+// k_conv3_halo with one plane per block, slower than with several)
 bool use_persistent_halo()
 {
     static const bool on = [] {
@@ -1602,42 +1717,33 @@ bool use_persistent_halo()
     return on;
 }
 
-// the halo kernel applies when all 27 taps' weights fit beside the halo and
-// the grid has at least 8 cells per edge
-bool halo_applies(int CK, int N, int lg) { return 27 * N * CK * 2 <= 64 * 1024 && lg >= 3 && CK <= 64; }
-
-template <int N, bool FLIP>
-cudaError_t conv_launch_halo(const bf16 *in, int CK, const bf16 *W, const float *bias, void *out, int out_bf16,
-                             int relu, int lg, int V, int *err, cudaStream_t s)
+template <int N, bool FLIP, int CK>
+cudaError_t conv_launch_halo(const bf16 *in, const bf16 *W, const float *bias, void *out, int out_bf16, int relu,
+                             int lg, int V, int *err, cudaStream_t s)
 {
-    const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc)
-        return cudaErrorNotSupported;
     const int n = 1 << lg, B = V >> (3 * lg);
-    CUtensorMap mi{};
-    const cuuint64_t di[5] = {(cuuint64_t)CK, (cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)B};
-    const cuuint64_t si[4] = {(cuuint64_t)CK * 2, (cuuint64_t)n * CK * 2, (cuuint64_t)n * n * CK * 2,
-                              (cuuint64_t)n * n * n * CK * 2};
-    const cuuint32_t bi[5] = {8, 10, 18, 3, 1}, e5[5] = {1, 1, 1, 1, 1};
-    if (enc(&mi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(in), di, si, bi, e5,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    const size_t smem = (size_t)(CK / 8) * kHaloChunk + (size_t)27 * (CK / 8) * N * 16;
-    static cudaError_t attr = cudaFuncSetAttribute(k_conv3_halo<N, FLIP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   200 * 1024);
+    static cudaError_t attr = cudaFuncSetAttribute(k_conv3_halo<N, FLIP, CK>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (attr)
         return attr;
-    const int tiles = B * n * ((n + 15) / 16) * (n / 8);
-    static const bool by_tma = [] {   // the halo by one TMA box per chunk; UNET_HALO_TMA=0: cp.async rows
-        const char *v = std::getenv("UNET_HALO_TMA");
-        return !(v && v[0] == '0');
-    }();
+    const int tiles = B * n * ((n + 15) / 16) * (n / 8);   // of one plane
     static const int fault = [] {   // UNET_FAULT_WAIT=1: the accumulator waits run out (test of that path)
         const char *v = std::getenv("UNET_FAULT_WAIT");
         return v && v[0] == '1' ? 1 : 0;
     }();
-    if (by_tma && use_persistent_halo()) {
+    if (halo_resident(CK, N) && use_persistent_halo()) {
+        const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+        if (!enc)
+            return cudaErrorNotSupported;
+        CUtensorMap mi{};
+        const cuuint64_t di[5] = {(cuuint64_t)CK, (cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)B};
+        const cuuint64_t si[4] = {(cuuint64_t)CK * 2, (cuuint64_t)n * CK * 2, (cuuint64_t)n * n * CK * 2,
+                                  (cuuint64_t)n * n * n * CK * 2};
+        const cuuint32_t bi[5] = {8, 10, 18, 3, 1}, e5[5] = {1, 1, 1, 1, 1};
+        if (enc(&mi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<bf16 *>(in), di, si, bi, e5,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
         // persistent form: as many blocks as fit on the SMs at once, but never
         // more per SM than TMEM holds (each block keeps two accumulators of
         // NCOL columns allocated for its whole life; a block that could not
@@ -1675,8 +1781,34 @@ cudaError_t conv_launch_halo(const bf16 *in, int CK, const bf16 *W, const float 
             return cudaGetLastError();
         }
     }
-    k_conv3_halo<N, FLIP><<<tiles, 128, smem, s>>>(mi, in, by_tma ? 1 : 0, W, CK, bias, out, out_bf16, relu, lg, B,
-                                                   fault, err);
+    // planes per block: fewer loads per voxel against fewer blocks.  Time of a
+    // wave of blocks on an SM in cycles: copies at 64 bytes and MMAs at 32
+    // cycles (each reads 4 KB of shared memory) overlap between the blocks of an
+    // SM; a block alone does one after the other.
+    int tz = 1, ncol = 32;
+    size_t smem = 0;
+    double best = 0.0;
+    for (int z = 1; z <= (halo_resident(CK, N) ? 4 : 1); z *= 2) {
+        const int cols = std::max(32, z * N);
+        const size_t sm =
+            (size_t)(CK / 8) * halo_chunk(z) + (size_t)(halo_resident(CK, N) ? 27 : 9) * (CK / 8) * (N + 1) * 16;
+        if (sm > 226 * 1024 || cols > 512)
+            continue;
+        const int per_sm = std::min((int)(227 * 1024 / (sm + 2048)), 512 / cols);
+        const double copy = sm / 64.0, mma = z * 27.0 * (CK / 16) * 32.0;
+        const int blocks = tiles / z, waves = (blocks + 152 * per_sm - 1) / (152 * per_sm);
+        const int co = std::min(per_sm, (blocks + 151) / 152);   // blocks at once on an SM
+        const double time = waves * (co * std::max(copy, mma) + std::min(copy, mma) + 3000.0);
+        if (best == 0.0 || time < best) {
+            best = time;
+            tz = z;
+            ncol = cols;
+            smem = sm;
+        }
+    }
+    if (!smem)
+        return cudaErrorInvalidValue;
+    k_conv3_halo<N, FLIP, CK><<<tiles / tz, 256, smem, s>>>(in, W, bias, out, out_bf16, relu, lg, tz, ncol, fault, err);
     return cudaGetLastError();
 }
 
@@ -1698,8 +1830,15 @@ cudaError_t conv_launch(const TIn *in, int CK, const bf16 *W, const float *bias,
 {
     if (!use_mma_sync()) {
         if constexpr (sizeof(TIn) == 2) {
-            if (use_halo() && halo_applies(CK, NT * 8, lg))
-                return conv_launch_halo<NT * 8, FLIP>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
+            if (use_halo() && lg >= 3) {
+#define HALO(ck)      \
+    if (CK == ck)     \
+        return conv_launch_halo<NT * 8, FLIP, ck>(in, W, bias, out, out_bf16, relu, lg, V, err, s);
+                HALO(16) HALO(32) HALO(64)
+                if constexpr (NT * 8 <= 32)
+                    HALO(128)
+#undef HALO
+            }
             return conv_launch_tc<NT * 8, FLIP>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
         }
         return cudaErrorInvalidValue;
@@ -1719,14 +1858,6 @@ cudaError_t conv_any(const TIn *in, int CK, const bf16 *W, const float *bias, in
     case 128: return conv_launch<16, FLIP, TIn>(in, CK, W, bias, out, out_bf16, relu, lg, V, err, s);
     }
     return cudaErrorInvalidValue;
-}
-
-int ilog2(int n)
-{
-    int l = 0;
-    while ((1 << l) < n)
-        l++;
-    return l;
 }
 
 cudaError_t pack_all(mg_unet *u)
@@ -1754,18 +1885,18 @@ cudaError_t forward(mg_unet *u, int B, int lg)
         return e;
     FWD(0, u->x0, u->a0, lg, V0);
     FWD(1, u->a0, u->s0, lg, V0);
-    k_pool<<<blocks_for((long)V1 * 16), kT, 0, s>>>(u->s0, u->p0, 16, lg - 1, V1);
+    k_pool<<<blocks_for((long)V1 * 2), kT, 0, s>>>(u->s0, u->p0, 16, lg - 1, V1);
     FWD(2, u->p0, u->a1, lg - 1, V1);
     FWD(3, u->a1, u->s1, lg - 1, V1);
-    k_pool<<<blocks_for((long)V2 * 32), kT, 0, s>>>(u->s1, u->p1, 32, lg - 2, V2);
+    k_pool<<<blocks_for((long)V2 * 4), kT, 0, s>>>(u->s1, u->p1, 32, lg - 2, V2);
     FWD(4, u->p1, u->s2, lg - 2, V2);
-    k_pool<<<blocks_for((long)V3 * 64), kT, 0, s>>>(u->s2, u->p2, 64, lg - 3, V3);
+    k_pool<<<blocks_for((long)V3 * 8), kT, 0, s>>>(u->s2, u->p2, 64, lg - 3, V3);
     FWD(5, u->p2, u->a3, lg - 3, V3);
-    k_upcat<<<blocks_for((long)V2 * 128), kT, 0, s>>>(u->a3, 64, u->s2, 64, u->u2, lg - 2, V2);
+    k_upcat<<<blocks_for((long)V2 * 16), kT, 0, s>>>(u->a3, 64, u->s2, 64, u->u2, lg - 2, V2);
     FWD(6, u->u2, u->d2, lg - 2, V2);
-    k_upcat<<<blocks_for((long)V1 * 64), kT, 0, s>>>(u->d2, 32, u->s1, 32, u->u1, lg - 1, V1);
+    k_upcat<<<blocks_for((long)V1 * 8), kT, 0, s>>>(u->d2, 32, u->s1, 32, u->u1, lg - 1, V1);
     FWD(7, u->u1, u->d1, lg - 1, V1);
-    k_upcat<<<blocks_for((long)V0 * 32), kT, 0, s>>>(u->d1, 16, u->s0, 16, u->u0, lg, V0);
+    k_upcat<<<blocks_for((long)V0 * 4), kT, 0, s>>>(u->d1, 16, u->s0, 16, u->u0, lg, V0);
     FWD(8, u->u0, u->d0, lg, V0);
 #undef FWD
     k_out1<<<blocks_for(V0), kT, 0, s>>>(u->d0, P + u->nparam - 17, P + u->nparam - 1, u->y, V0);
@@ -1865,26 +1996,26 @@ cudaError_t backward(mg_unet *u, int B, int lg)
         (e = dgrad(u, 8, gA, gB, lg, V0)))
         return e;                                                        // gB = du0 [V0][32]
     // split du0 -> dd1 (coarse) and ds0 (gC)
-    k_upcat_bwd<<<blocks_for((long)V0 * 16), kT, 0, s>>>(gB, 16, 16, gA, gC, lg - 1, V1);   // gA = dd1 [V1][16], gC = ds0 [V0][16]
+    k_upcat_bwd<<<blocks_for((long)V0 * 4), kT, 0, s>>>(gB, 16, 16, gA, gC, lg - 1, V1);   // gA = dd1 [V1][16], gC = ds0 [V0][16]
     if ((e = wgrad(u, 7, u->u1, u->d1, gA, lg - 1, V1)) ||
         (e = dgrad(u, 7, gA, gB, lg - 1, V1)))
         return e;                                                        // gB = du1 [V1][64]
     // ds1 lives behind ds0 in gC
     float *ds1 = gC + (size_t)V0 * 16;
-    k_upcat_bwd<<<blocks_for((long)V1 * 32), kT, 0, s>>>(gB, 32, 32, gA, ds1, lg - 2, V2);  // gA = dd2 [V2][32]
+    k_upcat_bwd<<<blocks_for((long)V1 * 8), kT, 0, s>>>(gB, 32, 32, gA, ds1, lg - 2, V2);  // gA = dd2 [V2][32]
     if ((e = wgrad(u, 6, u->u2, u->d2, gA, lg - 2, V2)) ||
         (e = dgrad(u, 6, gA, gB, lg - 2, V2)))
         return e;                                                        // gB = du2 [V2][128]
     float *ds2 = ds1 + (size_t)V1 * 32;
-    k_upcat_bwd<<<blocks_for((long)V2 * 64), kT, 0, s>>>(gB, 64, 64, gA, ds2, lg - 3, V3);  // gA = da3 [V3][64]
+    k_upcat_bwd<<<blocks_for((long)V2 * 16), kT, 0, s>>>(gB, 64, 64, gA, ds2, lg - 3, V3);  // gA = da3 [V3][64]
     if ((e = wgrad(u, 5, u->p2, u->a3, gA, lg - 3, V3)) ||
         (e = dgrad(u, 5, gA, gB, lg - 3, V3)))
         return e;                                                        // gB = dp2 [V3][64]
-    k_pool_bwd_add<<<blocks_for((long)V2 * 64), kT, 0, s>>>(gB, ds2, 64, lg - 2, V2);
+    k_pool_bwd_add<<<blocks_for((long)V2 * 16), kT, 0, s>>>(gB, ds2, 64, lg - 2, V2);
     if ((e = wgrad(u, 4, u->p1, u->s2, ds2, lg - 2, V2)) ||
         (e = dgrad(u, 4, ds2, gB, lg - 2, V2)))
         return e;                                                        // gB = dp1 [V2][32]
-    k_pool_bwd_add<<<blocks_for((long)V1 * 32), kT, 0, s>>>(gB, ds1, 32, lg - 1, V1);
+    k_pool_bwd_add<<<blocks_for((long)V1 * 8), kT, 0, s>>>(gB, ds1, 32, lg - 1, V1);
     if ((e = wgrad(u, 3, u->a1, u->s1, ds1, lg - 1, V1)) ||
         (e = dgrad(u, 3, ds1, gB, lg - 1, V1)))
         return e;                                                        // gB = da1 [V1][32]
@@ -1892,7 +2023,7 @@ cudaError_t backward(mg_unet *u, int B, int lg)
         (e = dgrad(u, 2, gB, gA, lg - 1, V1)))
         return e;                                                        // gA = dp0 [V1][16]
     float *ds0 = gC;
-    k_pool_bwd_add<<<blocks_for((long)V0 * 16), kT, 0, s>>>(gA, ds0, 16, lg, V0);
+    k_pool_bwd_add<<<blocks_for((long)V0 * 4), kT, 0, s>>>(gA, ds0, 16, lg, V0);
     if ((e = wgrad(u, 1, u->a0, u->s0, ds0, lg, V0)) ||
         (e = dgrad(u, 1, ds0, gB, lg, V0)))
         return e;                                                        // gB = da0 [V0][16]

@@ -461,3 +461,25 @@ def test_weight_gradients_by_rows_elementwise_dyadic(un, n, B):
         assert (gr != 0).mean() > 0.01
     finally:
         un.mg_unet_destroy(u)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,B", [(8, 1), (16, 3), (32, 2), (64, 1), (64, 4)])
+def test_forward_bitwise_dyadic_at_every_tile_shape(un, n, B):
+    """The forward output on the dyadic case (every sum exact) equals the
+    reference bit for bit where a convolution block takes one, two or four
+    planes of its grid and where its weights stay or stream."""
+    import torch
+    from oracle import unet_ref as R
+    rho, phi, res, tru, frho, p = _dyadic_case(2, n, B)
+    u = un.mg_unet_create(n, B, seed=0)
+    try:
+        un.mg_unet_set_params(u, p)
+        dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        y = un.mg_unet_forward(u, B, n, dev(rho), dev(phi), dev(res), frho)
+        T = torch.from_numpy
+        yr, _ = R.forward(T(p.astype(np.float64)), T(rho), T(phi), T(res), frho, emulate=True)
+        yr = yr.detach().numpy().astype(np.float32)
+        assert np.array_equal(np.asarray(y).reshape(yr.shape), yr)
+    finally:
+        un.mg_unet_destroy(u)
