@@ -579,46 +579,49 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(const bf16 *__restrict__ in, i
 // one plane z, all x) of the output gradient and the rows y0 - 1 .. of plane
 // z + dz of the input, per row one line of voxels per 8 channels.  A start
 // address 16 bytes on is a shift by one voxel (dx), and the lines of
-// consecutive rows are evenly spaced, so one MMA takes 128 / CK input rows
-// (M = row, channel) and TB gradient rows (N = row, channel) over 16 voxels of
-// x (two groups of 8 rows on the 8^3 grid): its D holds every dy = input row -
-// gradient row of them, and the rest of D (other row pairs, rows past the
-// tile) is ignored.  A block keeps the three dx (and the MA row groups that
-// TB + 2 input rows need) of one dz in TMEM over all its stages, two in
-// flight, and adds its sums into dW with 16-byte reductions.
+// consecutive rows are evenly spaced, so one MMA takes the input rows of all
+// three dy (M = row, channel; 128 / CK rows, what is past the third ignored)
+// over 16 voxels of x (two rows on the 8^3 grid).  A block keeps the ndx
+// shifts of one dz in TMEM over its stages, two in flight, and adds its sums
+// into dW with 16-byte reductions.  With NZ = 3 (planes of at least
+// kWgradChain voxels) a stage holds 4 rows of an input plane and of the gradient planes z
+// - dz of all three dz, side by side in N, which an MMA takes in the time of
+// one: a third of the MMAs.
+// The tensor core rounds each sum in its FP32 accumulators towards zero, an
+// error that grows with the number of MMAs that an accumulator takes.  A block
+// takes kWgradChain voxels in memory order, the products of k_wgrad_tc's
+// accumulators in the same order: the sums are equal bit for bit up to the
+// order of the reductions into dW.  Two or four gradient rows in N would need
+// as many times fewer MMAs, but other sums (up to 3e-5 relative off).
 // The gather by tap (k_wgrad_tc) spent its time in the transposing stores,
-// eight-way bank conflicts among them, once per tap: 4 x 64^3 voxels, 32 -> 16
-// channels 1022 -> 123 us and 16 -> 16 608 -> 56 us, 4 x 8^3, 64 -> 64 111 ->
-// 13 us.  What bounds it now is the MMAs' reading of A (4 KB of shared memory,
-// 32 cycles each, for 16 voxels of TB rows) beside the copies of a stage (59
-// KB for 512 voxels, from L2).  Error of the sums against FP64, relative in the
-// 2-norm: 3e-6 -> 2e-6 at 64^3, 1e-6 -> 1e-7 at 8^3 (shorter accumulator
-// chains, see kChain).  Grids of less than 8^3 voxels and layers whose stages
-// do not fit stay with k_wgrad_tc.
-template <int CK, int N>
+// eight-way bank conflicts among them, once per tap.
+// Training step of 4 samples of 64^3: 5538 us with the gather, 1998 us with
+// NZ = 1 everywhere, 1679 us with NZ = 3 at 64^3 (1416 us with two or four
+// gradient rows in N).  What bounds it is the MMAs, 32 cycles each for the 4
+// KB of A that they read.
+// Grids of less than 8^3 voxels and layers whose stages do not fit stay with
+// k_wgrad_tc.
+constexpr int kWgradChain = 4096;   // voxels per accumulator
+
+template <int CK, int N, int NZ>
 struct WgradTile {
-    static constexpr int kRA = 128 / CK;                              // input rows of one MMA
-    static constexpr int kTB = CK == 16 ? 4 : CK == 32 ? 2 : N == 16 ? 2 : 1;   // gradient rows of one MMA
-    static constexpr int kMA = (kTB + 2 + kRA - 1) / kRA;
-    static constexpr int kTY = 8;
-    static constexpr int kRows = kTY - kTB + kRA * kMA;               // input rows an MMA may read
-    // The tensor core adds to its FP32 accumulators with more error than a
-    // rounded addition, so no accumulator takes more than kChain MMAs: stages
-    // take kSets sets of accumulators in turn, and a block at most
-    // kChain kSets / (MMAs of one accumulator per stage) stages.
-    static constexpr int kChain = 256;
-    static constexpr int kSetCols = 3 * kMA * kTB * N;
-    static constexpr int kSets = kSetCols <= 128 ? 4 : 1;
-    static constexpr int kCols = kSets * kSetCols;
-    static constexpr int kAlloc = kCols <= 256 ? 256 : 512;
-    static int items_max(int n) { return kChain * kSets / (kTY / kTB * std::max(n, 16) / 16 / (n == 8 ? 2 : 1)); }
+    static constexpr int kRA = 128 / CK;              // input rows of one MMA
+    static constexpr int kMA = (3 + kRA - 1) / kRA;   // MMAs for the three dy
+    static constexpr int kTY = NZ == 3 ? 4 : 8;
+    static constexpr int kRows = kTY - 1 + kRA * kMA; // input rows an MMA may read
+    static constexpr int kCols = 3 * kMA * NZ * N;
+    static constexpr int kAlloc = kCols <= 64 ? 64 : kCols <= 128 ? 128 : kCols <= 256 ? 256 : 512;
     // voxels per line: x = -1 .. n and one more (odd: lines of different channels in different banks)
     __host__ __device__ static int pa(int n) { return n + 3; }
     __host__ __device__ static int pb(int n) { return n + 1; }
     __host__ __device__ static int a_bytes(int n) { return kRows * (CK / 8) * pa(n) * 16; }
-    __host__ __device__ static int stage(int n) { return a_bytes(n) + kTY * (N / 8) * pb(n) * 16; }
+    __host__ __device__ static int stage(int n) { return a_bytes(n) + kTY * NZ * (N / 8) * pb(n) * 16; }
     static constexpr int kSmemMax = 226 * 1024;
-    static bool applies(int lg) { return lg >= 3 && 2 * stage(1 << lg) <= kSmemMax; }
+    static bool applies(int lg)
+    {
+        return kCols <= 512 && lg >= 3 && (NZ == 1 || 1 << 2 * lg >= kWgradChain) && kTY << lg <= kWgradChain &&
+               2 * stage(1 << lg) <= kSmemMax;
+    }
 };
 
 __device__ __forceinline__ void red_add4(float *p, const float *v)
@@ -627,14 +630,14 @@ __device__ __forceinline__ void red_add4(float *p, const float *v)
                  : "memory");
 }
 
-template <int CK, int N>
+template <int CK, int N, int NZ>
 __global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in, int Cin, const bf16 *__restrict__ d,
-                                                    float *__restrict__ dW, int lg, int B, int *__restrict__ err)
+                                                    float *__restrict__ dW, int lg, int B, int ndx, int *__restrict__ err)
 {
-    typedef WgradTile<CK, N> W;
-    constexpr int CG = CK / 8, NG = N / 8, TY = W::kTY;
+    typedef WgradTile<CK, N, NZ> W;
+    constexpr int CG = CK / 8, NG = N / 8, TY = W::kTY, LTY = TY == 4 ? 2 : 3;
     // BF16 operands, both M- / N-major
-    constexpr uint32_t IDESC = tc_idesc_bf16(128, W::kTB * N) | (1u << 15) | (1u << 16);
+    constexpr uint32_t IDESC = tc_idesc_bf16(128, NZ * N) | (1u << 15) | (1u << 16);
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t mbar[2];
     __shared__ uint32_t tslot;
@@ -659,10 +662,12 @@ __global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in,
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tslot;
-    const int dz = (int)blockIdx.y - 1;
-    const int lgt = lg - 3, nitem = B << (lg + lgt);   // items: (sample, z, group of 8 rows)
+    // blockIdx.y: dz (NZ = 1) and the first dx (ndx = 3: all of them; else ndx = 1)
+    const int dz = NZ == 3 ? 0 : (int)blockIdx.y % 3 - 1, dx0 = NZ == 3 ? (int)blockIdx.y : (int)blockIdx.y / 3;
+    const int lgt = lg - LTY, chain = kWgradChain >> (lg + LTY);
+    const int it0 = blockIdx.x * chain, nitem = min(it0 + chain, B << (lg + lgt));   // items: (sample, z, TY rows)
     auto next_item = [&](int it) {
-        for (; it < nitem; it += gridDim.x) {
+        for (; it < nitem; it++) {
             const int z = ((it >> lgt) & (n - 1)) + dz;
             if ((unsigned)z < (unsigned)n)
                 break;
@@ -678,22 +683,28 @@ __global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in,
             const bool ok = (unsigned)y < (unsigned)n;
             cp16(As + ((row * CG + cg) * PA + x + 1) * 16, ok ? pa + ((size_t)(y << lg) + x) * CK + 8 * cg : pa, ok);
         }
-        const bf16 *pd = d + ((size_t)((((b << lg) + z) << lg) + y0) << lg) * N;
-        for (int e = tid; e < TY * n * NG; e += 256) {
-            const int ng = e & (NG - 1), x = (e / NG) & (n - 1), row = (e / NG) >> lg;
-            cp16(Bs + ((row * NG + ng) * PB + x) * 16, pd + ((size_t)(row << lg) + x) * N + 8 * ng, true);
+#pragma unroll
+        for (int q = 0; q < NZ; q++) {   // gradient planes z - dz (NZ = 3: dz = q - 1)
+            const int zg = NZ == 3 ? z - q + 1 : z;
+            const bool ok = (unsigned)zg < (unsigned)n;
+            const bf16 *pd = ok ? d + ((size_t)((((b << lg) + zg) << lg) + y0) << lg) * N : d;
+            for (int e = tid; e < TY * n * NG; e += 256) {
+                const int ng = e & (NG - 1), x = (e / NG) & (n - 1), row = (e / NG) >> lg;
+                cp16(Bs + (((row * NZ + q) * NG + ng) * PB + x) * 16,
+                     ok ? pd + ((size_t)(row << lg) + x) * N + 8 * ng : d, ok);
+            }
         }
     };
-    const uint32_t lboA = n == 8 ? W::kTB * CG * PA * 16 : 128, lboB = n == 8 ? W::kTB * NG * PB * 16 : 128;
-    const int ystep = n == 8 ? 2 * W::kTB : W::kTB;
-    int it = next_item(blockIdx.x), issued = 0;
+    const uint32_t lboA = n == 8 ? CG * PA * 16 : 128, lboB = n == 8 ? NG * PB * 16 : 128;
+    const int ystep = n == 8 ? 2 : 1;
+    int it = next_item(it0), issued = 0;
     uint32_t phases = 0u;
     bool bad = false;
     if (it < nitem)
         fill(it, 0);
     cp_commit();
     while (it < nitem) {
-        const int nx = next_item(it + gridDim.x), s = issued & 1;
+        const int nx = next_item(it + 1), s = issued & 1;
         if (nx < nitem) {
             if (issued > 0) {   // the other stage's MMAs have finished reading it
                 const bool done = mbar_wait_for(mb0 + 8 * (s ^ 1), (phases >> (s ^ 1)) & 1u, kTcBudget);
@@ -714,17 +725,18 @@ __global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in,
         if (tid == 0) {
             const uint64_t da0 = tc_sdesc(sm0 + s * sbytes, lboA, PA * 16);
             const uint64_t db0 = tc_sdesc(sm0 + s * sbytes + abytes, lboB, PB * 16);
-            bool first = issued < W::kSets;
-            const uint32_t acc = tmem + (issued & (W::kSets - 1)) * W::kSetCols, step = W::kRA * CG * PA;
+            const uint32_t lines = W::kRA * CG * PA;
+            bool first = issued == 0;
             for (int yb = 0; yb < TY; yb += ystep) {
-                uint64_t da = da0 + yb * CG * PA, db = db0 + yb * NG * PB;
+                uint64_t da = da0 + yb * CG * PA + dx0, db = db0 + yb * NZ * NG * PB;
                 for (int x0 = 0; x0 < n; x0 += 16, da += 16, db += 16) {
 #pragma unroll
                     for (int dx = 0; dx < 3; dx++)
+                        if (dx < ndx)
 #pragma unroll
-                        for (int ma = 0; ma < W::kMA; ma++)
-                            tc_mma(acc + (dx * W::kMA + ma) * W::kTB * N, da + dx + ma * step, db, IDESC,
-                                   first ? 0u : 1u);
+                            for (int ma = 0; ma < W::kMA; ma++)
+                                tc_mma(tmem + (dx * W::kMA + ma) * NZ * N, da + dx + ma * lines, db, IDESC,
+                                       first ? 0u : 1u);
                     first = false;
                 }
             }
@@ -744,21 +756,14 @@ __global__ void __launch_bounds__(256) k_wgrad_rows(const bf16 *__restrict__ in,
     if (done && !bad && issued > 0) {
         const int m = (warp & 3) * 32 + (tid & 31), ci = m & (CK - 1);
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        for (int q = warp >> 2; q < 3 * W::kMA * W::kTB; q += 2) {   // column blocks (dx, row group, gradient row)
-            const int b = q % W::kTB, ma = (q / W::kTB) % W::kMA, dx = q / (W::kTB * W::kMA);
-            const int dy = ma * W::kRA + m / CK - b;
-            float *o = dW + ((size_t)((blockIdx.y * 3 + dy) * 3 + dx) * Cin + ci) * N;
+        for (int q = warp >> 2; q < ndx * W::kMA * NZ; q += 2) {   // column blocks (dx, group of dy, dz)
+            const int ma = q / NZ % W::kMA, dx = dx0 + q / (NZ * W::kMA), dy = ma * W::kRA + m / CK;
+            const int tz = NZ == 3 ? q % NZ : dz + 1;
+            float *o = dW + ((size_t)(tz * 9 + dy * 3 + dx) * Cin + ci) * N;
             for (int c0 = 0; c0 < N; c0 += 16) {
                 float v[16];
                 tc_ld16(lane_base + q * N + c0, v);
-                for (int set = 1; set < min(W::kSets, issued); set++) {
-                    float w[16];
-                    tc_ld16(lane_base + set * W::kSetCols + q * N + c0, w);
-#pragma unroll
-                    for (int i = 0; i < 16; i++)
-                        v[i] += w[i];
-                }
-                if (dy >= 0 && dy < 3 && ci < Cin)
+                if (dy < 3 && ci < Cin)
 #pragma unroll
                     for (int i = 0; i < 16; i += 4)
                         red_add4(o + c0 + i, v + i);
@@ -1903,30 +1908,38 @@ cudaError_t forward(mg_unet *u, int B, int lg)
     return cudaGetLastError();
 }
 
+template <int CK, int N, int NZ>
+cudaError_t wgrad_rows(const bf16 *in, int Cin, const bf16 *gbf, float *dW, int lg, int V, int *err, cudaStream_t s)
+{
+    typedef WgradTile<CK, N, NZ> W;
+    static cudaError_t attr = cudaFuncSetAttribute(k_wgrad_rows<CK, N, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   W::kSmemMax);
+    if (attr)
+        return attr;
+    // no more blocks per SM than tensor memory has room for: a block never waits for its columns
+    const int most = 512 / W::kAlloc, smem = std::max(2 * W::stage(1 << lg), W::kSmemMax / (most + 1) + 1024);
+    // a block per chain (and dz with NZ = 1), and per dx where that leaves SMs without one
+    const int chains = (V + kWgradChain - 1) / kWgradChain, nz = NZ == 3 ? 1 : 3, ndx = nz * chains < 152 ? 1 : 3;
+    k_wgrad_rows<CK, N, NZ><<<dim3(chains, ndx == 1 ? 3 * nz : nz), 256, smem, s>>>(in, Cin, gbf, dW, lg,
+                                                                                   V >> (3 * lg), ndx, err);
+    return cudaGetLastError();
+}
+
 template <int CK, int N>
 cudaError_t wgrad_tc(const bf16 *in, int Cin, const float *g, const bf16 *gbf, float *dW, int lg, int V, int *err,
                      cudaStream_t s)
 {
-    typedef WgradTile<CK, N> W;
-    if (W::applies(lg)) {
-        static cudaError_t attr = cudaFuncSetAttribute(k_wgrad_rows<CK, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       W::kSmemMax);
-        if (attr)
-            return attr;
-        // no more blocks per SM than tensor memory has room for: a block never waits for its columns
-        const int most = 512 / W::kAlloc, smem = std::max(2 * W::stage(1 << lg), W::kSmemMax / (most + 1) + 1024);
-        const int B = V >> (3 * lg), items = B << (2 * lg - 3), per_sm = std::max(1, W::kSmemMax / smem);
-        const int most_items = W::items_max(1 << lg);
-        const dim3 grid(std::max(std::min(items, 152 * per_sm / 3), (items + most_items - 1) / most_items), 3);
-        k_wgrad_rows<CK, N><<<grid, 256, smem, s>>>(in, Cin, gbf, dW, lg, B, err);
-        return cudaGetLastError();
-    }
+    if constexpr (WgradTile<CK, N, 3>::kCols <= 512)
+        if (WgradTile<CK, N, 3>::applies(lg))
+            return wgrad_rows<CK, N, 3>(in, Cin, gbf, dW, lg, V, err, s);
+    if (WgradTile<CK, N, 1>::applies(lg))
+        return wgrad_rows<CK, N, 1>(in, Cin, gbf, dW, lg, V, err, s);
     constexpr size_t smem = 2 * ((size_t)128 * 64 * 2 + (size_t)N * 64 * 2);
     static cudaError_t attr = cudaFuncSetAttribute(k_wgrad_tc<CK, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)smem);
     if (attr)
         return attr;
-    const int vchunk = 4096;
+    const int vchunk = kWgradChain;
     dim3 grid((V + vchunk - 1) / vchunk, (27 + 128 / CK - 1) / (128 / CK));
     k_wgrad_tc<CK, N><<<grid, 128, smem, s>>>(in, Cin, g, dW, lg, V, vchunk, err);
     return cudaGetLastError();
@@ -1937,7 +1950,7 @@ bool wgrad_by_rows(int CK, int N, int lg)
 {
 #define WG(ck, nn)                   \
     if (CK == ck && N == nn)         \
-        return WgradTile<ck, nn>::applies(lg);
+        return WgradTile<ck, nn, 1>::applies(lg) || WgradTile<ck, nn, 3>::applies(lg);
     WG(16, 16) WG(16, 32) WG(32, 32) WG(32, 64) WG(64, 64) WG(128, 32) WG(64, 16) WG(32, 16)
 #undef WG
     return false;
