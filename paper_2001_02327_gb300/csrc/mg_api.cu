@@ -136,18 +136,23 @@ void plan_tiles(LevelData &ld, int dim, int nu_pre, int nu_post)
 // run the box-patch kernels (mg_box.cu), whose colour pass moves exactly its
 // algorithmic bytes; levels below stay plain for the bottom, plane-marching
 // and blocked kernels.  MG_SPLIT=S fixes S; without it (and without tuning)
-// the levels of 192 cells per edge or more are split (measured on 4 nested
-// 256^3 levels: the 258^3 level gains 33.4 -> 28.6 ms, splitting the 129^3
-// level as well costs 0.9 ms, and at 66^3 the tuner keeps plain), unless MG_WAVE,
-// MG_WAVE_PLAN or MG_TB_TILE ask for the plain-layout plans.  mg_autotune
+// the leading levels of kSplitMinN cells per edge or more are split, and in 3D
+// the first level from kSplitFirst (kSplitFirstBatch in batches) cells.
+// Measured in mixed precision, plain -> split first level: 3 nested 64^3 2.41
+// -> 2.45 ms, 96^3 3.59 -> 3.56, 128^3 5.14 -> 4.81, 160^3 7.55 -> 6.56; 4
+// nested 256^3 29.4 -> 20.8 ms, and 21.3 with the 129^3 level split as well.
+// Where the branches of a batch fill the SMs, the instructions count at
+// smaller sizes too: 32 hierarchies of 32 to 128 cells per edge 36.5 ms plain,
+// 30.0 split from 98 cells, 29.7 from 66 or from 50.  MG_WAVE,
+// MG_WAVE_PLAN or MG_TB_TILE ask for the plain-layout plans instead.  mg_autotune
 // times the choices; the batched kernels (MG_BATCHED=1) run plain levels
 // only.  Changing the layout clears the level's FP32 arrays (their ghost
 // layer must read zero in either layout).
 int first_fused(const LevelData &ld, bool fp32);
 constexpr int kTileSplit = 1 << 16;   // mg_tuning / tuning-cache code of a split level
-constexpr int kSplitMinN = 192;
+constexpr int kSplitMinN = 192, kSplitFirst = 100, kSplitFirstBatch = 60;
 
-int split_default(const LevelData &ld)
+int split_default(const LevelData &ld, int dim, int batch)
 {
     if (ld.Lc[1] >= 0 || ld.frozen)   // the cluster kernel runs plain levels
         return 0;
@@ -162,6 +167,8 @@ int split_default(const LevelData &ld)
     int S = 0;
     while (S < Ls && ld.g[S].N >= kSplitMinN)
         S++;
+    if (S == 0 && Ls > 0 && dim == 3 && ld.g[0].N >= (batch > 1 ? kSplitFirstBatch : kSplitFirst))
+        S = 1;
     return S;
 }
 
@@ -380,7 +387,9 @@ void build_geometry(LevelData &ld, int dim)
     ld.nsplit = 0;
 }
 
-#define MG_BRANCHES 8   // parallel branches of the solve graph (hierarchies of a batch)
+// parallel branches of the solve graph (hierarchies of a batch): 32 hierarchies of 32 to 128 cells per edge 29.7 ms
+// with 8, 28.8 with 16 or 24
+#define MG_BRANCHES 16
 
 enum KernelKind { KK_SMOOTH, KK_RESTRICT, KK_PROLONG, KK_NORM, KK_DEFECT, KK_ACCUM, KK_IFACE, KK_FORCES,
                   KK_SETDENS, KK_BOTTOM, KK_TB_PRE, KK_TB_POST, KK_CLUSTER, KK_SMOOTH0, KK_WAVE, KK_WAVE0, KK_COUNT };
@@ -2392,7 +2401,7 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
             if (e == cudaSuccess)
                 e = plan_slab(h, ld, true);
             if (e == cudaSuccess && o.precision == MG_MIXED)
-                e = plan_split(ld, dim, split_default(ld), h->stream);
+                e = plan_split(ld, dim, split_default(ld, dim, batch), h->stream);
         }
     if (e == cudaSuccess) {
         std::vector<double> fr((size_t)batch * MG_MAX_LEVELS, 0.0);
