@@ -1518,19 +1518,20 @@ bool persist_eligible(const mg_hierarchy *h)
 }
 
 // Which hierarchies of an eligible batch the persistent launch takes.  Cost
-// model, calibrated on GB300 batches of 512 hierarchies of 16-32 and 32-48
-// cells per edge and of 64 and 512 hierarchies of 32-128: a graph branch
-// costs about 2.3 us per kernel node (Ls (2 nu_pre + 1) + 1 + Ls (2 nu_post
-// + 1) nodes per V-cycle, 12 V-cycles per level assumed, 8 branches at once)
-// plus its cells at 1.5e9 per second; the persistent launch solves 6e6 cells
-// per second per block, 2 blocks per SM, largest hierarchy first.  The whole
-// batch goes to the persistent launch when that estimate is the shorter:
-// run beside graph branches it takes SMs and bandwidth from them (measured:
-// a split of the 512-hierarchy batch of 32-128 took 707 ms against 642 ms
-// with graph branches only).  MG_PERSIST=1 / 0 forces all / none (the
-// batched kernels, MG_BATCHED=1, exclude it); MG_PERSIST_COUNT=k gives the k
-// smallest hierarchies to it and the rest to graph branches in the same
-// graph.
+// model, calibrated on GB300: graph branches cost about 2.3 us per kernel node
+// (Ls (2 nu_pre + 1) + 1 + Ls (2 nu_post + 1) nodes per V-cycle, 12 V-cycles
+// per level assumed; eight at once, more branches launch no faster) plus the
+// cells at 1.5e9 per second; a block of the persistent launch, one per SM,
+// largest hierarchy first, takes 1.9 times a hierarchy's node time plus its
+// cells at 2e7 per second.  The whole batch goes to the persistent launch when
+// that estimate is the shorter.  Measured, persistent / branches: 32, 64 and
+// 512 hierarchies of 16 to 32 cells per edge 6.9 / 10.4, 7.5 / 20.9 and 23.9 /
+// 142 ms, 256 of 32 to 48 28 / 94 ms, 24 of 32 to 128 168 / 20.9 ms.  Run beside
+// graph branches it takes SMs and bandwidth from them (a split of a batch of
+// 512 of 32 to 128 took 707 ms against 642 ms with graph branches only).
+// MG_PERSIST=1 / 0 forces all / none (the batched kernels, MG_BATCHED=1, exclude
+// it); MG_PERSIST_COUNT=k gives the k smallest hierarchies to it and the rest to
+// graph branches in the same graph.
 void choose_persistent(mg_hierarchy *h)
 {
     const int nb = h->batch;
@@ -1564,14 +1565,16 @@ void choose_persistent(mg_hierarchy *h)
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    double g_lat = 0.0, all = 0.0, big = 0.0;
+    double g_lat = 0.0, all = 0.0, sum = 0.0, longest = 0.0;
     for (int b = 0; b < nb; b++) {
+        const double t = 1.9 * lat[b] + cells[b] / 2e7;
         g_lat += lat[b];
         all += cells[b];
-        big = std::max(big, cells[b]);
+        sum += t;
+        longest = std::max(longest, t);
     }
     const double tg = g_lat / 8.0 + all / 1.5e9;
-    const double tp = std::max(big / 6e6, all / (std::min((double)nb, 2.0 * nsm) * 6e6));
+    const double tp = std::max(longest, sum / std::min(nb, nsm));
     if (tp < tg)
         h->in_persist.assign(nb, 1);
 }
@@ -1592,7 +1595,7 @@ bool plan_persistent(mg_hierarchy *h, mg_status &err)
         double cellsum = 0.0;
         for (int l = 0; l < h->desc[b].num_levels; l++) {
             LevelData &ld = h->lev[b][l];
-            if (cudaError_t e = plan_split(ld, dim, 0, h->stream)) {
+            if (cudaError_t e = plan_split(ld, dim, ld.Ls[1], h->stream)) {
                 err = fail_cuda(h, e, "persistent plan");
                 return false;
             }

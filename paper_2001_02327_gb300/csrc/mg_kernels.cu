@@ -2518,7 +2518,7 @@ __global__ void __launch_bounds__(1024) kb_ctl(const MgBPart *__restrict__ parts
 // ---------------------------------------------------------------------------
 // persistent batched solve: one block per hierarchy at a time
 // ---------------------------------------------------------------------------
-constexpr int kPersistThreads = 512;
+constexpr int kPersistThreads = 768;   // one block per SM (figures at split_smooth)
 
 // Fixed-order sum over the block (up to 1024 threads); valid in thread 0.
 __device__ __forceinline__ double block_sum_all(double v, double *sm)
@@ -2535,10 +2535,258 @@ __device__ __forceinline__ double block_sum_all(double v, double *sm)
     return v;
 }
 
+// ---------------------------------------------------------------------------
+// Phases of the persistent kernel on colour-split FP32 levels (layout of
+// mg_idx32), several cells per thread from 16-byte loads.  The per-cell forms
+// above (op_smooth_colour, op_resid_restrict, op_prolong) on plain levels
+// issue about 60 to 80 instructions per cell, and a block is bound by that (the
+// schedulers of a busy SM issue in half of all cycles; DRAM 2 %, FP64 pipe 5 %);
+// here the index arithmetic, the ghost rule and the loads are shared by four
+// cells.  Per cell the arithmetic and its order are those of the per-cell
+// forms.  Ghost and padding positions are zero in these arrays (a correction's
+// ring is zero, coarse ghosts are folded), so whole vectors are stored, zero
+// outside the level.
+// The level's geometry is copied out of the part's descriptor first: the
+// compiler reloads what a store through a float pointer may have changed.  256
+// hierarchies of 16 to 32 cells per edge: 23.9 ms with the per-cell forms, 23.4
+// with copied geometry, 17.0 to 18.0 with these phases (27.9 without the copies), all with two
+// blocks of 512 threads per SM; 13.6 with one of 1024, 12.8 with one of 768,
+// whose longest hierarchy has the SM to itself and no register spills.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int axis_bits(int a, int N) { return (a == 1 ? 1 : 0) | (a == N ? 2 : 0); }
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+
+// Which neighbours along y and z of row (j, k) the ghost rule keeps, and the
+// row's boundary class.
+struct SplitRow {
+    bool yd, yu, zd, zu;
+    int cls;
+    template <int DIM>
+    static __device__ __forceinline__ SplitRow of(const MgGeom &g, int j, int k)
+    {
+        SplitRow r{true, true, true, true, 0};
+        if (g.L > 0) {
+            const int N = g.N;
+            const bool tieN = g.tie && N >= 2;
+            r.yd = j != 1 && !(j == N && tieN);
+            r.yu = j != N;
+            r.cls = axis_bits(j, N) << 2;
+            if (DIM == 3) {
+                r.zd = k != 1 && !(k == N && tieN);
+                r.zu = k != N;
+                r.cls |= axis_bits(k, N) << 4;
+            }
+        }
+        return r;
+    }
+};
+
+// One colour of a red-black sweep, four cells of the colour per thread: row
+// (j, k) holds cell i = 2m + par at position m.
+template <int DIM>
+__device__ __forceinline__ void split_smooth(float *__restrict__ phi, const float *__restrict__ f, const MgGeom &g_,
+                                             int colour, int t0, int stride)
+{
+    const MgGeom g = g_;   // out of memory that the stores may alias
+    const int N = g.N, H = g.sH, q = ((N >> 1) + 4) >> 2, half = (int)g.shalf, pl = g.E * H;
+    const int total = q * N * (DIM == 3 ? N : 1);
+    const float *oth = phi + (colour ^ 1) * half, *fc = f + colour * half;
+    float *own = phi + colour * half;
+    const bool tieN = g.tie && N >= 2;
+    Walk3 w(t0, stride, q, DIM == 3 ? N : total);
+    for (int t = t0; t < total; t += stride, w.next()) {
+        const int j = w.y + 1, k = DIM == 3 ? w.z + 1 : 0;
+        const int par = (colour - j - k) & 1, i0 = 8 * w.x + par;
+        if (i0 > N)
+            continue;
+        const int p = (DIM == 3 ? k * pl : 0) + j * H + 4 * w.x;
+        const SplitRow row = SplitRow::of<DIM>(g, j, k);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 c = ld4(oth + p);
+        const float s = oth[par ? p + 4 : p - 1];
+        const float4 yd = row.yd ? ld4(oth + p - H) : zero, yu = row.yu ? ld4(oth + p + H) : zero;
+        float4 zd = zero, zu = zero;
+        if (DIM == 3) {
+            if (row.zd)
+                zd = ld4(oth + p - pl);
+            if (row.zu)
+                zu = ld4(oth + p + pl);
+        }
+        const float4 fv = ld4(fc + p);
+        float xl[4] = {par ? c.x : s, par ? c.y : c.x, par ? c.z : c.y, par ? c.w : c.z};
+        float xr[4] = {par ? c.y : c.x, par ? c.z : c.y, par ? c.w : c.z, par ? s : c.w};
+        const float y[4] = {yd.x + yu.x, yd.y + yu.y, yd.z + yu.z, yd.w + yu.w};
+        const float z[4] = {zd.x + zu.x, zd.y + zu.y, zd.z + zu.z, zd.w + zu.w};
+        const float fe[4] = {fv.x, fv.y, fv.z, fv.w};
+        const float fac = neg_inv_diag<float, DIM>(g, row.cls);
+        float nv[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int i = i0 + 2 * e;
+            float fi = fac;
+            if (g.L > 0 && (i == 1 || i == N)) {
+                if (i == 1 || tieN)
+                    xl[e] = 0.f;
+                if (i == N)
+                    xr[e] = 0.f;
+                fi = neg_inv_diag<float, DIM>(g, row.cls | axis_bits(i, N));
+            }
+            float o = (xl[e] + xr[e]) + y[e];
+            if (DIM == 3)
+                o += z[e];
+            nv[e] = i >= 1 && i <= N ? (o - g.h2f * fe[e]) * fi : 0.f;
+        }
+        *reinterpret_cast<float4 *>(own + p) = make_float4(nv[0], nv[1], nv[2], nv[3]);
+    }
+}
+
+// Residual and restriction, two coarse cells 2u + 1 and 2u + 2 of a row per
+// thread: their children x = 4u + 1 .. 4u + 4 with the x neighbours are
+// positions 2u .. 2u + 2 of both colours.
+template <int DIM>
+__device__ __forceinline__ void split_restrict(const float *__restrict__ phi, const float *__restrict__ f,
+                                               const MgGeom &gf_, float *__restrict__ phi_c, float *__restrict__ f_c,
+                                               const MgGeom &gc_, int t0, int stride)
+{
+    const MgGeom gf = gf_, gc = gc_;
+    const int N = gf.N, Nc = gc.N, H = gf.sH, pl = gf.E * H, half = (int)gf.shalf, q = (Nc + 1) >> 1;
+    const int total = q * Nc * (DIM == 3 ? Nc : 1);
+    const bool tieN = gf.tie && N >= 2;
+    Walk3 w(t0, stride, q, DIM == 3 ? Nc : total);
+    for (int t = t0; t < total; t += stride, w.next()) {
+        const int J = w.y + 1, K = DIM == 3 ? w.z + 1 : 0, x0 = 4 * w.x;
+        float s[2] = {0.f, 0.f};
+#pragma unroll 1
+        for (int rr = 0; rr < (DIM == 3 ? 4 : 2); rr++) {
+            const int j = 2 * J - 1 + (rr & 1), k = DIM == 3 ? 2 * K - 1 + (rr >> 1) : 0;
+            if (j > N || (DIM == 3 && k > N))
+                continue;
+            const SplitRow row = SplitRow::of<DIM>(gf, j, k);
+            const int p = (DIM == 3 ? k * pl : 0) + j * H + 2 * w.x;
+            // this row's odd and even x; the rows next to it have them in the other array
+            const float *od = phi + ((1 + j + k) & 1) * half + p, *ev = phi + ((j + k) & 1) * half + p;
+            const float2 a = ld2(od), b = ld2(ev);
+            const float c[6] = {b.x, a.x, b.y, a.y, ev[2], od[2]};   // x0 .. x0 + 5
+            float o[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int i = x0 + 1 + e;
+                const bool lo = gf.L > 0 && i == 1, hi = gf.L > 0 && i == N;
+                o[e] = (lo || (hi && tieN) ? 0.f : c[e]) + (hi ? 0.f : c[e + 2]);
+            }
+            auto add_pair = [&](int off, bool keep_d, bool keep_u) {
+                float2 da = make_float2(0.f, 0.f), ua = da;
+                float d1 = 0.f, d3 = 0.f, u1 = 0.f, u3 = 0.f;
+                if (keep_d) {
+                    da = ld2(ev - off);
+                    d1 = od[1 - off];
+                    d3 = od[2 - off];
+                }
+                if (keep_u) {
+                    ua = ld2(ev + off);
+                    u1 = od[1 + off];
+                    u3 = od[2 + off];
+                }
+                o[0] += da.x + ua.x;
+                o[1] += d1 + u1;
+                o[2] += da.y + ua.y;
+                o[3] += d3 + u3;
+            };
+            add_pair(H, row.yd, row.yu);
+            if (DIM == 3)
+                add_pair(pl, row.zd, row.zu);
+            const float2 fa = ld2(f + (od - phi));
+            const float *fv = f + (ev - phi);
+            const float fe[4] = {fa.x, fv[1], fa.y, fv[2]};
+            const float dg = diag_of<float, DIM>(gf, row.cls);
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int i = x0 + 1 + e;
+                float di = dg;
+                if (gf.L > 0 && (i == 1 || i == N))
+                    di = diag_of<float, DIM>(gf, row.cls | axis_bits(i, N));
+                const float r = fe[e] - (o[e] + di * c[e + 1]) * gf.inv_h2f;
+                if (i <= N)
+                    s[e >> 1] += r;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            const int I = 2 * w.x + 1 + e;
+            if (I <= Nc) {
+                const int pc = (int)mg_idx32(gc, DIM, I, J, K);
+                f_c[pc] = (DIM == 3 ? 0.125f : 0.25f) * s[e];
+                phi_c[pc] = 0.f;
+            }
+        }
+    }
+}
+
+// Prolongation and correction, the four cells x = 4u .. 4u + 3 of a row per
+// thread from the coarse cells 2u .. 2u + 2 of its 2^(d-1) coarse rows.
+template <int DIM>
+__device__ __forceinline__ void split_prolong(const float *__restrict__ phi_c, const MgGeom &gc_,
+                                              float *__restrict__ phi, const MgGeom &gf_, int t0, int stride)
+{
+    const MgGeom gf = gf_, gc = gc_;
+    const int N = gf.N, H = gf.sH, pl = gf.E * H, half = (int)gf.shalf, q = (N >> 2) + 1;
+    const int total = q * N * (DIM == 3 ? N : 1);
+    Walk3 w(t0, stride, q, DIM == 3 ? N : total);
+    for (int t = t0; t < total; t += stride, w.next()) {
+        const int j = w.y + 1, k = DIM == 3 ? w.z + 1 : 0;
+        int jm[2], km[2] = {0, 0}, im[3];
+        float wj[2], wk[2] = {1.f, 1.f}, ci[3];
+        prolong_axis<float>(j, gc, jm[0], jm[1], wj[0], wj[1]);
+        if (DIM == 3)
+            prolong_axis<float>(k, gc, km[0], km[1], wk[0], wk[1]);
+#pragma unroll
+        for (int x = 0; x < 3; x++) {
+            const int I = 2 * w.x + x;
+            if (I <= gc.N + 1) {
+                ghost_map<float>(I, gc, im[x], ci[x]);
+            } else {   // only cells past the level take it
+                im[x] = 1;
+                ci[x] = 0.f;
+            }
+        }
+        float nv[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int z = 0; z < (DIM == 3 ? 2 : 1); z++) {
+            float ys[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int y = 0; y < 2; y++) {
+                float v[3];
+#pragma unroll
+                for (int x = 0; x < 3; x++)
+                    v[x] = phi_c[(int)mg_idx32(gc, DIM, im[x], jm[y], km[z])];
+#pragma unroll
+                for (int e = 0; e < 4; e++) {
+                    const int near = (e + 1) >> 1, far = (e & 1) ? near - 1 : near + 1;
+                    ys[e] += wj[y] * (0.75f * ci[near] * v[near] + 0.25f * ci[far] * v[far]);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                nv[e] += DIM == 3 ? wk[z] * ys[e] : ys[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e++)
+            if (4 * w.x + e < 1 || 4 * w.x + e > N)
+                nv[e] = 0.f;
+        const int p = (DIM == 3 ? k * pl : 0) + j * H + 2 * w.x;
+        float2 *pe = reinterpret_cast<float2 *>(phi + ((j + k) & 1) * half + p);
+        float2 *po = reinterpret_cast<float2 *>(phi + ((1 + j + k) & 1) * half + p);
+        const float2 a = *pe, b = *po;
+        *pe = make_float2(a.x + nv[0], a.y + nv[2]);
+        *po = make_float2(b.x + nv[1], b.y + nv[3]);
+    }
+}
+
 // One FP32 V-cycle (Sec. 2.3 steps 2-13) of part P by this block: per level
 // above the bottom, nu_pre sweeps and the residual restriction, the bottom
 // levels from the one-block plan, then prolongation and nu_post sweeps back
-// up.  The same per-cell functions as the one-kernel-per-phase launches.
+// up.  Levels above the bottom are colour-split.
 template <int DIM>
 __device__ void persist_vcycle(const MgBPart &P, int nu_pre, int nu_post, unsigned char *smem)
 {
@@ -2546,21 +2794,20 @@ __device__ void persist_vcycle(const MgBPart &P, int nu_pre, int nu_post, unsign
     for (int L = 0; L < Ls; L++) {
         for (int sw = 0; sw < nu_pre; sw++)
             for (int col = 0; col < 2; col++) {
-                op_smooth_colour<float, DIM>(P.phi32[L], P.f32[L], P.g[L], col, tid, nth);
+                split_smooth<DIM>(P.phi32[L], P.f32[L], P.g[L], col, tid, nth);
                 __syncthreads();
             }
-        op_resid_restrict<float, DIM>(P.phi32[L], P.f32[L], P.g[L], P.phi32[L + 1], P.f32[L + 1], P.g[L + 1], tid,
-                                      nth);
+        split_restrict<DIM>(P.phi32[L], P.f32[L], P.g[L], P.phi32[L + 1], P.f32[L + 1], P.g[L + 1], tid, nth);
         __syncthreads();
     }
     bottom_body<float, DIM>(P.phi32[Ls], P.f32[Ls], P.bt, nu_pre, nu_post, smem);
     __syncthreads();
     for (int L = Ls; L > 0; L--) {
-        op_prolong<float, DIM>(P.phi32[L], P.g[L], P.phi32[L - 1], P.g[L - 1], tid, nth);
+        split_prolong<DIM>(P.phi32[L], P.g[L], P.phi32[L - 1], P.g[L - 1], tid, nth);
         __syncthreads();
         for (int sw = 0; sw < nu_post; sw++)
             for (int col = 0; col < 2; col++) {
-                op_smooth_colour<float, DIM>(P.phi32[L - 1], P.f32[L - 1], P.g[L - 1], col, tid, nth);
+                split_smooth<DIM>(P.phi32[L - 1], P.f32[L - 1], P.g[L - 1], col, tid, nth);
                 __syncthreads();
             }
     }
@@ -2677,7 +2924,7 @@ __device__ void persist_level(const MgBPart &P, int nu_pre, int nu_post, double 
 // the counter (hierarchies ordered largest first on the host) and solves its
 // levels in order; no block waits for another.
 template <int DIM>
-__global__ void __launch_bounds__(kPersistThreads, 2) k_persist(const MgBPart *__restrict__ parts,
+__global__ void __launch_bounds__(kPersistThreads, 1) k_persist(const MgBPart *__restrict__ parts,
                                                                const MgPTask *__restrict__ tasks, int ntasks,
                                                                unsigned *__restrict__ next, int nu_pre, int nu_post,
                                                                double tol, int max_cycles, int inner0, int inner_max,
