@@ -71,6 +71,14 @@ __device__ __forceinline__ long long lidx(const BoxGeom &g, int i, int j, int k)
     return box_index(g, i, j, k);
 }
 
+// lidx of an array that fits shared memory
+template <bool S>
+__device__ __forceinline__ int tail_idx(const BoxGeom &g, int i, int j, int k)
+{
+    const int r = k * g.E[1] + j;
+    return S ? ((i + j + k) & 1) * (int)g.half + r * g.H + (i >> 1) : r * g.E[0] + i;
+}
+
 // Division of an unsigned 32-bit n by an invariant d with one multiply-high,
 // an add and shifts (Granlund and Montgomery, "Division by invariant integers
 // using multiplication", 1994, round-up method): l = ceil(log2 d),
@@ -461,7 +469,8 @@ __global__ void __launch_bounds__(256) kx_restrict32(const float *__restrict__ p
 // A coarse value read through the ghost rule of Sec. 2.4, applied axis after
 // axis (x, y, z) as a ghost fill would: index 0 -> -Phi_1; N+1 -> cR Phi_N,
 // or at a tie -Phi_{N-1} (+Phi_1 when N = 1).
-template <typename T, int DIM, bool S>
+// SMALL: an array that fits shared memory (32-bit indices).
+template <typename T, int DIM, bool S, bool SMALL = false>
 __device__ __forceinline__ T ghost_read(const T *__restrict__ phic, const BoxGeom &g, int i, int j, int k)
 {
     int id[3] = {i, j, k};
@@ -482,7 +491,11 @@ __device__ __forceinline__ T ghost_read(const T *__restrict__ phic, const BoxGeo
             }
         }
     }
-    T v = phic[lidx<S>(g, id[0], id[1], id[2])];
+    T v;
+    if constexpr (SMALL)
+        v = phic[tail_idx<S>(g, id[0], id[1], id[2])];
+    else
+        v = phic[lidx<S>(g, id[0], id[1], id[2])];
 #pragma unroll
     for (int a = 0; a < DIM; a++)
         v = v * c[a];
@@ -494,7 +507,7 @@ __device__ __forceinline__ T ghost_read(const T *__restrict__ phic, const BoxGeo
 // ceil(i/2) towards ceil(i/2) - 1 (i odd) or + 1 (i even): weights 3/4 and
 // 1/4; along the others it takes coarse cell i.  Interpolated x first, then
 // y, then z.  This is the correction at fine cell (i, j, k), coarse layout CS.
-template <typename T, int DIM, bool CS>
+template <typename T, int DIM, bool CS, bool SMALL = false>
 __device__ __forceinline__ T prolong_value(const BoxGeom &gf, const T *__restrict__ phic, const BoxGeom &gc, int cmask,
                                            int i, int j, int k)
 {
@@ -507,9 +520,9 @@ __device__ __forceinline__ T prolong_value(const BoxGeom &gf, const T *__restric
     const T w0 = T(0.75), w1 = T(0.25);
     auto row = [&](int y, int z) {   // interpolated along x
         if (!cx)
-            return T(0) + T(1) * ghost_read<T, DIM, CS>(phic, gc, ax0, y, z);
-        T v = T(0) + w0 * ghost_read<T, DIM, CS>(phic, gc, ax0, y, z);
-        return v + w1 * ghost_read<T, DIM, CS>(phic, gc, ax1, y, z);
+            return T(0) + T(1) * ghost_read<T, DIM, CS, SMALL>(phic, gc, ax0, y, z);
+        T v = T(0) + w0 * ghost_read<T, DIM, CS, SMALL>(phic, gc, ax0, y, z);
+        return v + w1 * ghost_read<T, DIM, CS, SMALL>(phic, gc, ax1, y, z);
     };
     auto plane = [&](int z) {        // then along y
         if (!cy)
@@ -673,13 +686,20 @@ __global__ void __launch_bounds__(256, 4) kx_prolong8(float *__restrict__ phif, 
 // as zero; the rule's part of the diagonal comes from a table by boundary
 // class (two bits per axis: first and last cell), since a division per
 // boundary cell would cost more than the rest of it.
-// Three nested patches, V(2,2) to 1e-10: 48x24x32 mixed 7.43 -> 4.03 ms, 128x96x80
-// mixed 9.58 -> 6.28 ms, 512x256x256 mixed 36.3 -> 33.3 ms, 64^3 FP64 11.9 -> 9.5 ms.
-constexpr int kTailMax = 12, kTailThreads = 512;
+// Three nested patches, V(2,2) to 1e-10, launches -> tail: 48x24x32 mixed 7.43 -> 3.32
+// ms, 34^3 7.25 -> 3.46, 128x96x80 9.58 -> 5.90, 512x256x256 36.3 -> 33.2, 64^3 FP64
+// 11.9 -> 9.5 ms.  What bounds it: the latency of the phases' dependent
+// shared-memory loads (32-bit indexes and division by multiplication took 34^3 from
+// 4.24 to 3.79 ms).
+constexpr int kTailMax = 12;
+// 34^3 mixed with 256 / 512 / 1024 threads 4.39 / 3.74 / 3.46 ms; 32^3 FP64 6.27 / 6.09 / 6.27
+template <typename T>
+constexpr int kTailThreads = sizeof(T) == 4 ? 1024 : 512;
 constexpr size_t kTailSmem = 200 * 1024;
 
 struct BoxTail {
     BoxGeom g[kTailMax];
+    FastDiv dhalf[kTailMax], dn0[kTailMax], dn1[kTailMax];   // by (N_x + 1) / 2, N_x, N_y
     int cmask[kTailMax];   // axes that coarsen from this level to the next
     int nlev, nu_pre, nu_post;
 };
@@ -703,12 +723,18 @@ template <typename T, int DIM>
 __device__ __forceinline__ T tail_other(const T *phi, const BoxGeom &g, int i, int j, int k, int cls)
 {
     constexpr bool S = sizeof(T) == 4;
+    // every neighbour has the other colour: its row in that array, or the cell itself
+    const int r = (k * g.E[1] + j) * (S ? g.H : g.E[0]);
+    const T *c = phi + r + (S ? ((i + j + k + 1) & 1) * (int)g.half : 0);
+    const int x = S ? i >> 1 : i, row = S ? g.H : g.E[0];
+    const int lo[3] = {S ? (i - 1) >> 1 : i - 1, x - row, x - row * g.E[1]};
+    const int hi[3] = {S ? (i + 1) >> 1 : i + 1, x + row, x + row * g.E[1]};
     T v[2 * DIM];
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
-        const bool lo = (cls >> (2 * a)) & 1, hi = (cls >> (2 * a + 1)) & 1;
-        v[2 * a] = lo || (hi && g.tie[a]) ? T(0) : phi[lidx<S>(g, i - (a == 0), j - (a == 1), k - (a == 2))];
-        v[2 * a + 1] = hi ? T(0) : phi[lidx<S>(g, i + (a == 0), j + (a == 1), k + (a == 2))];
+        const bool first = (cls >> (2 * a)) & 1, last = (cls >> (2 * a + 1)) & 1;
+        v[2 * a] = first || (last && g.tie[a]) ? T(0) : c[lo[a]];
+        v[2 * a + 1] = last ? T(0) : c[hi[a]];
     }
     if constexpr (sizeof(T) == sizeof(double)) {
         if (g.iso)
@@ -722,14 +748,14 @@ __device__ __forceinline__ T tail_other(const T *phi, const BoxGeom &g, int i, i
 }
 
 template <typename T, int DIM>
-__global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, const T *__restrict__ f_g,
+__global__ void __launch_bounds__(kTailThreads<T>) kx_tail(T *__restrict__ phi_g, const T *__restrict__ f_g,
                                                         const __grid_constant__ BoxTail t)
 {
     pdl_begin();
     constexpr bool S = sizeof(T) == 4;
     extern __shared__ __align__(16) unsigned char tail_smem[];
     T *const sm = reinterpret_cast<T *>(tail_smem);
-    const int tid = threadIdx.x, nth = kTailThreads;
+    const int tid = threadIdx.x, nth = kTailThreads<T>;
     // per level: a table of 64 diagonals and 64 reciprocals, phi, f
     int base[kTailMax];
     base[0] = 0;
@@ -763,8 +789,8 @@ __global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, c
     }
     __syncthreads();
     // item e of a level's rows of nx: cell x of row (j, k)
-    auto cell = [](int e, int nx, int ny, int &x, int &j, int &k) {
-        const int r = e / nx, z = DIM == 3 ? r / ny : 0;
+    auto cell = [](int e, int nx, int ny, const FastDiv &dx, const FastDiv &dy, int &x, int &j, int &k) {
+        const int r = (int)fdiv(dx, e), z = DIM == 3 ? (int)fdiv(dy, r) : 0;
         x = e - r * nx;
         j = r - z * ny + 1;
         k = DIM == 3 ? z + 1 : 0;
@@ -777,12 +803,12 @@ __global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, c
         for (int c = 0; c < 2 * sweeps; c++) {
             for (int e = tid; e < total; e += nth) {
                 int x, j, k;
-                cell(e, nx, g.N[1], x, j, k);
+                cell(e, nx, g.N[1], t.dhalf[q], t.dn1[q], x, j, k);
                 const int i = 2 * x + ((((c & 1) - j - k) & 1) ? 1 : 2);
                 if (i > g.N[0])
                     continue;
                 const int cls = tail_class<DIM>(g, i, j, k);
-                const int p = (int)lidx<S>(g, i, j, k);
+                const int p = tail_idx<S>(g, i, j, k);
                 phi[p] = (f[p] - tail_other<T, DIM>(phi, g, i, j, k, cls)) * inv[cls];
             }
             __syncthreads();
@@ -797,7 +823,7 @@ __global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, c
         const int total = gc.N[0] * gc.N[1] * (DIM == 3 ? gc.N[2] : 1);
         for (int e = tid; e < total; e += nth) {
             int I, J, K;
-            cell(e, gc.N[0], gc.N[1], I, J, K);
+            cell(e, gc.N[0], gc.N[1], t.dn0[q + 1], t.dn1[q + 1], I, J, K);
             I++;
             const int x0 = cx ? 2 * I - 1 : I, y0 = cy ? 2 * J - 1 : J, z0 = cz ? 2 * K - 1 : K;
             const int nx = cx && 2 * I <= gf.N[0] ? 2 : 1, ny = cy && 2 * J <= gf.N[1] ? 2 : 1,
@@ -809,14 +835,14 @@ __global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, c
                     T sx = T(0);
                     for (int dx = 0; dx < nx; dx++) {
                         const int i = x0 + dx, j = y0 + dy, k = z0 + dz, cls = tail_class<DIM>(gf, i, j, k);
-                        const int p = (int)lidx<S>(gf, i, j, k);
+                        const int p = tail_idx<S>(gf, i, j, k);
                         sx = sx + (f[p] - (tail_other<T, DIM>(phi, gf, i, j, k, cls) + dg[cls] * phi[p]));
                     }
                     sy = sy + sx;
                 }
                 sz = sz + sy;
             }
-            const int pc = (int)lidx<S>(gc, I, J, K);
+            const int pc = tail_idx<S>(gc, I, J, K);
             F(q + 1)[pc] = sz * wk;
             PHI(q + 1)[pc] = T(0);
         }
@@ -828,10 +854,10 @@ __global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, c
         const int total = gf.N[0] * gf.N[1] * (DIM == 3 ? gf.N[2] : 1);
         for (int e = tid; e < total; e += nth) {
             int i, j, k;
-            cell(e, gf.N[0], gf.N[1], i, j, k);
+            cell(e, gf.N[0], gf.N[1], t.dn0[q - 1], t.dn1[q - 1], i, j, k);
             i++;
-            PHI(q - 1)[lidx<S>(gf, i, j, k)] +=
-                prolong_value<T, DIM, S>(gf, (const T *)PHI(q), gc, t.cmask[q - 1], i, j, k);
+            PHI(q - 1)[tail_idx<S>(gf, i, j, k)] +=
+                prolong_value<T, DIM, S, true>(gf, (const T *)PHI(q), gc, t.cmask[q - 1], i, j, k);
         }
         __syncthreads();
         smooth(q - 1, t.nu_post);
@@ -840,8 +866,8 @@ __global__ void __launch_bounds__(kTailThreads) kx_tail(T *__restrict__ phi_g, c
     const int total = g.N[0] * g.N[1] * (DIM == 3 ? g.N[2] : 1);
     for (int e = tid; e < total; e += nth) {
         int i, j, k;
-        cell(e, g.N[0], g.N[1], i, j, k);
-        const int p = (int)lidx<S>(g, i + 1, j, k);
+        cell(e, g.N[0], g.N[1], t.dn0[0], t.dn1[0], i, j, k);
+        const int p = tail_idx<S>(g, i + 1, j, k);
         phi_g[p] = PHI(0)[p];
     }
 }
@@ -1409,9 +1435,9 @@ cudaError_t smooth(const mg_box *b, const BoxLevel &l, int sweeps, cudaStream_t 
 // The levels that kx_tail takes: from the first of at most tail_limit cells
 // (and not level 0, whose ghost layer holds data) whose arrays and those below
 // fit shared memory.  A level of more cells is faster spread over the SMs; limits
-// of 2000 / 6000 cells, mixed: 34^3 4.24 / 4.52 ms, 48x24x32 4.03 / 4.29; of 300 / 1000 /
-// 3000 cells, FP64: 64^3 10.43 / 9.53 / 9.52 ms, 100x60x80 10.86 / 10.86 / 10.71.
-int tail_limit(bool fp32) { return fp32 ? 2000 : 3000; }
+// of 2000 / 6000 cells, mixed: 34^3 3.79 / 3.75 ms, 64^3 5.14 / 4.95; of 300 / 1000 / 3000
+// cells, FP64: 64^3 10.43 / 9.53 / 9.52 ms, 100x60x80 10.86 / 10.86 / 10.71.
+int tail_limit(bool fp32) { return fp32 ? 6000 : 3000; }
 
 template <typename T>
 cudaError_t plan_tail(BoxPatch &P, int dim, const mg_options &o)
@@ -1435,6 +1461,9 @@ cudaError_t plan_tail(BoxPatch &P, int dim, const mg_options &o)
         for (int q = L; q <= Lc; q++) {
             P.tail.g[q - L] = P.lv[q].g;
             P.tail.cmask[q - L] = P.lv[q].cmask;
+            P.tail.dhalf[q - L] = fast_div((P.lv[q].g.N[0] + 1) / 2);
+            P.tail.dn0[q - L] = fast_div(P.lv[q].g.N[0]);
+            P.tail.dn1[q - L] = fast_div(P.lv[q].g.N[1]);
         }
         break;
     }
@@ -1477,7 +1506,7 @@ cudaError_t vcycle(const mg_box *b, const BoxPatch &P, cudaStream_t s)
     }
     if (P.Ltail && !e) {
         const BoxLevel &l = P.lv[P.Ltail];
-        mg_launch_kernel(dim == 3 ? kx_tail<T, 3> : kx_tail<T, 2>, dim3(1), dim3(kTailThreads), P.tail_smem, s,
+        mg_launch_kernel(dim == 3 ? kx_tail<T, 3> : kx_tail<T, 2>, dim3(1), dim3(kTailThreads<T>), P.tail_smem, s,
                          lphi<T>(l), (const T *)lf<T>(l), P.tail);
         e = cudaGetLastError();
     }

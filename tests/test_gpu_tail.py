@@ -27,7 +27,7 @@ def test_fp64_tail_matches_oracle(mg, dim, n, nu):  # noqa: F811
     assert relmax(got[0][0], ref[0][0]) < 1e-12
 
 
-@pytest.mark.parametrize("dim,n", SHAPES + [(3, (34, 34, 34)), (2, (150, 150))])
+@pytest.mark.parametrize("dim,n", SHAPES + [(3, (34, 34, 34)), (3, (36, 34, 34)), (2, (150, 150)), (2, (156, 154))])
 def test_mixed_tail_converges_as_fp64(mg, dim, n):  # noqa: F811
     """FP32 V-cycles through the tail reach the FP64 form's tolerance in its
     cycles, give or take one step, and its solution: a relative residual of
