@@ -1183,9 +1183,18 @@ struct Engine {
 
     // x 2^e (e any)
     __device__ __forceinline__ static double scaled(double x, int e) { return scalbn(scalbn(x, e / 2), e - e / 2); }
-    // |h^2 r|^2 over level 0 in units of 2^(-2 scale): every CTA gets the sum,
-    // added in a fixed order
-    __device__ __forceinline__ double square_sum(int K) const
+    // The CTAs' parts of the norm, two sets in turn: a CTA without a share in the
+    // level waits for nobody between two norms, so a part may arrive while
+    // another still reads the last norm's.  The second set takes the slots of
+    // the residual of the last possible level, which is solved and has none.
+    __device__ __forceinline__ double *parts(int odd) const
+    {
+        return odd ? reinterpret_cast<double *>(slots() + 32 * (MG_SLAB_MAXLEV - 1)) : sums() + 16;
+    }
+    // |h^2 r|^2 over level 0 after cycle n: every CTA gets the same sum, added
+    // in a fixed order.  A CTA scales its own part: a level that CTA 0 holds
+    // alone changes its scale there alone (prolong_scale).
+    __device__ __forceinline__ double square_sum(int K, int n) const
     {
         const Lev L = level(0);
         double acc = 0.0;
@@ -1215,13 +1224,13 @@ struct Engine {
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1)
                 acc += __shfl_down_sync(0xffffffffu, acc, o);
-            acc = __shfl_sync(0xffffffffu, acc, 0);
+            acc = scaled(__shfl_sync(0xffffffffu, acc, 0), -2 * sc()[0]);
             if (tid < pl.csize)
-                st_cluster(cluster_addr(shared_addr(sm + 16 + rank), tid), __double_as_longlong(acc));
+                st_cluster(cluster_addr(shared_addr(parts(n & 1) + rank), tid), __double_as_longlong(acc));
         }
         cluster_sync_();
         if (tid < 32) {
-            acc = tid < pl.csize ? sm[16 + tid] : 0.0;
+            acc = tid < pl.csize ? parts(n & 1)[tid] : 0.0;
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1)
                 acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -1422,10 +1431,8 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
         if constexpr (P::kFix)
             if (solve) {
                 r2 = CUDART_NAN;
-                if (!bad) {
-                    const double q = en.square_sum(pl.K[0]);
-                    r2 = en.scaled(q, -2 * en.sc()[0]) * g0.inv_h2 * g0.inv_h2;
-                }
+                if (!bad)
+                    r2 = en.square_sum(pl.K[0], n) * g0.inv_h2 * g0.inv_h2;
             }
         go = more();
     }

@@ -92,3 +92,22 @@ def test_fp64_slab_solve_of_nothing(mg):  # noqa: F811
     inp = [{"rho": np.zeros((n,) * 3), "bc_rho": np.zeros((n + 2,) * 3), "bc_phi": np.zeros((n + 4,) * 3)}]
     _, g = gpu_solve(mg, H, inp, max_cycles=5, rel_tol=1e-10)
     assert g[0]["cycles"] == 0 and np.all(g[0]["phi"] == 0.0)
+
+
+@pytest.mark.parametrize("dim,n", [(2, 20), (2, 22), (2, 23), (3, 5), (3, 7), (3, 8)])
+@pytest.mark.parametrize("nu", [(2, 1), (1, 0)])
+def test_fp64_slab_solve_of_a_level_in_one_cta(mg, monkeypatch, dim, n, nu):  # noqa: F811
+    """Levels that CTA 0 holds alone (and the first that it does not), with a
+    scale that gives way in the first ascent: every CTA of the cluster has to
+    stop after the same cycle, the one where the loop of launches stops.  The
+    residual of a potential of order one rounds below 1e-13 of the right-hand
+    side at these sizes."""
+    H = I.Hierarchy(dim, [n], [tuple([0.0] * dim)], 1.0 / n, 1.0, [], "const")
+    inp = [{"rho": np.ones((n,) * dim), "bc_rho": np.ones((n + 2,) * dim), "bc_phi": np.zeros((n + 4,) * dim)}]
+    kw = dict(nu_pre=nu[0], nu_post=nu[1], max_cycles=40, rel_tol=1e-8)
+    _, a = gpu_solve(mg, H, inp, **kw)
+    monkeypatch.setenv("MG_BOTTOM_N64", "8")
+    _, b = gpu_solve(mg, H, inp, **kw)
+    assert a[0]["cycles"] == b[0]["cycles"] and a[0]["status"] == b[0]["status"] == 0
+    assert abs(a[0]["rel_res"] - b[0]["rel_res"]) < 1e-12
+    assert relmax(a[0]["phi"], b[0]["phi"]) < 1e-12
