@@ -48,8 +48,9 @@
 // by the reciprocal diagonal is a 64 x 64 bit high product.  Every level has a
 // power-of-two scale of its own, taken from the largest right-hand side (and
 // potential) it starts from; a coarse correction too large for the finer
-// level's scale lowers that scale first (prolong_from), so nothing overflows
-// and a right-hand side keeps 53 bits or more below its largest value.
+// level's scale, or a potential that has outgrown it, lowers that scale first
+// (prolong_scale).  So a potential stays below 2^57 + 2^57 and what the sweeps
+// add, the sum of a pair's residuals (f + 12 Phi at most, twice) below 2^63.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -437,7 +438,8 @@ struct Engine {
     __device__ __forceinline__ int *sc() const { return ctrl(); }                       // fixed point: scale of every level
     __device__ __forceinline__ int *psc() const { return ctrl() + MG_SLAB_MAXLEV; }     // ... of its published potential
     // OR of magnitudes, [2 MAXLEV] pairs: residuals of level q at q, published
-    // potentials at MAXLEV + q; orw: over this CTA, slots: of every CTA
+    // potentials at MAXLEV + q (level 0's, which is not published, in a solve);
+    // orw: over this CTA, slots: of every CTA
     __device__ __forceinline__ unsigned *orw() const { return reinterpret_cast<unsigned *>(ctrl() + 2 * MG_SLAB_MAXLEV); }
     __device__ __forceinline__ unsigned *slots() const { return orw() + 4 * MG_SLAB_MAXLEV; }
     // per level, of the CTAs with the planes before and after its own: byte
@@ -715,16 +717,19 @@ struct Engine {
                 atomicOr(orw() + 2 * w + 1, lo);
         }
     }
-    // ... and to every CTA of the cluster
-    __device__ __forceinline__ void share_or(int w) const
+    // ... and to every CTA of the cluster; also that of word pair w2 (-1: none)
+    __device__ __forceinline__ void share_or(int w, int w2 = -1) const
     {
         __syncthreads();
-        if (tid < pl.csize) {
-            const unsigned dst = cluster_addr(shared_addr(slots() + (w * 16 + rank) * 2), tid);
+        if (w2 >= 0 && tid >= 32)
+            w = w2;
+        const int to = tid & 31;
+        if (to < pl.csize && tid < (w2 >= 0 ? 64 : 32)) {
+            const unsigned dst = cluster_addr(shared_addr(slots() + (w * 16 + rank) * 2), to);
             st_cluster(dst, orw()[2 * w]);
             st_cluster(dst + 4, orw()[2 * w + 1]);
             if (w >= MG_SLAB_MAXLEV && rank == 0)
-                st_cluster(cluster_addr(shared_addr(psc() + (w - MG_SLAB_MAXLEV)), tid),
+                st_cluster(cluster_addr(shared_addr(psc() + (w - MG_SLAB_MAXLEV)), to),
                            (unsigned)sc()[w - MG_SLAB_MAXLEV]);
         }
     }
@@ -750,9 +755,10 @@ struct Engine {
     }
     __device__ __forceinline__ static fix mag(fix v) { return v < 0 ? ~v : v; }
 
-    // Residual (step 4) of both cells of every pair, summed over the pair.
+    // Residual (step 4) of both cells of every pair, summed over the pair; the
+    // OR of the sums' magnitudes, and in `pot` that of the potentials'.
     template <int K>
-    __device__ __forceinline__ fix residual(int q, const Lev &L, const Items<K> &it, int u0) const
+    __device__ __forceinline__ fix residual(int q, const Lev &L, const Items<K> &it, int u0, fix &pot) const
     {
         const T *tb = tab(q);
         const float ih2 = pl.g[q].inv_h2f;
@@ -772,6 +778,7 @@ struct Engine {
                     if (cls)
                         d = tb[64 + cls] * v + qmul<30>(v, tb[128 + cls]);
                     d = it.f[c][u] - ns + d;
+                    pot |= mag(v);
                 } else {
                     d = it.f[c][u] - (ns + tb[64 + cls] * v) * ih2;
                 }
@@ -992,12 +999,15 @@ struct Engine {
     }
 
     // The shift of level q + 1's potential to level q's scale, which is lowered
-    // first if the correction is beyond its range.
+    // first if the correction is beyond its range, or (level 0 of a solve, whose
+    // potential stays from cycle to cycle; every other starts from the range of
+    // its right-hand side) the potential.
     __device__ __forceinline__ int prolong_scale(int q, const Lev &L) const
     {
         const bool cl = dist(q);
         const int bits = or_bits(MG_SLAB_MAXLEV + q + 1, cl), s1 = cl ? psc()[q + 1] : sc()[q + 1], s0 = sc()[q];
-        const int low = bits ? max(0, bits + s0 - s1 - pl.top[q]) : 0;
+        const int pot = q == 0 && pl.solve ? or_bits(MG_SLAB_MAXLEV, cl) : 0;
+        const int low = max(0, max(bits ? bits + s0 - s1 : 0, pot) - pl.top[q]);
         if (low) {
             __syncthreads();   // every thread has read the scale
             if (tid == 0)
@@ -1098,12 +1108,15 @@ struct Engine {
                 colour(std::integral_constant<int, 0>());
             colour(std::integral_constant<int, 1>());
         }
-        fix big = 0;
-        each(q, h, [&](auto &it, int u0) { big |= residual(q, L, it, u0); });
+        fix big = 0, pot = 0;
+        each(q, h, [&](auto &it, int u0) { big |= residual(q, L, it, u0, pot); });
         if constexpr (kFix) {
+            const bool both = q == 0 && pl.solve;
             block_or(big, q);
+            if (both)
+                block_or(pot, MG_SLAB_MAXLEV);
             if (cl)
-                share_or(q);
+                share_or(q, both ? MG_SLAB_MAXLEV : -1);
         }
         sync(cl);
     }

@@ -111,3 +111,19 @@ def test_fp64_slab_solve_of_a_level_in_one_cta(mg, monkeypatch, dim, n, nu):  # 
     assert a[0]["cycles"] == b[0]["cycles"] and a[0]["status"] == b[0]["status"] == 0
     assert abs(a[0]["rel_res"] - b[0]["rel_res"]) < 1e-12
     assert relmax(a[0]["phi"], b[0]["phi"]) < 1e-12
+
+
+@pytest.mark.parametrize("dim,n", [(3, 7), (3, 16), (3, 31), (2, 22), (2, 126)])
+@pytest.mark.parametrize("nu", [(1, 0), (0, 1)])
+def test_fp64_slab_solve_of_many_slow_cycles(mg, monkeypatch, dim, n, nu):  # noqa: F811
+    """Sixty cycles of one sweep each: the potential grows to nearly twice its
+    first value, and once it has outgrown the scale that gives way; the loop of
+    launches ends at the same potential."""
+    H = I.Hierarchy(dim, [n], [tuple([0.0] * dim)], 1.0 / n, 1.0, [], "const")
+    inp = [{"rho": np.ones((n,) * dim), "bc_rho": np.ones((n + 2,) * dim), "bc_phi": np.zeros((n + 4,) * dim)}]
+    kw = dict(nu_pre=nu[0], nu_post=nu[1], max_cycles=60, rel_tol=0.0)
+    _, a = gpu_solve(mg, H, inp, **kw)
+    monkeypatch.setenv("MG_BOTTOM_N64", "8")
+    _, b = gpu_solve(mg, H, inp, **kw)
+    assert a[0]["cycles"] == b[0]["cycles"] == 60
+    assert relmax(a[0]["phi"], b[0]["phi"]) < 1e-12
