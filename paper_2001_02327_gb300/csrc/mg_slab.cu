@@ -51,6 +51,20 @@
 // level's scale, or a potential that has outgrown it, lowers that scale first
 // (prolong_scale).  So a potential stays below 2^57 + 2^57 and what the sweeps
 // add, the sum of a pair's residuals (f + 12 Phi at most, twice) below 2^63.
+//
+// What that costs in accuracy: a level's arrays share a scale, so a value far
+// below the level's largest keeps fewer bits of its own than a double would.
+// What a finest level keeps from cycle to cycle has 56 to 57 bits for the
+// largest potential (ring included) and, without a potential that outweighs
+// it, 54 to 57 for the largest right-hand side; a level that is a correction
+// of a finer one starts from 50 to 57 bits.  Largest error of the converged
+// potential over its largest value, V(2,2), against a solution in 128 bits,
+// FP64 launches -> here: a sphere with its potential on the ring, 32^3 1.6e-15
+// -> 7.5e-17, 160^2 1.6e-14 -> 1.6e-16; random density and ring 3.0e-16 ->
+// 2.6e-16 and 5.7e-16 -> 2.9e-16; an amplitude growing by 2^30 across the level
+// 4.0e-16 -> 1.6e-16 and 5.4e-16 -> 4.9e-16.  There the cells of the median,
+// 2^-15 of the largest, are 1.9e-15 (32^3, launches 7e-16) and 2e-14 (160^2,
+// launches 4.6e-15) of their own value off.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -146,8 +160,14 @@ __device__ __forceinline__ unsigned shared_addr(const T *p)
     return (unsigned)__cvta_generic_to_shared(p);
 }
 
+// Everything that a level keeps is rounded to nearest: a rounding that leans to
+// one side adds up over the level.  With floors, half a unit on every
+// right-hand side moved the potential by N^2 / 16 units.
+
 // (v * K) >> (32 + S) for |v|, |K| < 2^62, K = kh 2^32 + kl with kl signed; the
-// product of the low words (below one unit) is dropped.
+// product of the low words (below one unit) is dropped.  It leans by half a unit
+// and more: update() rounds, the others scale corrections, whose last bits the
+// next cycle corrects.
 template <int S>
 __device__ __forceinline__ fix qmul(fix v, fix K)
 {
@@ -158,12 +178,23 @@ __device__ __forceinline__ fix qmul(fix v, fix K)
     return (((fix)vh * kh) << (32 - S)) + (mid >> S);
 }
 
-__device__ __forceinline__ fix shift_by(fix v, int s)   // v * 2^s, floor
+__device__ __forceinline__ fix shift_by(fix v, int s)   // v * 2^s, |v| < 2^62
 {
-    return s >= 0 ? v << min(s, 63) : v >> min(-s, 63);
+    if (s >= 0)
+        return v << min(s, 63);
+    s = min(-s, 63);
+    return (v + (1ll << (s - 1))) >> s;
 }
 
-// x * 2^scale, truncated (|result| < 2^62 by the choice of the scale; x finite)
+// v * 2^-s, ties to even: where the dropped bits are few, ties are many and
+// must not lean either (0 <= v < 2^63 or |v| < 2^62; s >= 0)
+template <typename V>
+__device__ __forceinline__ V shift_even(V v, int s)
+{
+    return s == 0 ? v : s > 63 ? V(0) : (v + ((V(1) << (s - 1)) - 1) + ((v >> s) & 1)) >> s;
+}
+
+// x * 2^scale (|result| < 2^62 by the choice of the scale; x finite)
 __device__ __forceinline__ fix to_fix(double x, int scale)
 {
     const int hi = __double2hiint(x);
@@ -171,8 +202,25 @@ __device__ __forceinline__ fix to_fix(double x, int scale)
     const int e = (hi >> 20) & 0x7ff;
     if (e == 0)
         return 0;   // zero or denormal
-    const fix m = (fix)(((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | lo);
-    const fix a = shift_by(m, e - 1075 + scale);
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | lo;
+    const int s = e - 1075 + scale;
+    const fix a = (fix)(s >= 0 ? m << min(s, 63) : shift_even(m, -s));
+    return hi < 0 ? -a : a;
+}
+
+// x * k * 2^(scale - 62) for 2^61 <= k < 2^62 (|result| < 2^58), rounded once
+__device__ __forceinline__ fix to_fix_times(double x, fix k, int scale)
+{
+    const int hi = __double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const int e = (hi >> 20) & 0x7ff;
+    if (e == 0)
+        return 0;
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 43) | ((unsigned long long)lo << 11);
+    const unsigned long long k2 = (unsigned long long)k << 1;
+    // the product's upper 64 bits, the last one set where lower ones are: 2^61 .. 2^63
+    const unsigned long long p = __umul64hi(m, k2) | (m * k2 ? 1 : 0);
+    const fix a = (fix)shift_even(p, 1085 - e - scale);
     return hi < 0 ? -a : a;
 }
 
@@ -679,8 +727,10 @@ struct Engine {
 
     __device__ __forceinline__ T update(int q, T s, T f, T n) const
     {
+        // rounded by what is added before the product: half of an inner cell's diagonal, and twice the
+        // mean of what qmul drops, kl / 2^32 = 1/3 for K = 2^63 / 6 (one addition of three terms)
         if constexpr (kFix)
-            return qmul<31>(s - f, n);
+            return qmul<31>(s - f + (DIM == 3 ? 5 : 2), n);
         else
             return (s - pl.g[q].h2f * f) * n;
     }
@@ -1013,10 +1063,10 @@ struct Engine {
             if (tid == 0)
                 sc()[q] = s0 - low;
             for (int t = tid; t < 2 * L.cs; t += kT)
-                W()[L.ph + t] = shift_by(W()[L.ph + t], -low);
+                W()[L.ph + t] = shift_even(W()[L.ph + t], low);
             T *f = fs() + 2 * pl.slot[q] * kT + tid;
             for (int u = 0; u < 2 * pl.K[q]; u++)
-                f[u * kT] = shift_by(f[u * kT], -low);
+                f[u * kT] = shift_even(f[u * kT], low);
             sync(cl);
         }
         return s0 - low - s1;
@@ -1031,7 +1081,7 @@ struct Engine {
         // 3/4 - 1/4 interpolation along one axis
         auto mix = [](T near, T far) -> T {
             if constexpr (kFix)
-                return (3 * near + far) >> 2;
+                return (3 * near + far + 2) >> 2;
             else
                 return 0.75f * near + 0.25f * far;
         };
@@ -1267,7 +1317,8 @@ struct Engine {
                 nid = g.tab64[64 + c];
             }
             if constexpr (kFix) {
-                tb[c] = (fix)(nid * 9223372036854775808.0);
+                // an inner cell's to the last bit: the double 1 / 6 is 2^-55 of it off, half a unit of 2^54
+                tb[c] = c ? (fix)(nid * 9223372036854775808.0) : (fix)(((1ull << 63) + DIM) / (2 * DIM));
                 const double fl = floor(-d);
                 tb[64 + c] = (fix)fl;
                 tb[128 + c] = (fix)((-d - fl) * 4611686018427387904.0);
@@ -1411,13 +1462,13 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
         }
         bad = mphi >= 0x7ff00000u || mf >= 0x7ff00000u;
         const int gb = mf ? exp_bound(mf) + pl.h2e : -4000;   // h^2 = h2k 2^(h2e - 62)
-        const int s0 = mf || mphi ? pl.tb[0] - max(gb, exp_bound(mphi)) : 0;
+        const int s0 = mf || mphi ? min(pl.tb[0] - gb, pl.top[0] - exp_bound(mphi)) : 0;
         if (tid == 0)
             en.sc()[0] = s0;
         if (!pl.zero_start)
             for (int t = tid; t < 2 * S.cs; t += kT)
                 ph0[t] = to_fix(__longlong_as_double(ph0[t]), s0);
-        keep([&](double f) { return qmul<30>(to_fix(f, s0 + pl.h2e), pl.h2k); });
+        keep([&](double f) { return to_fix_times(f, pl.h2k, s0 + pl.h2e); });
     } else {
         keep([](float f) { return f; });
     }
@@ -1620,6 +1671,13 @@ bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, in
         const int db = (int)std::ceil(std::log2(dmax / 6.0 > 1.0 ? dmax / 6.0 : 1.0));
         p.tb[q] = std::min(57 - db - lognu, q + 1 == nlev ? 54 : 57);
         p.top[q] = 57 - db;
+        // the finest level of a refinement level keeps its right-hand side and potential from cycle to
+        // cycle and their bits are those of the result: with a potential of 2^57, as much again from a
+        // correction and nu f / dim from the sweeps, 2 (f + 4 dim Phi) stays below 2^63
+        if (g[q].L == 0) {
+            const double room = (std::ldexp(1.0, 62) - std::ldexp(1.0, 57)) / (4 * dim) - std::ldexp(1.0, 58);
+            p.tb[q] = std::min(57, (int)std::floor(std::log2(room * dim / (nu_pre + nu_post))));
+        }
     }
     // plan words: A of every slot, B C D of the levels with one pair per thread, ghosts (copied to
     // shared memory), then B C D of the other levels

@@ -127,3 +127,50 @@ def test_fp64_slab_solve_of_many_slow_cycles(mg, monkeypatch, dim, n, nu):  # no
     _, b = gpu_solve(mg, H, inp, **kw)
     assert a[0]["cycles"] == b[0]["cycles"] == 60
     assert relmax(a[0]["phi"], b[0]["phi"]) < 1e-12
+
+
+def _discrete_solution(f, block, h):
+    """The discrete problem solved by sine transforms and refined with residuals in long doubles."""
+    import scipy.fft as sf
+    N, dim, LD = f.shape[0], f.ndim, np.longdouble
+    lam = 2.0 * np.cos(np.pi * np.arange(1, N + 1) / (N + 1)) - 2.0
+    eig = sum(lam.reshape([-1 if a == q else 1 for q in range(dim)]) for a in range(dim))
+    x, c = block.astype(LD), (slice(1, -1),) * dim
+    x[c] = 0
+    for _ in range(4):
+        lap = -2 * dim * x[c]
+        for a in range(dim):
+            for o in (0, 2):
+                lap = lap + x[tuple(slice(o, o + N) if q == a else slice(1, -1) for q in range(dim))]
+        r = f.astype(LD) * LD(h) ** 2 - lap
+        big = float(np.abs(r).max()) or 1.0
+        x[c] += sf.idstn(sf.dstn((r / big).astype(float), type=1) / eig, type=1).astype(LD) * big
+    return x
+
+
+@pytest.mark.parametrize("dim,n", [(3, 8), (3, 16), (3, 31), (2, 23), (2, 64), (2, 158)])
+@pytest.mark.parametrize("kind", ["sphere", "random", "constant"])
+@pytest.mark.parametrize("nu", [(2, 1), (4, 4)])
+def test_fp64_slab_converged_potential_is_unbiased(mg, dim, n, kind, nu):  # noqa: F811
+    """The converged potential against the discrete solution.  A right-hand
+    side is off by at most half a unit of the level's scale, which is at most
+    2^-56 of the largest potential, and half a unit everywhere moves the
+    potential by N^2 / 16 (2D 0.0737 N^2 / 2) units at most; as much again and
+    eight units are allowed for the sweeps' own rounding.  Floors instead of
+    rounding exceed this by ten and more."""
+    rng = np.random.default_rng(100 * dim + n)
+    h, N = 1.0 / n, n + 2
+    if kind == "random":
+        phi, rho = rng.standard_normal((n + 4,) * dim), rng.standard_normal((N,) * dim)
+    elif kind == "constant":
+        phi, rho = np.zeros((n + 4,) * dim), np.ones((N,) * dim)
+    else:
+        r2 = sum((a - 0.13) ** 2 for a in np.meshgrid(*[(np.arange(n + 4) - 1.5) * h - 0.5] * dim, indexing="ij"))
+        phi, rho = -1.0 / np.sqrt(r2 + 0.09), (np.maximum(0.0, 1.0 - r2 / 0.09) ** 3)[(slice(1, -1),) * dim]
+    H = I.Hierarchy(dim, [n], [tuple([0.0] * dim)], h, 1.0, [], kind)
+    inp = [{"rho": np.ascontiguousarray(rho[(slice(1, -1),) * dim]), "bc_rho": np.ascontiguousarray(rho), "bc_phi": phi}]
+    _, g = gpu_solve(mg, H, inp, nu_pre=nu[0], nu_post=nu[1], max_cycles=30, rel_tol=0.0)
+    x = _discrete_solution(4.0 * np.pi * rho, phi, h)
+    unit = 2.0 ** -56 * float(np.abs(x).max())
+    err = float(np.abs(g[0]["phi"] - x[(slice(2, -2),) * dim]).max())
+    assert err <= unit * ((1.0 / 8 if dim == 3 else 0.0737) * N ** 2 + 8.0)
