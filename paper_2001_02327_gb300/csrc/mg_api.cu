@@ -433,8 +433,9 @@ struct mg_hierarchy {
     double *frho = nullptr;         // device 4 pi G h_l^2 per (b, l) (input scaling of the learned guess)
     mg_unet *unet = nullptr;        // learned initial guess (MG_GUESS_LEARNED)
     MgSolveCtl *hctl = nullptr;     // pinned mirror
-    int *werr = nullptr;            // device word: MG_ETIMEOUT once a plane-marching load wait gave up
-    int wfault = 0;                 // MG_FAULT_WAVE_WAIT=1: those waits are made to run out (test of that path)
+    int *werr = nullptr;            // device word: MG_ETIMEOUT once a wait of the plane-marching or slab kernel gave up
+    int wfault = 0;                 // MG_FAULT_WAVE_WAIT=1: the former's are made to run out (test of that path)
+    int sfault = 0;                 // MG_FAULT_SLAB_WAIT=1: the latter's
     bool poisoned = false, solved = false;
     std::string err;
     Profiler prof;
@@ -652,8 +653,8 @@ mg_status check_desc(const mg_hierarchy_desc &d, int b, int dim0)
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// After device work that ran plane-marching sweeps: MG_ETIMEOUT (and the
-// handle poisoned) when one of their bounded load waits gave up.
+// After device work that ran plane-marching sweeps or the slab kernel:
+// MG_ETIMEOUT (and the handle poisoned) when one of their bounded waits gave up.
 mg_status wave_status(mg_hierarchy *h)
 {
     int w = 0;
@@ -835,6 +836,7 @@ cudaError_t vcycle(mg_hierarchy *h, const LevelData &ld, bool fp32, cudaStream_t
             p.hi = hi;
         }
         p.err = h->werr;
+        p.fault = h->sfault;
         return timed_slab(h, 3.0 * w * cells_d(ld.g[Lslab].E, dim) * cycles,
                           [&] { return mg_launch_slab(dim, fp32, p, s); });
     };
@@ -1142,6 +1144,7 @@ cudaError_t slab_solve(mg_hierarchy *h, int b, int l, cudaStream_t s)
     p.scal = level_scal(h, b, l);
     p.ctl = level_ctl(h, b, l);
     p.err = h->werr;
+    p.fault = h->sfault;
     return timed_slab(h, 3.0 * 8.0 * cells_d(ld.g[0].E, h->dim),
                       [&] { return mg_launch_slab(h->dim, false, p, s); });
 }
@@ -2362,6 +2365,8 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
         h->use_graph = !(v && v[0] == '0');
         const char *fw = std::getenv("MG_FAULT_WAVE_WAIT");
         h->wfault = fw && fw[0] == '1';
+        const char *fs = std::getenv("MG_FAULT_SLAB_WAIT");
+        h->sfault = fs && fs[0] == '1';
     }
     // ghost layers and rings start at zero
     e = mg_bottom_prepare();

@@ -173,6 +173,7 @@ struct MgSlabPlan {
     double tol;
     const double *scal;
     int *err;                      // MG_ETIMEOUT once a wait for a neighbour's values ran out
+    int fault;                     // test of that path: one CTA's first wait runs out, after about 1 ms
 };
 int mg_slab_prepare();             // CTAs per cluster (0: unavailable); once per device before the first launch
 bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, int cut, int nu_pre, int nu_post,

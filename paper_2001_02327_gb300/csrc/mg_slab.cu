@@ -78,7 +78,8 @@
 namespace {
 
 constexpr int kT = MG_SLAB_THREADS;
-constexpr long long kWaitCycles = 2000000000ll;   // bound of one wait, about 1 s
+constexpr int kWaitUnits = 954;                   // bound of one wait in 2^21 cycles (1 ms), about 1 s
+constexpr long long kDrainCycles = 1ll << 19;     // time that values sent before a failure have to arrive
 
 typedef long long fix;   // fixed-point value: real * 2^scale
 
@@ -135,9 +136,9 @@ __device__ __forceinline__ void st_async(unsigned a, long long v, unsigned mb)
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a), "l"(v), "r"(mb)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_init(unsigned mb)
+__device__ __forceinline__ void mbar_init(unsigned mb, unsigned count)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_expect(unsigned mb, unsigned bytes)
 {
@@ -467,7 +468,10 @@ struct Engine {
     const MgSlabPlan &pl;
     int rank, tid;
     unsigned npass = 0;     // colour passes on distributed levels so far (the same in every CTA)
-    unsigned phase = 0;     // phase bits of the four mbarriers: [from the previous, next CTA][even, odd pass]
+    // phase bits of the four mbarriers: [from the previous, next CTA][even, odd pass]; kDead: this thread
+    // has left a wait that had not ended
+    unsigned phase = 0;
+    static constexpr unsigned kDead = 16;
 
     __device__ explicit Engine(const MgSlabPlan &p) : pl(p), rank((int)cluster_rank_()), tid((int)threadIdx.x) {}
 
@@ -500,6 +504,8 @@ struct Engine {
         return shared_addr(nbr() + 4 * MG_SLAB_MAXLEV) + 8 * (2 * dir + par);
     }
     __device__ __forceinline__ int *failed() const { return reinterpret_cast<int *>(nbr() + 4 * MG_SLAB_MAXLEV + 8); }
+    // bound of a wait (here, not in a register or the parameters: either cost 1.5 % of an FP64 V-cycle)
+    __device__ __forceinline__ volatile int *wait_units() const { return failed() + 1; }
     // norm of the residual: 16 warps' and 16 CTAs' sums, the total
     __device__ __forceinline__ double *sums() const { return reinterpret_cast<double *>(nbr() + 4 * MG_SLAB_MAXLEV + 10); }
     __device__ __forceinline__ int *img() const { return ctrl() + MG_SLAB_CTRL; }
@@ -572,9 +578,14 @@ struct Engine {
         const bool more = DIM == 3 ? ((c + k) & 1) == 0 : ((c + k) & 1) == 1;
         return (unsigned)(kW * ((cells + (more ? 1 : 0)) >> 1));
     }
+    __device__ __forceinline__ bool has_failed() const { return *(volatile int *)failed() != 0; }
     // After a colour pass on level q: the neighbours' new values have arrived
-    // (bounded: a wait that runs out marks the launch failed, after which no
-    // further wait waits) and every thread of this CTA has written its own.
+    // and every thread of this CTA has written its own.  The wait is bounded;
+    // after one that ran out this CTA waits for nothing more, sends what its
+    // neighbours wait for, and the launch runs to its end and reports the
+    // failure (k_slab).  Thread 0 no longer arrives then: no phase gets a second
+    // arrival.  (Its test is of a register: this step is on the critical path, a
+    // load from shared memory here cost 1 to 2 % of a V-cycle.)
     __device__ __forceinline__ void pass_sync(int q, const Lev &L, int c)
     {
         if (!dist(q)) {
@@ -583,7 +594,7 @@ struct Engine {
         }
         const int par = npass & 1;
         npass++;
-        if (tid == 0) {
+        if (tid == 0 && !(phase & kDead)) {
             if (L.mprev)
                 mbar_expect(mbar(0, par), plane_bytes(q, c, plane_first(pl, q, rank) - 1));
             if (L.mnext)
@@ -593,11 +604,12 @@ struct Engine {
         for (int dir = 0; dir < 2; dir++)
             if (dir ? L.mnext : L.mprev) {
                 const unsigned bit = 1u << (2 * dir + par);
-                if (!mbar_try(mbar(dir, par), phase & bit ? 1u : 0u) && !*failed()) {
+                if (!mbar_try(mbar(dir, par), phase & bit ? 1u : 0u)) {
                     const long long t0 = clock64();
                     while (!mbar_try(mbar(dir, par), phase & bit ? 1u : 0u))
-                        if (clock64() - t0 > kWaitCycles) {
-                            *failed() = 1;
+                        if (has_failed() || (int)((clock64() - t0) >> 21) >= *wait_units()) {
+                            *(volatile int *)failed() = 1;
+                            phase |= kDead;
                             break;
                         }
                 }
@@ -1287,7 +1299,7 @@ struct Engine {
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1)
                 acc += __shfl_down_sync(0xffffffffu, acc, o);
-            acc = scaled(__shfl_sync(0xffffffffu, acc, 0), -2 * sc()[0]);
+            acc = has_failed() ? CUDART_NAN : scaled(__shfl_sync(0xffffffffu, acc, 0), -2 * sc()[0]);
             if (tid < pl.csize)
                 st_cluster(cluster_addr(shared_addr(parts(n & 1) + rank), tid), __double_as_longlong(acc));
         }
@@ -1368,8 +1380,11 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
     if (tid < 2)
         s_max[tid] = 0u;
     __syncthreads();
+    if (tid == 0)
+        *en.wait_units() = pl.fault ? 1 : kWaitUnits;
     if (tid < 4) {
-        mbar_init(en.mbar(tid >> 1, tid & 1));
+        // (pl.fault: CTA 1's even passes wait for an arrival that does not come)
+        mbar_init(en.mbar(tid >> 1, tid & 1), pl.fault && rank == 1 && !(tid & 1) ? 2 : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < pl.nlev)
@@ -1508,11 +1523,6 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
         c.status = isfinite(c.bnorm) && (n == 0 || isfinite(c.rel)) ? 0 : 6;
         *pl.ctl = c;
     }
-    if (*en.failed()) {   // (a wait for a neighbour ran out)
-        bad = true;
-        if (pl.err && tid == 0)
-            *pl.err = 7;   // MG_ETIMEOUT
-    }
     // the potential of the plan's first level back to global memory
     if (n > 0) {
         G *out = static_cast<G *>(pl.phi);
@@ -1541,7 +1551,31 @@ __global__ void __launch_bounds__(kT, 1) k_slab(const __grid_constant__ MgSlabPl
     }
     if (pl.ctl && !solve && rank == 0 && tid == 0)
         inner_step_count(pl.ctl, pl.hi);
+    if (tid < C && en.has_failed())
+        st_cluster(cluster_addr(shared_addr(en.failed()), tid), 1u);
     cluster_sync_();   // no CTA leaves while another may still write to its shared memory
+    // A wait ran out, in whichever CTA: the potential becomes NaN, and what was
+    // sent but never waited for gets time to arrive before its destination
+    // leaves.
+    if (en.has_failed()) {
+        for (int u = 0; u < pl.K[0]; u++) {
+            const int A = en.word_a(u), d = en.word(0, u, kD);
+            G *dst = static_cast<G *>(pl.phi) + gidx(2 * (d & 0x3ff) + 1, (d >> 10) & 0x3ff, d >> 20);
+            if ((A >> 15) & 1)
+                dst[0] = G(CUDART_NAN);
+            if ((A >> 16) & 1)
+                dst[1] = G(CUDART_NAN);
+        }
+        if (rank == 0 && tid == 0) {
+            if (pl.err)
+                *pl.err = 7;   // MG_ETIMEOUT
+            if (solve)
+                pl.ctl->status = 6;
+        }
+        const long long t0 = clock64();
+        while (clock64() - t0 < kDrainCycles)
+            ;
+    }
 }
 
 template <class P, int DIM>

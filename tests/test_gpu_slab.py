@@ -174,3 +174,36 @@ def test_fp64_slab_converged_potential_is_unbiased(mg, dim, n, kind, nu):  # noq
     unit = 2.0 ** -56 * float(np.abs(x).max())
     err = float(np.abs(g[0]["phi"] - x[(slice(2, -2),) * dim]).max())
     assert err <= unit * ((1.0 / 8 if dim == 3 else 0.0737) * N ** 2 + 8.0)
+
+
+@pytest.mark.parametrize("dim,n,prec,solve", [(3, 16, "fp64", True), (2, 64, "fp64", True), (3, 62, "fp64", False),
+                                              (3, 30, "mixed", False), (2, 126, "mixed", False)])
+@pytest.mark.parametrize("graph", ["1", "0"])
+def test_slab_wait_timeout_reports_etimeout(mg, monkeypatch, dim, n, prec, solve, graph):  # noqa: F811
+    """With MG_FAULT_SLAB_WAIT=1 one CTA's first wait for its neighbours runs
+    out (limit about 1 ms): the launch ends, mg_solve reports MG_ETIMEOUT, the
+    handle refuses further work, and a new handle solves as one without the
+    fault; for levels that one launch solves and for single V-cycles."""
+    import torch
+    H, inp = random_single_level(dim, n, 3 * n + dim)
+    kw = dict(max_cycles=4, rel_tol=0.0)
+    if prec == "mixed":
+        kw.update(precision=mg.MG_MIXED, inner_cycles=2)
+    monkeypatch.setenv("MG_SOLVE_GRAPH", graph)
+    _, before = gpu_solve(mg, H, inp, **kw)
+    monkeypatch.setenv("MG_FAULT_SLAB_WAIT", "1")
+    h = mg.mg_create_hierarchy([mg.desc_from(H)], mg.options(**kw))
+    try:
+        dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        mg.mg_set_density(h, 0, 0, dev(inp[0]["rho"]), dev(inp[0]["bc_rho"]), dev(inp[0]["bc_phi"]))
+        with pytest.raises(mg.MGError) as ei:
+            mg.mg_solve(h, 1, allow_noconv=True)
+        assert ei.value.status == mg.MG_ETIMEOUT, ei.value
+        with pytest.raises(mg.MGError) as ei:
+            mg.mg_solve(h, 1, allow_noconv=True)
+        assert ei.value.status == mg.MG_ESTATE, ei.value
+    finally:
+        mg.mg_destroy(h)
+    monkeypatch.delenv("MG_FAULT_SLAB_WAIT")
+    _, after = gpu_solve(mg, H, inp, **kw)
+    assert np.array_equal(before[0]["phi"], after[0]["phi"])
