@@ -914,7 +914,7 @@ __global__ void __launch_bounds__(256, 5) kx_norm_march(const double *__restrict
     pdl_begin();
     MarchResidual<BoxIndex> fn{phi, f, m.sy, m.sz, g.N[0], g.N[1], g.N[2], g.ih2[0], false, f32, e32,
                                {g.half, g.E[1], g.H}, 0.0, 0.0, 0.0};
-    march<1, 6>(phi, m, fn);
+    march<1, 6, false>(phi, m, fn);
     const double s = block_sum(fn.r2);
     if (threadIdx.x == 0)
         part[blockIdx.x] = s;
@@ -1130,7 +1130,7 @@ __global__ void __launch_bounds__(256, 4) kx_forces_march(PatchDims d, double c,
 {
     pdl_begin();
     MarchForces fn{phi, m.sy, m.sz, (long long)d.n[0] * d.n[1] * d.n[2], d.n[0], d.n[1], stencil, c, F, phi_out, 0.0};
-    march<2, 5>(phi, m, fn);
+    march<2, 6, true>(phi, m, fn);
 }
 __global__ void __launch_bounds__(256) kx_forces(PatchDims d, int dim, double i2h, double i4h,
                                                  const double *__restrict__ phi, double *__restrict__ F,

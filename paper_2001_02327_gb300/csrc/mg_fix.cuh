@@ -152,11 +152,14 @@ __device__ __forceinline__ double fx_interp(const double (&v)[1 << DIM], const b
     return DIM == 3 ? fx_rare_add(fx_rare_mul(far[2] ? 0.25 : 0.75, z[0]), fx_rare_mul(far[2] ? 0.75 : 0.25, z[1])) : z[0];
 }
 
-// 8 (a - b) - (c - d), the numerator of the fourth-order difference
+// 8 (a - b) - (c - d), the numerator of the fourth-order difference: exact and
+// rounded once where no term loses bits, else by the FP64 instructions (the
+// terms may cancel, so a bound by the largest of them would not do)
 __device__ __forceinline__ double fx_diff4(double a, double b, double c, double d)
 {
-    const int e = max(max(fx_exp(a), fx_exp(b)), max(fx_exp(c), fx_exp(d)));
-    if (!fx_ok(e))
+    const int ea = fx_exp(a), eb = fx_exp(b), ec = fx_exp(c), ed = fx_exp(d);
+    const int e = max(max(ea, eb), max(ec, ed));
+    if (!fx_ok(e) || min(min(ea, eb), min(ec, ed)) < e - 5)
         return fx_rare_diff4(a, b, c, d);
     return fx_round<5>(8 * (fx_align<5>(a, e) - fx_align<5>(b, e)) - (fx_align<5>(c, e) - fx_align<5>(d, e)), e);
 }

@@ -1647,7 +1647,7 @@ __global__ void __launch_bounds__(256, 5) k_norms_march(const double *__restrict
 {
     pdl_begin();
     MarchResidual<SplitIndex> fn{phi, f, m.sy, m.sz, g.N, g.N, g.N, g.inv_h2, (which & 1) != 0, r32, e32, {g}, 0.0, 0.0, 0.0};
-    march<1, 6>(phi, m, fn);
+    march<1, 6, false>(phi, m, fn);
     norms_reduce(fn.b2, fn.r2, which, partials, counter, out2);
 }
 
@@ -2055,7 +2055,7 @@ __global__ void __launch_bounds__(256, 4) k_forces_march(int n, double c, const 
 {
     pdl_begin();
     MarchForces fn{phi, m.sy, m.sz, (long long)n * n * n, n, n, stencil, c, F, phi_out, 0.0};
-    march<2, 5>(phi, m, fn);
+    march<2, 6, true>(phi, m, fn);
 }
 
 // Stopping test of Sec. 3: max over Omega of |F(phi) - F(prev)|^2 into *cmax

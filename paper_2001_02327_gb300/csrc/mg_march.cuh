@@ -10,9 +10,12 @@
 // along z from a window in registers.  All values of a block share one
 // exponent, the largest seen so far plus a bit; a plane that exceeds it shifts
 // what the block holds (the test rides on the barrier that each plane needs
-// anyway); cells far below that exponent take the FP64 instructions, so that no
-// result is less accurate than they would give.  Two planes are in flight ahead
-// of the one being aligned, and the functor's own loads one plane ahead.
+// anyway).  Cells for which that exponent is too large take the FP64
+// instructions: residuals whose centre is below 2^-6 of it (else the truncation
+// of the terms is of the size of FP64's own rounding, 12 units of 2^-53 of the
+// centre at most), forces of which a term lost a bit (else their sum is exact
+// and rounded once).  Two planes are in flight ahead of the one being aligned,
+// and the functor's own loads one plane ahead.
 #pragma once
 
 #include "mg_fix.cuh"
@@ -52,10 +55,25 @@ inline MarchGrid march_grid(int n0, int n1, int n2, long long sy, long long sz, 
     return m;
 }
 
+// v * 2^-d, the last bit set where bits are lost
+__device__ __forceinline__ long long fx_shift_mark(long long v, int d)
+{
+    const long long r = v >> d;
+    return (long long)((unsigned long long)r << d) == v ? r : r | 1;
+}
+// fx_align, the last bit set where x has bits there or below (it is clear otherwise)
+template <int P>
+__device__ __forceinline__ long long fx_align_mark(double x, int emax)
+{
+    const bool lost = emax - fx_exp(x) >= P && ((__double2hiint(x) << 1) | __double2loint(x)) != 0;
+    return fx_align<P>(x, emax) | (lost ? 1 : 0);
+}
+
 // R rings; fn.prefetch(i, j, k) a plane ahead and fn(i, j, k, b, w, bound) for every active cell
 // (storage indices): b points at the cell in its aligned plane of row pitch
-// 32 + 2 R, w[0..2R] is its column, both multiples of 2^(bound - 1023 - 52 - P).
-template <int R, int P, class Fn>
+// 32 + 2 R, w[0..2R] is its column, both multiples of 2^(bound - 1023 - 52 - P)
+// and below 2^(52 + P) of them; with MARK the last bit says that bits were lost.
+template <int R, int P, bool MARK, class Fn>
 __device__ __forceinline__ void march(const double *__restrict__ src, const MarchGrid &g, Fn &fn)
 {
     constexpr int TX = 32, TY = 8, W = TX + 2 * R, H = TY + 2 * R, NB = R + 1, HALO = 2 * R * (TX + TY);
@@ -120,9 +138,11 @@ __device__ __forceinline__ void march(const double *__restrict__ src, const Marc
                 const int d = min(nb - bound, 63);
 #pragma unroll
                 for (int u = 0; u <= 2 * R; u++)
-                    w[u] >>= d;
-                for (int u = t; u < NB * H * W; u += TX * TY)
-                    (&buf[0][0])[u] >>= d;
+                    w[u] = MARK ? fx_shift_mark(w[u], d) : w[u] >> d;
+                for (int u = t; u < NB * H * W; u += TX * TY) {
+                    long long &v = (&buf[0][0])[u];
+                    v = MARK ? fx_shift_mark(v, d) : v >> d;
+                }
             }
             bound = nb;
             first = false;
@@ -131,10 +151,10 @@ __device__ __forceinline__ void march(const double *__restrict__ src, const Marc
 #pragma unroll
         for (int u = 0; u < 2 * R; u++)
             w[u] = w[u + 1];
-        w[2 * R] = fx_align<P>(c0, bound);
+        w[2 * R] = MARK ? fx_align_mark<P>(c0, bound) : fx_align<P>(c0, bound);
         buf[cur][at] = w[2 * R];
         if (t < HALO)
-            buf[cur][hat] = fx_align<P>(h0, bound);
+            buf[cur][hat] = MARK ? fx_align_mark<P>(h0, bound) : fx_align<P>(h0, bound);
         cur = cur == NB - 1 ? 0 : cur + 1;   // now the plane k = p - R: written R planes ago
         if (k >= z0 && active) {
             const auto ahead = fn.taken();
@@ -247,23 +267,31 @@ struct MarchForces {
         const long long t = ((long long)(k - 2) * n1 + (j - 2)) * n0 + (i - 2);
         double d[3];
         {
+            // the differences of aligned terms, and whether one of these lost bits (march)
             long long s[3];
+            int lost[3];
             if (stencil == 0) {
-                s[0] = fx_d4(b[1], b[-1], b[2], b[-2]);
-                s[1] = fx_d4(b[W], b[-W], b[2 * W], b[-2 * W]);
-                s[2] = fx_d4(w[3], w[1], w[4], w[0]);
+                auto diff = [&](int a, long long p1, long long m1, long long p2, long long m2) {
+                    s[a] = fx_d4(p1, m1, p2, m2);
+                    lost[a] = ((int)p1 | (int)m1 | (int)p2 | (int)m2) & 1;
+                };
+                diff(0, b[1], b[-1], b[2], b[-2]);
+                diff(1, b[W], b[-W], b[2 * W], b[-2 * W]);
+                diff(2, w[3], w[1], w[4], w[0]);
             } else {
-                s[0] = b[1] - b[-1];
-                s[1] = b[W] - b[-W];
-                s[2] = w[3] - w[1];
+                auto diff = [&](int a, long long p1, long long m1) {
+                    s[a] = p1 - m1;
+                    lost[a] = ((int)p1 | (int)m1) & 1;
+                };
+                diff(0, b[1], b[-1]);
+                diff(1, b[W], b[-W]);
+                diff(2, w[3], w[1]);
             }
-            // a difference below 2^-10 of the block's exponent could be more than
-            // 2^-43 of its terms off by the truncation of 18 of them
             const bool ok = fx_ok(bound);
 #pragma unroll
             for (int a = 0; a < 3; a++) {
-                d[a] = fx_round<5>(s[a], bound);
-                if (!ok || (unsigned long long)(s[a] + (1ll << 48)) < (1ull << 49))
+                d[a] = fx_round<6>(s[a], bound);
+                if (!ok || lost[a])
                     d[a] = plain(p, a == 0 ? 1 : a == 1 ? sy : sz, stencil);
             }
         }
