@@ -37,6 +37,7 @@ struct LevelData {
     bool frozen = false;           // MG_IFACE_FROZEN level: multigrid on Omega only
     double *prev = nullptr;        // MG_STOP_FORCE: the (n+4)^d block before the iteration
     float *phi32[MG_MAX_MG] = {};  // mixed precision correction, all multigrid levels
+    size_t fp32_bytes = 0;         // phi32, phi32b and f32 of all levels, from phi32[0] on
     float *phi32b[MG_MAX_MG] = {}; // second FP32 buffer of the temporally blocked levels
     int tile[MG_MAX_MG] = {};      // FP32 temporal-blocking tile per level (0: one kernel per phase)
     int nsplit = 0;                // FP32 levels 0..nsplit-1 stored colour-split (MgGeom::sH > 0), tile 0
@@ -146,8 +147,9 @@ void plan_tiles(LevelData &ld, int dim, int nu_pre, int nu_post)
 // 30.0 split from 98 cells, 29.7 from 66 or from 50.  MG_WAVE,
 // MG_WAVE_PLAN or MG_TB_TILE ask for the plain-layout plans instead.  mg_autotune
 // times the choices; the batched kernels (MG_BATCHED=1) run plain levels
-// only.  Changing the layout clears the level's FP32 arrays (their ghost
-// layer must read zero in either layout).
+// only.  Changing the layout clears the level's FP32 arrays once something has
+// been written to them (their ghost layer must read zero in either layout): one
+// memset, the arrays lie side by side.
 int first_fused(const LevelData &ld, bool fp32);
 constexpr int kTileSplit = 1 << 16;   // mg_tuning / tuning-cache code of a split level
 constexpr int kSplitMinN = 192, kSplitFirst = 100, kSplitFirstBatch = 60;
@@ -172,7 +174,7 @@ int split_default(const LevelData &ld, int dim, int batch)
     return S;
 }
 
-cudaError_t plan_split(LevelData &ld, int dim, int S, cudaStream_t s)
+cudaError_t plan_split(LevelData &ld, int dim, int S, bool written, cudaStream_t s)
 {
     S = std::max(0, std::min(S, first_fused(ld, true)));
     if (ld.Lc[1] >= 0)
@@ -190,13 +192,9 @@ cudaError_t plan_split(LevelData &ld, int dim, int S, cudaStream_t s)
         }
     }
     ld.nsplit = S;
-    if (!changed || !ld.phi32[0])
+    if (!changed || !written || !ld.phi32[0])
         return cudaSuccess;
-    for (int L = 0; L < ld.nmg; L++)
-        for (float *a : {ld.phi32[L], ld.phi32b[L], ld.f32[L]})
-            if (cudaError_t e = cudaMemsetAsync(a, 0, mg_fp32_cells(ld.g[L].E, dim) * sizeof(float), s))
-                return e;
-    return cudaSuccess;
+    return cudaMemsetAsync(ld.phi32[0], 0, ld.fp32_bytes, s);
 }
 
 void plan_bottom(LevelData &ld, int dim, int lim32 = -1)
@@ -441,6 +439,7 @@ struct mg_hierarchy {
     Profiler prof;
     // solve graph
     bool use_graph = true;          // MG_SOLVE_GRAPH=0: host-driven loop (for kernel profilers)
+    bool fp32_written = false;      // something has run on the FP32 arrays: until then they are zero in any layout
     int csize = 0;                  // CTAs per cluster of the cluster kernel (0: unavailable)
     int ssize = 0;                  // the same of the slab kernel
     std::map<std::pair<int, int>, int *> slab_img;   // its plan images by (M, first level)
@@ -1184,6 +1183,7 @@ mg_status solve_level_host(mg_hierarchy *h, int b, int l, mg_level_stats *st)
     cudaStream_t s = h->stream;
     double *hs = h->hscal + 2 * ((size_t)b * MG_MAX_LEVELS + l);
     double *ds = level_scal(h, b, l);
+    h->fp32_written = true;
     CK(h, level_prelude(h, b, l, s, 0));
     CK(h, cudaMemcpyAsync(hs, ds, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(h, cudaStreamSynchronize(s));
@@ -1598,7 +1598,7 @@ bool plan_persistent(mg_hierarchy *h, mg_status &err)
         double cellsum = 0.0;
         for (int l = 0; l < h->desc[b].num_levels; l++) {
             LevelData &ld = h->lev[b][l];
-            if (cudaError_t e = plan_split(ld, dim, ld.Ls[1], h->stream)) {
+            if (cudaError_t e = plan_split(ld, dim, ld.Ls[1], h->fp32_written, h->stream)) {
                 err = fail_cuda(h, e, "persistent plan");
                 return false;
             }
@@ -1805,7 +1805,7 @@ mg_status build_graph(mg_hierarchy *h)
         if (v && v[0] == '1') {
             for (auto &hl : h->lev)
                 for (auto &ld : hl)
-                    CK(h, plan_split(ld, h->dim, 0, h->stream));
+                    CK(h, plan_split(ld, h->dim, 0, h->fp32_written, h->stream));
             mg_status perr;
             h->batched = plan_batched(h, perr);
             if (perr)
@@ -1891,6 +1891,7 @@ mg_status solve_graph(mg_hierarchy *h, mg_level_stats *stats)
             return s;
     }
     const size_t nctl = (size_t)h->batch * MG_MAX_LEVELS;
+    h->fp32_written = true;
     CK(h, cudaGraphLaunch(h->gexec, h->stream));
     CK(h, cudaMemcpyAsync(h->hctl, h->ctl, nctl * sizeof(MgSolveCtl), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
@@ -2016,7 +2017,7 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
             return false;
         plan_tiles(ld, dim, o.nu_pre, o.nu_post);
         plan_cluster(ld, h->dim, h->csize, h->opt);
-        if ((err = plan_split(ld, dim, 0, h->stream)))
+        if ((err = plan_split(ld, dim, 0, true, h->stream)))
             return false;
         const float ms = time_ms(h, 10, [&](cudaStream_t cs) { return vcycle(h, ld, true, cs); }, err);
         if (err)
@@ -2032,7 +2033,7 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
     if ((err = refresh_bottom_plan(h, ld)))
         return false;
     plan_cluster(ld, h->dim, h->csize, h->opt);
-    if ((err = plan_split(ld, dim, 0, h->stream)))
+    if ((err = plan_split(ld, dim, 0, true, h->stream)))
         return false;
     te.bottom_n = bestnb;
     // 2. per level above the bottom: the tile of its pre/post pair
@@ -2115,7 +2116,7 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
         int bestS = 0;
         for (int S = 0; S <= Ls; S++) {
             std::copy(tiles, tiles + MG_MAX_MG, ld.tile);
-            if ((err = plan_split(ld, dim, S, h->stream)))
+            if ((err = plan_split(ld, dim, S, true, h->stream)))
                 return false;
             const float ms = time_ms(h, 10, [&](cudaStream_t cs) { return vcycle(h, ld, true, cs); }, err);
             if (err)
@@ -2126,7 +2127,7 @@ bool tune_level(mg_hierarchy *h, LevelData &ld, TuneEntry &te, cudaError_t &err)
             }
         }
         std::copy(tiles, tiles + MG_MAX_MG, ld.tile);
-        if ((err = plan_split(ld, dim, bestS, h->stream)))
+        if ((err = plan_split(ld, dim, bestS, true, h->stream)))
             return false;
         for (int L = 0; L < bestS; L++)
             te.tile[L] = kTileSplit;
@@ -2148,7 +2149,7 @@ cudaError_t apply_entry(mg_hierarchy *h, LevelData &ld, const TuneEntry &te)
         ld.tile[L] = L < Ls && te.tile[L] != kTileSplit ? te.tile[L] : 0;
     plan_cluster(ld, h->dim, h->csize, h->opt);
     if (!e)
-        e = plan_split(ld, h->dim, S, h->stream);
+        e = plan_split(ld, h->dim, S, h->fp32_written, h->stream);
     return e;
 }
 
@@ -2294,12 +2295,12 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
                 const size_t c = (size_t)cells(ld.g[L].E, dim);
                 slots.push_back({(void **)&ld.phi[L], align256(c * sizeof(double))});
                 slots.push_back({(void **)&ld.f[L], align256(c * sizeof(double))});
-                if (o.precision == MG_MIXED) {   // room for the plain and the colour-split layout
-                    const size_t c32 = mg_fp32_cells(ld.g[L].E, dim);
-                    slots.push_back({(void **)&ld.phi32[L], align256(c32 * sizeof(float))});
-                    slots.push_back({(void **)&ld.phi32b[L], align256(c32 * sizeof(float))});
-                    slots.push_back({(void **)&ld.f32[L], align256(c32 * sizeof(float))});
-                }
+            }
+            for (int L = 0; L < ld.nmg && o.precision == MG_MIXED; L++) {   // room for the plain and the colour-split layout
+                const size_t c32 = align256(mg_fp32_cells(ld.g[L].E, dim) * sizeof(float));
+                for (float **a : {&ld.phi32[L], &ld.phi32b[L], &ld.f32[L]})
+                    slots.push_back({(void **)a, c32});
+                ld.fp32_bytes += 3 * c32;
             }
             for (int L = 1; L < ld.nmg; L++) {
                 slots.push_back({(void **)&ld.tab64[L], align256(128 * sizeof(double))});
@@ -2409,7 +2410,7 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
             if (e == cudaSuccess)
                 e = plan_slab(h, ld, true);
             if (e == cudaSuccess && o.precision == MG_MIXED)
-                e = plan_split(ld, dim, split_default(ld, dim, batch), h->stream);
+                e = plan_split(ld, dim, split_default(ld, dim, batch), false, h->stream);
         }
     if (e == cudaSuccess) {
         std::vector<double> fr((size_t)batch * MG_MAX_LEVELS, 0.0);
@@ -2724,6 +2725,7 @@ mg_status mg_autotune(mg_hierarchy *h, const char *cache_path)
             }
             TuneEntry te{};
             cudaError_t e = cudaSuccess;
+            h->fp32_written = true;
             if (!tune_level(h, ld, te, e))
                 return fail_cuda(h, e, "autotune timing");
             fresh.push_back(te);
@@ -2764,6 +2766,7 @@ mg_status mg_time_smoothing(mg_hierarchy *h, int b, int level, int L, int launch
         return fail(h, MG_EINVAL, "multigrid level %d runs the temporally blocked legs", L);
     const mg_options &o = h->opt;
     cudaError_t err = cudaSuccess;
+    h->fp32_written = true;
     const float ms = time_ms(h, 5, [&](cudaStream_t s) {
         cudaError_t e = cudaSuccess;
         for (int r = 0; r < launches && !e; r++) {
