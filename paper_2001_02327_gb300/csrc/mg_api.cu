@@ -52,6 +52,7 @@ struct LevelData {
     int Llim[2] = {0, 0};          // the level-size limit that chose it
     MgBottom bt[2];
     int Lslab[2] = {-1, -1};       // first level handled by the slab kernel (-1: none)
+    int slab_first = -1;           // ... if it is put to use (-1: does not apply)
     MgSlabPlan slab;               // its plan, for the precision of the V-cycles
     // device image of the one-block kernel's plan for the precision the
     // V-cycles run in, sized for the largest bottom the level admits
@@ -323,7 +324,7 @@ void plan_cluster(LevelData &ld, int dim, int csize, const mg_options &o, int li
 // per edge are split over its CTAs.  The limits are the largest levels whose
 // V-cycle is shorter there than as launches of the whole GPU (3D 34^3: 31 us
 // FP32 and 48 us FP64 against 52 and 70 us) and that fit its shared memory.
-int slab_limit(int dim, bool) { return dim == 3 ? 34 : 160; }
+int slab_limit(int dim) { return dim == 3 ? 34 : 160; }
 int slab_cut(int dim) { return dim == 3 ? 9 : 24; }
 
 bool slab_wanted(bool fp32)
@@ -411,6 +412,12 @@ struct Profiler {
 
 }  // namespace
 
+// A plan image of the slab kernel in the arena
+struct SlabImage {
+    char *mem = nullptr;
+    bool written = false;
+};
+
 struct mg_hierarchy {
     int batch = 0, dim = 0;
     std::vector<mg_hierarchy_desc> desc;
@@ -442,7 +449,7 @@ struct mg_hierarchy {
     bool fp32_written = false;      // something has run on the FP32 arrays: until then they are zero in any layout
     int csize = 0;                  // CTAs per cluster of the cluster kernel (0: unavailable)
     int ssize = 0;                  // the same of the slab kernel
-    std::map<std::pair<int, int>, int *> slab_img;   // its plan images by (M, first level)
+    std::map<std::pair<int, int>, SlabImage> slab_img;   // its plan images by (M, first level)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
     std::vector<char> graph_sig;
@@ -722,58 +729,68 @@ cudaError_t refresh_bottom_plan(mg_hierarchy *h, LevelData &ld)
     return e;
 }
 
-// The slab kernel's plan of a level, for the precision of the V-cycles; its
-// image is shared by all levels of the handle with the same sizes and built
-// at creation or tuning (synchronous).
-cudaError_t plan_slab(mg_hierarchy *h, LevelData &ld, bool on)
+// Lays out the slab kernel's plan of a level, for the precision of the
+// V-cycles, whether or not it will run (plan_slab).
+void layout_slab(const mg_hierarchy *h, LevelData &ld)
 {
     const bool fp32 = h->opt.precision == MG_MIXED;
-    const int w = fp32 ? 1 : 0, lim = slab_limit(h->dim, fp32);
-    ld.Lslab[w] = -1;
+    const int lim = slab_limit(h->dim);
     // mixed batches: graph branches of several hierarchies share the SMs, which
     // small launches of all of them fill better than clusters of 16 (batch of 32
     // uneven hierarchies: 40 ms against 47 ms)
-    if (!on || h->ssize <= 0 || !slab_wanted(fp32) || (fp32 && h->batch > 1))
+    if (h->ssize <= 0 || (fp32 && h->batch > 1))
+        return;
+    for (int L = 0; L + 1 < ld.nmg && ld.slab_first < 0; L++)
+        if (ld.g[L].N <= lim && mg_slab_layout(h->dim, fp32, h->ssize, &ld.g[L], ld.nmg - L, slab_cut(h->dim),
+                                               h->opt.nu_pre, h->opt.nu_post, ld.slab))
+            ld.slab_first = L;
+}
+
+// bytes of a plan's image with the dense matrix behind the plan words
+size_t slab_image_bytes(const MgSlabPlan &p, bool fp32)
+{
+    return align256(mg_slab_image_bytes(p)) + align256((size_t)p.dn * p.dn * (fp32 ? 4 : 8));
+}
+
+// The slab kernel's plan of a level put to use (or not).  Its image is shared by
+// all levels of the handle with the same sizes and written for the first of
+// them, on the handle's stream; nothing waits for it here.
+cudaError_t plan_slab(mg_hierarchy *h, LevelData &ld, bool on)
+{
+    const bool fp32 = h->opt.precision == MG_MIXED;
+    const int w = fp32 ? 1 : 0, L = ld.slab_first;
+    ld.Lslab[w] = -1;
+    if (!on || L < 0 || !slab_wanted(fp32))
         return cudaSuccess;
-    for (int L = 0; L + 1 < ld.nmg; L++) {
-        if (ld.g[L].N > lim)
-            continue;
-        MgSlabPlan &p = ld.slab;
-        if (!mg_slab_layout(h->dim, fp32, h->ssize, &ld.g[L], ld.nmg - L, slab_cut(h->dim), h->opt.nu_pre,
-                            h->opt.nu_post, p))
-            continue;
-        int *&img = h->slab_img[{ld.M, L}];
-        const size_t ib = align256(mg_slab_image_bytes(p)), nd = (size_t)p.dn * p.dn;
-        if (!img) {
-            // the dense matrix behind the plan words
-            const int Ld = L + p.nlev - 1;
-            std::vector<double> mat(nd);
-            mg_slab_dense(h->dim, &ld.g[Ld], ld.nmg - Ld, h->opt.nu_pre, h->opt.nu_post, mat.data());
-            std::vector<float> m32(nd);
-            std::vector<long long> m64(nd);
-            for (size_t i = 0; i < nd; i++) {
-                m32[i] = (float)mat[i];
-                m64[i] = std::llrint(std::ldexp(mat[i], 60));
-            }
-            cudaError_t e = cudaMalloc((void **)&img, ib + nd * (fp32 ? 4 : 8));
-            if (e == cudaSuccess)
-                e = mg_launch_slab_plan(h->dim, p, img, h->stream);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync((char *)img + ib, fp32 ? (const void *)m32.data() : (const void *)m64.data(),
-                                    nd * (fp32 ? 4 : 8), cudaMemcpyHostToDevice, h->stream);
-            if (e == cudaSuccess)
-                e = cudaStreamSynchronize(h->stream);
-            if (e)
-                return e;
+    MgSlabPlan &p = ld.slab;
+    for (int q = 0; q < p.nlev; q++)
+        p.g[q] = ld.g[L + q];   // with the tables made since
+    SlabImage &img = h->slab_img[{ld.M, L}];
+    const size_t ib = align256(mg_slab_image_bytes(p)), nd = (size_t)p.dn * p.dn;
+    if (!img.written) {
+        const int Ld = L + p.nlev - 1;
+        std::vector<double> mat(nd);
+        mg_slab_dense(h->dim, &ld.g[Ld], ld.nmg - Ld, h->opt.nu_pre, h->opt.nu_post, mat.data());
+        std::vector<float> m32(nd);
+        std::vector<long long> m64(nd);
+        for (size_t i = 0; i < nd; i++) {
+            m32[i] = (float)mat[i];
+            m64[i] = std::llrint(std::ldexp(mat[i], 60));
         }
-        p.dense = (const char *)img + ib;
-        p.img = img;
-        p.zero_start = L > 0;
-        p.phi = fp32 ? (void *)ld.phi32[L] : (void *)ld.phi[L];
-        p.f = fp32 ? (const void *)ld.f32[L] : (const void *)ld.f[L];
-        ld.Lslab[w] = L;
-        break;
+        cudaError_t e = mg_launch_slab_plan(h->dim, p, (int *)img.mem, h->stream);
+        if (e == cudaSuccess)   // (from pageable memory: staged when the call returns)
+            e = cudaMemcpyAsync(img.mem + ib, fp32 ? (const void *)m32.data() : (const void *)m64.data(),
+                                nd * (fp32 ? 4 : 8), cudaMemcpyHostToDevice, h->stream);
+        if (e)
+            return e;
+        img.written = true;
     }
+    p.img = (const int *)img.mem;
+    p.dense = img.mem + ib;
+    p.zero_start = L > 0;
+    p.phi = fp32 ? (void *)ld.phi32[L] : (void *)ld.phi[L];
+    p.f = fp32 ? (const void *)ld.f32[L] : (const void *)ld.f[L];
+    ld.Lslab[w] = L;
     return cudaSuccess;
 }
 
@@ -2272,6 +2289,7 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
     }
 
     // geometry and arena layout
+    h->ssize = mg_slab_prepare();
     h->lev.resize(batch);
     size_t bytes = 0, stage = 0;
     struct Slot { void **dst; size_t bytes; };
@@ -2309,6 +2327,12 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
             ld.bplan_bytes = max_bottom_plan_bytes(ld, dim, o.precision == MG_MIXED);
             if (ld.bplan_bytes)
                 slots.push_back({(void **)&ld.bplan, align256(ld.bplan_bytes)});
+            layout_slab(h, ld);
+            if (ld.slab_first >= 0) {
+                const auto at = h->slab_img.insert({{ld.M, ld.slab_first}, SlabImage{}});
+                if (at.second)
+                    slots.push_back({(void **)&at.first->second.mem, slab_image_bytes(ld.slab, o.precision == MG_MIXED)});
+            }
             if (o.stop == MG_STOP_FORCE)
                 slots.push_back({(void **)&ld.prev, align256((size_t)cells(ld.n + 4, dim) * sizeof(double))});
             if (ld.frozen) {
@@ -2380,8 +2404,6 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
     if (e == cudaSuccess)
         h->csize = mg_cluster_prepare();
     if (e == cudaSuccess)
-        h->ssize = mg_slab_prepare();
-    if (e == cudaSuccess)
         e = mg_launch_zero(h->arena, bytes, h->stream);
     if (e == cudaSuccess)   // the table copies below do not run on the caller's stream
         e = cudaStreamSynchronize(h->stream);
@@ -2404,11 +2426,11 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
             }
             plan_bottom(ld, dim);
             if (e == cudaSuccess)
+                e = plan_slab(h, ld, true);
+            if (e == cudaSuccess && ld.Lslab[o.precision == MG_MIXED ? 1 : 0] < 0)   // the slab kernel's levels need none
                 e = refresh_bottom_plan(h, ld);
             plan_tiles(ld, dim, o.nu_pre, o.nu_post);
             plan_cluster(ld, h->dim, h->csize, h->opt);
-            if (e == cudaSuccess)
-                e = plan_slab(h, ld, true);
             if (e == cudaSuccess && o.precision == MG_MIXED)
                 e = plan_split(ld, dim, split_default(ld, dim, batch), false, h->stream);
         }
@@ -2425,8 +2447,6 @@ mg_status mg_create_hierarchy(const mg_hierarchy_desc *descs, int batch, const m
         e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        for (auto &im : h->slab_img)
-            cudaFree(im.second);
         cudaFreeHost(h->hscal);
         cudaFreeHost(h->hctl);
         cudaFree(h->arena);
@@ -2825,8 +2845,6 @@ mg_status mg_destroy(mg_hierarchy *h)
     for (cudaEvent_t e : h->prof.pool)
         cudaEventDestroy(e);
     destroy_graph(h);
-    for (auto &im : h->slab_img)
-        cudaFree(im.second);
     if (h->persist_mem)
         cudaFree(h->persist_mem);
     if (h->cap_p)

@@ -1754,57 +1754,26 @@ bool mg_slab_layout(int dim, bool fp32, int csize, const MgGeom *g, int nlev, in
 // Matrix of one V-cycle from a zero potential on levels g[0..nlev-1] (all of
 // them, down to one cell): column j holds the potential of level 0 for the
 // right-hand side h^2 f = unit vector j, cells x fastest.  FP64 on the host,
-// at most 64 cells.
+// at most 64 cells.  The columns go through each step side by side (a row of n0
+// values per cell), along lists of neighbours made once: creating a handle
+// waits for this (4^3, V(2,2): 0.4 ms one column at a time).
 void mg_slab_dense(int dim, const MgGeom *g, int nlev, int nu_pre, int nu_post, double *mat)
 {
-    struct L {
-        int N, E, n;
-        std::vector<double> phi, f;   // (N + 2)^d, ghosts zero; f as h^2 f
+    struct Cell {
+        int nb[6], nn, parent, colour;   // neighbours in the order of the stencil's sum
+        double d;                        // diagonal with the ghost rule folded in
+        int at[8];                       // the coarse cells that it is interpolated from
+        double w[8];
     };
-    std::vector<L> v(nlev);
-    for (int q = 0; q < nlev; q++) {
-        v[q].N = g[q].N;
-        v[q].E = g[q].N + 2;
-        v[q].n = dim == 3 ? v[q].E * v[q].E * v[q].E : v[q].E * v[q].E;
-        v[q].phi.assign(v[q].n, 0.0);
-        v[q].f.assign(v[q].n, 0.0);
-    }
-    auto id = [&](const L &l, int i, int j, int k) { return (k * l.E + j) * l.E + i; };
-    auto cells = [&](const L &l, auto &&fn) {
-        for (int k = dim == 3 ? 1 : 0; k <= (dim == 3 ? l.N : 0); k++)
-            for (int j = 1; j <= l.N; j++)
-                for (int i = 1; i <= l.N; i++)
-                    fn(i, j, k);
+    struct Level {
+        std::vector<Cell> cell;
+        std::vector<double> phi, f;      // f as h^2 f
     };
-    // neighbour sum and diagonal with the ghost rule folded in
-    auto stencil = [&](int q, int i, int j, int k, double &s, double &d) {
-        const L &l = v[q];
-        const MgGeom &G = g[q];
-        const int st[3] = {1, l.E, l.E * l.E}, a[3] = {i, j, k}, p = id(l, i, j, k);
-        s = d = 0.0;
-        for (int x = 0; x < dim; x++) {
-            const bool lo = a[x] == 1, hi = a[x] == l.N;
-            d += mg_axis_diag((lo ? 1 : 0) | (hi ? 2 : 0), G);
-            if (!lo && !(hi && G.tie && l.N >= 2))
-                s += l.phi[p - st[x]];
-            if (!hi)
-                s += l.phi[p + st[x]];
-        }
-    };
-    auto smooth = [&](int q, int sweeps) {
-        for (int sw = 0; sw < (v[q].N == 1 && sweeps > 0 ? 1 : sweeps); sw++)
-            for (int c = 0; c < 2; c++)
-                cells(v[q], [&](int i, int j, int k) {
-                    if (((i + j + k) & 1) != c)
-                        return;
-                    double s, d;
-                    stencil(q, i, j, k, s, d);
-                    const int p = id(v[q], i, j, k);
-                    v[q].phi[p] = (s - v[q].f[p]) / -d;
-                });
-    };
-    auto ghost = [&](int q, int I, double &c) {   // coarse index with ghosts -> active index, factor
-        const int N = v[q].N;
+    auto cells = [&](int q) { return (dim == 3 ? g[q].N : 1) * g[q].N * g[q].N; };
+    const int n0 = cells(0), corners = 1 << dim;
+    // coarse index with ghosts -> active index, factor
+    auto ghost = [&](int q, int I, double &c) {
+        const int N = g[q].N;
         c = 1.0;
         if (I >= 1 && I <= N)
             return I;
@@ -1819,49 +1788,102 @@ void mg_slab_dense(int dim, const MgGeom *g, int nlev, int nu_pre, int nu_post, 
         c = g[q].cR;
         return N;
     };
-    const int N0 = v[0].N, n0 = dim == 3 ? N0 * N0 * N0 : N0 * N0;
-    for (int col = 0; col < n0; col++) {
-        std::fill(v[0].phi.begin(), v[0].phi.end(), 0.0);
-        std::fill(v[0].f.begin(), v[0].f.end(), 0.0);
-        v[0].f[id(v[0], 1 + col % N0, 1 + (col / N0) % N0, dim == 3 ? 1 + col / (N0 * N0) : 0)] = 1.0;
-        smooth(0, nu_pre);
-        for (int q = 0; q + 1 < nlev; q++) {
-            L &c = v[q + 1];
-            std::fill(c.phi.begin(), c.phi.end(), 0.0);
-            std::fill(c.f.begin(), c.f.end(), 0.0);
-            cells(v[q], [&](int i, int j, int k) {   // h_c^2 = 4 h_f^2, 2^-d average
-                const int I = (i + 1) / 2, J = (j + 1) / 2, K = (k + 1) / 2;
-                if (I > c.N || J > c.N || K > c.N)
-                    return;
-                double s, d;
-                stencil(q, i, j, k, s, d);
-                const int p = id(v[q], i, j, k);
-                c.f[id(c, I, J, K)] += (dim == 3 ? 0.5 : 1.0) * (v[q].f[p] - s - d * v[q].phi[p]);
-            });
-            smooth(q + 1, nu_pre);
-        }
-        for (int q = nlev - 2; q >= 0; q--) {
-            cells(v[q], [&](int i, int j, int k) {
-                double e = 0.0;
-                for (int m = 0; m < (1 << dim); m++) {
-                    double w = 1.0;
-                    int at[3] = {0, 0, 0};
-                    const int a[3] = {i, j, k};
-                    for (int x = 0; x < dim; x++) {
-                        const int near = (a[x] + 1) / 2, far = near + (a[x] & 1 ? -1 : 1);
-                        double c;
-                        at[x] = ghost(q + 1, (m >> x) & 1 ? far : near, c);
-                        w *= c * ((m >> x) & 1 ? 0.25 : 0.75);
-                    }
-                    e += w * v[q + 1].phi[id(v[q + 1], at[0], at[1], at[2])];
+    std::vector<Level> lev(nlev);
+    for (int q = 0; q < nlev; q++) {
+        Level &l = lev[q];
+        const int N = g[q].N, Nc = q + 1 < nlev ? g[q + 1].N : 0;
+        l.cell.resize(cells(q));
+        l.phi.assign((size_t)cells(q) * n0, 0.0);
+        l.f.assign((size_t)cells(q) * n0, 0.0);
+        for (int t = 0; t < cells(q); t++) {
+            Cell &c = l.cell[t];
+            const int a[3] = {t % N + 1, t / N % N + 1, dim == 3 ? t / (N * N) + 1 : 0}, st[3] = {1, N, N * N};
+            c.colour = (a[0] + a[1] + a[2]) & 1;
+            c.nn = 0;
+            c.d = 0.0;
+            for (int x = 0; x < dim; x++) {
+                const bool lo = a[x] == 1, hi = a[x] == N;
+                c.d += mg_axis_diag((lo ? 1 : 0) | (hi ? 2 : 0), g[q]);
+                if (!lo && !(hi && g[q].tie && N >= 2))
+                    c.nb[c.nn++] = t - st[x];
+                if (!hi)
+                    c.nb[c.nn++] = t + st[x];
+            }
+            c.parent = -1;
+            if (!Nc)
+                continue;
+            const int P[3] = {(a[0] + 1) / 2, (a[1] + 1) / 2, (a[2] + 1) / 2};
+            if (P[0] <= Nc && P[1] <= Nc && P[2] <= Nc)
+                c.parent = (dim == 3 ? (P[2] - 1) * Nc * Nc : 0) + (P[1] - 1) * Nc + P[0] - 1;
+            for (int m = 0; m < corners; m++) {
+                c.w[m] = 1.0;
+                int at[3] = {1, 1, 1};
+                for (int x = 0; x < dim; x++) {
+                    const int near = (a[x] + 1) / 2, far = near + (a[x] & 1 ? -1 : 1);
+                    double k;
+                    at[x] = ghost(q + 1, (m >> x) & 1 ? far : near, k);
+                    c.w[m] *= k * ((m >> x) & 1 ? 0.25 : 0.75);
                 }
-                v[q].phi[id(v[q], i, j, k)] += e;
-            });
-            smooth(q, nu_post);
+                c.at[m] = (at[2] - 1) * Nc * Nc + (at[1] - 1) * Nc + at[0] - 1;
+            }
         }
-        int row = 0;
-        cells(v[0], [&](int i, int j, int k) { mat[(size_t)col * n0 + row++] = v[0].phi[id(v[0], i, j, k)]; });
     }
+    std::vector<double> sum(n0);
+    auto neighbours = [&](const Level &l, const Cell &c) {
+        std::fill(sum.begin(), sum.end(), 0.0);
+        for (int e = 0; e < c.nn; e++) {
+            const double *v = &l.phi[(size_t)c.nb[e] * n0];
+            for (int k = 0; k < n0; k++)
+                sum[k] += v[k];
+        }
+    };
+    auto smooth = [&](int q, int sweeps) {
+        Level &l = lev[q];
+        for (int sw = 0; sw < (g[q].N == 1 && sweeps > 0 ? 1 : sweeps); sw++)
+            for (int colour = 0; colour < 2; colour++)
+                for (size_t t = 0; t < l.cell.size(); t++) {
+                    const Cell &c = l.cell[t];
+                    if (c.colour != colour)
+                        continue;
+                    neighbours(l, c);
+                    for (int k = 0; k < n0; k++)
+                        l.phi[t * n0 + k] = (sum[k] - l.f[t * n0 + k]) / -c.d;
+                }
+    };
+    for (int k = 0; k < n0; k++)
+        lev[0].f[(size_t)k * n0 + k] = 1.0;
+    smooth(0, nu_pre);
+    for (int q = 0; q + 1 < nlev; q++) {
+        Level &l = lev[q];
+        for (size_t t = 0; t < l.cell.size(); t++) {   // h_c^2 = 4 h_f^2, 2^-d average
+            const Cell &c = l.cell[t];
+            if (c.parent < 0)
+                continue;
+            neighbours(l, c);
+            double *fc = &lev[q + 1].f[(size_t)c.parent * n0];
+            for (int k = 0; k < n0; k++)
+                fc[k] += (dim == 3 ? 0.5 : 1.0) * (l.f[t * n0 + k] - sum[k] - c.d * l.phi[t * n0 + k]);
+        }
+        smooth(q + 1, nu_pre);
+    }
+    for (int q = nlev - 2; q >= 0; q--) {
+        Level &l = lev[q];
+        for (size_t t = 0; t < l.cell.size(); t++) {
+            const Cell &c = l.cell[t];
+            std::fill(sum.begin(), sum.end(), 0.0);
+            for (int m = 0; m < corners; m++) {
+                const double *v = &lev[q + 1].phi[(size_t)c.at[m] * n0];
+                for (int k = 0; k < n0; k++)
+                    sum[k] += c.w[m] * v[k];
+            }
+            for (int k = 0; k < n0; k++)
+                l.phi[t * n0 + k] += sum[k];
+        }
+        smooth(q, nu_post);
+    }
+    for (int t = 0; t < n0; t++)
+        for (int k = 0; k < n0; k++)
+            mat[(size_t)k * n0 + t] = lev[0].phi[(size_t)t * n0 + k];
 }
 
 size_t mg_slab_image_bytes(const MgSlabPlan &p) { return (size_t)p.csize * p.words * kT * sizeof(int); }

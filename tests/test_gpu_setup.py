@@ -83,3 +83,26 @@ def test_layout_change_after_a_solve_clears_the_arrays(mg, monkeypatch):  # noqa
                 assert np.max(np.abs(a - b)) <= 1e-10 * np.max(np.abs(b))
     finally:
         mg.mg_destroy(h)
+
+
+def test_creation_with_the_slab_kernel_costs_little_more_than_without(mg, monkeypatch):  # noqa: F811
+    """Three levels of three sizes: the slab kernel's plans (a matrix of 64
+    columns on the host, a launch and a copy per size, no allocation, no wait)
+    in place of the one-block kernel's (a launch and a wait per level).  With an
+    allocation and two waits per size, and both plans, it took twice the time."""
+    H = I.Hierarchy(3, [30, 28, 26], [(-0.5,) * 3, (-0.5 + 8 / 30,) * 3, (-0.5 + 12 / 30,) * 3], 1.0 / 30, 1.0, [], "abc")
+
+    def create_ms():
+        t = []
+        for _ in range(25):
+            t0 = time.perf_counter()
+            h = mg.mg_create_hierarchy([mg.desc_from(H)], mg.options())
+            t.append(1e3 * (time.perf_counter() - t0))
+            mg.mg_destroy(h)
+        return sorted(t)[12]
+
+    monkeypatch.setenv("MG_BOTTOM_N64", "8")
+    create_ms()
+    without = create_ms()
+    monkeypatch.delenv("MG_BOTTOM_N64")
+    assert create_ms() < 1.5 * without
