@@ -734,20 +734,13 @@ cudaError_t refresh_bottom_plan(mg_hierarchy *h, LevelData &ld)
 void layout_slab(const mg_hierarchy *h, LevelData &ld)
 {
     const bool fp32 = h->opt.precision == MG_MIXED;
-    const int lim = slab_limit(h->dim), nb = h->batch;
-    // Batches: graph branches of several hierarchies share the SMs, which small
-    // launches of all of them fill better than clusters of 16, of which nine run at
-    // once.  Mixed: none (32 uneven hierarchies: 40 ms against 47 ms).  FP64, without
-    // -> with the slab kernel: levels that it solves whole gain in every batch (three
-    // levels of 16^3, 4 / 32 hierarchies, 4.0 -> 1.6 and 13.3 -> 6.6 ms; 64^2 1.37 ->
-    // 0.52 and 4.1 -> 2.4); as the coarse part of larger levels it gains in small
-    // batches (2D 256^2, 2 / 4 / 8: 1.41 -> 1.08, 1.51 -> 1.34, 1.68 -> 2.24; 3D 64^3, 2 /
-    // 4 / 8: 5.61 -> 5.72, 7.7 -> 9.9, 10.9 -> 14.8; 32^3, 2 / 8 / 16: 4.2 -> 2.8, 6.1 -> 5.8,
-    // 10.3 -> 11.0).
-    if (h->ssize <= 0 || (fp32 && nb > 1))
+    const int lim = slab_limit(h->dim);
+    // mixed batches: graph branches of several hierarchies share the SMs, which
+    // small launches of all of them fill better than clusters of 16 (batch of 32
+    // uneven hierarchies: 40 ms against 47 ms)
+    if (h->ssize <= 0 || (fp32 && h->batch > 1))
         return;
-    const bool coarse = nb <= 2 || (h->dim == 2 ? nb <= 4 : nb <= 8 && ld.g[0].N <= 40);
-    for (int L = 0; L + 1 < ld.nmg && ld.slab_first < 0 && (L == 0 || coarse); L++)
+    for (int L = 0; L + 1 < ld.nmg && ld.slab_first < 0; L++)
         if (ld.g[L].N <= lim && mg_slab_layout(h->dim, fp32, h->ssize, &ld.g[L], ld.nmg - L, slab_cut(h->dim),
                                                h->opt.nu_pre, h->opt.nu_post, ld.slab))
             ld.slab_first = L;

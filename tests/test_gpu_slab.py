@@ -207,31 +207,3 @@ def test_slab_wait_timeout_reports_etimeout(mg, monkeypatch, dim, n, prec, solve
     monkeypatch.delenv("MG_FAULT_SLAB_WAIT")
     _, after = gpu_solve(mg, H, inp, **kw)
     assert np.array_equal(before[0]["phi"], after[0]["phi"])
-
-
-@pytest.mark.parametrize("dim,edges,count", [(3, (14, 30, 62), 3), (3, (14, 30, 62), 9), (2, (30, 254), 2), (2, (30, 254), 6)])
-def test_fp64_batch_equals_single_solves(mg, dim, edges, count):  # noqa: F811
-    """Batches on both sides of the sizes from which the slab kernel runs: whole
-    levels always, the coarse part of larger ones in small batches.  Cycles and
-    potentials of each hierarchy solved alone (the parity bar of the FP64 path)."""
-    import torch
-    Hs = [random_single_level(dim, edges[b % len(edges)], 7 * b + dim) for b in range(count)]
-    kw = dict(max_cycles=30, rel_tol=1e-9)
-    h = mg.mg_create_hierarchy([mg.desc_from(H) for H, _ in Hs], mg.options(**kw))
-    try:
-        dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
-        for b, (_, inp) in enumerate(Hs):
-            mg.mg_set_density(h, b, 0, dev(inp[0]["rho"]), dev(inp[0]["bc_rho"]), dev(inp[0]["bc_phi"]))
-        _, st = mg.mg_solve(h, count)
-        got = []
-        for b, (H, _) in enumerate(Hs):
-            phi = torch.zeros((H.n[0],) * dim, dtype=torch.float64, device="cuda")
-            mg.mg_forces(h, b, 0, phi, None)
-            torch.cuda.synchronize()
-            got.append(phi.cpu().numpy())
-    finally:
-        mg.mg_destroy(h)
-    for b, (H, inp) in enumerate(Hs):
-        _, one = gpu_solve(mg, H, inp, **kw)
-        assert st[b][0]["cycles"] == one[0]["cycles"]
-        assert relmax(got[b], one[0]["phi"]) < 1e-12
