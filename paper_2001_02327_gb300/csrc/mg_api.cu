@@ -735,9 +735,16 @@ void layout_slab(const mg_hierarchy *h, LevelData &ld)
 {
     const bool fp32 = h->opt.precision == MG_MIXED;
     const int lim = slab_limit(h->dim);
-    // mixed batches: graph branches of several hierarchies share the SMs, which
-    // small launches of all of them fill better than clusters of 16 (batch of 32
-    // uneven hierarchies: 40 ms against 47 ms)
+    // Batches: graph branches of several hierarchies share the SMs, which small
+    // launches of all of them fill better than clusters of 16, of which nine run at
+    // once.  Mixed: none (32 uneven hierarchies: 40 ms against 47 ms).  FP64: as
+    // alone, so that a hierarchy's result does not depend, in any bit, on the batch
+    // it is in.  There levels that the kernel solves whole gain (three levels of
+    // 16^3, 4 / 32 hierarchies, without -> with: 4.0 -> 1.6 and 13.3 -> 6.6 ms; 64^2 1.37
+    // -> 0.52 and 4.1 -> 2.4), the coarse part of larger ones gains in batches of two
+    // to four and loses in larger ones (32 uneven hierarchies of 16 to 32 cells 16.5
+    // -> 14.4 ms, of 32 to 128 86 -> 102; 8 of 64^3 10.9 -> 14.8; 8 / 32 of 256^2 1.68 ->
+    // 2.24 and 4.7 -> 7.2).
     if (h->ssize <= 0 || (fp32 && h->batch > 1))
         return;
     for (int L = 0; L + 1 < ld.nmg && ld.slab_first < 0; L++)
@@ -1544,9 +1551,10 @@ bool persist_eligible(const mg_hierarchy *h)
 // cells at 1.5e9 per second; a block of the persistent launch, one per SM,
 // largest hierarchy first, takes 1.9 times a hierarchy's node time plus its
 // cells at 2e7 per second.  The whole batch goes to the persistent launch when
-// that estimate is the shorter.  Measured, persistent / branches: 32, 64 and
-// 512 hierarchies of 16 to 32 cells per edge 6.9 / 10.4, 7.5 / 20.9 and 23.9 /
-// 142 ms, 256 of 32 to 48 28 / 94 ms, 24 of 32 to 128 168 / 20.9 ms.  Run beside
+// that estimate is the shorter.  Measured, persistent / branches (densities
+// handed over and solved): 32, 64, 256 and 512 hierarchies of 16 to 32 cells per
+// edge 6.8 / 10.9, 8.1 / 18.9, 13.0 / 69 and 25 / 144 ms, 256 of 32 to 48 26.5 / 92
+// ms, 24 of 32 to 128 170 / 24.3 ms.  Run beside
 // graph branches it takes SMs and bandwidth from them (a split of a batch of
 // 512 of 32 to 128 took 707 ms against 642 ms with graph branches only).
 // MG_PERSIST=1 / 0 forces all / none (the batched kernels, MG_BATCHED=1, exclude

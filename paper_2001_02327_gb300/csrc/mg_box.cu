@@ -1120,18 +1120,21 @@ __global__ void __launch_bounds__(256) kx_zero_gamma(PatchDims d, int dim, doubl
         phi[t] = 0.0;
 }
 
-// F = -grad Phi on Omega (Eq. 2: 4/3 of the centred difference over 2h minus
-// 1/3 of the one over 4h, i2h = 1/(2h), i4h = 1/(4h); stencil 1: the
-// two-point centred difference), and the potential on Omega.  Component a at
-// F[a * cells + cell].
-__global__ void __launch_bounds__(256, kMarchForce) kx_forces_march(PatchDims d, double c, const double *__restrict__ phi, MarchGrid m,
-                                                          double *__restrict__ F, double *__restrict__ phi_out,
-                                                          int stencil)
+// The forces of kx_forces for large 3D patches (mg_march.cuh); c = -1 / (12 h)
+// or, stencil 1, -1 / (2 h).
+__global__ void __launch_bounds__(256, kMarchForce) kx_forces_march(PatchDims d, double c,
+                                                                   const double *__restrict__ phi, MarchGrid m,
+                                                                   double *__restrict__ F, double *__restrict__ phi_out,
+                                                                   int stencil)
 {
     pdl_begin();
     MarchForces fn{phi, m.sy, m.sz, (long long)d.n[0] * d.n[1] * d.n[2], d.n[0], d.n[1], stencil, c, F, phi_out, 0.0};
     march<2, 6, true>(phi, m, fn);
 }
+// F = -grad Phi on Omega (Eq. 2: 4/3 of the centred difference over 2h minus
+// 1/3 of the one over 4h, i2h = 1/(2h), i4h = 1/(4h); stencil 1: the
+// two-point centred difference), and the potential on Omega.  Component a at
+// F[a * cells + cell].
 __global__ void __launch_bounds__(256) kx_forces(PatchDims d, int dim, double i2h, double i4h,
                                                  const double *__restrict__ phi, double *__restrict__ F,
                                                  double *__restrict__ phi_out, int stencil)

@@ -37,7 +37,7 @@
 //     three 16^3 levels 2.05 -> 1.28 ms, of three 64^2 levels 1.35 -> 0.90 ms
 //     (one launch per phase: 2.73 and 2.34 ms).
 //
-// One V-cycle, launch to launch: 33^3 31 us in FP32 and 47 us in FP64, 17^3 15
+// One V-cycle, launch to launch: 33^3 31 us in FP32 and 48 us in FP64, 17^3 15
 // us (FP32), 18^3 30 us and 66^2 28 us (FP64).
 //
 // FP64 V-cycles run in 64-bit fixed point.  The part issues one FP64

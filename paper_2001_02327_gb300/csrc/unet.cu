@@ -827,16 +827,16 @@ __global__ void __launch_bounds__(256) k_grad_prep(float *__restrict__ d, const 
 }
 
 // ---------------------------------------------------------------------------
-// The same convolution from a TMA-loaded halo: a tile of 8 (x) x 16 (y) x 1
-// (z) voxels of one sample; one TMA box per 8 input channels brings the
-// 10 x 18 x 3 voxels around it (zero outside the grid) into shared memory as
-// 16-byte rows, x fastest.  Tap (dz, dy, dx) is then the 128 x CK operand
-// whose row (x, y) is halo row ((dz+1) 18 + y + dy + 1) 10 + x + dx + 1: a
-// descriptor at that start with 8-row groups one halo row (160 B) apart
-// (SBO) and the channel chunks one chunk apart (LBO) -- no copy per tap.
-// All 27 taps' weights (N x CK each) come in by cp.async from every thread,
-// N rows of 16 B per chunk.  One thread issues the TMA and every MMA; the
-// block waits once for the accumulator.
+// The same convolution from a halo in shared memory: a tile of 8 (x) x 16 (y)
+// voxels of one plane of one sample with the 10 x 18 x 3 voxels around it (zero
+// outside the grid), per 8 input channels a chunk of 16-byte rows, x fastest.
+// Tap (dz, dy, dx) is then the 128 x CK operand whose row (x, y) is halo row
+// ((dz+1) 18 + y + dy + 1) 10 + x + dx + 1: a descriptor at that start with
+// 8-row groups one halo row (160 B) apart (SBO) and the channel chunks one
+// chunk apart (LBO) -- no copy per tap.  One thread issues every MMA.
+// k_conv3_halo takes up to four planes per block and copies halo and weights by
+// cp.async; k_conv3_halo_p, the persistent form, loads its halos with one TMA
+// box per 8 channels.
 // ---------------------------------------------------------------------------
 constexpr int kHaloRows = 10 * 18 * 3;                 // 540 rows of one channel chunk
 constexpr int kHaloChunk = (kHaloRows * 16 + 127) / 128 * 128;   // 8704 B, 128-byte aligned chunks
