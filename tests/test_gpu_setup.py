@@ -41,10 +41,10 @@ def test_first_solve_of_a_persistent_batch_costs_little_more_than_the_next(mg): 
         try:
             first.append(_solve_ms(mg, h, count))
             assert mg.mg_persistent_count(h) == count
-            later.append(_solve_ms(mg, h, count))
+            later.append(min(_solve_ms(mg, h, count) for _ in range(2)))
         finally:
             mg.mg_destroy(h)
-    assert sorted(first)[1] < 2.0 * sorted(later)[1]
+    assert min(first) < 2.0 * min(later)
 
 
 def test_layout_change_after_a_solve_clears_the_arrays(mg, monkeypatch):  # noqa: F811
@@ -92,17 +92,16 @@ def test_creation_with_the_slab_kernel_costs_little_more_than_without(mg, monkey
     allocation and two waits per size, and both plans, it took twice the time."""
     H = I.Hierarchy(3, [30, 28, 26], [(-0.5,) * 3, (-0.5 + 8 / 30,) * 3, (-0.5 + 12 / 30,) * 3], 1.0 / 30, 1.0, [], "abc")
 
-    def create_ms():
-        t = []
-        for _ in range(25):
-            t0 = time.perf_counter()
-            h = mg.mg_create_hierarchy([mg.desc_from(H)], mg.options())
-            t.append(1e3 * (time.perf_counter() - t0))
-            mg.mg_destroy(h)
-        return sorted(t)[12]
+    def create_ms(env):
+        if env:
+            monkeypatch.setenv("MG_BOTTOM_N64", "8")
+        else:
+            monkeypatch.delenv("MG_BOTTOM_N64", raising=False)
+        t0 = time.perf_counter()
+        h = mg.mg_create_hierarchy([mg.desc_from(H)], mg.options())
+        t = 1e3 * (time.perf_counter() - t0)
+        mg.mg_destroy(h)
+        return t
 
-    monkeypatch.setenv("MG_BOTTOM_N64", "8")
-    create_ms()
-    without = create_ms()
-    monkeypatch.delenv("MG_BOTTOM_N64")
-    assert create_ms() < 1.5 * without
+    pairs = [(create_ms(True), create_ms(False)) for _ in range(30)]   # in turn, the quickest of each
+    assert min(b for _, b in pairs) < 1.5 * min(a for a, _ in pairs)
