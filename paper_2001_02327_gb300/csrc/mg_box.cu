@@ -907,7 +907,7 @@ struct BoxIndex {
         return ((i + j + k) & 1) * half + ((long long)k * E1 + j) * H + (i >> 1);
     }
 };
-__global__ void __launch_bounds__(256, kMarchResid) kx_norm_march(const double *__restrict__ phi, const double *__restrict__ f,
+__global__ void __launch_bounds__(256, 5) kx_norm_march(const double *__restrict__ phi, const double *__restrict__ f,
                                                         BoxGeom g, MarchGrid m, double *__restrict__ part,
                                                         float *__restrict__ f32, float *__restrict__ e32)
 {
@@ -1122,7 +1122,7 @@ __global__ void __launch_bounds__(256) kx_zero_gamma(PatchDims d, int dim, doubl
 
 // The forces of kx_forces for large 3D patches (mg_march.cuh); c = -1 / (12 h)
 // or, stencil 1, -1 / (2 h).
-__global__ void __launch_bounds__(256, kMarchForce) kx_forces_march(PatchDims d, double c,
+__global__ void __launch_bounds__(256, 4) kx_forces_march(PatchDims d, double c,
                                                                    const double *__restrict__ phi, MarchGrid m,
                                                                    double *__restrict__ F, double *__restrict__ phi_out,
                                                                    int stencil)
@@ -1541,7 +1541,7 @@ cudaError_t resid_norm(const mg_box *b, const BoxPatch &P, int zero_inside, bool
     int mblocks = 0;
     MarchGrid m{};
     if (b->dim == 3 && !zero_inside && march_fits(l.g.N))
-        m = march_grid(l.g.N[0], l.g.N[1], l.g.N[2], l.g.E[0], (long long)l.g.E[0] * l.g.E[1], 1, kMarchResid, &mblocks);
+        m = march_grid(l.g.N[0], l.g.N[1], l.g.N[2], l.g.E[0], (long long)l.g.E[0] * l.g.E[1], 1, &mblocks);
     if (mblocks > 0 && mblocks <= MG_MARCH_BLOCKS) {
         blocks = mblocks;
         mg_launch_kernel(kx_norm_march, dim3(blocks), dim3(256), 0, s, (const double *)l.phi64, (const double *)l.f64,
@@ -2103,7 +2103,7 @@ mg_status mg_box_forces(mg_box *b, int patch, double *phi_out, double *F_out)
     if (dim == 3 && march_fits(P.n)) {
         int blocks = 0;
         const MarchGrid m =
-            march_grid(P.n[0], P.n[1], P.n[2], P.d.B[0], (long long)P.d.B[0] * P.d.B[1], 2, kMarchForce, &blocks);
+            march_grid(P.n[0], P.n[1], P.n[2], P.d.B[0], (long long)P.d.B[0] * P.d.B[1], 2, &blocks);
         mg_launch_kernel(kx_forces_march, dim3(blocks), dim3(256), 0, b->stream, P.d,
                          -1.0 / ((b->opt.force_stencil == 0 ? 12.0 : 2.0) * P.h), (const double *)P.phi, m, dF, dP,
                          b->opt.force_stencil);

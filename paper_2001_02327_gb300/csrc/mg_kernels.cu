@@ -1639,7 +1639,7 @@ struct SplitIndex {
     MgGeom g;
     __device__ __forceinline__ long long operator()(int i, int j, int k) const { return mg_idx32(g, 3, i, j, k); }
 };
-__global__ void __launch_bounds__(256, kMarchResid) k_norms_march(const double *__restrict__ phi, const double *__restrict__ f,
+__global__ void __launch_bounds__(256, 5) k_norms_march(const double *__restrict__ phi, const double *__restrict__ f,
                                                         MgGeom g, MarchGrid m, int which,
                                                         double *__restrict__ partials, unsigned *__restrict__ counter,
                                                         double *__restrict__ out2, float *__restrict__ r32,
@@ -2049,7 +2049,7 @@ __global__ void __launch_bounds__(kThreads) k_forces(int n, double h, const doub
 // The same for large 3D levels (mg_march.cuh): 500 us at 256^3 with FP64
 // instructions, 275 us with integer sums per cell, 205 us here (cold caches); the
 // bytes take 100 us.
-__global__ void __launch_bounds__(256, kMarchForce) k_forces_march(int n, double c, const double *__restrict__ phi, MarchGrid m,
+__global__ void __launch_bounds__(256, 4) k_forces_march(int n, double c, const double *__restrict__ phi, MarchGrid m,
                                                          double *__restrict__ F, double *__restrict__ phi_out,
                                                          int stencil)
 {
@@ -3224,7 +3224,7 @@ cudaError_t mg_launch_norms2(int dim, const double *phi, const double *f, const 
 {
     if (dim == 3 && g.N >= kMarchMinN && (which & 2)) {
         int blocks = 0;
-        const MarchGrid m = march_grid(g.N, g.N, g.N, g.E, (long long)g.E * g.E, 1, kMarchResid, &blocks);
+        const MarchGrid m = march_grid(g.N, g.N, g.N, g.E, (long long)g.E * g.E, 1, &blocks);
         if (blocks <= MG_MARCH_BLOCKS) {
             mg_launch_kernel(k_norms_march, blocks, 256, 0, s, phi, f, g, m, which, partials, counter, out2, r32, e32);
             return cudaGetLastError();
@@ -3322,7 +3322,7 @@ cudaError_t mg_launch_forces(int dim, int n, double h, const double *phi_blk, do
     if (dim == 3 && n >= kMarchMinN) {
         int blocks = 0;
         const int E = n + 4;
-        const MarchGrid m = march_grid(n, n, n, E, (long long)E * E, 2, kMarchForce, &blocks);
+        const MarchGrid m = march_grid(n, n, n, E, (long long)E * E, 2, &blocks);
         mg_launch_kernel(k_forces_march, blocks, 256, 0, s, n, -1.0 / ((stencil == 0 ? 12.0 : 2.0) * h), phi_blk, m, F,
                          phi_out, stencil);
         return cudaGetLastError();

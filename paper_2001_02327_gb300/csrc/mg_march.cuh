@@ -20,9 +20,6 @@
 
 #include "mg_fix.cuh"
 
-// resident blocks per SM that the kernels ask for: residuals, forces (registers)
-constexpr int kMarchResid = 5, kMarchForce = 4;
-
 struct MarchGrid {
     int n[3];         // active cells per axis; storage extents are n + 2 R
     int nx, ny, zc;   // tiles along x and y, planes per block
@@ -31,12 +28,9 @@ struct MarchGrid {
 };
 
 // Tiles and z ranges: of the splits with at least 8 planes a block and at most
-// MG_MARCH_BLOCKS blocks, the one whose waves of 152 x per_sm resident blocks march
-// the fewest planes in all (each block also loads 2 R planes around its own).
-// Forces with 4 instead of 5 counted (they have 4): 128^3 34.3 -> 33.7 us, 160^3
-// 61.0 -> 56.8, 192^3 97.4 -> 96.8, 256^3 208.8 -> 204.1, 112^3 26.7 -> 27.7, 144^3 49.7
-// -> 51.0 (mg_forces).
-inline MarchGrid march_grid(int n0, int n1, int n2, long long sy, long long sz, int R, int per_sm, int *blocks)
+// MG_MARCH_BLOCKS blocks, the one whose waves of 152 x 5 resident blocks march the
+// fewest planes in all (each block also loads 2 R planes around its own).
+inline MarchGrid march_grid(int n0, int n1, int n2, long long sy, long long sz, int R, int *blocks)
 {
     MarchGrid m;
     m.n[0] = n0;
@@ -51,7 +45,7 @@ inline MarchGrid march_grid(int n0, int n1, int n2, long long sy, long long sz, 
     long best = 0;
     for (int c = 1; c == 1 || (c * 8 <= n2 && (long)tiles * c <= MG_MARCH_BLOCKS); c++) {
         const int zc = (n2 + c - 1) / c;
-        const long wave = 152L * per_sm, cost = ((tiles * c + wave - 1) / wave) * (zc + 2 * R);
+        const long cost = (((long)tiles * c + 759) / 760) * (zc + 2 * R);
         if (best == 0 || cost < best) {
             best = cost;
             m.zc = zc;
