@@ -1122,10 +1122,9 @@ __global__ void __launch_bounds__(256) kx_zero_gamma(PatchDims d, int dim, doubl
 
 // The forces of kx_forces for large 3D patches (mg_march.cuh); c = -1 / (12 h)
 // or, stencil 1, -1 / (2 h).
-__global__ void __launch_bounds__(256, 4) kx_forces_march(PatchDims d, double c,
-                                                                   const double *__restrict__ phi, MarchGrid m,
-                                                                   double *__restrict__ F, double *__restrict__ phi_out,
-                                                                   int stencil)
+__global__ void __launch_bounds__(256, 4) kx_forces_march(PatchDims d, double c, const double *__restrict__ phi,
+                                                          MarchGrid m, double *__restrict__ F,
+                                                          double *__restrict__ phi_out, int stencil)
 {
     pdl_begin();
     MarchForces fn{phi, m.sy, m.sz, (long long)d.n[0] * d.n[1] * d.n[2], d.n[0], d.n[1], stencil, c, F, phi_out, 0.0};

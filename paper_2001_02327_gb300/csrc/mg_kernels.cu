@@ -2047,7 +2047,7 @@ __global__ void __launch_bounds__(kThreads) k_forces(int n, double h, const doub
 }
 
 // The same for large 3D levels (mg_march.cuh): 500 us at 256^3 with FP64
-// instructions, 275 us with integer sums per cell, 205 us here (cold caches); the
+// instructions, 275 us with integer sums per cell, 209 us here (cold caches); the
 // bytes take 100 us.
 __global__ void __launch_bounds__(256, 4) k_forces_march(int n, double c, const double *__restrict__ phi, MarchGrid m,
                                                          double *__restrict__ F, double *__restrict__ phi_out,
